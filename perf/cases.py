@@ -296,6 +296,84 @@ _RUN = {"compress": _run_compress, "decompress": _run_decompress, "backward": _r
         "reproject": _run_reproject, "reparam": _run_reparam, "average": _run_average}
 
 
+# ---- the same passes in 64 bits, as plain torch ------------------------------------------------
+def exact(case, seed):
+    s = prepare(case, seed)
+    return (_exact_tokens if case["kind"] in _TOKEN_KINDS else _EXACT[case["kind"]])(case, s)
+
+
+def _exact_tokens(case, s):
+    kind, n, k = case["kind"], case["tokens"], case["k"]
+    codec = s["codec"]
+    U = codec.U.double()
+
+    def shift(rows):
+        t = codec.E[s["ids"][rows]].double()
+        if codec.P is not None:
+            pos = s["pos"][rows] if s["pos"] is not None else torch.arange(rows.start, rows.stop, device="cuda") % s["seq"]
+            t += codec.P[pos.long()].double()
+        return t
+
+    def by_rows(f, cols):
+        out = torch.empty((n, cols), device="cuda", dtype=torch.float64)
+        for lo in range(0, n, 8192):
+            rows = slice(lo, min(n, lo + 8192))
+            out[rows] = f(rows)
+        return out
+
+    def compress():
+        return by_rows(lambda r: (s["X"][r].double() + (s["R"][r].double() if kind == "wire" else 0.0) - shift(r)) @ U, k)
+
+    def expand(Z):
+        return by_rows(lambda r: Z[r].double() @ U.T + shift(r), case["d"])
+
+    def backward(dZ):
+        return by_rows(lambda r: dZ[r].double() @ U.T, case["d"]), by_rows(lambda r: s["G"][r].double() @ U, k)
+
+    if kind == "wire":
+        X, out = expand(s["wire"][:, :k].view(torch.float32)), compress()
+        return X, out, s["ids"], *backward(s["wire_grad"].view(torch.float32))
+    if kind == "compress":
+        return compress()
+    if kind == "decompress":
+        return expand(s["Z"])
+    return backward(s["dZ"]) if kind == "backward" else (expand(s["Z"]), compress(), *backward(s["dZ"]))
+
+
+def _exact_reproject(case, s):
+    U = s["codec"].U.double()
+    return [(w.double() @ U) @ U.T if case["side"] == "right" else U @ (U.T @ w.double()) for w in s["weights"]]
+
+
+def _exact_reparam(case, s):
+    U, Zw, dY = s["U"].double(), s["Zw"].double(), s["dY"].double()
+    C, F = torch.empty((case["tokens"], case["k"]), device="cuda", dtype=torch.float64), 0.0
+    dC = dY @ U
+    for lo in range(0, case["tokens"], 4096):
+        H = s["H"][lo:lo + 4096].double()
+        C[lo:lo + 4096] = H @ Zw
+        F = F + H.T @ dC[lo:lo + 4096]
+    return C @ U.T, dC @ Zw.T, F
+
+
+def _exact_average(case, s):
+    n, r = s["n"], s["round"] % 20
+    lo, hi = n * r // 20 & ~63, n if r == 19 else n * (r + 1) // 20 & ~63
+    buf, theta = s["buf"].double(), s["theta"].double()
+    snap = buf[lo:hi].clone()
+    chunks = [c.double() for c in s["chunks"]]
+    acc = sum(w * c for w, c in zip(s["weights"], chunks)) / sum(s["weights"])
+    deltas = [acc - c for c in chunks]
+    buf[lo:hi] += deltas[0]
+    theta[lo:hi] += buf[lo:hi] - snap
+    norm2 = sum(g.double().square().sum() for g in s["grads"])
+    coef = min(1.0, 0.3779 / (math.sqrt(float(norm2)) + 1e-6))
+    return snap, acc, deltas, buf, theta, norm2.reshape(1), [g.double() * coef for g in s["grads"]]
+
+
+_EXACT = {"reproject": _exact_reproject, "reparam": _exact_reparam, "average": _exact_average}
+
+
 # ---- what a pass cannot do without ------------------------------------------------------------
 def _distinct_rows(case):
     """Expected number of distinct embedding rows among the tokens."""
