@@ -402,14 +402,18 @@ enum {
   SSN_KERNEL_UMMA_PROJECT = 5,     /* tcgen05 + TMA projection                                 */
   SSN_KERNEL_UMMA_EXPAND = 6,      /* tcgen05 + TMA expansion                                  */
   SSN_KERNEL_UMMA_ROUNDTRIP = 7,   /* tcgen05 + TMA project-then-expand                        */
-  SSN_KERNEL_UMMA_TOKENS = 8       /* tcgen05 + TMA contraction over tokens                    */
+  SSN_KERNEL_UMMA_TOKENS = 8,      /* tcgen05 + TMA contraction over tokens                    */
+  SSN_KERNEL_SPLIT_PROJECT = 9,    /* tcgen05 projection, operands split into bf16 parts: fp32 and
+                                      the bf16 calls TMA cannot fetch                          */
+  SSN_KERNEL_SPLIT_EXPAND = 10     /* the same for the expansion                               */
 };
 #define SSN_KVAR_E 1      /* the kernel reads E rows                                            */
 #define SSN_KVAR_P 2      /* the kernel reads P rows                                            */
 #define SSN_KVAR_WIDE 4   /* rank above 64 (two 64-coordinate groups / the wide row tiles)      */
 #define SSN_KVAR_ALT 8    /* MMA_SYNC: 32 rows per warp; EXPAND64: one P row per 16-sequence tile;
                              UMMA_PROJECT: positional product shared per block; UMMA_EXPAND:
-                             tiles of 8 sequences x 16 positions; UMMA_ROUNDTRIP: LEFT          */
+                             tiles of 8 sequences x 16 positions; UMMA_ROUNDTRIP: LEFT;
+                             SPLIT_PROJECT: several CTAs per tile; SPLIT_EXPAND: fp32 wire rows */
 #define SSN_KVAR_ROWSUMSQ 16 /* UMMA_EXPAND / GENERIC: the row statistic is produced              */
 #define SSN_KVAR_TWO_RUNS 64  /* UMMA_EXPAND: head and remainder of fp32 wire rows as two runs against one chunk of U */
 #define SSN_KVAR_FEWSEQ 32   /* UMMA_EXPAND: tiles of 4, 2 or 1 sequences (a batch that is not groups of 8) */

@@ -1,0 +1,99 @@
+// Launcher of the split-operand projection kernel (see codec_split_project.cuh).
+#include "codec_split_project.cuh"
+
+#include "codec_mma_launch.h"
+#include "codec_split.h"
+
+namespace ssn {
+namespace {
+
+// CTAs per tile.  With enough tiles every CTA takes whole ones.  Fewer tiles than half the SMs: the
+// largest cluster that still runs in one wave.  In between, two CTAs per tile where the halves pack
+// the last wave better than whole tiles do (by more than a tenth of a tile, about what the exchange
+// and a second set-up cost).
+int cluster_of(int64_t ntiles, int nst, int sms) {
+  int c = 1;
+  while (c < 8 && 2 * c <= nst && ntiles * 2 * c <= sms - (2 * c == 8 ? 20 : 0)) c *= 2;
+  if (c == 1 && nst >= 2 && ntiles > sms && ntiles < 8 * (int64_t)sms) {
+    const int64_t whole = (ntiles + sms - 1) / sms, halves = (2 * ntiles + sms - 1) / sms;
+    if (10 * halves + 2 < 20 * whole - 2) c = 2;
+  }
+  return c;
+}
+
+template <typename T, int KN, int NSLOT>
+cudaError_t launch_one(const SplitProjectArgs &a, int sms, cudaStream_t stream) {
+  auto kernel = codec_split_project_kernel<T, KN, NSLOT>;
+  constexpr int smem = SplitProjectConfig<T, KN, NSLOT>::kSmemBytes;
+  static std::atomic<uint64_t> configured{0};
+  cudaError_t e = allow_dynamic_smem(kernel, smem, configured);
+  if (e != cudaSuccess) return e;
+  const int64_t ntiles = (a.n + kUmmaTile - 1) / kUmmaTile;
+  const int c = cluster_of(ntiles, (a.d + kSplitCols - 1) / kSplitCols, sms);
+  const int64_t most = (int64_t)sms * SplitProjectConfig<T, KN, NSLOT>::kCtasPerSm;
+  const int64_t single = ntiles < most ? ntiles : most, grid = c > 1 ? ntiles * c : single;
+  e = launch_dependent(kernel, (unsigned)grid, kSplitProjectThreads, smem, stream, c, a);
+  if (e != cudaSuccess && c > 1) {   // a device that cannot co-schedule the cluster
+    cudaGetLastError();
+    e = launch_dependent(kernel, (unsigned)single, kSplitProjectThreads, smem, stream, 1, a);
+  }
+  note_kernel(SSN_KERNEL_SPLIT_PROJECT,
+              (a.has_e ? SSN_KVAR_E : 0) | (a.has_p ? SSN_KVAR_P : 0) | (KN > 64 ? SSN_KVAR_WIDE : 0) | (c > 1 ? SSN_KVAR_ALT : 0));
+  return e;
+}
+
+template <typename T, int KN>
+cudaError_t launch_slots(const SplitProjectArgs &a, int slots, int sms, cudaStream_t s) {
+  if (slots == 0) return launch_one<T, KN, 0>(a, sms, s);
+  if (slots == 1) return launch_one<T, KN, 1>(a, sms, s);
+  if (slots == 2) return launch_one<T, KN, 2>(a, sms, s);
+  return launch_one<T, KN, 3>(a, sms, s);
+}
+
+template <typename T>
+cudaError_t launch_rank(const SplitProjectArgs &a, int slots, int sms, cudaStream_t s) {
+  if (a.k <= 32) return launch_slots<T, 32>(a, slots, sms, s);
+  if (a.k <= 64) return launch_slots<T, 64>(a, slots, sms, s);
+  return launch_slots<T, 128>(a, slots, sms, s);
+}
+
+bool rows16(const void *p, int64_t ld, int esz) {
+  return (reinterpret_cast<uintptr_t>(p) & 15) == 0 && (ld * esz) % 16 == 0;
+}
+
+}  // namespace
+
+cudaError_t launch_codec_split_project(const TokenArgs &a, int32_t dtype, int sm_count, cudaStream_t stream) {
+  if (a.src == nullptr || a.zout == nullptr || a.dst != nullptr || a.rowsumsq != nullptr || a.k > kSplitMaxRank ||
+      a.U2 != nullptr || a.n > 0x7fffffffLL || sm_count < 1)
+    return cudaErrorNotSupported;
+  const int esz = dtype == SSN_F32 ? 4 : 2;
+  SplitProjectArgs p{};
+  p.src = a.src;
+  p.src2 = a.src2;
+  p.U = a.U;
+  p.zout = a.zout;
+  p.lds = a.lds;
+  p.lds2 = a.lds2;
+  p.ldu = a.ldu;
+  p.ldzout = a.ldzout;
+  p.n = a.n;
+  p.d = a.d;
+  p.k = a.k;
+  p.wire = a.wire;
+  p.wire_ids = a.wire_ids;
+  p.shift = a.shift;
+  p.has_e = a.sub_shift && a.shift.E != nullptr;
+  p.has_p = a.sub_shift && a.shift.P != nullptr;
+  p.vec_rows = (int64_t)a.d * esz % 16 == 0 && rows16(a.src, a.lds, esz) &&
+               (a.src2 == nullptr || rows16(a.src2, a.lds2, esz)) &&
+               (!p.has_e || rows16(a.shift.E, a.shift.lde, esz)) && (!p.has_p || rows16(a.shift.P, a.shift.ldp, esz));
+  p.vec_u = pairs_aligned(a.U, a.ldu, esz);
+  // four coordinates are 16 bytes of words or 8 bytes of bf16
+  p.vec_out = (a.ldzout & 3) == 0 && (reinterpret_cast<uintptr_t>(a.zout) & (a.wire || dtype == SSN_F32 ? 15 : 7)) == 0;
+  const int slots = (a.src2 != nullptr) + p.has_e + p.has_p;
+  return dtype == SSN_F32 ? launch_rank<float>(p, slots, sm_count, stream)
+                          : launch_rank<__nv_bfloat16>(p, slots, sm_count, stream);
+}
+
+}  // namespace ssn

@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "codec_mma_launch.h"
+#include "codec_split.h"
 #include "generic_kernels.cuh"
 #include "ssn_common.cuh"
 
@@ -154,6 +155,18 @@ ssn_status_t launch_token_kernel(const TokenArgs &a, int32_t dtype, cudaStream_t
         g_launches.fetch_add(1, std::memory_order_relaxed);
         return e == cudaSuccess ? SSN_OK : SSN_ERR_CUDA;
       }
+    }
+  }
+  // everything else that is a projection or an expansion of rank up to 128: fp32 storage, operands off
+  // the 16-byte grid, wire rows and addends the kernels above do not take
+  const int sms = sm_count_of_current_device();
+  if (sms > 0) {
+    const cudaError_t e = a.src != nullptr ? launch_codec_split_project(a, dtype, sms, stream)
+                                           : launch_codec_split_expand(a, dtype, sms, stream);
+    if (e == cudaSuccess) return launch_status();
+    if (e != cudaErrorNotSupported) {
+      cudaGetLastError();
+      return SSN_ERR_CUDA;
     }
   }
   return launch_generic_token_kernel(a, dtype, stream);

@@ -1,0 +1,120 @@
+"""The split-operand tcgen05 kernels (fp32 storage, and the bf16 calls TMA cannot fetch) at the sizes
+where they can go wrong: edges of the 128-token tiles, the 64-column stages and the 128-column chunks,
+one and several CTAs per tile, every rank variant, leading dimensions off the 16-byte grid, positions
+per token; and rows whose magnitudes the three-part split does not hold."""
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import ssn_oracle as oracle
+from paper_2607_13332_b200 import binding as B
+from paper_2607_13332_b200 import synth
+from tests.harness import Codec, assert_close, f64, guards_intact, host64, padded, to_device
+
+pytestmark = pytest.mark.gpu
+
+# fp32 sums of at most 2176 products of size ~1/sqrt(d): 64-column chains of fp32 additions err by a few
+# 2^-24 of the partial sums, 1e-6 of the rms at the outer tail over all elements of a result
+F32_SUM_TOL = 1e-6
+
+CASES = [   # n, d, k, leading dimension excess (elements)
+    (1, 64, 1, 1), (127, 65, 7, 0), (128, 127, 32, 1), (129, 128, 33, 0), (300, 192, 64, 3), (513, 130, 65, 1),
+    (2000, 2176, 40, 0), (2000, 1088, 128, 1), (10007, 256, 51, 0), (19100, 136, 9, 1), (40000, 72, 17, 0),
+]
+
+
+def _inputs(n, d, k, dt, seed):
+    wl = synth.Workload("split", d, k, 97, 1, n, dt)
+    return synth.codec_inputs(wl, seed=seed, noise_std=0.05)
+
+
+def _strided(t, dt, excess):
+    t = to_device(t, dt)
+    view, _ = padded(t.shape[0], t.shape[1], t.shape[1] + excess, dt, fill=t)
+    return view
+
+
+@pytest.mark.parametrize("n,d,k,excess", CASES)
+@pytest.mark.parametrize("dt", [synth.F32, synth.BF16])
+@pytest.mark.parametrize("tables", ["EP", "E", "none"])
+def test_split_kernels_match_the_oracle(n, d, k, excess, dt, tables):
+    if dt == synth.BF16 and excess == 0 and k % 8 == 0 and d % 8 == 0:
+        excess = 1   # an aligned bf16 call belongs to the TMA kernels
+    rng = np.random.default_rng(n + d)
+    t = _inputs(n, d, k, dt, seed=n + k)
+    E0, P0 = (t["E"] if "E" in tables else None), (t["P"][:50] if "P" in tables else None)
+    pos = rng.integers(0, min(50, n), n).astype(np.int32)
+    dev = {x: _strided(t[x], dt, excess) for x in ("X", "G", "U", "Z0")}
+    codec = Codec(dt, dev["U"], None if E0 is None else _strided(E0, dt, excess), None if P0 is None else _strided(P0, dt, excess))
+    ids, dpos = torch.from_numpy(t["ids"]).cuda(), torch.from_numpy(pos).cuda()
+    f = {x: f64(t[x], dt) for x in ("X", "G", "U", "Z0")}
+    E, P = f64(E0, dt), f64(P0, dt)
+
+    Z, buf = padded(n, k, k + excess, dt)
+    codec.compress(dev["X"], ids, pos=dpos, out=Z)
+    assert B.ssn_last_kernel()[0] == B.SSN_KERNEL_SPLIT_PROJECT
+    expect, _ = oracle.compress(f["X"], f["U"], E, t["ids"], P, pos)
+    assert_close(host64(Z, dt), expect, dt, "compress", tol=F32_SUM_TOL if dt == synth.F32 else None)
+    assert guards_intact(Z, buf, dt)
+
+    # a residual addend beside the tables, fp32 words out with the token id
+    wire = codec.compress_sum(dev["X"], dev["G"], ids, pos=dpos, wire=True, with_ids=True)
+    expect, _ = oracle.compress_sum(f["X"], f["G"], f["U"], E, t["ids"], P, pos)
+    coords, got_ids = oracle.wire_unpack(wire.cpu().numpy(), k, True)
+    if tables != "none" or excess or dt == synth.F32:
+        assert B.ssn_last_kernel()[0] == B.SSN_KERNEL_SPLIT_PROJECT
+        assert_close(coords, expect, dt, "compress_sum wire", tol=F32_SUM_TOL)
+    assert np.array_equal(got_ids, t["ids"])
+
+    out, buf = padded(n, d, d + excess, dt)
+    codec.decompress(dev["Z0"], ids, pos=dpos, out=out)
+    assert B.ssn_last_kernel()[0] == B.SSN_KERNEL_SPLIT_EXPAND
+    expect, _ = oracle.decompress(f["Z0"], f["U"], E, t["ids"], P, pos)
+    assert_close(host64(out, dt), expect, dt, "decompress", tol=F32_SUM_TOL if dt == synth.F32 else None)
+    assert guards_intact(out, buf, dt)
+
+    Xw = codec.decompress_wire(wire, pos=dpos, with_ids=True, use_workspace=False)
+    assert B.ssn_last_kernel()[0] == B.SSN_KERNEL_SPLIT_EXPAND
+    expect, _ = oracle.decompress(coords, f["U"], E, t["ids"], P, pos)
+    assert_close(host64(Xw, dt), expect, dt, "decompress_wire", tol=F32_SUM_TOL if dt == synth.F32 else None)
+    assert codec.take_status() == 0
+
+
+def _same_as_plain_sums(got, expect, what):
+    """Infinities and NaN where plain sums have them; each other row within the fp32 tolerance of its own scale."""
+    assert np.array_equal(np.isnan(got), np.isnan(expect)), what
+    inf = np.isinf(expect)
+    assert np.array_equal(np.isinf(got), inf) and np.array_equal(np.sign(got[inf]), np.sign(expect[inf])), what
+    for r in range(expect.shape[0]):
+        if np.isfinite(expect[r]).all():
+            scale = max(np.abs(expect[r]).max(), 1e-300)
+            assert np.abs(got[r] - expect[r]).max() <= 1e-5 * scale, (what, r)
+
+
+@pytest.mark.parametrize("n,d,k", [(300, 256, 40), (19100, 128, 16)])
+def test_rows_the_split_does_not_hold(n, d, k):
+    """Infinite, NaN, enormous and tiny rows (and one row of zeros) give what plain fp32 sums give."""
+    dt = synth.F32
+    t = _inputs(n, d, k, dt, seed=3)
+    t["X"][0, 5], t["X"][7, 9], t["X"][8, 9] = np.inf, -np.inf, np.nan
+    t["X"][20] *= 1e36
+    t["X"][130] *= 1e-30
+    t["X"][131] = 0
+    t["Z0"][0, 3], t["Z0"][9, 0] = np.inf, np.nan
+    t["Z0"][21] *= 1e36
+    t["Z0"][130] *= 1e-30
+    codec = Codec(dt, to_device(t["U"], dt))
+    f = {x: f64(t[x], dt) for x in ("X", "U", "Z0")}
+    with np.errstate(invalid="ignore"):
+        _same_as_plain_sums(host64(codec.grad_project(to_device(t["X"], dt)), dt), f["X"] @ f["U"], "projection")
+        _same_as_plain_sums(host64(codec.decompress(to_device(t["Z0"], dt)), dt), f["Z0"] @ f["U"].T, "expansion")
+        # an infinity in the basis concerns every row
+        t["U"][3, 1] = np.inf
+        U = f64(t["U"], dt)
+        codec = Codec(dt, to_device(t["U"], dt))
+        finite = _inputs(n, d, k, dt, seed=4)
+        X, Z = f64(finite["X"], dt), f64(finite["Z0"], dt)
+        _same_as_plain_sums(host64(codec.grad_project(to_device(finite["X"], dt)), dt), X @ U, "projection, U")
+        _same_as_plain_sums(host64(codec.decompress(to_device(finite["Z0"], dt)), dt), Z @ U.T, "expansion, U")
+    assert codec.take_status() == 0
