@@ -11,7 +11,7 @@
 //
 // The split needs room below and above x: rows whose largest magnitude is under kSplitTiny (the low
 // terms would leave the range of bf16) or at or over kSplitHuge (h, or a partial sum of it, would
-// overflow; infinities and NaN too) are flagged and computed with plain fp32 FMAs instead.
+// overflow; infinities too) are flagged and computed with plain fp32 FMAs instead.
 #pragma once
 
 #include "codec_umma.cuh"
@@ -19,12 +19,22 @@
 
 namespace ssn {
 
-constexpr uint32_t kSplitHugeBits = 0x7B800000u;   // 2^120
-constexpr uint32_t kSplitTinyBits = 0x17800000u;   // 2^-80
+constexpr float kSplitHuge = 0x1p120f, kSplitTiny = 0x1p-80f;
 
-__device__ __forceinline__ uint32_t magnitude_bits(float v) { return __float_as_uint(v) & 0x7FFFFFFFu; }
-__device__ __forceinline__ bool split_unsafe(uint32_t largest_bits) {
-  return largest_bits >= kSplitHugeBits || (largest_bits != 0 && largest_bits < kSplitTinyBits);
+// `largest`: by fmaxf over magnitudes, which skips NaN: a NaN stays one through its leading part, and makes
+// every sum it enters NaN, as it does in plain FMAs.
+__device__ __forceinline__ bool split_unsafe(float largest) {
+  return largest >= kSplitHuge || (largest != 0.f && largest < kSplitTiny);
+}
+
+// Two fp32 operations in one instruction.
+__device__ __forceinline__ void sub2(float &a0, float &a1, float b0, float b1) {
+  asm("{\n.reg .b64 a, b;\nmov.b64 a, {%0, %1};\nmov.b64 b, {%2, %3};\nsub.rn.f32x2 a, a, b;\nmov.b64 {%0, %1}, a;\n}\n"
+      : "+f"(a0), "+f"(a1) : "f"(b0), "f"(b1));
+}
+__device__ __forceinline__ void add2(float &a0, float &a1, float b0, float b1) {
+  asm("{\n.reg .b64 a, b;\nmov.b64 a, {%0, %1};\nmov.b64 b, {%2, %3};\nadd.rn.f32x2 a, a, b;\nmov.b64 {%0, %1}, a;\n}\n"
+      : "+f"(a0), "+f"(a1) : "f"(b0), "f"(b1));
 }
 
 // Parts h, m, l (NP = 3) or h alone (NP = 1) of the pair (v0, v1), v0 in the low half.
@@ -33,10 +43,7 @@ __device__ __forceinline__ void split_pair(float v0, float v1, uint32_t (&p)[NP]
 #pragma unroll
   for (int i = 0; i < NP; ++i) {
     p[i] = pack_bf16(v0, v1);
-    if (i + 1 < NP) {
-      v0 -= __uint_as_float(p[i] << 16);
-      v1 -= __uint_as_float(p[i] & 0xFFFF0000u);
-    }
+    if (i + 1 < NP) sub2(v0, v1, __uint_as_float(p[i] << 16), __uint_as_float(p[i] & 0xFFFF0000u));
   }
 }
 
@@ -55,34 +62,105 @@ __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t
   asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};\n" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
 
-// Two neighbouring elements as stored, zeros past `valid` of them; `vec`: the pair may be read at once.
-template <typename T> struct Pair { uint32_t w[sizeof(T) / 2]; };
+__device__ __forceinline__ uint4 ld_shared_v4(uint32_t addr) {
+  uint4 v;
+  asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];\n" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
+  return v;
+}
+
+// Loads that are predicated where they have to be, never branched around, and not touched where they are
+// issued: the values are consumed a step later, and anything done to them here would wait for memory.
+__device__ __forceinline__ uint4 load_global_v4_if(const void *p, bool ok) {
+  uint4 v;
+  asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %5, 0;\n"
+               "mov.b32 %0, 0;\nmov.b32 %1, 0;\nmov.b32 %2, 0;\nmov.b32 %3, 0;\n"
+               "@p ld.global.nc.v4.b32 {%0,%1,%2,%3}, [%4];\n}\n"
+               : "=&r"(v.x), "=&r"(v.y), "=&r"(v.z), "=&r"(v.w) : "l"(p), "r"((int)ok));
+  return v;
+}
+__device__ __forceinline__ uint2 load_global_v2_if(const void *p, bool ok) {
+  uint2 v;
+  asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %3, 0;\nmov.b32 %0, 0;\nmov.b32 %1, 0;\n"
+               "@p ld.global.nc.v2.b32 {%0,%1}, [%2];\n}\n" : "=&r"(v.x), "=&r"(v.y) : "l"(p), "r"((int)ok));
+  return v;
+}
+__device__ __forceinline__ uint32_t load_global_b32_if(const void *p, bool ok) {
+  uint32_t v;
+  asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %2, 0;\nmov.b32 %0, 0;\n@p ld.global.nc.b32 %0, [%1];\n}\n"
+               : "=&r"(v) : "l"(p), "r"((int)ok));
+  return v;
+}
+__device__ __forceinline__ uint32_t load_global_b16_if(const void *p, bool ok) {
+  uint16_t v;
+  asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %2, 0;\nmov.b16 %0, 0;\n@p ld.global.nc.b16 %0, [%1];\n}\n"
+               : "=&h"(v) : "l"(p), "r"((int)ok));
+  return v;
+}
+__device__ __forceinline__ uint2 load_global_v2(const void *p) {
+  uint2 v;
+  asm volatile("ld.global.nc.v2.b32 {%0,%1}, [%2];\n" : "=r"(v.x), "=r"(v.y) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ uint32_t load_global_b32(const void *p) {
+  uint32_t v;
+  asm volatile("ld.global.nc.b32 %0, [%1];\n" : "=r"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ uint32_t load_global_b16(const void *p) {
+  uint16_t v;
+  asm volatile("ld.global.nc.b16 %0, [%1];\n" : "=h"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];\n" ::"l"(p)); }
+
+// Two neighbouring elements as loaded.  A bf16 pair has one word per element until joined() puts them
+// into w[0] (w[1] = 0: read at once).
+template <typename T> struct Pair { uint32_t w[2]; };
+// The pairs at at(0) .. at(N - 1): `valid` says how many of a pair's elements exist (the same for all; the
+// others read as 0, and none at all leaves v as it is), `vec` whether a pair may be read at once.  One branch
+// for all of them: with one per pair the loads and what follows them were serialised.
+template <int N, typename T, typename At>
+__device__ __forceinline__ void load_pairs(Pair<T> (&v)[N], At at, int valid, bool vec) {
+  if (valid > 1 && vec) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      if constexpr (sizeof(T) == 4) {
+        const uint2 x = load_global_v2(at(i));
+        v[i].w[0] = x.x;
+        v[i].w[1] = x.y;
+      } else {
+        v[i].w[0] = load_global_b32(at(i));
+        v[i].w[1] = 0;
+      }
+    }
+  } else if (valid > 1) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      const T *p = at(i);
+      v[i].w[0] = sizeof(T) == 4 ? load_global_b32(p) : load_global_b16(p);
+      v[i].w[1] = sizeof(T) == 4 ? load_global_b32(p + 1) : load_global_b16(p + 1);
+    }
+  } else if (valid > 0) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      v[i].w[0] = sizeof(T) == 4 ? load_global_b32(at(i)) : load_global_b16(at(i));
+      v[i].w[1] = 0;
+    }
+  }
+}
+// The pair as used: two fp32 words, or both bf16 values in w[0].
 template <typename T>
-__device__ __forceinline__ Pair<T> load_pair(const T *p, int valid, bool vec) {
-  Pair<T> v;
-  if constexpr (sizeof(T) == 4) {
-    if (vec && valid > 1) {
-      const uint2 x = __ldg(reinterpret_cast<const uint2 *>(p));
-      v.w[0] = x.x;
-      v.w[1] = x.y;
-    } else {
-      v.w[0] = valid > 0 ? __float_as_uint(p[0]) : 0u;
-      v.w[1] = valid > 1 ? __float_as_uint(p[1]) : 0u;
-    }
-  } else {
-    if (vec && valid > 1) {
-      v.w[0] = __ldg(reinterpret_cast<const uint32_t *>(p));
-    } else {
-      v.w[0] = valid > 0 ? __bfloat16_as_ushort(p[0]) : 0u;
-      if (valid > 1) v.w[0] |= (uint32_t)__bfloat16_as_ushort(p[1]) << 16;
-    }
+__device__ __forceinline__ Pair<T> joined(Pair<T> v) {
+  if constexpr (sizeof(T) == 2) {
+    v.w[0] |= v.w[1] << 16;
+    v.w[1] = 0;
   }
   return v;
 }
 template <typename T>
-__device__ __forceinline__ uint32_t pair_magnitude(const Pair<T> &v) {   // of the larger one, as fp32 bits
-  if constexpr (sizeof(T) == 4) return max(v.w[0] & 0x7FFFFFFFu, v.w[1] & 0x7FFFFFFFu);
-  else return max(v.w[0] & 0x7FFF0000u, (v.w[0] << 16) & 0x7FFF0000u);
+__device__ __forceinline__ float pair_magnitude(const Pair<T> &v) {   // of the larger one
+  if constexpr (sizeof(T) == 4) return fmaxf(fabsf(__uint_as_float(v.w[0])), fabsf(__uint_as_float(v.w[1])));
+  else return fmaxf(fabsf(__uint_as_float(v.w[0] << 16)), fabsf(__uint_as_float(v.w[0] & 0xFFFF0000u)));
 }
 // Its bf16 parts: three of an fp32 pair (or NP = 1), itself for a bf16 pair.
 template <typename T, int NP>

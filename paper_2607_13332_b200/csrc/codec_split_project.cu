@@ -29,9 +29,8 @@ cudaError_t launch_one(const SplitProjectArgs &a, int sms, cudaStream_t stream) 
   cudaError_t e = allow_dynamic_smem(kernel, smem, configured);
   if (e != cudaSuccess) return e;
   const int64_t ntiles = (a.n + kUmmaTile - 1) / kUmmaTile;
-  const int c = cluster_of(ntiles, (a.d + kSplitCols - 1) / kSplitCols, sms);
-  const int64_t most = (int64_t)sms * SplitProjectConfig<T, KN, NSLOT>::kCtasPerSm;
-  const int64_t single = ntiles < most ? ntiles : most, grid = c > 1 ? ntiles * c : single;
+  const int c = cluster_of(ntiles, (a.d + 63) / 64, sms);
+  const int64_t single = ntiles < sms ? ntiles : sms, grid = c > 1 ? ntiles * c : single;
   e = launch_dependent(kernel, (unsigned)grid, kSplitProjectThreads, smem, stream, c, a);
   if (e != cudaSuccess && c > 1) {   // a device that cannot co-schedule the cluster
     cudaGetLastError();
@@ -85,7 +84,7 @@ cudaError_t launch_codec_split_project(const TokenArgs &a, int32_t dtype, int sm
   p.shift = a.shift;
   p.has_e = a.sub_shift && a.shift.E != nullptr;
   p.has_p = a.sub_shift && a.shift.P != nullptr;
-  p.vec_rows = (int64_t)a.d * esz % 16 == 0 && rows16(a.src, a.lds, esz) &&
+  p.vec_rows = (int64_t)a.d * esz % 16 == 0 && (int64_t)a.d * esz <= kZeroRowBytes && rows16(a.src, a.lds, esz) &&
                (a.src2 == nullptr || rows16(a.src2, a.lds2, esz)) &&
                (!p.has_e || rows16(a.shift.E, a.shift.lde, esz)) && (!p.has_p || rows16(a.shift.P, a.shift.ldp, esz));
   p.vec_u = pairs_aligned(a.U, a.ldu, esz);

@@ -3,23 +3,21 @@
 // for fp32 storage, and for the bf16 calls whose operands the TMA projection cannot fetch: leading
 // dimensions or addresses off the 16-byte grid, positions per token, a residual addend beside row tables.
 //
-// Threads load the rows straight into registers (any alignment, any row per token), form the residual
-// in fp32 as the general kernel does, split it into bf16 parts (codec_split.cuh) and write them as
-// swizzled operand tiles; the basis is split the same way, stage by stage.  With bf16 rows and no
-// subtraction one part is exact, and bf16 bases have one part.
+// cp.async brings the rows in, 16 bytes at a time and any row per token, several steps ahead (what is in
+// flight is bounded by shared memory, not by registers); the residual is formed in fp32 as the general
+// kernel does, split into bf16 parts (codec_split.cuh) and written as swizzled operand tiles; the basis is split
+// the same way, step by step.  With bf16 rows and no subtraction one part is exact, and bf16 bases have
+// one part.  A step is 128 bytes of every row: 32 columns of fp32, 64 of bf16.
 //
-// Sixteen warps (128 registers a thread), all in the same roles, one 64-column stage per step:
-//   - the residuals of the stage are formed from the rows in flight, and the rows of the next one are
-//     requested (16 values per thread and operand: what covers the HBM latency);
-//   - one thread issues the MMAs of the stage before: Ah x (Uh|Um|Ul), Am x (Uh|Um), Al x Uh, the parts of U
-//     side by side on N so that three instructions per K step cover the six products (rank above
-//     64: five instructions, (Uh|Um) being 256 columns wide);
-//   - the finished accumulator of the stage two back is added to the fp32 sums in registers (see
-//     codec_split.cuh on why the chains are this short); warp w reads TMEM lanes 32 (w % 4) .. +31 and a
-//     quarter of the columns;
-//   - the residuals and the slice of U are split and written to the stage.
-// Waiting for the accumulator of step s - 2 before writing step s is also what makes two stages of
-// shared memory enough, with no barrier for a free stage or a free accumulator.
+//   warps 0-15  every thread reads back the pieces it copied itself (no barrier), writes their parts and its
+//               share of U to the step's operand stage, and requests the rows of the step RD - 1 ahead.
+//               Every 64 columns a finished accumulator is added to fp32 sums in registers (see
+//               codec_split.cuh on why the chains are this short): warp w reads TMEM lanes 32 (w % 4) .. +31
+//               and a quarter of the columns.
+//   warp 16     one thread issues the MMAs: Ah x (Uh|Um|Ul), Am x (Uh|Um), Al x Uh, the parts of U side by
+//               side on N so that three instructions per K step cover the six products (rank above 64:
+//               five instructions, (Uh|Um) being 256 columns wide).  It is a warp of its own because each
+//               of these instructions blocks its thread for about 100 clocks.
 //
 // A CTA takes whole tiles of 128 tokens; when there are fewer tiles than SMs, a cluster of 2, 4 or 8
 // CTAs shares one tile, each contracting a slice of d, and the partial sums meet through distributed
@@ -37,15 +35,14 @@ struct SplitProjectArgs {
   int32_t d, k;
   int32_t wire, wire_ids;      // fp32 words out, word k of a row = the token id
   int32_t has_e, has_p;
-  int32_t vec_rows;            // every row operand may be read 16 bytes at a time
+  int32_t vec_rows;            // every row operand may be read 16 bytes at a time and g_zero_row holds a row
   int32_t vec_u, vec_out;      // two coordinates of U may be read, four coordinates stored at a time
   ShiftTables shift;
 };
 
-constexpr int kSplitProjectWarps = 16;
-constexpr int kSplitProjectThreads = 32 * kSplitProjectWarps;
-constexpr int kSplitCols = 64;                        // columns of d per stage
-constexpr int kSplitPartBytes = kUmmaTile * 128;      // one bf16 part of a [128 x 64] operand
+constexpr int kSplitRowWarps = 16, kSplitRowThreads = 32 * kSplitRowWarps;
+constexpr int kSplitProjectThreads = kSplitRowThreads + 32;
+constexpr int kSplitRawBytes = kUmmaTile * 128;       // one operand's rows of one step
 
 template <typename T, int KN, int NSLOT>
 struct SplitProjectConfig {
@@ -57,35 +54,49 @@ struct SplitProjectConfig {
   static constexpr int kDCols = kNX == 1 ? KN : (kStack == 3 ? 3 : 2) * KN;
   static constexpr int kDStride = kDCols <= 32 ? 32 : (kDCols <= 64 ? 64 : (kDCols <= 128 ? 128 : 256));
   static constexpr int kTmemCols = 2 * kDStride;
-  static constexpr int kABytes = kNX * kSplitPartBytes;
+  static constexpr int kCols = kF32 ? 32 : 64;              // columns of d per step
+  static constexpr int kPartBytes = kUmmaTile * kCols * 2;  // one bf16 part of a [128 x kCols] operand
+  static constexpr int kRowBytes = kCols * 2;               // its rows, swizzled within 64 or 128 bytes
+  static constexpr int kABytes = kNX * kPartBytes;
   static constexpr int kBGroups = (kNU * KN + 63) / 64;     // 64-coordinate groups of all parts
-  static constexpr int kGroupBytes = kSplitCols * 128;
+  static constexpr int kGroupBytes = kCols * 128;
   static constexpr int kStageBytes = kABytes + kBGroups * kGroupBytes;
+  static constexpr int kRawStepBytes = (1 + NSLOT) * kSplitRawBytes;
   static constexpr int kSumPitch = KN + 4;                  // floats per row of the exchanged sums
-  // two stages, or the exchanged sums in their place
-  static constexpr int kRingBytes = 2 * kStageBytes > kUmmaTile * kSumPitch * 4 ? 2 * kStageBytes : kUmmaTile * kSumPitch * 4;
-  static constexpr int kBars = 4;
+  static constexpr int kSumBytes = kUmmaTile * kSumPitch * 4;
+  static constexpr int kRoom = 227 * 1024 - 1024 - 256;
+  // two operand stages unless that leaves no two steps of rows (bf16, three more operands)
+  static constexpr int kStages = kRoom - 2 * kStageBytes >= 2 * kRawStepBytes ? 2 : 1;
+  static constexpr int kFit = (kRoom - kStages * kStageBytes) / kRawStepBytes;
+  static constexpr int kRaw = kFit < 6 ? kFit : 6;          // steps of rows in flight or being read
+  static_assert(kRaw >= 2, "no room for two steps of rows");
+  static constexpr int kRingBytes = kStages * kStageBytes + kRaw * kRawStepBytes;
+  static_assert(kRingBytes >= kSumBytes, "the exchanged sums take the place of the rings");
+  static constexpr int kBars = 8;
   static constexpr int kSmemBytes = 1024 + kRingBytes + kBars * 8 + 16;   // barriers, TMEM address, unsafe-value flags
-  static_assert(kSmemBytes <= 227 * 1024, "no room for two stages");
-  static constexpr int kCtasPerSm = kNX == 1 && KN <= 64 ? 2 : 1;   // one part and few sums: two CTAs hide each other's waits
-  static constexpr int kPairs = KN / 16;                    // pairs of U per thread and stage
+  static constexpr int kChain = 64 / kCols;                 // steps per accumulator
+  static constexpr int kPairs = kCols * KN / 2 / kSplitRowThreads;   // pairs of U per thread and step
   static constexpr int kSums = KN / 4;                      // coordinates of one row per thread
-  static constexpr int kVecs = kF32 ? 4 : 2;                // 16-byte pieces per thread, operand and stage
-  static constexpr int kVecElems = kF32 ? 4 : 8;
+  static constexpr int kVecElems = kF32 ? 4 : 8;            // of a 16-byte piece; a thread has two per operand and step
 };
 
-// 16 bytes of a row from column c on (zeros past column d and for a missing row).
+// 16 bytes of a row from column c on, element by element (zeros past column d and for a missing row).
 template <typename T>
-__device__ __forceinline__ uint4 load_row_piece(const T *row, int c, int d, bool vec) {
-  constexpr int E = 16 / (int)sizeof(T);
-  uint4 raw = make_uint4(0, 0, 0, 0);
-  if (row == nullptr || c >= d) return raw;
-  if (vec) return __ldg(reinterpret_cast<const uint4 *>(row + c));   // vec: d is a multiple of E
-  T e[E];
+__device__ __forceinline__ uint4 load_row_piece(const T *row, int c, int d) {
+  uint32_t w[4];
+  const bool ok = row != nullptr;
 #pragma unroll
-  for (int i = 0; i < E; ++i) e[i] = c + i < d ? row[c + i] : from_f32<T>(0.f);
-  memcpy(&raw, e, 16);
-  return raw;
+  for (int i = 0; i < 4; ++i) {
+    if constexpr (sizeof(T) == 4)
+      w[i] = load_global_b32_if(row + c + i, ok && c + i < d);
+    else
+      w[i] = load_global_b16_if(row + c + 2 * i, ok && c + 2 * i < d) | load_global_b16_if(row + c + 2 * i + 1, ok && c + 2 * i + 1 < d) << 16;
+  }
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+// The same with an asynchronous copy to shared memory; `ok` = false writes zeros.
+__device__ __forceinline__ void cp_async16_if(uint32_t dst, const void *src, bool ok) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src), "r"(ok ? 16 : 0) : "memory");
 }
 
 template <typename T> __device__ __forceinline__ void widen_piece(const uint4 &raw, float *f);
@@ -131,8 +142,9 @@ __device__ __forceinline__ void store_coords4(const SplitProjectArgs &a, int64_t
 template <typename T>
 __device__ __noinline__ void project_unsafe_rows(const SplitProjectArgs &a, int64_t tile, int row0, int rows, bool all) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (warp >= kSplitRowWarps) return;
   const T *U = static_cast<const T *>(a.U);
-  for (int rr = row0 + warp; rr < row0 + rows; rr += kSplitProjectWarps) {
+  for (int rr = row0 + warp; rr < row0 + rows; rr += kSplitRowWarps) {
     const int64_t t = tile * kUmmaTile + rr;
     if (t >= a.n) return;
     const T *x = static_cast<const T *>(a.src) + t * a.lds;
@@ -147,9 +159,10 @@ __device__ __noinline__ void project_unsafe_rows(const SplitProjectArgs &a, int6
       if (p != nullptr) r -= to_f32(p[i]);
       return r;
     };
-    uint32_t m = 0;
-    for (int i = lane; i < a.d; i += 32) m = max(m, magnitude_bits(residual(i)));
-    m = __reduce_max_sync(0xffffffffu, m);
+    float m = 0.f;
+    for (int i = lane; i < a.d; i += 32) m = fmaxf(m, fabsf(residual(i)));
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
     if (!all && !split_unsafe(m)) continue;
     for (int j = lane; j < a.k; j += 32) {
       float acc = 0.f;
@@ -163,10 +176,9 @@ __device__ __noinline__ void project_unsafe_rows(const SplitProjectArgs &a, int6
 }
 
 template <typename T, int KN, int NSLOT>
-__global__ void __launch_bounds__(kSplitProjectThreads, (SplitProjectConfig<T, KN, NSLOT>::kCtasPerSm))
-codec_split_project_kernel(const SplitProjectArgs a) {
+__global__ void __launch_bounds__(kSplitProjectThreads, 1) codec_split_project_kernel(const SplitProjectArgs a) {
   using Cfg = SplitProjectConfig<T, KN, NSLOT>;
-  constexpr int NX = Cfg::kNX, NU = Cfg::kNU;
+  constexpr int NX = Cfg::kNX, NU = Cfg::kNU, S = Cfg::kStages, RD = Cfg::kRaw, G = Cfg::kChain;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -176,16 +188,18 @@ codec_split_project_kernel(const SplitProjectArgs a) {
   asm volatile("mov.u32 %0, %%cluster_ctarank;\n" : "=r"(cta_rank));
   const int64_t ntiles = (a.n + kUmmaTile - 1) / kUmmaTile;
   const int64_t groups = gridDim.x / cluster_size, group = blockIdx.x / cluster_size;
-  const int nst = (a.d + kSplitCols - 1) / kSplitCols;
+  const int nst = (a.d + Cfg::kCols - 1) / Cfg::kCols;
   const int st_lo = (int)((int64_t)nst * cta_rank / cluster_size);
   const int nloc = (int)((int64_t)nst * (cta_rank + 1) / cluster_size) - st_lo;   // >= 1: cluster_size <= nst
   const int my_tiles = (int)((ntiles - group + groups - 1) / groups);             // 1 with clusters
   const int steps = my_tiles * nloc;
 
   const uint32_t smem_u = smem_u32(smem_raw), smem0 = (smem_u + 1023u) & ~1023u;
-  const uint32_t bars = smem0 + Cfg::kRingBytes;
+  const uint32_t raw0 = smem0 + S * Cfg::kStageBytes, bars = smem0 + Cfg::kRingBytes;
   auto full_bar = [&](int s) { return bars + s * 8; };
-  auto acc_full_bar = [&](int b) { return bars + (2 + b) * 8; };
+  auto empty_bar = [&](int s) { return bars + (2 + s) * 8; };
+  auto acc_full_bar = [&](int b) { return bars + (4 + b) * 8; };
+  auto acc_empty_bar = [&](int b) { return bars + (6 + b) * 8; };
   unsigned char *tail = smem_raw + (bars - smem_u) + Cfg::kBars * 8;
   volatile uint32_t *tmem_slot_ptr = reinterpret_cast<volatile uint32_t *>(tail);
   // bit 0: some row may hold values its split does not; bit 1: U does
@@ -193,13 +207,15 @@ codec_split_project_kernel(const SplitProjectArgs a) {
 
   if (tid == 0) {
     for (int s = 0; s < 2; ++s) {
-      mbar_init(full_bar(s), kSplitProjectWarps);
+      mbar_init(full_bar(s), kSplitRowWarps);
+      mbar_init(empty_bar(s), 1);
       mbar_init(acc_full_bar(s), 1);
+      mbar_init(acc_empty_bar(s), kSplitRowWarps);
     }
     *unsafe = 0;
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
-  if (warp == 1) {
+  if (warp == kSplitRowWarps) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tail)),
                  "r"(Cfg::kTmemCols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
@@ -222,247 +238,311 @@ codec_split_project_kernel(const SplitProjectArgs a) {
   const int quarter = warp & 3, part = warp >> 2;     // TMEM lanes and columns of this warp's sums
   const int sum_row = quarter * 32 + lane, sum_col = part * Cfg::kSums;
 
-  // Four lanes per row; the order of a warp's eight rows makes the swizzled stores conflict-free
-  // (8-byte stores per half warp, 16-byte ones per quarter).
-  const int idx = lane >> 2, q = lane & 3;
-  const int row = warp * 8 + (Cfg::kF32 ? ((idx & 3) << 1 | idx >> 2) : ((idx & 1) << 2 | idx >> 1));
-  const bool vec = a.vec_rows != 0;
-  const T *U = static_cast<const T *>(a.U);
-  const T *ptr[1 + NSLOT];                 // this thread's row: X, then R, E, P as far as present
-  uint4 in[1 + NSLOT][Cfg::kVecs];
-  Pair<T> ureg[Cfg::kPairs];
-  const bool has_r = NSLOT > 0 && a.src2 != nullptr;
-
-  auto row_pointers = [&](int64_t tile) {
-    const int64_t t = tile * kUmmaTile + row;
-    const bool live = t < a.n;
-    ptr[0] = live ? static_cast<const T *>(a.src) + t * a.lds : nullptr;
-    if (NSLOT > 0) {
-      int s = 1;
-      const T *r = nullptr, *e = nullptr, *p = nullptr;
-      if (live) {
-        if (has_r) r = static_cast<const T *>(a.src2) + t * a.lds2;
-        const int64_t er = a.has_e ? embedding_row(a.shift, t) : -1, pr = a.has_p ? position_row(a.shift, t) : -1;
-        if (er >= 0) e = static_cast<const T *>(a.shift.E) + er * a.shift.lde;
-        if (pr >= 0) p = static_cast<const T *>(a.shift.P) + pr * a.shift.ldp;
-      }
-      // slots in the order R, E, P; with constant indexes so that the array stays in registers
-      const T *list[3] = {r, e, p};
-      const bool present[3] = {has_r, a.has_e != 0, a.has_p != 0};
+  if (warp == kSplitRowWarps) {
+    // ------------------------------------------------------------------------- MMA issuer
+    if (lane == 0) {
+      // A: K-major rows of kRowBytes, 8-row groups 8 kRowBytes apart, one part after the other.  B: MN-major,
+      // 64-coordinate groups kGroupBytes apart, 8-row groups 1024 bytes apart.
+      constexpr uint32_t kLayoutA = Cfg::kF32 ? 4 : 2;       // 64- or 128-byte swizzle
+      constexpr uint32_t id1 = umma_idesc(KN, false), id2 = umma_idesc(Cfg::kStack >= 2 ? 2 * KN : KN, false),
+                         id3 = umma_idesc(Cfg::kStack == 3 ? 3 * KN : KN, false);
+      constexpr uint32_t kPart = Cfg::kPartBytes >> 4;                             // next part of A
+      constexpr uint32_t kBPart = (uint32_t)(KN / 64) * (Cfg::kGroupBytes >> 4);   // next part of B (KN = 128 only)
+      int slot = 0, st = 0, in_chain = 0, chain = 0;
+      uint32_t parity = 0;
+      for (int step = 0; step < steps; ++step) {
+        const int buf = chain & 1;
+        if (in_chain == 0 && !dead && !mbar_wait(acc_empty_bar(buf), (uint32_t)(((chain >> 1) & 1) ^ 1))) timed_out();
+        if (!dead && !mbar_wait(full_bar(slot), parity)) timed_out();
+        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+        const uint32_t base = smem0 + (uint32_t)slot * Cfg::kStageBytes;
+        const uint32_t D = tmem_base + (uint32_t)buf * Cfg::kDStride;
+        const uint64_t ad = umma_desc(base, 16, 8 * Cfg::kRowBytes, kLayoutA);
+        const uint64_t bd = umma_desc(base + Cfg::kABytes, Cfg::kGroupBytes, 1024, 2);
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        if (!present[c]) continue;
-#pragma unroll
-        for (int i = 1; i <= NSLOT; ++i)
-          if (i == s) ptr[i] = list[c];
-        ++s;
-      }
-    }
-  };
-  auto issue = [&](int st) {               // rows and slice of U of a stage into registers
-    const int c0 = (st_lo + st) * kSplitCols;
-#pragma unroll
-    for (int i = 0; i < Cfg::kPairs; ++i) {
-      const int p = tid + i * kSplitProjectThreads, kk = p / (KN / 2), j = 2 * (p % (KN / 2));
-      ureg[i] = load_pair<T>(U + (int64_t)(c0 + kk) * a.ldu + j, c0 + kk < a.d ? a.k - j : 0, a.vec_u != 0);
-    }
-#pragma unroll
-    for (int o = 0; o < 1 + NSLOT; ++o)
-#pragma unroll
-      for (int i = 0; i < Cfg::kVecs; ++i)
-        in[o][i] = load_row_piece<T>(ptr[o], c0 + (4 * i + q) * Cfg::kVecElems, a.d, vec);
-  };
-  auto issue_mma = [&](int step) {         // one thread
-    const int buf = step & 1;
-    if (!dead && !mbar_wait(full_bar(buf), (uint32_t)((step >> 1) & 1))) timed_out();
-    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    // A: K-major rows of 128 bytes, 8-row groups 1024 bytes apart, one part after the other.  B: MN-major,
-    // 64-coordinate groups kGroupBytes apart, 8-row groups 1024 bytes apart.
-    constexpr uint32_t id1 = umma_idesc(KN, false), id2 = umma_idesc(Cfg::kStack >= 2 ? 2 * KN : KN, false),
-                       id3 = umma_idesc(Cfg::kStack == 3 ? 3 * KN : KN, false);
-    const uint32_t base = smem0 + (uint32_t)buf * Cfg::kStageBytes;
-    const uint32_t D = tmem_base + (uint32_t)buf * Cfg::kDStride;
-    const uint64_t ad = umma_desc(base, 16, 1024, 2), bd = umma_desc(base + Cfg::kABytes, Cfg::kGroupBytes, 1024, 2);
-    constexpr uint32_t kPart = kSplitPartBytes >> 4;                             // next part of A
-    constexpr uint32_t kBPart = (uint32_t)(KN / 64) * (Cfg::kGroupBytes >> 4);   // next part of B (KN = 128 only)
-#pragma unroll
-    for (int j = 0; j < kSplitCols / 16; ++j) {
-      const uint64_t A = ad + j * 2, B = bd + j * 128;   // 32 bytes of an A row; 16 rows of B
-      const uint32_t more = j > 0 ? 1u : 0u;
-      if (NX == 1) {
-        umma_bf16(D, A, B, id1, more);
-      } else if (NU == 1) {
-        umma_bf16(D, A, B, id1, more);
-        umma_bf16(D + KN, A + kPart, B, id1, more);
-        umma_bf16(D + KN, A + 2 * kPart, B, id1, 1u);
-      } else if (Cfg::kStack == 3) {
-        umma_bf16(D, A, B, id3, more);
-        umma_bf16(D + KN, A + kPart, B, id2, 1u);
-        umma_bf16(D + 2 * KN, A + 2 * kPart, B, id1, 1u);
-      } else {
-        umma_bf16(D, A, B, id2, more);
-        umma_bf16(D + KN, A + kPart, B, id1, 1u);
-        umma_bf16(D + KN, A + kPart, B + kBPart, id1, 1u);
-        umma_bf16(D + KN, A + 2 * kPart, B, id1, 1u);
-        umma_bf16(D + KN, A, B + 2 * kBPart, id1, 1u);
-      }
-    }
-    umma_commit(acc_full_bar(buf));
-  };
-
-  int ld_tile = 0, ld_st = 0;              // the step whose rows are in flight
-  row_pointers(group);
-  issue(0);
-  int fin_tile = 0, fin_st = 0;            // the step whose accumulator is being added
-  uint32_t u_max = 0, row_max = 0;
-  for (int step = 0; step < steps + 2; ++step) {
-    const bool writing = step < steps;
-    float r[NX == 3 ? 16 : 1];             // the residuals of the step, or its rows as they are
-    uint4 raw[NX == 3 ? 1 : Cfg::kVecs];
-    Pair<T> u[Cfg::kPairs];
-    if (writing) {
-#pragma unroll
-      for (int i = 0; i < Cfg::kPairs; ++i) u[i] = ureg[i];
-      if constexpr (NX == 1) {
-#pragma unroll
-        for (int i = 0; i < Cfg::kVecs; ++i) raw[i] = in[0][i];
-      } else {
-        constexpr int E = Cfg::kVecElems;
-#pragma unroll
-        for (int i = 0; i < Cfg::kVecs; ++i) {
-          widen_piece<T>(in[0][i], r + E * i);
-#pragma unroll
-          for (int o = 1; o <= NSLOT; ++o) {
-            float w[E];
-            widen_piece<T>(in[o][i], w);
-            const bool plus = o == 1 && has_r;
-#pragma unroll
-            for (int e = 0; e < E; ++e) r[E * i + e] = plus ? r[E * i + e] + w[e] : r[E * i + e] - w[e];
+        for (int j = 0; j < Cfg::kCols / 16; ++j) {
+          const uint64_t A = ad + j * 2, B = bd + j * 128;   // 32 bytes of an A row; 16 rows of B
+          const uint32_t more = in_chain > 0 || j > 0 ? 1u : 0u;
+          if (NX == 1) {
+            umma_bf16(D, A, B, id1, more);
+          } else if (NU == 1) {
+            umma_bf16(D, A, B, id1, more);
+            umma_bf16(D + KN, A + kPart, B, id1, more);
+            umma_bf16(D + KN, A + 2 * kPart, B, id1, 1u);
+          } else if (Cfg::kStack == 3) {
+            umma_bf16(D, A, B, id3, more);
+            umma_bf16(D + KN, A + kPart, B, id2, 1u);
+            umma_bf16(D + 2 * KN, A + 2 * kPart, B, id1, 1u);
+          } else {
+            umma_bf16(D, A, B, id2, more);
+            umma_bf16(D + KN, A + kPart, B, id1, 1u);
+            umma_bf16(D + KN, A + kPart, B + kBPart, id1, 1u);
+            umma_bf16(D + KN, A + 2 * kPart, B, id1, 1u);
+            umma_bf16(D + KN, A, B + 2 * kBPart, id1, 1u);
           }
         }
-#pragma unroll
-        for (int i = 0; i < 16; ++i) row_max = max(row_max, magnitude_bits(r[i]));
-#pragma unroll
-        for (int i = 0; i < Cfg::kPairs; ++i) u_max = max(u_max, pair_magnitude<T>(u[i]));
-      }
-      if (step + 1 < steps) {
-        if (++ld_st == nloc) {
-          ld_st = 0;
-          ++ld_tile;
-          row_pointers(group + ld_tile * groups);
-          // this thread's part of the row: a row can be unsafe only if one of its parts is
-          if (NX == 3 && split_unsafe(row_max)) atomicOr(unsafe, 1u);
-          row_max = 0;
+        umma_commit(empty_bar(slot));
+        if (++st == nloc) st = 0;
+        if (++in_chain == G || st == 0) {    // chains never reach into the next tile
+          umma_commit(acc_full_bar(buf));
+          in_chain = 0;
+          ++chain;
         }
-        issue(ld_st);
+        if (++slot == S) {
+          slot = 0;
+          parity ^= 1u;
+        }
       }
     }
-    if (warp == 0 && step >= 1 && step <= steps) {
-      if (lane == 0) issue_mma(step - 1);
-      __syncwarp();
-    }
-    if (step >= 2) {
-      // -------- the accumulator of two steps back into the sums
-      const int s2 = step - 2, buf = s2 & 1;
-      if (!dead && !mbar_wait(acc_full_bar(buf), (uint32_t)((s2 >> 1) & 1))) timed_out();
+    __syncwarp();
+  } else {
+    // ------------------------------------------------------------------------- rows, basis, sums
+    // Two 16-byte pieces per operand and step: rows tid / 8 and tid / 8 + 64, piece tid % 8.
+    const int row = tid >> 3, unit = tid & 7;
+    const bool vec = a.vec_rows != 0;
+    // the pairs of U this thread moves: rows u_row, u_row + kURows, ... of the step (8 divides kURows)
+    constexpr int kURows = 2 * kSplitRowThreads / KN;
+    const int u_row = tid / (KN / 2), u_col = 2 * (tid % (KN / 2)), u_valid = max(a.k - u_col, 0);
+    const int64_t u_step = kURows * a.ldu;
+    const bool vec_u = a.vec_u != 0;
+    const T *U = static_cast<const T *>(a.U);
+    const T *ptr[1 + NSLOT][2];              // this thread's rows: X, then R, E, P as far as present
+    Pair<T> ureg[Cfg::kPairs];
+    const bool has_r = NSLOT > 0 && a.src2 != nullptr;
+
+    auto row_pointers = [&](int64_t tile) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int64_t t = min(tile * kUmmaTile + row + 64 * h, a.n - 1);   // past the end: the last row again, never stored
+        ptr[0][h] = static_cast<const T *>(a.src) + t * a.lds;
+        if (NSLOT > 0) {
+          int s = 1;
+          const T *none = vec ? reinterpret_cast<const T *>(g_zero_row) : nullptr;   // an id or position outside its table
+          const T *r = has_r ? static_cast<const T *>(a.src2) + t * a.lds2 : none, *e = none, *p = none;
+          const int64_t er = a.has_e ? embedding_row(a.shift, t) : -1, pr = a.has_p ? position_row(a.shift, t) : -1;
+          if (er >= 0) e = static_cast<const T *>(a.shift.E) + er * a.shift.lde;
+          if (pr >= 0) p = static_cast<const T *>(a.shift.P) + pr * a.shift.ldp;
+          // slots in the order R, E, P; with constant indexes so that the array stays in registers
+          const T *list[3] = {r, e, p};
+          const bool present[3] = {has_r, a.has_e != 0, a.has_p != 0};
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            if (!present[c]) continue;
+#pragma unroll
+            for (int i = 1; i <= NSLOT; ++i)
+              if (i == s) ptr[i][h] = list[c];
+            ++s;
+          }
+        }
+      }
+    };
+    const uint32_t raw_off = (uint32_t)tid * 16;             // + 8192: the second piece
+    auto issue_rows = [&](int st, int rslot) {
+      const int c = (st_lo + st) * Cfg::kCols + unit * Cfg::kVecElems;
+      const uint32_t dst = raw0 + (uint32_t)rslot * Cfg::kRawStepBytes + raw_off;
+      if (vec) {
+        const bool ok = c < a.d;                             // d is a multiple of the piece
+#pragma unroll
+        for (int o = 0; o < 1 + NSLOT; ++o)
+#pragma unroll
+          for (int h = 0; h < 2; ++h) cp_async16_if(dst + o * kSplitRawBytes + h * 8192, ptr[o][h] + (ok ? c : 0), ok);
+      } else {
+#pragma unroll
+        for (int o = 0; o < 1 + NSLOT; ++o)
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const uint4 v = load_row_piece<T>(ptr[o][h], c, a.d);
+            st_shared_v4(dst + o * kSplitRawBytes + h * 8192, v.x, v.y, v.z, v.w);
+          }
+      }
+    };
+    auto issue_u = [&](int st) {
+      const int c0 = (st_lo + st) * Cfg::kCols;
+      const T *up = U + (int64_t)(c0 + u_row) * a.ldu + u_col;
+      if (c0 + Cfg::kCols <= a.d) {          // whole step; a pair past column k stays the zero it is
+        load_pairs<Cfg::kPairs, T>(ureg, [&](int i) { return up + i * u_step; }, u_valid, vec_u);
+      } else {
+#pragma unroll
+        for (int i = 0; i < Cfg::kPairs; ++i) {
+          const bool in = c0 + u_row + i * kURows < a.d;
+          if constexpr (Cfg::kF32) {
+            ureg[i].w[0] = load_global_b32_if(up + i * u_step, in && u_valid > 0);
+            ureg[i].w[1] = load_global_b32_if(up + i * u_step + 1, in && u_valid > 1);
+          } else {
+            ureg[i].w[0] = load_global_b16_if(up + i * u_step, in && u_valid > 0);
+            ureg[i].w[1] = load_global_b16_if(up + i * u_step + 1, in && u_valid > 1);
+          }
+        }
+      }
+    };
+    int chain = 0, fin_tile = 0;             // accumulators written so far, tiles finished
+    // adds accumulator c to the sums; `last`: it completes a tile
+    auto take_chain = [&](int c, bool last) {
+      const int buf = c & 1;
+      if (!dead && !mbar_wait(acc_full_bar(buf), (uint32_t)((c >> 1) & 1))) timed_out();
       asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
       if (sum_col < a.k) {
         const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)buf * Cfg::kDStride + sum_col;
 #pragma unroll
-        for (int c = 0; c < Cfg::kSums; c += 8) {
+        for (int i = 0; i < Cfg::kSums; i += 8) {
           uint32_t v0[8], v1[8], v2[8];
-          tmem_ld8(taddr + c, v0);
-          if (NX > 1) tmem_ld8(taddr + KN + c, v1);
-          if (Cfg::kStack == 3) tmem_ld8(taddr + 2 * KN + c, v2);
+          tmem_ld8(taddr + i, v0);
+          if (NX > 1) tmem_ld8(taddr + KN + i, v1);
+          if (Cfg::kStack == 3) tmem_ld8(taddr + 2 * KN + i, v2);
           asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
 #pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            float v = __uint_as_float(v0[e]);
-            if (Cfg::kStack == 3)
-              v += __uint_as_float(v1[e]) + __uint_as_float(v2[e]);
-            else if (NX > 1)
-              v += __uint_as_float(v1[e]);
-            sum[c + e] += v;
+          for (int e = 0; e < 8; e += 2) {
+            float w0 = __uint_as_float(v0[e]), w1 = __uint_as_float(v0[e + 1]);
+            if (Cfg::kStack == 3) {
+              float x0 = __uint_as_float(v1[e]), x1 = __uint_as_float(v1[e + 1]);
+              add2(x0, x1, __uint_as_float(v2[e]), __uint_as_float(v2[e + 1]));
+              add2(w0, w1, x0, x1);
+            } else if (NX > 1) {
+              add2(w0, w1, __uint_as_float(v1[e]), __uint_as_float(v1[e + 1]));
+            }
+            add2(sum[i + e], sum[i + e + 1], w0, w1);
           }
         }
       }
       asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-      if (++fin_st == nloc) {              // a tile is complete
-        fin_st = 0;
+      __syncwarp();
+      if (lane == 0) mbar_arrive(acc_empty_bar(buf));
+      if (last) {
         const int64_t t = (group + (int64_t)fin_tile * groups) * kUmmaTile + sum_row;
         ++fin_tile;
         if (cluster_size == 1) {
           if (t < a.n) {
 #pragma unroll
-            for (int c = 0; c < Cfg::kSums; c += 4)
-              store_coords4<T>(a, t, sum_col + c, {sum[c], sum[c + 1], sum[c + 2], sum[c + 3]});
+            for (int i = 0; i < Cfg::kSums; i += 4)
+              store_coords4<T>(a, t, sum_col + i, {sum[i], sum[i + 1], sum[i + 2], sum[i + 3]});
             if (a.wire_ids && part == 0) static_cast<int32_t *>(a.zout)[t * a.ldzout + a.k] = a.shift.ids[t];
           }
 #pragma unroll
           for (int i = 0; i < Cfg::kSums; ++i) sum[i] = 0.f;
         }
       }
-    }
-    if (writing) {
-      // -------- residuals and basis into the stage
-      const uint32_t base = smem0 + (uint32_t)(step & 1) * Cfg::kStageBytes;
-      const uint32_t arow = base + row * 128;
-      if constexpr (NX == 1) {             // columns 32 i + 8 q .. +7
-#pragma unroll
-        for (int i = 0; i < Cfg::kVecs; ++i)
-          st_shared_v4(arow + (((4 * i + q) ^ (row & 7)) << 4), raw[i].x, raw[i].y, raw[i].z, raw[i].w);
-      } else if constexpr (Cfg::kF32) {    // columns 16 i + 4 q .. +3
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          uint32_t lo[3], hi[3];
-          split_pair<3>(r[4 * i], r[4 * i + 1], lo);
-          split_pair<3>(r[4 * i + 2], r[4 * i + 3], hi);
-          const uint32_t addr = arow + (((2 * i + (q >> 1)) ^ (row & 7)) << 4) + (q & 1) * 8;
-#pragma unroll
-          for (int p = 0; p < 3; ++p) st_shared_v2(addr + p * kSplitPartBytes, lo[p], hi[p]);
+    };
+
+    int ld_tile = 0, ld_st = 0, ld_slot = 0;
+    auto advance_rows = [&](bool more) {     // requests one more step (or commits an empty group)
+      if (more) {
+        if (ld_st == 0) row_pointers(group + (int64_t)ld_tile * groups);
+        issue_rows(ld_st, ld_slot);
+        if (++ld_st == nloc) {
+          ld_st = 0;
+          ++ld_tile;
         }
-      } else {                             // columns 32 i + 8 q .. +7
+        if (++ld_slot == RD) ld_slot = 0;
+      }
+      cp_async_commit();
+    };
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-          uint32_t w[4][3];
+    for (int i = 0; i < Cfg::kPairs; ++i) ureg[i].w[0] = ureg[i].w[1] = 0;
+    issue_u(0);
+    for (int i = 0; i < RD - 1; ++i) advance_rows(i < steps);
+
+    int slot = 0, rslot = 0, st = 0, in_chain = 0;
+    uint32_t parity = 1;
+    bool prev_last = false;
+    float u_max = 0.f, row_max[2] = {0.f, 0.f};
+    const uint32_t a_off = Cfg::kF32 ? row * 64 + (((unit >> 1) ^ ((row >> 1) & 3)) << 4) + (unit & 1) * 8
+                                     : row * 128 + ((unit ^ (row & 7)) << 4);   // + 64 rows: the second piece
+    for (int step = 0; step < steps; ++step) {
+      cp_async_wait<RD - 2>();
+      const int next_st = st + 1 == nloc ? 0 : st + 1;
+      uint4 x[2], w[NSLOT > 0 ? NSLOT : 1][2];
+      const uint32_t src = raw0 + (uint32_t)rslot * Cfg::kRawStepBytes + raw_off;
 #pragma unroll
-          for (int e = 0; e < 4; ++e) split_pair<3>(r[8 * i + 2 * e], r[8 * i + 2 * e + 1], w[e]);
-          const uint32_t addr = arow + (((4 * i + q) ^ (row & 7)) << 4);
+      for (int h = 0; h < 2; ++h) {
+        x[h] = ld_shared_v4(src + h * 8192);
 #pragma unroll
-          for (int p = 0; p < 3; ++p) st_shared_v4(addr + p * kSplitPartBytes, w[0][p], w[1][p], w[2][p], w[3][p]);
+        for (int o = 0; o < NSLOT; ++o) w[o][h] = ld_shared_v4(src + (o + 1) * kSplitRawBytes + h * 8192);
+      }
+      if (!dead && !mbar_wait(empty_bar(slot), parity)) timed_out();
+      const uint32_t base = smem0 + (uint32_t)slot * Cfg::kStageBytes;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const uint32_t addr = base + a_off + h * 64 * Cfg::kRowBytes;
+        if constexpr (NX == 1) {
+          st_shared_v4(addr, x[h].x, x[h].y, x[h].z, x[h].w);
+        } else {
+          constexpr int E = Cfg::kVecElems;
+          float r[E];
+          widen_piece<T>(x[h], r);
+#pragma unroll
+          for (int o = 0; o < NSLOT; ++o) {
+            float v[E];
+            widen_piece<T>(w[o][h], v);
+            const bool plus = o == 0 && has_r;
+#pragma unroll
+            for (int e = 0; e < E; e += 2) {
+              if (plus) add2(r[e], r[e + 1], v[e], v[e + 1]);
+              else sub2(r[e], r[e + 1], v[e], v[e + 1]);
+            }
+          }
+#pragma unroll
+          for (int e = 0; e < E; ++e) row_max[h] = fmaxf(row_max[h], fabsf(r[e]));
+          uint32_t p[E / 2][3];
+#pragma unroll
+          for (int e = 0; e < E / 2; ++e) split_pair<3>(r[2 * e], r[2 * e + 1], p[e]);
+#pragma unroll
+          for (int i = 0; i < 3; ++i) {
+            if constexpr (Cfg::kF32) st_shared_v2(addr + i * Cfg::kPartBytes, p[0][i], p[1][i]);
+            else st_shared_v4(addr + i * Cfg::kPartBytes, p[0][i], p[1][i], p[2][i], p[3][i]);
+          }
         }
       }
-      const uint32_t bbase = base + Cfg::kABytes;
 #pragma unroll
       for (int i = 0; i < Cfg::kPairs; ++i) {
-        const int p = tid + i * kSplitProjectThreads, kk = p / (KN / 2), j = 2 * (p % (KN / 2));
+        const Pair<T> u = joined<T>(ureg[i]);
+        if (NX == 3) u_max = fmaxf(u_max, pair_magnitude<T>(u));
         uint32_t up[NU];
-        split_pair<T, NU>(u[i], up);
+        split_pair<T, NU>(u, up);
 #pragma unroll
         for (int s = 0; s < NU; ++s) {
-          const int n = s * KN + j;
-          st_shared_b32(bbase + (n >> 6) * Cfg::kGroupBytes + kk * 128 + ((((n & 63) >> 3) ^ (kk & 7)) << 4) + (n & 7) * 2,
-                        up[s]);
+          const int n = s * KN + u_col;
+          st_shared_b32(base + Cfg::kABytes + (n >> 6) * Cfg::kGroupBytes + (u_row + i * kURows) * 128 +
+                            ((((n & 63) >> 3) ^ (u_row & 7)) << 4) + (n & 7) * 2, up[s]);
         }
       }
       asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
       __syncwarp();
-      if (lane == 0) mbar_arrive(full_bar(step & 1));
+      if (lane == 0) mbar_arrive(full_bar(slot));
+      if (step + 1 < steps) issue_u(next_st);
+      advance_rows(step + RD - 1 < steps);   // into the slot read in the step before
+      if (++slot == S) {
+        slot = 0;
+        parity ^= 1u;
+      }
+      if (++rslot == RD) rslot = 0;
+      st = next_st;
+      if (st == 0 && NX == 3) {
+        // the tile's rows are complete: a row can be unsafe only if this thread's part of it is
+        if (split_unsafe(row_max[0]) || split_unsafe(row_max[1])) atomicOr(unsafe, 1u);
+        row_max[0] = row_max[1] = 0.f;
+      }
+      if (++in_chain == G || st == 0) {      // the accumulator before the one just filled
+        if (chain > 0) take_chain(chain - 1, prev_last);
+        prev_last = st == 0;
+        in_chain = 0;
+        ++chain;
+      }
     }
-  }
-  if (NX == 3) {
-    if (split_unsafe(row_max)) atomicOr(unsafe, 1u);
-    if (u_max >= kSplitHugeBits) atomicOr(unsafe, 2u);
+    take_chain(chain - 1, true);
+    cp_async_wait<0>();
+    if (NX == 3 && u_max >= kSplitHuge) atomicOr(unsafe, 2u);
   }
 
   if (cluster_size > 1) {
-    // Every accumulator has been read, so every stage is consumed and the ring can carry the sums.
+    // Every accumulator has been read, so every stage is consumed and the rings can carry the sums.
     __syncthreads();
-    const uint32_t dst = smem0 + (uint32_t)(sum_row * Cfg::kSumPitch + sum_col) * 4;
+    if (warp < kSplitRowWarps) {
+      const uint32_t dst = smem0 + (uint32_t)(sum_row * Cfg::kSumPitch + sum_col) * 4;
 #pragma unroll
-    for (int c = 0; c < Cfg::kSums; c += 4)
-      st_shared_v4(dst + c * 4, __float_as_uint(sum[c]), __float_as_uint(sum[c + 1]), __float_as_uint(sum[c + 2]),
-                   __float_as_uint(sum[c + 3]));
+      for (int c = 0; c < Cfg::kSums; c += 4)
+        st_shared_v4(dst + c * 4, __float_as_uint(sum[c]), __float_as_uint(sum[c + 1]), __float_as_uint(sum[c + 2]),
+                     __float_as_uint(sum[c + 3]));
+    }
     asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
     const int rows = kUmmaTile / (int)cluster_size, row0 = rows * (int)cta_rank;
     auto peer = [](uint32_t addr, uint32_t rank) {
@@ -493,13 +573,13 @@ codec_split_project_kernel(const SplitProjectArgs a) {
         bad |= f;
       }
     }
-    // nobody leaves while its sums can still be read
+    // nobody leaves while its sums can still be read; and the rows above are stored
     asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
     if (NX == 3 && bad != 0) project_unsafe_rows<T>(a, group, row0, rows, (bad & 2) != 0);
   }
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   __syncthreads();
-  if (warp == 1) {
+  if (warp == kSplitRowWarps) {
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem_base), "r"(Cfg::kTmemCols)
                  : "memory");
