@@ -149,7 +149,13 @@ bool codec_mma_supports(int d, int k) {
 
 cudaError_t launch_codec_mma(const MmaArgs &a, bool shift, int mode, int sm_count,
                              cudaStream_t stream) {
-  if (mode == kModeProject) {
+  // Up to 16 tokens per SM the few-rows kernel has the shorter start: it wins until its own work (its warps
+  // read all of U) outgrows that, at about 65536 elements of U.  us, E and P rows, tcgen05 -> few rows: 2048
+  // tokens, rank 40: 512 columns 10.0 -> 6.8, 1536 columns 13.1 -> 10.5, 4096 columns 21.1 -> 21.1 (no tables: 15.9
+  // -> 18.9); rank 16, 4096 columns 20.2 -> 13.6.  Wire rows keep their kernel.
+  const bool few_rows = a.n <= 16 * (int64_t)sm_count && a.k <= 64 && (int64_t)a.d * a.k <= 65536 &&
+                        a.zout32 == nullptr && a.src2 == nullptr;
+  if (mode == kModeProject && !few_rows) {
     cudaError_t e = launch_codec_umma_project(a, shift, sm_count, stream);
     if (e != cudaErrorNotSupported) return e;
   }
@@ -168,8 +174,12 @@ cudaError_t launch_codec_mma(const MmaArgs &a, bool shift, int mode, int sm_coun
   // The tcgen05 expansion deals (tile, chunk) units to the SMs, so it fills the machine from 512
   // tokens on; measured against the few-rows kernel it wins wherever the output is 8 MB or more,
   // the model is wide or the rank needs the wide mma.sync tiles (16384 tokens, d = 4096: 48 us
-  // against 127 us), and loses a few microseconds of set-up on the smallest outputs.
-  if (small && mode == kModeExpand && (a.n * a.d >= (1 << 22) || a.d >= 2048 || nt > 8)) {
+  // against 127 us), and on smaller ones from 32768 elements of U per 16 tokens of an SM on (E and P rows, few
+  // rows -> tcgen05: rank 40, 2048 x 1024 8.8 -> 8.4 us, 3072 x 512 10.4 -> 8.1, 7168 x 256 16.3 -> 8.4; rank 16,
+  // 7168 x 512 12.7 -> 10.7); below that it loses a few microseconds of set-up (rank 16, 2048 x 1024 6.3 -> 8.4).
+  const int64_t row_groups = (a.n + 16 * (int64_t)sm_count - 1) / (16 * (int64_t)sm_count);
+  if (small && mode == kModeExpand &&
+      (a.n * a.d >= (1 << 22) || a.d >= 2048 || nt > 8 || (int64_t)a.d * a.k * row_groups >= 32768)) {
     cudaError_t e = launch_codec_umma_expand(a, shift, sm_count, stream);
     if (e != cudaErrorNotSupported) return e;
   }

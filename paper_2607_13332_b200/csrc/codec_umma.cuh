@@ -17,9 +17,11 @@
 //   warps 4-7  epilogue: tcgen05.ld their 32 TMEM lanes (one token per thread), combine the
 //            accumulators, round to bf16, store the Z rows; two sets of accumulators let a tile's
 //            epilogue overlap the next tile's MMAs.
-//   warps 8-11 (with E rows only)  gather the E rows of the tile: 8 lanes copy one 128-byte row
-//            piece with cp.async straight into the swizzled tile, some stages ahead of the
-//            barrier arrival that publishes them (an id outside the table points at a row of zeros).
+//   warps 8-11 (with E rows, or P rows that TMA cannot fetch)  gather those rows of the tile: 8 lanes
+//            copy one 128-byte row piece with cp.async straight into the swizzled tile, some stages ahead of
+//            the barrier arrival that publishes them (an id or position outside the table points at a row
+//            of zeros).  P rows are gathered (kPGather) when positions are given per token or a tile's are
+//            not consecutive; otherwise they come by TMA (kPTma).
 //   A launch carries only the warps its roles need (8, 12 or 13).
 //
 // X, E and P tiles use the 128-byte swizzled K-major layout (rows of 128 bytes); U arrives as a
@@ -230,8 +232,12 @@ __device__ __forceinline__ void store_projected_row(const MmaArgs &a, int64_t t,
   }
 }
 
-template <int NTP, bool HAS_E, bool HAS_P>
+enum { kPNone = 0, kPTma = 1, kPGather = 2 };   // where the P rows of a projection come from
+
+template <int NTP, bool HAS_E, int PMODE>
 struct UmmaProjectConfig {
+  static constexpr bool HAS_P = PMODE != kPNone;
+  static constexpr bool kGathers = HAS_E || PMODE == kPGather;
   static_assert(NTP % 2 == 0 && NTP >= 2 && NTP <= 16, "N = 8*NTP must be a multiple of 16 up to 128");
   static constexpr int kN = NTP * 8;
   static constexpr int kATileBytes = kUmmaTile * 128;               // 128 rows of 128 bytes
@@ -240,7 +246,7 @@ struct UmmaProjectConfig {
   static constexpr int kUGroupBytes = kUmmaCols * 128;              // 64 rows of 128 bytes
   static constexpr int kUBytes = kUGroups * kUGroupBytes;
   static constexpr int kStageBytes = kATiles * kATileBytes + kUBytes;
-  static constexpr int kTmaBytes = kStageBytes - (HAS_E ? kATileBytes : 0);
+  static constexpr int kTmaBytes = kStageBytes - (HAS_E ? kATileBytes : 0) - (PMODE == kPGather ? kATileBytes : 0);
   static constexpr int kMaxSmem = 227 * 1024;
   static constexpr int kFit = (kMaxSmem - 1024 - 512) / kStageBytes;
   static constexpr int kStagesN = kFit < 10 ? kFit : 10;
@@ -266,7 +272,7 @@ struct UmmaProjectConfig {
   // warp 12 is the fourth issuer (E only, k <= 64).  A launch has only the warps its roles need, so
   // that the register budget of the epilogue (a whole accumulator row per thread) is not cut by
   // warps that would idle: 256 threads without E rows, 384 or 416 with them.
-  static constexpr int kWarps = !HAS_E ? 8 : (kIssuers == 4 ? 13 : 12);
+  static constexpr int kWarps = !kGathers ? 8 : (kIssuers == 4 ? 13 : 12);
   static constexpr int kThreads = 32 * kWarps;
   static constexpr int kBufs = 2 * kIssuers * kAccCols <= 512 ? 2 : 1;   // accumulator sets (tiles in flight)
   // accumulator slots: kIssuers per buffer; a launch that shares the positional product keeps it
@@ -308,10 +314,11 @@ cudaError_t launch_tile_pairs(Kernel kernel, int threads, int smem, const MmaArg
   return launch_dependent(kernel, (unsigned)grid, threads, smem, stream, 1, a, maps);
 }
 
-template <int NTP, bool HAS_E, bool HAS_P>
-__global__ void __launch_bounds__((UmmaProjectConfig<NTP, HAS_E, HAS_P>::kThreads), 1)
+template <int NTP, bool HAS_E, int PMODE>
+__global__ void __launch_bounds__((UmmaProjectConfig<NTP, HAS_E, PMODE>::kThreads), 1)
 codec_umma_project_kernel(const MmaArgs a, const __grid_constant__ UmmaMaps maps) {
-  using Cfg = UmmaProjectConfig<NTP, HAS_E, HAS_P>;
+  using Cfg = UmmaProjectConfig<NTP, HAS_E, PMODE>;
+  constexpr bool HAS_P = Cfg::HAS_P;
   constexpr int kETile = 1, kPTile = HAS_E ? 2 : 1;   // order of the tiles inside a stage
   constexpr int S = Cfg::kStagesN;
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -349,7 +356,7 @@ codec_umma_project_kernel(const MmaArgs a, const __grid_constant__ UmmaMaps maps
   // enumerated position-block-major (L = block * sequences + sequence), every pair takes a
   // contiguous range of L, and a CTA keeps P U of its current block in a persistent accumulator:
   // the P rows are loaded and contracted only when the block changes.
-  constexpr bool kCanShare = HAS_E && HAS_P && Cfg::kN <= 64;
+  constexpr bool kCanShare = HAS_E && PMODE == kPTma && Cfg::kN <= 64;
   const bool pshare = kCanShare && a.pshare != 0;
   const int64_t nseq = pshare ? a.n / a.shift.seq_len : 1;
   const int64_t nblk = pshare ? a.shift.seq_len / kUmmaTile : 1;
@@ -397,7 +404,7 @@ codec_umma_project_kernel(const MmaArgs a, const __grid_constant__ UmmaMaps maps
     mbar_init(partial_ready_bar, 64);   // the threads of the peer's two sending warps
     mbar_init(ring_free_bar, 2);        // the peer's two receiving warps
     for (int s = 0; s < S; ++s) {
-      mbar_init(full_bar(s), HAS_E ? 5 : 1);
+      mbar_init(full_bar(s), Cfg::kGathers ? 5 : 1);
       mbar_init(empty_bar(s), Cfg::kATiles);   // one commit per operand (the X threads take turns)
     }
     for (int b = 0; b < 2; ++b) {
@@ -438,14 +445,14 @@ codec_umma_project_kernel(const MmaArgs a, const __grid_constant__ UmmaMaps maps
       bool split;
       schedule(it, tile, st_lo, st_hi, split);
       const int64_t tok0 = tile * kUmmaTile;
-      const int pos0 = HAS_P ? (int)(tok0 % a.shift.seq_len) : 0;
-      const bool load_p = HAS_P && p_action(it, split, cached_blk) == 0;
+      const int pos0 = PMODE == kPTma ? (int)(tok0 % a.shift.seq_len) : 0;
+      const bool load_p = PMODE == kPTma && p_action(it, split, cached_blk) == 0;
       for (int st = st_lo; st < st_hi; ++st) {
         if (!dead && !mbar_wait(empty_bar(slot), parity)) timed_out();
         const uint32_t base = smem0 + (uint32_t)slot * Cfg::kStageBytes;
         const uint32_t bar = full_bar(slot);
         if (lane == 0) {
-          mbar_expect_tx(bar, Cfg::kTmaBytes - (HAS_P && !load_p ? Cfg::kATileBytes : 0));
+          mbar_expect_tx(bar, Cfg::kTmaBytes - (PMODE == kPTma && !load_p ? Cfg::kATileBytes : 0));
           const int su = st < nstage1 ? st : st - nstage1;   // slice of U; the second matrix starts over
           tma_load_2d_hint(base, st < nstage1 ? &maps.x : &maps.x2, bar, su * kUmmaCols, (int)tok0, stream_in);
           if (load_p) tma_load_2d_hint(base + kPTile * Cfg::kATileBytes, &maps.p, bar, st * kUmmaCols, pos0, keep);
@@ -534,8 +541,8 @@ codec_umma_project_kernel(const MmaArgs a, const __grid_constant__ UmmaMaps maps
       }
     }
   } else if (warp >= 8) {
-    // ------------------------------------------------------------------------- E row gather
-    if (HAS_E) {
+    // ------------------------------------------------------------------------- row gather (E, P)
+    if (Cfg::kGathers) {
       const int gw = warp - 8;                 // rows 32*gw .. 32*gw+31 of the tile
       const int piece = lane & 7, sub = lane >> 3;
       int slot = 0, pub_slot = 0, pending = 0;
@@ -553,23 +560,34 @@ codec_umma_project_kernel(const MmaArgs a, const __grid_constant__ UmmaMaps maps
         bool split;
         schedule(it, tile, st_lo, st_hi, split);
         const int64_t tok0 = tile * kUmmaTile;
-        const unsigned char *src[8];
+        const unsigned char *src[8], *psrc[8];
         uint32_t dst[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
           const int r = gw * 32 + i * 4 + sub;
           const int64_t t = tok0 + r;
-          const int64_t er = t < a.n ? embedding_row(a.shift, t) : -1;
-          src[i] = (er >= 0 ? reinterpret_cast<const unsigned char *>(
-                                  static_cast<const __nv_bfloat16 *>(a.shift.E) + er * a.shift.lde)
-                            : g_zero_row) + piece * 16;
-          dst[i] = kETile * Cfg::kATileBytes + r * 128 + ((piece ^ (r & 7)) << 4);
+          if (HAS_E) {
+            const int64_t er = t < a.n ? embedding_row(a.shift, t) : -1;
+            src[i] = (er >= 0 ? reinterpret_cast<const unsigned char *>(
+                                    static_cast<const __nv_bfloat16 *>(a.shift.E) + er * a.shift.lde)
+                              : g_zero_row) + piece * 16;
+          }
+          if (PMODE == kPGather) {
+            const int64_t pr = t < a.n ? position_row(a.shift, t) : -1;
+            psrc[i] = (pr >= 0 ? reinterpret_cast<const unsigned char *>(
+                                     static_cast<const __nv_bfloat16 *>(a.shift.P) + pr * a.shift.ldp)
+                               : g_zero_row) + piece * 16;
+          }
+          dst[i] = r * 128 + ((piece ^ (r & 7)) << 4);
         }
         for (int st = st_lo; st < st_hi; ++st) {
           if (!dead && !mbar_wait(empty_bar(slot), parity)) timed_out();
           const uint32_t base = smem0 + (uint32_t)slot * Cfg::kStageBytes;
 #pragma unroll
-          for (int i = 0; i < 8; ++i) cp_async16_cg(base + dst[i], src[i] + st * 128);
+          for (int i = 0; i < 8; ++i) {
+            if (HAS_E) cp_async16_cg(base + kETile * Cfg::kATileBytes + dst[i], src[i] + st * 128);
+            if (PMODE == kPGather) cp_async16_cg(base + kPTile * Cfg::kATileBytes + dst[i], psrc[i] + st * 128);
+          }
           cp_async_commit();
           if (++pending > Cfg::kGatherLag) {
             cp_async_wait<Cfg::kGatherLag>();

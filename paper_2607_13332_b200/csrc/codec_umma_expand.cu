@@ -6,6 +6,15 @@
 namespace ssn {
 namespace {
 
+// Whether the P rows may be gathered: us against the mma.sync kernels, E and P rows (theirs -> this one),
+// 10007 tokens: 512 columns 28 -> 16, 2048 columns 56 -> 25; 40000 x 512: 32 -> 28.  Narrower rows gain nothing
+// (10007 x 256, rank 72: 12 -> 15), nor do E and P rows of up to 16 tokens per SM (2155 x 2048: 13.6 -> 13.8,
+// rank 24 11.0 -> 13.6) unless the rank or a second run of coordinates needs their wide tiles (45 -> 14).
+bool gathers_positions(const MmaArgs &a, bool has_e, int sm_count) {
+  if (a.d < 512 || a.rowsumsq != nullptr) return false;
+  return !has_e || a.k > 64 || a.zin2 != nullptr || a.n > 16 * (int64_t)sm_count;
+}
+
 template <int KG, bool HAS_E, bool HAS_P, int PROWS = kGridPos>
 cudaError_t launch_umma_expand_one(const MmaArgs &a, const ExpandGeometry &geo, const UmmaExpandMaps &maps,
                                    int sm_count, cudaStream_t stream) {
@@ -21,16 +30,17 @@ cudaError_t launch_umma_expand_one(const MmaArgs &a, const ExpandGeometry &geo, 
   const cudaError_t launched = launch_dependent(kernel, (unsigned)grid, kExpandThreads, smem, stream, 1, a, geo, maps);
   note_kernel(SSN_KERNEL_UMMA_EXPAND, (HAS_E ? SSN_KVAR_E : 0) | (HAS_P ? SSN_KVAR_P : 0) | (KG == 2 ? SSN_KVAR_WIDE : 0) |
                                           (geo.grid_mode ? SSN_KVAR_ALT : 0) | (a.rowsumsq != nullptr ? SSN_KVAR_ROWSUMSQ : 0) |
-                                          (PROWS != kGridPos ? SSN_KVAR_FEWSEQ : 0) | (a.zin2 != nullptr ? SSN_KVAR_TWO_RUNS : 0));
+                                          (PROWS == kUmmaTile ? SSN_KVAR_FEWSEQ : 0) | (a.zin2 != nullptr ? SSN_KVAR_TWO_RUNS : 0));
   return launched;
 }
 
 }  // namespace
 
 // Expansion (decompress) on tcgen05.  Returns cudaErrorNotSupported when the call should take the
-// mma.sync kernel instead: k > 128, d not a multiple of 128, few tokens, no tensor map, or a
-// position table with explicit positions / a batch that is not made of whole sequences that tile
-// into g sequences x 128/g positions (g = 8: length a multiple of 16; else g = 4, 2, 1 with k <= 64).
+// mma.sync kernel instead: k > 128, d not a multiple of 128, few tokens, no tensor map, or narrow rows
+// whose positions no tile of sequences fits.  A tile is g sequences x 128/g positions (g = 8: length a multiple
+// of 16; else g = 4, 2, 1 with k <= 64) of a batch of whole sequences with implicit positions; with any
+// other positions its P rows are gathered.
 cudaError_t launch_codec_umma_expand(const MmaArgs &a, bool shift, int sm_count, cudaStream_t stream) {
   if (a.zin == nullptr || a.dst == nullptr || a.src != nullptr) return cudaErrorNotSupported;
   if (a.d % kChunkCols != 0 || a.k > 128 || a.n < 4 * kUmmaTile || a.n > 0x7fffffffLL)
@@ -39,23 +49,28 @@ cudaError_t launch_codec_umma_expand(const MmaArgs &a, bool shift, int sm_count,
   const bool has_e = shift && a.shift.E != nullptr, has_p = shift && a.shift.P != nullptr;
   ExpandGeometry geo{};
   geo.seq_len = a.shift.seq_len;
+  bool gather_p = false;
   if (has_p) {
     const int64_t L = a.shift.seq_len;
-    if (a.shift.pos != nullptr || L < 1 || L > a.shift.max_pos || a.n % L != 0) return cudaErrorNotSupported;
+    const bool whole = a.shift.pos == nullptr && L >= 1 && L <= a.shift.max_pos && a.n % L == 0;
     // tiles of gseqs sequences x gpos positions: 8 x 16 when the batch allows, else the widest
     // group of sequences that divides it (a small call of 1 to 6 sequences)
-    const int64_t B = a.n / L;
+    const int64_t B = whole ? a.n / L : 0;
     int gseqs = 0;
-    for (int g = kGridSeqs; g >= 1 && gseqs == 0; g >>= 1)
+    for (int g = kGridSeqs; whole && g >= 1 && gseqs == 0; g >>= 1)
       if (B % g == 0 && L % (kUmmaTile / g) == 0) gseqs = g;
-    if (gseqs == 0 || (gseqs != kGridSeqs && a.k > 64)) return cudaErrorNotSupported;
-    geo.grid_mode = 1;
-    geo.gseqs = gseqs;
-    geo.gpos = kUmmaTile / gseqs;
-    geo.nsg = (int32_t)(B / gseqs);
-    geo.ntiles = (int64_t)geo.nsg * (L / geo.gpos);
-  } else {
-    geo.grid_mode = 0;
+    if (gseqs == 0 || (gseqs != kGridSeqs && a.k > 64)) {
+      if (!gathers_positions(a, has_e, sm_count)) return cudaErrorNotSupported;
+      gather_p = true;
+    } else {
+      geo.grid_mode = 1;
+      geo.gseqs = gseqs;
+      geo.gpos = kUmmaTile / gseqs;
+      geo.nsg = (int32_t)(B / gseqs);
+      geo.ntiles = (int64_t)geo.nsg * (L / geo.gpos);
+    }
+  }
+  if (!geo.grid_mode) {
     geo.nsg = 1;
     geo.ntiles = (a.n + kUmmaTile - 1) / kUmmaTile;
   }
@@ -88,6 +103,13 @@ cudaError_t launch_codec_umma_expand(const MmaArgs &a, bool shift, int sm_count,
   }
   if (!make_sw128_map(&maps.u, a.U, a.d, a.k, a.ldu, kUmmaCols)) return cudaErrorNotSupported;
   if (!make_sw128_map(&maps.u_wide, a.U, a.d, a.k <= 64 ? 64 : 128, a.ldu, kUmmaCols)) return cudaErrorNotSupported;
+  if (gather_p) {
+    if (a.k > 64)
+      return has_e ? launch_umma_expand_one<2, true, true, 0>(a, geo, maps, sm_count, stream)
+                   : launch_umma_expand_one<2, false, true, 0>(a, geo, maps, sm_count, stream);
+    return has_e ? launch_umma_expand_one<1, true, true, 0>(a, geo, maps, sm_count, stream)
+                 : launch_umma_expand_one<1, false, true, 0>(a, geo, maps, sm_count, stream);
+  }
   if (has_p && geo.gseqs != kGridSeqs) {   // few sequences: room for up to 128 rows of P per chunk
     if (has_e) return launch_umma_expand_one<1, true, true, kUmmaTile>(a, geo, maps, sm_count, stream);
     return launch_umma_expand_one<1, false, true, kUmmaTile>(a, geo, maps, sm_count, stream);

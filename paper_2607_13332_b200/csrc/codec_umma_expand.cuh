@@ -14,7 +14,9 @@
 // 8 sequences take g = 8: 16 rows of P and ONE more MMA per chunk (PROWS = 16).  Other batches
 // (the 1 to 6 sequences of a small call) take g = 4, 2 or 1 in the PROWS = 128 variant, which
 // reserves shared memory for up to 128 rows of P per chunk and issues 128/(16 g) MMAs for them.
-// Without P a tile is 128 consecutive tokens.
+// Without P a tile is 128 consecutive tokens.  Positions per token, and lengths no such tile fits, take
+// the PROWS = 0 variant: 128 consecutive tokens whose P rows are gathered like the E rows, into the
+// same ring (E piece, then P piece), and added by the epilogue.
 //
 //   warp 0     producer: per tile the Z tile; per chunk the 128 rows of U (K-major operand)
 //              and the 16 rows of P.
@@ -69,32 +71,35 @@ __device__ __forceinline__ void tma_store_3d(const CUtensorMap *map, uint32_t sr
 
 template <int KG, bool HAS_E, bool HAS_P, int PROWS = kGridPos>
 struct UmmaExpandConfig {
-  static_assert(PROWS == 16 || PROWS == 128, "rows of P per chunk the kernel reserves room for");
+  static_assert(PROWS == 0 || PROWS == 16 || PROWS == 128, "rows of P per chunk the kernel reserves room for");
+  static constexpr bool kPGathered = HAS_P && PROWS == 0, kPOperand = HAS_P && PROWS != 0;
+  // tables whose rows are gathered: stages of the ring per 64 columns
+  static constexpr int kGathered = (HAS_E ? 1 : 0) + (kPGathered ? 1 : 0);
   static constexpr int kTileBytes = kUmmaTile * 128;            // [128 rows x 128 B]
   static constexpr int kZBytes = KG * kTileBytes;               // one Z tile: KG groups of 64 coordinates
   // With E and two coordinate groups the E ring would have 4 stages only: one Z tile instead of two
   // buys two more (the MMAs run up to two chunks ahead of the epilogue, which hides most of the
   // load of the next tile's Z).  With one group the ring is deep enough and the second tile pays.
-  static constexpr int kZBufs = (HAS_E && KG == 2) ? 1 : 2;
+  static constexpr int kZBufs = (kGathered > 0 && KG == 2) ? 1 : 2;
   static constexpr int kU2Bytes = KG * kChunkCols * 128;        // 128 rows of U, K-major, KG groups
-  static constexpr int kPBytes = HAS_P ? 2 * PROWS * 128 : 0;      // PROWS rows of P, two 64-column groups
-  static constexpr int kSelBytes = HAS_P ? (PROWS <= 64 ? 1 : 2) * kTileBytes : 0;   // one tile per 64 positions
+  static constexpr int kPBytes = kPOperand ? 2 * PROWS * 128 : 0;      // PROWS rows of P, two 64-column groups
+  static constexpr int kSelBytes = kPOperand ? (PROWS <= 64 ? 1 : 2) * kTileBytes : 0;   // one tile per 64 positions
   static constexpr int kUStageBytes = kU2Bytes + kPBytes;
   // with E the shared memory is better spent on its ring; 128 rows of P per stage leave room for two
-  static constexpr int kUStages = (HAS_E || KG == 2 || (HAS_P && PROWS > kGridPos)) ? 2 : 3;
+  static constexpr int kUStages = (kGathered > 0 || KG == 2 || (HAS_P && PROWS > kGridPos)) ? 2 : 3;
   static constexpr int kEStageBytes = kTileBytes;               // E rows of 64 columns of a chunk
   // Without E the epilogue warps stage their output in two [32 x 128 B] slabs each; with E the
   // sum is formed in place in the E stage, which is then the source of the TMA store.
-  static constexpr int kStagingBytes = HAS_E ? 0 : 8 * 2 * 4096;
+  static constexpr int kStagingBytes = kGathered > 0 ? 0 : 8 * 2 * 4096;
   static constexpr int kFixedBytes =
       kZBufs * kZBytes + kSelBytes + kUStages * kUStageBytes + kStagingBytes;
   static constexpr int kMaxSmem = 227 * 1024;
   static constexpr int kEFit = (kMaxSmem - 1024 - 1024 - kFixedBytes) / kEStageBytes;
-  static constexpr int kEStages = HAS_E ? (kEFit < 12 ? kEFit : 12) : 0;
-  static_assert(!HAS_E || kEStages >= 4, "no room for the E ring");
+  static constexpr int kEStages = kGathered > 0 ? (kEFit < 12 ? kEFit : 12) : 0;
+  static_assert(kGathered == 0 || kEStages >= 4, "no room for the E ring");
   static constexpr int kDBufs = 2;                 // accumulators of 128 columns: one per epilogue group
   static constexpr int kTmemCols = 256;
-  static constexpr int SE = HAS_E ? kEStages : 1;
+  static constexpr int SE = kGathered > 0 ? kEStages : 1;
   static constexpr int kBars = 4 + 2 * kUStages + 8 * SE + 2 * kDBufs;   // the E ring has a full and an empty barrier per stage and QUARTER
   static constexpr int kSmemBytes = 1024 + kFixedBytes + kEStages * kEStageBytes + kBars * 8 + 16;
   static_assert(kSmemBytes <= kMaxSmem, "the rings do not fit in shared memory");
@@ -121,8 +126,10 @@ __global__ void __launch_bounds__(kExpandThreads, 1)
 codec_umma_expand_kernel(const MmaArgs a, const ExpandGeometry geo, const __grid_constant__ UmmaExpandMaps maps) {
   using Cfg = UmmaExpandConfig<KG, HAS_E, HAS_P, PROWS>;
   // positions and sequences of a tile: fixed in the PROWS = 16 variant, the launch's otherwise
-  const int gpos = PROWS == kGridPos ? kGridPos : geo.gpos, gseqs = PROWS == kGridPos ? kGridSeqs : geo.gseqs;
-  constexpr int SU = Cfg::kUStages, SE = Cfg::SE;
+  const int gpos = PROWS == kGridPos ? kGridPos : (PROWS == 0 ? kUmmaTile : geo.gpos);
+  const int gseqs = PROWS == kGridPos ? kGridSeqs : (PROWS == 0 ? 1 : geo.gseqs);
+  constexpr int SU = Cfg::kUStages, SE = Cfg::SE, NG = Cfg::kGathered;
+  constexpr bool kPOperand = Cfg::kPOperand;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");   // the next kernel may set up behind this one
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -155,7 +162,7 @@ codec_umma_expand_kernel(const MmaArgs a, const ExpandGeometry geo, const __grid
   volatile uint32_t *tmem_slot_ptr =
       reinterpret_cast<volatile uint32_t *>(smem_raw + (tmem_slot - smem_u32(smem_raw)));
 
-  if (HAS_P) {
+  if constexpr (kPOperand) {
     // Sel[r][j] = 1 for j == r mod gpos (K-major, 128-byte rows of 64 positions, swizzled; a second
     // tile holds positions 64..127); only K = gpos is read
     for (uint32_t i = threadIdx.x; i < Cfg::kSelBytes / 16; i += blockDim.x) {
@@ -260,14 +267,14 @@ codec_umma_expand_kernel(const MmaArgs a, const ExpandGeometry geo, const __grid
         if (!dead && !mbar_wait(u_empty_bar(slot), parity)) timed_out();
         const uint32_t base = u_ring + (uint32_t)slot * Cfg::kUStageBytes;
         if (lane == 0) {
-          mbar_expect_tx(u_full_bar(slot), Cfg::kU2Bytes + (HAS_P ? 2 * gpos * 128 : 0));
+          mbar_expect_tx(u_full_bar(slot), Cfg::kU2Bytes + (kPOperand ? 2 * gpos * 128 : 0));
 #pragma unroll
           for (int kg = 0; kg < KG; ++kg) {   // per group of 64 coordinates: 128 rows of 128 bytes
             tma_load_2d(base + kg * Cfg::kTileBytes, &maps.u_wide, u_full_bar(slot), kg * 64, q * kChunkCols);
             tma_load_2d(base + kg * Cfg::kTileBytes + 8192, q == nchunks - 1 ? &maps.u : &maps.u_wide,
                         u_full_bar(slot), kg * 64, q * kChunkCols + 64);
           }
-          if (HAS_P) {
+          if (kPOperand) {
             // both 64-column groups of the 16 P rows in one copy (a 3-D view of P)
             tma_load_3d_hint(base + Cfg::kU2Bytes, &maps.p, u_full_bar(slot), 0, c1, q * (kChunkCols / kUmmaCols),
                              keep);
@@ -312,7 +319,7 @@ codec_umma_expand_kernel(const MmaArgs a, const ExpandGeometry geo, const __grid
           }
           if (two_runs)
             for (int j = 0; j < ksteps; ++j) umma_bf16(dacc, zd2 + (uint32_t)j * 2, bd + (uint32_t)j * 2, idesc_kk, 1u);
-          if (HAS_P) {
+          if (kPOperand) {
             // K step j: 16 positions = 32 bytes of a Sel row (a second tile from position 64 on)
             // and 16 rows = 2048 bytes of the P operand
             const uint64_t pd = pdesc + umma_desc_addr(base + Cfg::kU2Bytes);
@@ -331,11 +338,11 @@ codec_umma_expand_kernel(const MmaArgs a, const ExpandGeometry geo, const __grid
       }
     }
   } else if (warp >= 10) {
-    // ------------------------------------------------------------------------- E row gather
+    // ------------------------------------------------------------------------- row gather (E, P)
     // 8 lanes copy one 128-byte row piece with cp.async straight into the swizzled stage; the
     // stage's "full" barrier counts one arrival per gather thread, made by the hardware when
     // that thread's copies have landed, so nothing waits between issuing stages.
-    if (HAS_E) {
+    if (NG > 0) {
       const int gw = warp - 10;                // rows 32*gw .. 32*gw+31 of the tile
       const int piece = lane & 7, sub = lane >> 3;
       int slot = 0;
@@ -343,30 +350,41 @@ codec_umma_expand_kernel(const MmaArgs a, const ExpandGeometry geo, const __grid
       for (int64_t tile = tile_lo; tile <= tile_hi; ++tile) {
         int c1, c2;
         tile_coords(tile, c1, c2);
-        const unsigned char *src[8];
+        const unsigned char *src[NG > 0 ? NG : 1][8];
         uint32_t dst[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
           const int r = gw * 32 + i * 4 + sub;
-          const int64_t t = geo.grid_mode ? (int64_t)(c2 + r / gpos) * geo.seq_len + c1 + r % gpos
-                                          : (int64_t)c1 + r;
-          const int64_t er = t < a.n ? embedding_row(a.shift, t) : -1;
-          src[i] = (er >= 0 ? reinterpret_cast<const unsigned char *>(
-                                  static_cast<const __nv_bfloat16 *>(a.shift.E) + er * a.shift.lde)
-                            : g_zero_row) + piece * 16;
+          const int64_t t = kPOperand && geo.grid_mode ? (int64_t)(c2 + r / gpos) * geo.seq_len + c1 + r % gpos
+                                                       : (int64_t)c1 + r;
+          if (HAS_E) {
+            const int64_t er = t < a.n ? embedding_row(a.shift, t) : -1;
+            src[0][i] = (er >= 0 ? reinterpret_cast<const unsigned char *>(
+                                       static_cast<const __nv_bfloat16 *>(a.shift.E) + er * a.shift.lde)
+                                 : g_zero_row) + piece * 16;
+          }
+          if (Cfg::kPGathered) {
+            const int64_t pr = t < a.n ? position_row(a.shift, t) : -1;
+            src[NG - 1][i] = (pr >= 0 ? reinterpret_cast<const unsigned char *>(
+                                            static_cast<const __nv_bfloat16 *>(a.shift.P) + pr * a.shift.ldp)
+                                      : g_zero_row) + piece * 16;
+          }
           dst[i] = r * 128 + ((piece ^ (r & 7)) << 4);
         }
         int q0, q1;
         chunk_range(tile, q0, q1);
         for (int qg = 2 * q0; qg < 2 * q1; ++qg) {     // 64-column groups of the row
-          if (!dead && !mbar_wait(e_empty_bar(slot, gw), parity)) timed_out();
-          const uint32_t base = e_ring + (uint32_t)slot * Cfg::kEStageBytes;
 #pragma unroll
-          for (int i = 0; i < 8; ++i) cp_async16_cg(base + dst[i], src[i] + qg * 128);
-          asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];\n" ::"r"(e_full_bar(slot, gw)) : "memory");
-          if (++slot == SE) {
-            slot = 0;
-            parity ^= 1u;
+          for (int o = 0; o < NG; ++o) {
+            if (!dead && !mbar_wait(e_empty_bar(slot, gw), parity)) timed_out();
+            const uint32_t base = e_ring + (uint32_t)slot * Cfg::kEStageBytes;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) cp_async16_cg(base + dst[i], src[o][i] + qg * 128);
+            asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];\n" ::"r"(e_full_bar(slot, gw)) : "memory");
+            if (++slot == SE) {
+              slot = 0;
+              parity ^= 1u;
+            }
           }
         }
       }
@@ -404,7 +422,7 @@ codec_umma_expand_kernel(const MmaArgs a, const ExpandGeometry geo, const __grid
         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
 #pragma unroll
         for (int g = 0; g < kChunkCols / 64; ++g) {
-          const int64_t ecount = 2 * ccount + g;
+          const int64_t ecount = (2 * ccount + g) * (NG > 0 ? NG : 1);
           const int eslot = (int)(ecount % SE);
           uint32_t v[4][16];
 #pragma unroll
@@ -416,7 +434,7 @@ codec_umma_expand_kernel(const MmaArgs a, const ExpandGeometry geo, const __grid
             if (lane == 0) mbar_arrive(d_empty_bar(db));
           }
           uint32_t slab;   // 32 rows x 128 B handed to the TMA store
-          if (HAS_E) {
+          if (NG > 0) {
             if (!dead && !mbar_wait(e_full_bar(eslot, quarter), (uint32_t)((ecount / SE) & 1))) timed_out();
             slab = e_ring + (uint32_t)eslot * Cfg::kEStageBytes + (uint32_t)quarter * 4096;
           } else {
@@ -426,9 +444,29 @@ codec_umma_expand_kernel(const MmaArgs a, const ExpandGeometry geo, const __grid
             slab = slab0 + (uint32_t)g * 4096;
           }
           const uint32_t srow = slab + lane * 128;
-          // all eight E pieces of the row first, so that their latencies overlap
+          if (NG == 2) {   // the P pieces from the next stage, which goes back at once
+            const int64_t pcount = ecount + 1;
+            const int pslot = (int)(pcount % SE);
+            if (!dead && !mbar_wait(e_full_bar(pslot, quarter), (uint32_t)((pcount / SE) & 1))) timed_out();
+            const uint32_t prow = e_ring + (uint32_t)pslot * Cfg::kEStageBytes + (uint32_t)quarter * 4096 + lane * 128;
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+              uint32_t p[4];
+              asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];\n"
+                           : "=r"(p[0]), "=r"(p[1]), "=r"(p[2]), "=r"(p[3]) : "r"(prow + ((c ^ (lane & 7)) << 4)));
+              uint32_t *w = &v[c >> 1][(c & 1) * 8];
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                w[2 * i] = __float_as_uint(__uint_as_float(w[2 * i]) + __uint_as_float(p[i] << 16));
+                w[2 * i + 1] = __float_as_uint(__uint_as_float(w[2 * i + 1]) + __uint_as_float(p[i] & 0xFFFF0000u));
+              }
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(e_empty_bar(pslot, quarter));
+          }
+          // all eight gathered pieces of the row first, so that their latencies overlap
           uint32_t e[8][4];
-          if (HAS_E) {
+          if (NG > 0) {
 #pragma unroll
             for (int c = 0; c < 8; ++c)
               asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];\n"
@@ -442,7 +480,7 @@ codec_umma_expand_kernel(const MmaArgs a, const ExpandGeometry geo, const __grid
             float f[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) f[i] = __uint_as_float(w[i]);
-            if (HAS_E) {   // the sum replaces the E piece
+            if (NG > 0) {   // the sum replaces the gathered piece
 #pragma unroll
               for (int i = 0; i < 4; ++i) {
                 f[2 * i] += __uint_as_float(e[c][i] << 16);
@@ -461,7 +499,7 @@ codec_umma_expand_kernel(const MmaArgs a, const ExpandGeometry geo, const __grid
           if (lane == 0) {
             if (rows_live) tma_store_3d_hint(&maps.out, slab, q * kChunkCols + g * 64, s1, s2, stream_out);
             bulk_commit();
-            if (HAS_E) {
+            if (NG > 0) {
               // the store before this one is done reading its stage: hand that stage back; after
               // the chunk's last store wait for that one too, since this warp's next store is
               // two chunks away and the stage would sit idle until then
@@ -480,7 +518,7 @@ codec_umma_expand_kernel(const MmaArgs a, const ExpandGeometry geo, const __grid
         if (a.rowsumsq != nullptr && tok < a.n) atomicAdd(a.rowsumsq + tok, ss);
       }
     }
-    if (HAS_E && lane == 0) {
+    if (NG > 0 && lane == 0) {
       bulk_wait_read<0>();
       if (held >= 0) mbar_arrive(e_empty_bar(held, quarter));
     }
