@@ -7,18 +7,26 @@
 namespace ssn {
 namespace {
 
-// CTAs per tile.  With enough tiles every CTA takes whole ones.  Fewer tiles than half the SMs: the
-// largest cluster that still runs in one wave.  In between, two CTAs per tile where the halves pack
-// the last wave better than whole tiles do (by more than a tenth of a tile, about what the exchange
-// and a second set-up cost).
+// CTAs per tile: the c whose waves of tiles, each 1 / c of a tile's time plus a fixed cost, end first.  The fixed
+// cost of a wave (set-up, first loads, exchange of the sums) is about that of kWaveStages stages of 64 columns.
+// Large batches keep whole tiles, which one persistent CTA runs back to back.  43 tiles of 64 stages: two CTAs per
+// tile 110 us, three 80 us.
+constexpr int kWaveStages = 5;
+// clusters of 1 .. 8 CTAs of one per SM that a B200's 148 SMs run at once (cudaOccupancyMaxActiveClusters)
+constexpr int kClustersAtOnce[8] = {148, 74, 45, 33, 26, 22, 15, 15};
 int cluster_of(int64_t ntiles, int nst, int sms) {
-  int c = 1;
-  while (c < 8 && 2 * c <= nst && ntiles * 2 * c <= sms - (2 * c == 8 ? 20 : 0)) c *= 2;
-  if (c == 1 && nst >= 2 && ntiles > sms && ntiles < 8 * (int64_t)sms) {
-    const int64_t whole = (ntiles + sms - 1) / sms, halves = (2 * ntiles + sms - 1) / sms;
-    if (10 * halves + 2 < 20 * whole - 2) c = 2;
+  int best = 1;
+  double best_cost = (double)((ntiles + sms - 1) / sms) * nst + kWaveStages;
+  for (int c = 2; c <= 8 && c <= nst; ++c) {
+    const int at_once = kClustersAtOnce[c - 1] * sms / 148;
+    if (at_once < 1) break;
+    const double cost = (double)((ntiles + at_once - 1) / at_once) * ((double)((nst + c - 1) / c) + kWaveStages);
+    if (cost < 0.97 * best_cost) {
+      best = c;
+      best_cost = cost;
+    }
   }
-  return c;
+  return best;
 }
 
 template <typename T, int KN, int NSLOT>

@@ -19,9 +19,9 @@
 //               five instructions, (Uh|Um) being 256 columns wide).  It is a warp of its own because each
 //               of these instructions blocks its thread for about 100 clocks.
 //
-// A CTA takes whole tiles of 128 tokens; when there are fewer tiles than SMs, a cluster of 2, 4 or 8
-// CTAs shares one tile, each contracting a slice of d, and the partial sums meet through distributed
-// shared memory, every CTA finishing its share of the rows.
+// A CTA takes whole tiles of 128 tokens, or a cluster of 2 to 8 CTAs shares one tile where that fills the
+// SMs better: each contracts a slice of d, and the partial sums meet through distributed shared memory, every
+// CTA finishing its share of the rows.
 #pragma once
 
 #include "codec_split.cuh"
@@ -544,7 +544,7 @@ __global__ void __launch_bounds__(kSplitProjectThreads, 1) codec_split_project_k
                      __float_as_uint(sum[c + 3]));
     }
     asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
-    const int rows = kUmmaTile / (int)cluster_size, row0 = rows * (int)cta_rank;
+    const int row0 = (int)(kUmmaTile * cta_rank / cluster_size), rows = (int)(kUmmaTile * (cta_rank + 1) / cluster_size) - row0;
     auto peer = [](uint32_t addr, uint32_t rank) {
       uint32_t r;
       asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(r) : "r"(addr), "r"(rank));
