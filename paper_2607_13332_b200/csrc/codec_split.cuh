@@ -111,6 +111,7 @@ __device__ __forceinline__ uint32_t load_global_b16(const void *p) {
   asm volatile("ld.global.nc.b16 %0, [%1];\n" : "=h"(v) : "l"(p));
   return v;
 }
+
 __device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];\n" ::"l"(p)); }
 
 // Two neighbouring elements as loaded.  A bf16 pair has one word per element until joined() puts them
@@ -174,6 +175,39 @@ __device__ __forceinline__ void split_pair(const Pair<T> &v, uint32_t (&p)[NP]) 
 }
 inline bool pairs_aligned(const void *p, int64_t ld, int esz) {
   return (reinterpret_cast<uintptr_t>(p) & (2 * esz - 1)) == 0 && (ld & 1) == 0;
+}
+
+// 16 bytes of a row from column c on, element by element (zeros past column d and for a missing row).
+template <typename T>
+__device__ __forceinline__ uint4 load_row_piece(const T *row, int c, int d) {
+  uint32_t w[4];
+  const bool ok = row != nullptr;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    if constexpr (sizeof(T) == 4)
+      w[i] = load_global_b32_if(row + c + i, ok && c + i < d);
+    else
+      w[i] = load_global_b16_if(row + c + 2 * i, ok && c + 2 * i < d) | load_global_b16_if(row + c + 2 * i + 1, ok && c + 2 * i + 1 < d) << 16;
+  }
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+// The same with an asynchronous copy to shared memory; `ok` = false writes zeros.
+__device__ __forceinline__ void cp_async16_if(uint32_t dst, const void *src, bool ok) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src), "r"(ok ? 16 : 0) : "memory");
+}
+
+template <typename T> __device__ __forceinline__ void widen_piece(const uint4 &raw, float *f);
+template <> __device__ __forceinline__ void widen_piece<float>(const uint4 &raw, float *f) {
+  f[0] = __uint_as_float(raw.x); f[1] = __uint_as_float(raw.y);
+  f[2] = __uint_as_float(raw.z); f[3] = __uint_as_float(raw.w);
+}
+template <> __device__ __forceinline__ void widen_piece<__nv_bfloat16>(const uint4 &raw, float *f) {
+  const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    f[2 * i] = __uint_as_float(w[i] << 16);
+    f[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
+  }
 }
 
 }  // namespace ssn

@@ -5,16 +5,18 @@
 //
 // A unit is 128 tokens x 128 output columns; the units are dealt to the CTAs in contiguous ranges.
 //
-//   warps 0-15   output: TMEM -> a staging tile in shared memory (half a unit, 64 columns, at a time)
-//                -> rows again, 16 lanes per row, so that the E and P rows are read and the output is
-//                written in whole sectors whatever their alignment; the row pieces of the next
-//                half are in flight while this one is staged, and their lines two units on are
-//                requested into L2 (the loads in registers alone do not cover HBM latency).
-//   warps 16-23  operands: Z once per tile and 128 rows of U per unit, loaded pair by pair of elements, split
+//   warps 0-7    epilogue, two warps per 32 rows: TMEM lane = row; 128 bytes of every row at a time (a piece),
+//                half of it per warp, the E and P pieces added from shared memory, the sum written in place and
+//                handed to a TMA store (or, off the 16-byte grid, stored by the warps themselves).  Plain stores
+//                of the whole output blocked the load pipe for everyone else (8192 x 2048 fp32: E and P rows
+//                76 -> 45 us with TMA stores and gathered rows, no tables 35 -> 31 us).  Both warps take every piece, so each follows the phases of
+//                every stage of the ring.
+//   warps 8-11   gather the E and P rows with cp.async into a ring of such pieces (E, then P), 32 rows each; a
+//                quarter of a stage is handed over at a time.
+//   warps 12-19  operands: Z once per tile and 128 rows of U per unit, loaded pair by pair of elements, split
 //                into bf16 parts (codec_split.cuh) and written as swizzled K-major tiles of 64 coordinates; a
-//                ring of such U tiles runs ahead of the MMAs.  One warp per scheduler could not keep up
-//                with the splitting.
-//   warp 24      one thread issues the MMAs (M = 128, N = 128): the leading product into one accumulator,
+//                ring of such U tiles runs ahead of the MMAs.
+//   warp 20      one thread issues the MMAs (M = 128, N = 128): the leading product into one accumulator,
 //                the small ones (hm, mh, mm, hl, lh) into a second, two sets of both.  A warp of its own, since
 //                every MMA blocks its thread for about 80 clocks.
 //
@@ -35,15 +37,15 @@ struct SplitExpandArgs {
   int32_t d, k;
   int32_t has_e, has_p;
   int32_t vec_z, vec_u;        // two coordinates of Z / U may be read at a time
-  int32_t vec_out;             // four elements of the output and of the E and P rows may be moved at a time
+  int32_t vec_rows;            // E and P rows may be read 16 bytes at a time and g_zero_row holds a row
+  int32_t tma_out;             // the output is stored through the tensor map
   ShiftTables shift;
 };
 
-constexpr int kSplitOutWarps = 16, kSplitOperandWarps = 8;
-constexpr int kSplitOutThreads = 32 * kSplitOutWarps;
-constexpr int kSplitExpandThreads = 32 * (kSplitOutWarps + kSplitOperandWarps + 1);
-constexpr int kSplitTileBytes = kUmmaTile * 128;     // one part of [128 rows x 64 coordinates]
-constexpr int kSplitHalf = 64;                       // output columns staged at a time
+constexpr int kSplitEpilogueWarps = 8, kSplitGatherWarps = 4, kSplitOperandWarps = 8;
+constexpr int kSplitOperandWarp0 = kSplitEpilogueWarps + kSplitGatherWarps, kSplitMmaWarp = kSplitOperandWarp0 + kSplitOperandWarps;
+constexpr int kSplitExpandThreads = 32 * (kSplitMmaWarp + 1);
+constexpr int kSplitTileBytes = kUmmaTile * 128;     // one part of [128 rows x 64 coordinates]; one piece of 128 rows
 
 // TZ: type of the coordinates (float for fp32 storage and wire rows), T: storage type, KG: groups of 64 coordinates
 template <typename T, typename TZ, int KG, int NSLOT>
@@ -53,56 +55,36 @@ struct SplitExpandConfig {
   static constexpr int kZBufs = kNZ == 1 ? 2 : 1;
   static constexpr int kUStageBytes = kNU * kSplitTileBytes;
   static constexpr int kUStages = kNU == 3 ? 2 : 3;
-  static constexpr int kHalfBytes = kUmmaTile * kSplitHalf * 4;
-  static constexpr int kStagings = kNU == 3 && KG == 2 ? 1 : 2;
   static constexpr bool kLow = kNZ > 1 || kNU > 1;          // a second accumulator for the small products
   static constexpr int kDCols = (kLow ? 2 : 1) * kChunkCols;
   static constexpr int kTmemCols = 2 * kDCols;
+  static constexpr int kPieceCols = 128 / (int)sizeof(T), kPieces = kChunkCols / kPieceCols;
   static constexpr int kOperandBytes = kZBufs * kZBytes + kUStages * kUStageBytes;
-  static constexpr int kBars = 4 + 2 * kUStages + 4;
+  static constexpr int kRoom = 227 * 1024 - 1024 - 2048 - kOperandBytes;
+  // the ring of pieces: gathered rows that become output, or output alone
+  static constexpr int kFit = kRoom / kSplitTileBytes;
+  static constexpr int kRing = NSLOT == 0 ? (kFit < 4 ? kFit : 4) : (kFit < 10 ? kFit : 10);
+  static_assert(kRing >= 2, "no room for the output");
+  // a stage goes back when the next store is under way, unless the ring is too short to wait for that
+  static constexpr bool kHold = NSLOT == 0 ? kRing > 2 : kRing >= 4 * NSLOT;
+  static constexpr int kOutBytes = kRing * kSplitTileBytes;
+  static constexpr int kBars = 4 + 2 * kUStages + 4 + 8 * kRing;
   static constexpr int kUnsafeSlots = 8;                    // units whose U values may be flagged at a time
-  static constexpr int kTailBytes = kBars * 8 + 16 + kUnsafeSlots * kSplitOperandWarps;
-  static constexpr int kSmemBytes = 1024 + kOperandBytes + kStagings * kHalfBytes + kTailBytes;
+  static constexpr int kTailBytes = kBars * 8 + 16 + kUnsafeSlots * kSplitOperandWarps + 4 * kUmmaTile;
+  static constexpr int kSmemBytes = 1024 + kOperandBytes + kOutBytes + kTailBytes;
   static_assert(kSmemBytes <= 227 * 1024, "the operands do not fit in shared memory");
 };
 
-// Four elements of a row from column c on (zeros past column d and for a missing row), as stored.
-template <typename T> struct RowPiece4 { uint32_t w[sizeof(T)]; };
-template <typename T>
-__device__ __forceinline__ RowPiece4<T> load_row4(const T *row, int c, int d, bool vec) {
-  RowPiece4<T> f;
-  const bool ok = row != nullptr;
-  if constexpr (sizeof(T) == 4) {
-    if (vec) {   // d is a multiple of 4 then
-      const uint4 v = load_global_v4_if(row + c, ok && c < d);
-      f.w[0] = v.x; f.w[1] = v.y; f.w[2] = v.z; f.w[3] = v.w;
-    } else {
-#pragma unroll
-      for (int e = 0; e < 4; ++e) f.w[e] = load_global_b32_if(row + c + e, ok && c + e < d);
-    }
-  } else {
-    if (vec) {
-      const uint2 v = load_global_v2_if(row + c, ok && c < d);
-      f.w[0] = v.x; f.w[1] = v.y;
-    } else {
-#pragma unroll
-      for (int e = 0; e < 2; ++e)
-        f.w[e] = load_global_b16_if(row + c + 2 * e, ok && c + 2 * e < d) |
-                 load_global_b16_if(row + c + 2 * e + 1, ok && c + 2 * e + 1 < d) << 16;
-    }
-  }
-  return f;
-}
-template <typename T>
-__device__ __forceinline__ float piece_element(const RowPiece4<T> &f, int e) {
-  if constexpr (sizeof(T) == 4) return __uint_as_float(f.w[e]);
-  else return __uint_as_float(e & 1 ? f.w[e >> 1] & 0xFFFF0000u : f.w[e >> 1] << 16);
+// What a row's largest magnitude says about its split, ordered so that the larger class of two halves is
+// that of the whole row.
+__device__ __forceinline__ unsigned char magnitude_class(float largest) {
+  return largest == 0.f ? 0 : (largest < kSplitTiny ? 1 : (largest < kSplitHuge ? 2 : 3));
 }
 
 template <typename T, typename TZ, int KG, int NSLOT>
-__global__ void __launch_bounds__(kSplitExpandThreads, 1) codec_split_expand_kernel(const SplitExpandArgs a) {
+__global__ void __launch_bounds__(kSplitExpandThreads, 1) codec_split_expand_kernel(const SplitExpandArgs a, const __grid_constant__ CUtensorMap out_map) {
   using Cfg = SplitExpandConfig<T, TZ, KG, NSLOT>;
-  constexpr int NZ = Cfg::kNZ, NU = Cfg::kNU, SU = Cfg::kUStages;
+  constexpr int NZ = Cfg::kNZ, NU = Cfg::kNU, SU = Cfg::kUStages, SE = Cfg::kRing;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -110,18 +92,22 @@ __global__ void __launch_bounds__(kSplitExpandThreads, 1) codec_split_expand_ker
   const int64_t ntiles = (a.n + kUmmaTile - 1) / kUmmaTile;
 
   const uint32_t smem_u = smem_u32(smem_raw), smem0 = (smem_u + 1023u) & ~1023u;
-  const uint32_t z_base = smem0, u_ring = z_base + Cfg::kZBufs * Cfg::kZBytes, staging = smem0 + Cfg::kOperandBytes;
-  const uint32_t bars = staging + Cfg::kStagings * Cfg::kHalfBytes;
+  const uint32_t z_base = smem0, u_ring = z_base + Cfg::kZBufs * Cfg::kZBytes, out_base = smem0 + Cfg::kOperandBytes;
+  const uint32_t bars = out_base + Cfg::kOutBytes;
   auto z_full_bar = [&](int b) { return bars + b * 8; };
   auto z_empty_bar = [&](int b) { return bars + (2 + b) * 8; };
   auto u_full_bar = [&](int s) { return bars + (4 + s) * 8; };
   auto u_empty_bar = [&](int s) { return bars + (4 + SU + s) * 8; };
   auto d_full_bar = [&](int b) { return bars + (4 + 2 * SU + b) * 8; };
   auto d_empty_bar = [&](int b) { return bars + (4 + 2 * SU + 2 + b) * 8; };
+  auto e_full_bar = [&](int s, int q) { return bars + (4 + 2 * SU + 4 + 4 * s + q) * 8; };
+  auto e_empty_bar = [&](int s, int q) { return bars + (4 + 2 * SU + 4 + 4 * SE + 4 * s + q) * 8; };
   unsigned char *tail = smem_raw + (bars - smem_u) + Cfg::kBars * 8;
   volatile uint32_t *tmem_slot_ptr = reinterpret_cast<volatile uint32_t *>(tail);
   // [unit % kUnsafeSlots][operand warp]: U of the unit holds values its split does not
   volatile unsigned char *unit_flags = tail + 16;
+  // [tile & 3][row]: magnitude class of the row of Z
+  volatile unsigned char *row_class = unit_flags + Cfg::kUnsafeSlots * kSplitOperandWarps;
 
   if (a.k % 16 != 0) {   // the coordinates a K step reads past k
     for (uint32_t i = tid; i < Cfg::kOperandBytes / 16; i += kSplitExpandThreads) st_shared_v4(smem0 + i * 16, 0, 0, 0, 0);
@@ -132,15 +118,20 @@ __global__ void __launch_bounds__(kSplitExpandThreads, 1) codec_split_expand_ker
       mbar_init(z_full_bar(b), kSplitOperandWarps);
       mbar_init(z_empty_bar(b), 1);
       mbar_init(d_full_bar(b), 1);
-      mbar_init(d_empty_bar(b), kSplitOutWarps);
+      mbar_init(d_empty_bar(b), kSplitEpilogueWarps);
     }
+    for (int s = 0; s < SE; ++s)
+      for (int q = 0; q < 4; ++q) {
+        mbar_init(e_full_bar(s, q), 32);
+        mbar_init(e_empty_bar(s, q), 1);
+      }
     for (int s = 0; s < SU; ++s) {
       mbar_init(u_full_bar(s), kSplitOperandWarps);
       mbar_init(u_empty_bar(s), 1);
     }
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
-  if (warp == kSplitOutWarps + kSplitOperandWarps) {
+  if (warp == kSplitMmaWarp) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tail)),
                  "r"(Cfg::kTmemCols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
@@ -164,19 +155,19 @@ __global__ void __launch_bounds__(kSplitExpandThreads, 1) codec_split_expand_ker
   const int64_t tile_lo = u_lo / nchunks;
   const int chunk_lo = (int)(u_lo - tile_lo * nchunks);
 
-  if (warp >= kSplitOutWarps && warp < kSplitOutWarps + kSplitOperandWarps) {
+  if (warp >= kSplitOperandWarp0 && warp < kSplitMmaWarp) {
     // ------------------------------------------------------------------------- operands
     // Lane = pair of coordinates (32, or 16 or 8 lanes per row where the rank leaves the others without
     // work), so the loads are coalesced and the swizzled stores hit all banks once.  The rows of a lane are
     // 8 or more apart, so its place in the swizzled rows never changes.
-    const int ow = warp - kSplitOutWarps;
+    const int ow = warp - kSplitOperandWarp0;
     const int lpr_log = KG == 2 || a.k > 32 ? 5 : (a.k > 16 ? 4 : 3), rpw = 32 >> lpr_log;
     const int row0 = ow * rpw + (lane >> lpr_log), pair = lane & ((1 << lpr_log) - 1);
     const int nit = kUmmaTile / (kSplitOperandWarps * rpw), row_step = kSplitOperandWarps * rpw;
     const uint32_t off0 = row0 * 128 + (((pair >> 2) ^ (row0 & 7)) << 4) + (pair & 3) * 4;
     // rows first .. first + 127 of a matrix (the last one repeated), coordinates 64 kg ..: parts into smem
     auto move_tile = [&](auto np, auto batch, const auto *M, int64_t ld, int64_t first, int64_t rows, int kg, bool vec_m,
-                         uint32_t base, uint32_t part_bytes, auto wait_free) {
+                         uint32_t base, uint32_t part_bytes, int class_slot, auto wait_free) {
       constexpr int NP = decltype(np)::value, B = decltype(batch)::value;   // B: rows in flight per lane
       using E = std::remove_const_t<std::remove_pointer_t<decltype(M)>>;
       const int j = kg * 64 + 2 * pair, valid = a.k - j;
@@ -194,6 +185,20 @@ __global__ void __launch_bounds__(kSplitExpandThreads, 1) codec_split_expand_ker
           load_pairs<B, E>(v, [&](int i) { return M + min(first + row0 + (int64_t)(b + i) * row_step, rows - 1) * ld + j; }, valid, vec_m);
         }
         if (b == 0) wait_free();
+        if (NZ == 3 && class_slot >= 0) {                // a row of Z: its lanes agree on its class
+#pragma unroll
+          for (int i = 0; i < B; ++i) {
+            float m = valid > 0 ? pair_magnitude<E>(joined<E>(v[i])) : 0.f;
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1)
+              if (off < (1 << lpr_log)) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+            if (pair == 0) {
+              volatile unsigned char *c = row_class + class_slot * kUmmaTile + row0 + (b + i) * row_step;
+              const unsigned char cls = magnitude_class(m);
+              *c = kg == 0 ? cls : max(cls, (unsigned char)*c);
+            }
+          }
+        }
         if (valid > 0) {
           const uint32_t dst = base + off0 + (uint32_t)b * row_step * 128;
 #pragma unroll
@@ -221,7 +226,7 @@ __global__ void __launch_bounds__(kSplitExpandThreads, 1) codec_split_expand_ker
         for (int kg = 0; kg < KG; ++kg) {
           auto z_tile = [&](auto batch) {
             move_tile(std::integral_constant<int, NZ>{}, batch, static_cast<const TZ *>(a.zin), a.ldzin, tile * kUmmaTile, a.n, kg,
-                      a.vec_z != 0, z_base + zb * Cfg::kZBytes + kg * kSplitTileBytes, KG * kSplitTileBytes, [&]() {
+                      a.vec_z != 0, z_base + zb * Cfg::kZBytes + kg * kSplitTileBytes, KG * kSplitTileBytes, tcount & 3, [&]() {
                         if (kg == 0 && !dead && !mbar_wait(z_empty_bar(zb), z_parity)) timed_out();
                       });
           };
@@ -238,7 +243,7 @@ __global__ void __launch_bounds__(kSplitExpandThreads, 1) codec_split_expand_ker
       for (int kg = 0; kg < KG; ++kg) {
         auto u_tile = [&](auto batch) {
           return move_tile(std::integral_constant<int, NU>{}, batch, U, a.ldu, (int64_t)col0, (int64_t)a.d, kg, a.vec_u != 0,
-                           u_ring + (uint32_t)slot * Cfg::kUStageBytes, kSplitTileBytes, [&]() {
+                           u_ring + (uint32_t)slot * Cfg::kUStageBytes, kSplitTileBytes, -1, [&]() {
                              if (!dead && !mbar_wait(u_empty_bar(slot), parity)) timed_out();
                            });
         };
@@ -260,7 +265,7 @@ __global__ void __launch_bounds__(kSplitExpandThreads, 1) codec_split_expand_ker
         ++tile;
       }
     }
-  } else if (warp == kSplitOutWarps + kSplitOperandWarps) {
+  } else if (warp == kSplitMmaWarp) {
     // ------------------------------------------------------------------------- MMA issuer
     if (lane == 0) {
       constexpr uint32_t idesc = umma_idesc_kk(kChunkCols);
@@ -309,183 +314,243 @@ __global__ void __launch_bounds__(kSplitExpandThreads, 1) codec_split_expand_ker
       }
     }
     __syncwarp();
-  } else {
-    // ------------------------------------------------------------------------- output
-    const int quarter = warp & 3, cpart = warp >> 2;       // TMEM lanes; 16 of the 64 columns of a half
-    const int trow = quarter * 32 + lane;                  // row this thread stages
-    const int sub = lane >> 4, c4 = (lane & 15) * 4;       // rows 2 i + sub of the warp's eight, columns c4 .. +3
-    const bool vec = a.vec_out != 0;
-    int64_t tile = tile_lo;
-    int chunk = chunk_lo;
-    int32_t er = -1, pr = -1;                              // lanes 0-7: table rows of the warp's rows
-    uint32_t unsafe_rows = 0;
-    int live_rows = 0;                                     // of the warp's eight, those before row n
-    T *out0 = nullptr;                                     // column c4 of row `sub` of the warp's eight
-    RowPiece4<T> in[NSLOT > 0 ? NSLOT : 1][4];
-    const T *E = a.has_e ? static_cast<const T *>(a.shift.E) : nullptr, *P = a.has_p ? static_cast<const T *>(a.shift.P) : nullptr;
-    auto row_of = [&](bool want_e, int i) -> const T * {   // E or P row of the warp's row i
-      const int32_t r = __shfl_sync(0xffffffffu, want_e ? er : pr, i);
-      return r < 0 ? nullptr : (want_e ? E + (int64_t)r * a.shift.lde : P + (int64_t)r * a.shift.ldp);
-    };
-    auto issue = [&](int col) {                            // E and P pieces of the warp's rows
+  } else if (warp >= kSplitEpilogueWarps) {
+    // ------------------------------------------------------------------------- row gather (E, P)
+    // 8 lanes copy 128 bytes of one row; the stage's quarter is full when every thread's copies have landed.
+    if (NSLOT > 0) {
+      const int gw = warp - kSplitEpilogueWarps, piece = lane & 7, sub = lane >> 3;   // rows 32 gw .. +31
+      constexpr int kUnitElems = 16 / (int)sizeof(T);
+      const bool vec = a.vec_rows != 0;
+      const T *E = a.has_e ? static_cast<const T *>(a.shift.E) : nullptr, *P = a.has_p ? static_cast<const T *>(a.shift.P) : nullptr;
+      const T *src[NSLOT > 0 ? NSLOT : 1][8];
+      uint32_t dst[8];
 #pragma unroll
-      for (int i = 0; i < (NSLOT > 0 ? 4 : 0); ++i) {
-        in[0][i] = load_row4<T>(row_of(NSLOT == 2 || a.has_e, 2 * i + sub), col + c4, a.d, vec);
-        if (NSLOT == 2) in[NSLOT - 1][i] = load_row4<T>(row_of(false, 2 * i + sub), col + c4, a.d, vec);
+      for (int i = 0; i < 8; ++i) {
+        const int r = gw * 32 + i * 4 + sub;
+        dst[i] = r * 128 + ((piece ^ (r & 7)) << 4);
       }
-    };
-    auto prefetch = [&](int col) {                         // the lines of 128 columns of the warp's rows
-      constexpr int kLines = kChunkCols * (int)sizeof(T) / 128, kLineElems = 128 / (int)sizeof(T);
-      if (NSLOT == 0 || col >= a.d) return;
-      const int r = lane / kLines, c = col + (lane % kLines) * kLineElems;   // bf16: the upper lanes have no row
+      int64_t tile = tile_lo;
+      int chunk = chunk_lo, slot = 0;
+      uint32_t parity = 1;
+      for (int unit = 0; unit < count_units; ++unit) {
+        if (unit == 0 || chunk == 0) {
+          const T *none = vec ? reinterpret_cast<const T *>(g_zero_row) : nullptr;
 #pragma unroll
-      for (int o = 0; o < NSLOT; ++o) {
-        const T *row = row_of(NSLOT == 2 ? o == 0 : a.has_e != 0, r & 7);
-        if (r < 8 && row != nullptr && c < a.d) prefetch_l2(row + c);
-      }
-    };
-    auto enter_tile = [&](int64_t ut) {
-      const int64_t t0 = ut * kUmmaTile + warp * 8, t = t0 + lane;
-      live_rows = (int)max((int64_t)0, min((int64_t)8, a.n - t0));
-      out0 = static_cast<T *>(a.dst) + (t0 + sub) * a.lddst + c4;
-      er = pr = -1;
-      if (NSLOT > 0 && lane < live_rows) {
-        if (a.has_e) er = (int32_t)embedding_row(a.shift, t);
-        if (a.has_p) pr = (int32_t)position_row(a.shift, t);
-      }
-      if (NZ == 3) {                                       // rows whose split does not hold
-        unsafe_rows = 0;
-        for (int r = 0; r < live_rows; ++r) {
-          const TZ *z = static_cast<const TZ *>(a.zin) + (t0 + r) * a.ldzin;
-          float m = 0.f;
-          for (int j = lane; j < a.k; j += 32) m = fmaxf(m, fabsf(to_f32(z[j])));
-          m = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(m)));   // floats >= 0 order like their bits
-          if (split_unsafe(m)) unsafe_rows |= 1u << r;
+          for (int i = 0; i < 8; ++i) {
+            const int64_t t = tile * kUmmaTile + gw * 32 + i * 4 + sub;
+            const int64_t er = t < a.n && E != nullptr ? embedding_row(a.shift, t) : -1;
+            const int64_t pr = t < a.n && P != nullptr ? position_row(a.shift, t) : -1;
+            const T *erow = er >= 0 ? E + er * a.shift.lde : none, *prow = pr >= 0 ? P + pr * a.shift.ldp : none;
+            src[0][i] = NSLOT == 2 || E != nullptr ? erow : prow;
+            if (NSLOT == 2) src[NSLOT - 1][i] = prow;
+          }
+        }
+        // the lines of the next unit into L2: the ring alone does not hold enough in flight for HBM latency
+        if (vec && piece < Cfg::kPieces && (chunk + 1) * kChunkCols + piece * Cfg::kPieceCols < a.d) {
+#pragma unroll
+          for (int o = 0; o < NSLOT; ++o)
+#pragma unroll
+            for (int i = 0; i < 8; ++i) prefetch_l2(src[o][i] + (chunk + 1) * kChunkCols + piece * Cfg::kPieceCols);
+        }
+#pragma unroll 1
+        for (int g = 0; g < Cfg::kPieces; ++g) {
+          const int c = chunk * kChunkCols + g * Cfg::kPieceCols + piece * kUnitElems;
+          const bool ok = c < a.d;
+#pragma unroll
+          for (int o = 0; o < NSLOT; ++o) {
+            if (!dead && !mbar_wait(e_empty_bar(slot, gw), parity)) timed_out();
+            const uint32_t base = out_base + (uint32_t)slot * kSplitTileBytes;
+            if (vec) {
+#pragma unroll
+              for (int i = 0; i < 8; ++i) cp_async16_if(base + dst[i], src[o][i] + (ok ? c : 0), ok);
+              asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];\n" ::"r"(e_full_bar(slot, gw)) : "memory");
+            } else {
+#pragma unroll 1
+              for (int i = 0; i < 8; ++i) {
+                const T *row = nullptr;
+                uint32_t to = 0;
+#pragma unroll
+                for (int h = 0; h < 8; ++h)
+                  if (h == i) {
+                    row = src[o][h];
+                    to = dst[h];
+                  }
+                const uint4 v = load_row_piece<T>(row, c, a.d);
+                st_shared_v4(base + to, v.x, v.y, v.z, v.w);
+              }
+              mbar_arrive(e_full_bar(slot, gw));
+            }
+            if (++slot == SE) {
+              slot = 0;
+              parity ^= 1u;
+            }
+          }
+        }
+        if (++chunk == nchunks) {
+          chunk = 0;
+          ++tile;
         }
       }
-    };
-    if (count_units > 0) {
-      enter_tile(tile);
-      issue(chunk * kChunkCols);
-      prefetch((chunk + 1) * kChunkCols);
+      cp_async_commit();
+      cp_async_wait<0>();
     }
+  } else {
+    // ------------------------------------------------------------------------- epilogue
+    const int quarter = warp & 3, half = warp >> 2;        // TMEM lanes 32 quarter .. +31; half of every piece
+    constexpr int kHalfCols = Cfg::kPieceCols / 2, kUnitElems = 16 / (int)sizeof(T);
+    const uint32_t lane_addr = tmem_base + ((uint32_t)(quarter * 32) << 16);
+    const uint64_t stream_out = l2_policy_evict_first();   // the output is written once and not read here
+    auto meet = [&]() { asm volatile("bar.sync %0, 64;\n" ::"r"(1 + quarter) : "memory"); };   // the quarter's two warps
+    int64_t tile = tile_lo;
+    int chunk = chunk_lo, tcount = 0, slot = 0;
+    uint32_t parity = 0;
+    int held = -1;                                         // stage whose store may still be reading it
     for (int unit = 0; unit < count_units; ++unit) {
-      const int col0 = chunk * kChunkCols, db = unit & 1;
+      const int db = unit & 1, col0 = chunk * kChunkCols;
+      const int64_t row0 = tile * kUmmaTile + quarter * 32, t = row0 + lane;
       if (!dead && !mbar_wait(d_full_bar(db), (uint32_t)((unit >> 1) & 1))) timed_out();
       asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-      uint32_t bad = 0;
+      bool bad = false;                                    // this row by plain FMAs
       if (Cfg::kLow) {
-        bad = unsafe_rows;
-        if (reinterpret_cast<volatile unsigned long long *>(tail + 16)[unit % Cfg::kUnsafeSlots] != 0) bad = 0xFFu;
+        const unsigned char cls = NZ == 3 ? row_class[(tcount & 3) * kUmmaTile + quarter * 32 + lane] : 2;
+        bad = t < a.n && (cls == 1 || cls == 3 ||
+                          reinterpret_cast<volatile unsigned long long *>(tail + 16)[unit % Cfg::kUnsafeSlots] != 0);
       }
-      prefetch(col0 + 2 * kChunkCols);
-#pragma unroll
-      for (int g = 0; g < kChunkCols / kSplitHalf; ++g) {
-        uint32_t v[2][8];
-        const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)db * Cfg::kDCols + g * kSplitHalf + cpart * 16;
-        tmem_ld8(taddr, v[0]);
-        tmem_ld8(taddr + 8, v[1]);
-        if (Cfg::kLow) {
-          uint32_t w[2][8];
-          tmem_ld8(taddr + kChunkCols, w[0]);
-          tmem_ld8(taddr + kChunkCols + 8, w[1]);
-          asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-#pragma unroll
-          for (int h = 0; h < 2; ++h)
-#pragma unroll
-            for (int e = 0; e < 8; ++e) v[h][e] = __float_as_uint(__uint_as_float(v[h][e]) + __uint_as_float(w[h][e]));
+#pragma unroll 1
+      for (int g = 0; g < Cfg::kPieces; ++g) {
+        // the piece's stage: full of E or P rows, or (no tables) free; and the P stage behind an E stage
+        const int eslot = slot;
+        if (NSLOT > 0) {
+          if (!dead && !mbar_wait(e_full_bar(slot, quarter), parity)) timed_out();
         } else {
-          asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+          if (!dead && !mbar_wait(e_empty_bar(slot, quarter), parity ^ 1u)) timed_out();
         }
-        if (g == kChunkCols / kSplitHalf - 1) {
-          asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-          __syncwarp();
-          if (lane == 0) mbar_arrive(d_empty_bar(db));
+        if (++slot == SE) {
+          slot = 0;
+          parity ^= 1u;
         }
-        // staging row: 64 floats, 16-byte units XORed with the row so that neither side conflicts
-        const uint32_t stage = staging + (Cfg::kStagings == 2 ? g : 0) * Cfg::kHalfBytes;
-        if (Cfg::kStagings == 1) asm volatile("bar.sync 1, %0;\n" ::"n"(kSplitOutThreads) : "memory");   // read by everyone
-#pragma unroll
-        for (int h = 0; h < 4; ++h) {
-          const uint32_t *w = &v[h >> 1][(h & 1) * 4];
-          st_shared_v4(stage + trow * 256 + (((cpart * 4 + h) ^ (trow & 15)) << 4), w[0], w[1], w[2], w[3]);
+        const int pslot = slot;
+        if (NSLOT == 2) {
+          if (!dead && !mbar_wait(e_full_bar(slot, quarter), parity)) timed_out();
+          if (++slot == SE) {
+            slot = 0;
+            parity ^= 1u;
+          }
         }
-        asm volatile("bar.sync 1, %0;\n" ::"n"(kSplitOutThreads) : "memory");
-        float o[4][4];
+        const uint32_t out = out_base + (uint32_t)eslot * kSplitTileBytes + (uint32_t)quarter * 4096;   // 32 rows x 128 bytes
+        const uint32_t orow = out + lane * 128;
+        const uint32_t prow = out_base + (uint32_t)pslot * kSplitTileBytes + (uint32_t)quarter * 4096 + lane * 128;
+        const int pcol = g * Cfg::kPieceCols + half * kHalfCols;   // this warp's columns of the unit
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int r = warp * 8 + 2 * i + sub;
-          const uint4 w = ld_shared_v4(stage + r * 256 + (((lane & 15) ^ (r & 15)) << 4));
-          o[i][0] = __uint_as_float(w.x); o[i][1] = __uint_as_float(w.y);
-          o[i][2] = __uint_as_float(w.z); o[i][3] = __uint_as_float(w.w);
-        }
-        const int col = col0 + g * kSplitHalf;
-        if (Cfg::kLow && bad != 0) {                       // plain FMAs for the flagged rows
+        for (int h = 0; h < kHalfCols / 16; ++h) {         // 16 columns at a time
+          const uint32_t taddr = lane_addr + (uint32_t)db * Cfg::kDCols + pcol + h * 16;
+          uint32_t v[16];
+          tmem_ld16(taddr, v);
+          if (Cfg::kLow) {
+            uint32_t w[16];
+            tmem_ld16(taddr + kChunkCols, w);
+            asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            if (!(bad >> (2 * i + sub) & 1) || 2 * i + sub >= live_rows) continue;
-            const TZ *z = static_cast<const TZ *>(a.zin) + (tile * kUmmaTile + warp * 8 + 2 * i + sub) * a.ldzin;
+            for (int e = 0; e < 16; ++e) v[e] = __float_as_uint(__uint_as_float(v[e]) + __uint_as_float(w[e]));
+          } else {
+            asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+          }
+          if (Cfg::kLow && bad) {
+            const TZ *z = static_cast<const TZ *>(a.zin) + t * a.ldzin;
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const int c = col + c4 + e;
+            for (int e = 0; e < 16; ++e) {
+              const int c = col0 + pcol + h * 16 + e;
               if (c >= a.d) continue;
               float acc = 0.f;
 #pragma unroll 1
               for (int j = 0; j < a.k; ++j) acc = fmaf(to_f32(z[j]), to_f32(U[(int64_t)c * a.ldu + j]), acc);
-              o[i][e] = acc;
+              v[e] = __float_as_uint(acc);
             }
           }
-        }
-        if (NSLOT > 0) {
 #pragma unroll
-          for (int i = 0; i < 4; ++i)
+          for (int c = 0; c < 16 / kUnitElems; ++c) {      // 16 bytes of the row
+            const uint32_t off = (((half * 4 + h * (16 / kUnitElems) + c) ^ (lane & 7)) << 4);
+            float f[kUnitElems];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              o[i][e] += piece_element<T>(in[0][i], e);
-              if (NSLOT == 2) o[i][e] += piece_element<T>(in[NSLOT - 1][i], e);
+            for (int e = 0; e < kUnitElems; ++e) f[e] = __uint_as_float(v[c * kUnitElems + e]);
+            if (NSLOT > 0) {
+              float e0[kUnitElems];
+              widen_piece<T>(ld_shared_v4(orow + off), e0);
+#pragma unroll
+              for (int e = 0; e < kUnitElems; ++e) f[e] += e0[e];
             }
+            if (NSLOT == 2) {
+              float p0[kUnitElems];
+              widen_piece<T>(ld_shared_v4(prow + off), p0);
+#pragma unroll
+              for (int e = 0; e < kUnitElems; ++e) f[e] += p0[e];
+            }
+            if constexpr (sizeof(T) == 4)
+              st_shared_v4(orow + off, __float_as_uint(f[0]), __float_as_uint(f[1]), __float_as_uint(f[2]), __float_as_uint(f[3]));
+            else
+              st_shared_v4(orow + off, pack_bf16(f[0], f[1]), pack_bf16(f[2], f[3]), pack_bf16(f[4], f[5]), pack_bf16(f[6], f[7]));
+          }
         }
-        T *out = out0 + col;
-        const int live = live_rows, cols = a.d - (col + c4);
-        if (g == 0) {
-          issue(col + kSplitHalf);
+        if (g == Cfg::kPieces - 1) {                       // the accumulator has been read
+          asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+          __syncwarp();
+          if (lane == 0) mbar_arrive(d_empty_bar(db));
+        }
+        const int col = col0 + g * Cfg::kPieceCols;
+        if (a.tma_out) {
+          asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+          meet();
+          if (half == 0 && lane == 0) {
+            if (NSLOT == 2) mbar_arrive(e_empty_bar(pslot, quarter));
+            if (row0 < a.n && col < a.d) tma_store_2d_hint(&out_map, out, col, (int)row0, stream_out);
+            bulk_commit();
+            // hand back the stage of the store before this one, and this one's too where the ring is short
+            if (Cfg::kHold) {
+              bulk_wait_read<1>();
+              if (held >= 0) mbar_arrive(e_empty_bar(held, quarter));
+              held = eslot;
+            } else {
+              bulk_wait_read<0>();
+              mbar_arrive(e_empty_bar(eslot, quarter));
+            }
+          }
         } else {
-          if (++chunk == nchunks) {
-            chunk = 0;
-            ++tile;
-            if (unit + 1 < count_units) {
-              enter_tile(tile);
-              prefetch(kChunkCols);
+          // any alignment: row by row, 128 bytes of it by one of the two warps
+          meet();
+#pragma unroll 1
+          for (int r = half; r < 32; r += 2) {
+            if (row0 + r >= a.n) break;
+            uint32_t w;
+            asm volatile("ld.shared.b32 %0, [%1];\n"
+                         : "=r"(w) : "r"(out + r * 128 + (((lane >> 2) ^ (r & 7)) << 4) + (lane & 3) * 4) : "memory");
+            T *o = static_cast<T *>(a.dst) + (row0 + r) * a.lddst;
+            if constexpr (sizeof(T) == 4) {
+              if (col + lane < a.d) o[col + lane] = __uint_as_float(w);
+            } else {
+              const int c = col + 2 * lane;
+              if (c < a.d) o[c] = __ushort_as_bfloat16((unsigned short)w);
+              if (c + 1 < a.d) o[c + 1] = __ushort_as_bfloat16((unsigned short)(w >> 16));
             }
           }
-          if (unit + 1 < count_units) issue(chunk * kChunkCols);
-        }
-        if (vec && live == 8) {                            // d is a multiple of 4
-          if (cols > 0) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              if constexpr (sizeof(T) == 4)
-                *reinterpret_cast<float4 *>(out + 2 * i * a.lddst) = make_float4(o[i][0], o[i][1], o[i][2], o[i][3]);
-              else
-                *reinterpret_cast<uint2 *>(out + 2 * i * a.lddst) = make_uint2(pack_bf16(o[i][0], o[i][1]), pack_bf16(o[i][2], o[i][3]));
-            }
-          }
-        } else {
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            if (2 * i + sub >= live) continue;
-#pragma unroll
-            for (int e = 0; e < 4; ++e)
-              if (e < cols) out[2 * i * a.lddst + e] = from_f32<T>(o[i][e]);
+          meet();
+          if (half == 0 && lane == 0) {
+            mbar_arrive(e_empty_bar(eslot, quarter));
+            if (NSLOT == 2) mbar_arrive(e_empty_bar(pslot, quarter));
           }
         }
       }
+      if (++chunk == nchunks) {
+        chunk = 0;
+        ++tile;
+        ++tcount;
+      }
     }
+    if (half == 0 && lane == 0) bulk_wait<0>();
   }
 
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   __syncthreads();
-  if (warp == kSplitOutWarps + kSplitOperandWarps) {
+  if (warp == kSplitMmaWarp) {
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem_base), "r"(Cfg::kTmemCols)
                  : "memory");
