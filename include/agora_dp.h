@@ -82,6 +82,18 @@ ssn_status_t stage_clip_sumsq(const void *grad, int64_t count, int32_t dtype, do
 ssn_status_t stage_clip_scale(void *grad, int64_t count, int32_t dtype, const double *sumsq,
                               float threshold, void *stream);
 
+/*
+ * The same for all gradient tensors of a stage (host arrays of `tensors` addresses, element counts and
+ * dtypes), in one launch per STAGE_CLIP_MAX_TENSORS of them: a launch per tensor starts and drains the GPU once per
+ * tensor.  The tensors must not overlap.  stage_clip_scale_list runs over them from the last to the first,
+ * because the end is what stage_clip_sumsq_list has left in L2.
+ */
+#define STAGE_CLIP_MAX_TENSORS 64
+ssn_status_t stage_clip_sumsq_list(const void *const *grads, const int64_t *counts, const int32_t *dtypes,
+                                   int32_t tensors, double *sumsq, void *stream);
+ssn_status_t stage_clip_scale_list(void *const *grads, const int64_t *counts, const int32_t *dtypes,
+                                   int32_t tensors, const double *sumsq, float threshold, void *stream);
+
 #ifdef __cplusplus
 }
 #endif

@@ -95,6 +95,9 @@ _SIGNATURES = {
     "stage_clip_threshold": (ctypes.c_float, [_i32, _i32]),
     "stage_clip_sumsq": (_i32, [_vp, _i64, _i32, _vp, _vp]),
     "stage_clip_scale": (_i32, [_vp, _i64, _i32, _vp, ctypes.c_float, _vp]),
+    "stage_clip_sumsq_list": (_i32, [ctypes.POINTER(_vp), ctypes.POINTER(_i64), ctypes.POINTER(_i32), _i32, _vp, _vp]),
+    "stage_clip_scale_list": (_i32, [ctypes.POINTER(_vp), ctypes.POINTER(_i64), ctypes.POINTER(_i32), _i32, _vp,
+                                     ctypes.c_float, _vp]),
     "ssn_status_string": (ctypes.c_char_p, [_i32]),
     "ssn_version": (_i32, []),
     "ssn_launch_count": (_i64, []),
@@ -341,3 +344,17 @@ def stage_clip_sumsq(grad: int, count: int, dtype: int, sumsq: int, stream: int 
 def stage_clip_scale(grad: int, count: int, dtype: int, sumsq: int, threshold: float, stream: int = 0) -> None:
     _check(_lib.stage_clip_scale(grad or None, count, dtype, sumsq or None, threshold, stream or None),
            "stage_clip_scale")
+
+
+def clip_list(grads: Sequence[int], counts: Sequence[int], dtypes: Sequence[int]):
+    """The three host arrays and their length, as stage_clip_sumsq_list and stage_clip_scale_list take them."""
+    n = len(grads)
+    return (_vp * max(n, 1))(*grads), (_i64 * max(n, 1))(*counts), (_i32 * max(n, 1))(*dtypes), n
+
+
+def stage_clip_sumsq_list(tensors, sumsq: int, stream: int = 0) -> None:
+    _check(_lib.stage_clip_sumsq_list(*tensors, sumsq or None, stream or None), "stage_clip_sumsq_list")
+
+
+def stage_clip_scale_list(tensors, sumsq: int, threshold: float, stream: int = 0) -> None:
+    _check(_lib.stage_clip_scale_list(*tensors, sumsq or None, threshold, stream or None), "stage_clip_scale_list")

@@ -9,6 +9,7 @@
 
 #include <cmath>
 #include <cstdint>
+#include <utility>
 
 namespace {
 
@@ -204,6 +205,184 @@ __global__ void __launch_bounds__(kThreads) clip_scale_kernel(T *g, int64_t n, c
   }
 }
 
+// ---- clipping of a whole stage: many tensors per launch ------------------------------------------
+// The tensors are cut into chunks of kClipChunkBytes; a block strides over the chunks of all of them.  36 tensors of
+// 973 M bf16 parameters, norm and scaling: a launch per tensor 1219 us, this 945 us (6.2 TB/s).
+constexpr int kClipBlocksPerSm = 8;   // one wave of 2048 threads per SM
+constexpr int kClipChunkBytes = 32768, kClipVecs = kClipChunkBytes / 16 / kThreads;   // 16-byte accesses per thread and chunk
+struct ClipList {
+  void *p[STAGE_CLIP_MAX_TENSORS];
+  int64_t n[STAGE_CLIP_MAX_TENSORS];
+  int32_t first[STAGE_CLIP_MAX_TENSORS + 1];   // first chunk of each tensor
+  uint8_t bf16[STAGE_CLIP_MAX_TENSORS], vec[STAGE_CLIP_MAX_TENSORS];
+  int32_t tensors;
+};
+
+// Elements [lo, hi) of g, 16 bytes at a time where the tensor is aligned.
+template <typename T>
+__device__ __forceinline__ double chunk_sumsq(const T *g, int64_t lo, int64_t hi, bool vec) {
+  constexpr int E = 16 / (int)sizeof(T);
+  double acc = 0.0;
+  int64_t done = lo;
+  if (vec) {
+    const uint4 *gv = reinterpret_cast<const uint4 *>(g + lo);
+    const int nv = (int)((hi - lo) / E);
+    uint4 raw[kClipVecs];
+#pragma unroll
+    for (int j = 0; j < kClipVecs; ++j) {
+      const int i = j * kThreads + threadIdx.x;
+      raw[j] = i < nv ? gv[i] : make_uint4(0, 0, 0, 0);
+    }
+#pragma unroll
+    for (int j = 0; j < kClipVecs; ++j) {
+      const T *e = reinterpret_cast<const T *>(&raw[j]);
+      float part = 0.f;   // the squares of one access in fp32, then into the fp64 sum
+#pragma unroll
+      for (int q = 0; q < E; ++q) {
+        const float v = widen<T>(e[q]);
+        part = fmaf(v, v, part);
+      }
+      acc += (double)part;
+    }
+    done = lo + (int64_t)nv * E;
+  }
+  for (int64_t i = done + threadIdx.x; i < hi; i += kThreads) {
+    const float v = widen<T>(g[i]);
+    acc += (double)v * (double)v;
+  }
+  return acc;
+}
+
+template <typename T>
+__device__ __forceinline__ void chunk_scale(T *g, int64_t lo, int64_t hi, bool vec, float coef) {
+  constexpr int E = 16 / (int)sizeof(T);
+  int64_t done = lo;
+  if (vec) {
+    uint4 *gv = reinterpret_cast<uint4 *>(g + lo);
+    const int nv = (int)((hi - lo) / E);
+    uint4 raw[kClipVecs];
+#pragma unroll
+    for (int j = 0; j < kClipVecs; ++j) {
+      const int i = j * kThreads + threadIdx.x;
+      if (i < nv) raw[j] = gv[i];
+    }
+#pragma unroll
+    for (int j = 0; j < kClipVecs; ++j) {
+      const int i = j * kThreads + threadIdx.x;
+      T *e = reinterpret_cast<T *>(&raw[j]);
+#pragma unroll
+      for (int q = 0; q < E; ++q) e[q] = narrow<T>(widen<T>(e[q]) * coef);
+      if (i < nv) gv[i] = raw[j];
+    }
+    done = lo + (int64_t)nv * E;
+  }
+  for (int64_t i = done + threadIdx.x; i < hi; i += kThreads) g[i] = narrow<T>(widen<T>(g[i]) * coef);
+}
+
+// Tensor of chunk c (the chunks of a block go up or down, so the search starts where the last one ended) and the
+// chunk's elements.
+__device__ __forceinline__ void locate_chunk(const ClipList &a, int c, int &t, int64_t &lo, int64_t &hi) {
+  while (c >= a.first[t + 1]) ++t;
+  while (c < a.first[t]) --t;
+  const int64_t per = kClipChunkBytes / (a.bf16[t] ? 2 : 4);
+  lo = (int64_t)(c - a.first[t]) * per;
+  hi = lo + per < a.n[t] ? lo + per : a.n[t];
+}
+
+__global__ void __launch_bounds__(kThreads) sumsq_list_kernel(const __grid_constant__ ClipList a, double *sumsq) {
+  double acc = 0.0;
+  int t = 0;
+  for (int c = blockIdx.x; c < a.first[a.tensors]; c += gridDim.x) {
+    int64_t lo, hi;
+    locate_chunk(a, c, t, lo, hi);
+    acc += a.bf16[t] ? chunk_sumsq(static_cast<const __nv_bfloat16 *>(a.p[t]), lo, hi, a.vec[t])
+                     : chunk_sumsq(static_cast<const float *>(a.p[t]), lo, hi, a.vec[t]);
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+  __shared__ double warp_sums[kThreads / 32];
+  if ((threadIdx.x & 31) == 0) warp_sums[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double total = 0.0;
+    for (int w = 0; w < kThreads / 32; ++w) total += warp_sums[w];
+    atomicAdd(sumsq, total);
+  }
+}
+
+__global__ void __launch_bounds__(kThreads) clip_scale_list_kernel(const __grid_constant__ ClipList a, const double *sumsq, float threshold) {
+  const float norm = (float)sqrt(*sumsq);
+  const float coef = fminf(1.f, threshold / (norm + 1e-6f));
+  if (!(coef < 1.f)) return;   // inside the budget: nothing to write
+  int t = a.tensors - 1;
+  for (int c = a.first[a.tensors] - 1 - (int)blockIdx.x; c >= 0; c -= gridDim.x) {
+    int64_t lo, hi;
+    locate_chunk(a, c, t, lo, hi);
+    if (a.bf16[t])
+      chunk_scale(static_cast<__nv_bfloat16 *>(a.p[t]), lo, hi, a.vec[t], coef);
+    else
+      chunk_scale(static_cast<float *>(a.p[t]), lo, hi, a.vec[t], coef);
+  }
+}
+
+ssn_status_t check_clip_list(const void *const *grads, const int64_t *counts, const int32_t *dtypes, int32_t tensors) {
+  if (tensors < 0) return SSN_ERR_SHAPE;
+  if (tensors > 0 && (grads == nullptr || counts == nullptr || dtypes == nullptr)) return SSN_ERR_NULL;
+  for (int32_t i = 0; i < tensors; ++i) {
+    if (dtypes[i] != SSN_F32 && dtypes[i] != SSN_BF16) return SSN_ERR_DTYPE;
+    if (counts[i] < 0 || counts[i] > (int64_t)1 << 42) return SSN_ERR_SHAPE;
+    if (counts[i] > 0 && grads[i] == nullptr) return SSN_ERR_NULL;
+  }
+  return SSN_OK;
+}
+
+// Groups of up to STAGE_CLIP_MAX_TENSORS tensors (and fewer than 2^31 chunks), handed to launch(list, blocks).
+template <typename Launch>
+ssn_status_t for_clip_groups(const void *const *grads, const int64_t *counts, const int32_t *dtypes, int32_t tensors, bool backwards,
+                             Launch launch) {
+  int32_t done = 0;
+  while (done < tensors) {
+    ClipList a{};
+    int64_t chunks = 0;
+    for (; done < tensors && a.tensors < STAGE_CLIP_MAX_TENSORS; ++done) {
+      // backwards: the groups from the last tensor on, each still in ascending order inside
+      const int32_t i = backwards ? tensors - 1 - done : done;
+      const int64_t per = kClipChunkBytes / (dtypes[i] == SSN_BF16 ? 2 : 4), c = (counts[i] + per - 1) / per;
+      if (chunks + c > 0x7fffffffLL - 65536) {
+        if (a.tensors == 0) return SSN_ERR_SHAPE;
+        break;
+      }
+      if (c == 0) continue;
+      const int32_t k = a.tensors++;
+      a.p[k] = const_cast<void *>(grads[i]);
+      a.n[k] = counts[i];
+      a.bf16[k] = dtypes[i] == SSN_BF16;
+      a.vec[k] = aligned16(grads[i]);
+      chunks += c;
+      a.first[k + 1] = (int32_t)chunks;
+    }
+    if (chunks == 0) continue;
+    if (backwards) {   // ascending order inside the group: turn the list around
+      for (int32_t l = 0, r = a.tensors - 1; l < r; ++l, --r) {
+        std::swap(a.p[l], a.p[r]);
+        std::swap(a.n[l], a.n[r]);
+        std::swap(a.bf16[l], a.bf16[r]);
+        std::swap(a.vec[l], a.vec[r]);
+      }
+      int32_t at = 0;
+      for (int32_t k = 0; k < a.tensors; ++k) {
+        const int64_t per = kClipChunkBytes / (a.bf16[k] ? 2 : 4);
+        at += (int32_t)((a.n[k] + per - 1) / per);
+        a.first[k + 1] = at;
+      }
+    }
+    const int64_t cap = (int64_t)(sm_count() > 0 ? sm_count() : 148) * kClipBlocksPerSm;
+    launch(a, (unsigned)(chunks < cap ? chunks : cap));
+    if (finish() != SSN_OK) return SSN_ERR_CUDA;
+  }
+  return SSN_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -320,6 +499,29 @@ ssn_status_t stage_clip_scale(void *grad, int64_t count, int32_t dtype, const do
     else clip_scale_kernel<__nv_bfloat16, false><<<grid_for(count), kThreads, 0, s>>>(g, count, sumsq, threshold);
   }
   return finish();
+}
+
+ssn_status_t stage_clip_sumsq_list(const void *const *grads, const int64_t *counts, const int32_t *dtypes, int32_t tensors,
+                                   double *sumsq, void *stream) {
+  const ssn_status_t st = check_clip_list(grads, counts, dtypes, tensors);
+  if (st != SSN_OK) return st;
+  if (sumsq == nullptr) return SSN_ERR_NULL;
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  return for_clip_groups(grads, counts, dtypes, tensors, false, [&](const ClipList &a, unsigned blocks) {
+    sumsq_list_kernel<<<blocks, kThreads, 0, s>>>(a, sumsq);
+  });
+}
+
+ssn_status_t stage_clip_scale_list(void *const *grads, const int64_t *counts, const int32_t *dtypes, int32_t tensors,
+                                   const double *sumsq, float threshold, void *stream) {
+  const ssn_status_t st = check_clip_list(grads, counts, dtypes, tensors);
+  if (st != SSN_OK) return st;
+  if (!(threshold > 0.f)) return SSN_ERR_SHAPE;
+  if (sumsq == nullptr) return SSN_ERR_NULL;
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  return for_clip_groups(grads, counts, dtypes, tensors, true, [&](const ClipList &a, unsigned blocks) {
+    clip_scale_list_kernel<<<blocks, kThreads, 0, s>>>(a, sumsq, threshold);
+  });
 }
 
 }  // extern "C"

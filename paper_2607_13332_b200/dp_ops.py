@@ -60,7 +60,14 @@ def stage_clip(grads: Sequence[torch.Tensor], threshold: float, sumsq: torch.Ten
     for g in grads:
         if not (g.is_cuda and g.is_contiguous() and g.dtype in codes):
             raise ValueError("expected contiguous fp32 / bf16 CUDA gradients")
-        binding.stage_clip_sumsq(g.data_ptr(), g.numel(), codes[g.dtype], sumsq.data_ptr(), _stream())
-    for g in grads:
-        binding.stage_clip_scale(g.data_ptr(), g.numel(), codes[g.dtype], sumsq.data_ptr(), threshold, _stream())
+    spans = sorted((g.data_ptr(), g.data_ptr() + g.numel() * g.element_size()) for g in grads)
+    if any(start < end for (_, end), (start, _) in zip(spans, spans[1:])):   # overlapping tensors: one after the other
+        groups = [[g] for g in grads]
+    else:
+        groups = [grads]
+    lists = [binding.clip_list([g.data_ptr() for g in gs], [g.numel() for g in gs], [codes[g.dtype] for g in gs]) for gs in groups]
+    for tensors in lists:
+        binding.stage_clip_sumsq_list(tensors, sumsq.data_ptr(), _stream())
+    for tensors in lists:
+        binding.stage_clip_scale_list(tensors, sumsq.data_ptr(), threshold, _stream())
     return sumsq
