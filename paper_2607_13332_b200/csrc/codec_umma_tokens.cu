@@ -14,9 +14,9 @@ cudaError_t launch_tokens_ntp(const TokensArgs &t, const UmmaTokensMaps &maps, i
     cudaError_t e = allow_dynamic_smem(kernel, smem, configured);
     if (e != cudaSuccess) return e;
   }
-  kernel<<<(unsigned)grid, kTokensThreads, smem, stream>>>(t, maps);
+  const cudaError_t e = launch_dependent(kernel, (unsigned)grid, kTokensThreads, smem, stream, 1, t, maps);
   note_kernel(SSN_KERNEL_UMMA_TOKENS, NTP > 8 ? SSN_KVAR_WIDE : 0);
-  return cudaGetLastError();
+  return e;
 }
 }  // namespace
 
@@ -31,30 +31,19 @@ cudaError_t launch_codec_umma_tokens(const __nv_bfloat16 *H, int64_t ldh, const 
   if (!make_sw128_map(&maps.c_wide, C, n, k <= 64 ? 64 : 128, ldc, kUmmaCols)) return cudaErrorNotSupported;
   const int nblk = (m + kUmmaTile - 1) / kUmmaTile;
   const int64_t nstage = (n + kUmmaCols - 1) / kUmmaCols;
-  // CTAs per column block: the count (up to 16) that fills whole waves of SMs best
-  int64_t splits = 1;
-  double best = 0.0;
-  for (int64_t s = 1; s <= 16 && s <= nstage; ++s) {
-    const int64_t ctas = nblk * s, waves = (ctas + sm_count - 1) / sm_count;
-    const double fill = (double)ctas / (double)(waves * sm_count);
-    if (fill > best + 1e-9) {
-      best = fill;
-      splits = s;
-    }
-  }
+  const int64_t units = nblk * nstage;
+  const int grid = (int)(units < sm_count ? units : sm_count);
   TokensArgs t{};
   t.out = out;
   t.ldout = ldout;
   t.n = n;
   t.m = m;
   t.k = k;
-  t.splits = (int32_t)splits;
   t.dev_status = dev_status;
-  if (splits > 1) {
+  if (nblk % grid != 0 || nstage > kTokensChain) {   // some block is summed in parts
     cudaError_t e = cudaMemset2DAsync(out, (size_t)ldout * sizeof(float), 0, (size_t)k * sizeof(float), (size_t)m, stream);
     if (e != cudaSuccess) return e;
   }
-  const int grid = (int)(nblk * splits);
   const int ntp = 2 * ((k + 15) / 16);
   if (ntp <= 2) return launch_tokens_ntp<2>(t, maps, grid, stream);
   if (ntp <= 4) return launch_tokens_ntp<4>(t, maps, grid, stream);
