@@ -11,8 +11,9 @@
 // One CTA per SM takes an equal, contiguous range of all (column block, stage) pairs, so it streams without a
 // pause and ends with the others.  At the end of a block, and after kTokensChain stages of one, the fp32 partial
 // sums are added to the (zeroed) output with red.global, from one of two accumulators while the next stages
-// go on in the other.  A block summed at once is stored.  (As a grid of one CTA per block and token
-// range, ten waves of 20 stages for 14336 columns: 140 us for 16384 tokens, rank 40; this TIME us.)
+// go on in the other.  A block summed at once is stored.  (As a grid of one CTA per block and token range, ten
+// waves of 20 stages for 14336 columns: 170 us with the projection in front of it, 16384 tokens, rank 40; like
+// this 131 us.  CTAs that walk the blocks in step, so that together they read whole rows of H: 142 us.)
 //
 //   warp 0  producer     warp 1  MMA issuer, owns the TMEM allocation     warps 2-5  epilogue
 // Every wait is bounded; a wait that runs out sets the status word (when given) and the kernel
