@@ -47,8 +47,9 @@
  *     tail of the earlier one (programmatic dependent launch); what either reads or writes is as
  *     if the calls ran one after the other.
  *   - bf16 buffers whose pointers are 16-byte aligned and whose leading dimensions are
- *     multiples of 8 take the vectorised tensor-core kernels; anything else (fp32, odd
- *     leading dimensions, unaligned views) is still computed, by slower general kernels.
+ *     multiples of 8 take the TMA kernels; anything else (fp32, odd leading dimensions,
+ *     unaligned views) is computed by tensor-core kernels that split their operands in
+ *     registers (rank up to 128), or by slower general kernels.
  */
 #ifndef SSN_H_
 #define SSN_H_
@@ -94,8 +95,9 @@ typedef enum { SSN_GRAD_COEFF = 1, SSN_GRAD_FULL = 2 } ssn_grad_mode_t;
  * dimensions that are multiples of 8 elements (bf16) for U, X / G / Xhat, E, P and the weights,
  * and for Z where it is read (decompress).  A rank that is not a multiple of 8 (the paper's 8B
  * run uses ~51) is fine as long as U and Z are STORED with such a leading dimension (ldu = 56,
- * say; the padding columns are never read as data).  Anything else still gives the same results,
- * through the general kernels, two orders of magnitude slower.
+ * say; the padding columns are never read as data).  Anything else still gives the same results:
+ * projections and expansions of rank up to 128 about three times slower, the rest through the
+ * general kernels, two orders of magnitude slower.
  */
 typedef struct ssn_codec {
   int32_t d;            /* model width, >= 1                                              */
@@ -307,7 +309,7 @@ ssn_status_t ssn_head_embed(const ssn_codec_t *codec, const void *Elow, int64_t 
  *                         of a coordinate, far below the single bf16 rounding of X^; for that the
  *                         call needs a 256-byte aligned workspace of
  *                         ssn_decompress_wire_workspace_bytes() bytes.  With a smaller (or
- *                         misaligned) workspace the general kernel runs; with_ids always needs
+ *                         misaligned) workspace the fp32 words are split in the kernel; with_ids always needs
  *                         at least n_tokens * 4 bytes (rounded up to 256).
  * Errors as for the calls they mirror, plus SSN_ERR_WORKSPACE.
  */
@@ -335,8 +337,8 @@ ssn_status_t ssn_decompress_wire(const ssn_codec_t *codec, const void *wire, int
  *   SSN_OUT_WIRE      wire rows, ldout >= k words                          (as ssn_compress_wire)
  *   SSN_OUT_WIRE_IDS  wire rows with the id word, ldout >= k + 1 words
  * Everything else as for ssn_compress.  Performance note: the tensor-core kernel takes this call
- * for a codec without E and P or with the prepared tables (ssn_prepare_tables); a codec that has
- * to gather E or P rows runs the general kernel here.
+ * for a codec without E and P or with the prepared tables (ssn_prepare_tables); for a codec that
+ * has to gather E or P rows the split projection adds R to the residual.
  */
 enum { SSN_OUT_STORAGE = 0, SSN_OUT_WIRE = 1, SSN_OUT_WIRE_IDS = 2 };
 ssn_status_t ssn_compress_sum(const ssn_codec_t *codec, const void *X, int64_t ldx, const void *R,

@@ -95,7 +95,11 @@ struct UmmaExpandConfig {
       kZBufs * kZBytes + kSelBytes + kUStages * kUStageBytes + kStagingBytes;
   static constexpr int kMaxSmem = 227 * 1024;
   static constexpr int kEFit = (kMaxSmem - 1024 - 1024 - kFixedBytes) / kEStageBytes;
-  static constexpr int kEStages = kGathered > 0 ? (kEFit < 12 ? kEFit : 12) : 0;
+  // A chunk takes 2 kGathered stages and the two epilogue groups take alternate chunks, so with E and P pieces a
+  // ring of 8 brings every group back to stages it consumed itself.  (A wait on a phase is only sound when the
+  // phase before it is known to be over; with 10 stages that would be the other group's, two chunks back.)
+  static constexpr int kEMost = kGathered == 2 ? 8 : 12;
+  static constexpr int kEStages = kGathered > 0 ? (kEFit < kEMost ? kEFit : kEMost) : 0;
   static_assert(kGathered == 0 || kEStages >= 4, "no room for the E ring");
   static constexpr int kDBufs = 2;                 // accumulators of 128 columns: one per epilogue group
   static constexpr int kTmemCols = 256;
