@@ -51,7 +51,12 @@ struct SplitProjectConfig {
   static constexpr int kNX = kF32 || NSLOT > 0 ? 3 : 1;    // parts of the residual
   static constexpr int kNU = kF32 ? 3 : 1;                 // parts of U
   static constexpr int kStack = kNU == 3 ? (KN <= 64 ? 3 : 2) : 1;   // parts of U under one Ah product
-  static constexpr int kDCols = kNX == 1 ? KN : (kStack == 3 ? 3 : 2) * KN;
+  // KN-wide accumulators of a chain, all of them summed in fp32 where it ends.  fp32: hi and low products, side by
+  // side.  bf16 bases leave room to deal the K steps of the leading product to several: gradients
+  // of 4096 columns, rank 51, one accumulator 1.6e-7 from 64-bit sums, four 9.2e-8, plain FMAs 9.5e-8.
+  static constexpr int kHiAccs = kNU == 3 ? 1 : (kNX == 1 ? (KN <= 64 ? 4 : 2) : (KN <= 64 ? 2 : 1));
+  static constexpr int kAccs = kNU == 3 ? kStack : kHiAccs + (kNX == 3 ? 1 : 0);
+  static constexpr int kDCols = kAccs * KN;
   static constexpr int kDStride = kDCols <= 32 ? 32 : (kDCols <= 64 ? 64 : (kDCols <= 128 ? 128 : 256));
   static constexpr int kTmemCols = 2 * kDStride;
   static constexpr int kCols = kF32 ? 32 : 64;              // columns of d per step
@@ -230,12 +235,12 @@ __global__ void __launch_bounds__(kSplitProjectThreads, 1) codec_split_project_k
         for (int j = 0; j < Cfg::kCols / 16; ++j) {
           const uint64_t A = ad + j * 2, B = bd + j * 128;   // 32 bytes of an A row; 16 rows of B
           const uint32_t more = in_chain > 0 || j > 0 ? 1u : 0u;
-          if (NX == 1) {
-            umma_bf16(D, A, B, id1, more);
-          } else if (NU == 1) {
-            umma_bf16(D, A, B, id1, more);
-            umma_bf16(D + KN, A + kPart, B, id1, more);
-            umma_bf16(D + KN, A + 2 * kPart, B, id1, 1u);
+          if (NU == 1) {                       // a bf16 chain is one step
+            umma_bf16(D + (j % Cfg::kHiAccs) * KN, A, B, id1, j >= Cfg::kHiAccs ? 1u : 0u);
+            if (NX == 3) {
+              umma_bf16(D + Cfg::kHiAccs * KN, A + kPart, B, id1, more);
+              umma_bf16(D + Cfg::kHiAccs * KN, A + 2 * kPart, B, id1, 1u);
+            }
           } else if (Cfg::kStack == 3) {
             umma_bf16(D, A, B, id3, more);
             umma_bf16(D + KN, A + kPart, B, id2, 1u);
@@ -352,21 +357,16 @@ __global__ void __launch_bounds__(kSplitProjectThreads, 1) codec_split_project_k
         const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)buf * Cfg::kDStride + sum_col;
 #pragma unroll
         for (int i = 0; i < Cfg::kSums; i += 8) {
-          uint32_t v0[8], v1[8], v2[8];
-          tmem_ld8(taddr + i, v0);
-          if (NX > 1) tmem_ld8(taddr + KN + i, v1);
-          if (Cfg::kStack == 3) tmem_ld8(taddr + 2 * KN + i, v2);
+          uint32_t v[Cfg::kAccs][8];
+#pragma unroll
+          for (int c2 = 0; c2 < Cfg::kAccs; ++c2) tmem_ld8(taddr + c2 * KN + i, v[c2]);
           asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
 #pragma unroll
           for (int e = 0; e < 8; e += 2) {
-            float w0 = __uint_as_float(v0[e]), w1 = __uint_as_float(v0[e + 1]);
-            if (Cfg::kStack == 3) {
-              float x0 = __uint_as_float(v1[e]), x1 = __uint_as_float(v1[e + 1]);
-              add2(x0, x1, __uint_as_float(v2[e]), __uint_as_float(v2[e + 1]));
-              add2(w0, w1, x0, x1);
-            } else if (NX > 1) {
-              add2(w0, w1, __uint_as_float(v1[e]), __uint_as_float(v1[e + 1]));
-            }
+            // from the last on: the low products come last
+            float w0 = __uint_as_float(v[Cfg::kAccs - 1][e]), w1 = __uint_as_float(v[Cfg::kAccs - 1][e + 1]);
+#pragma unroll
+            for (int c2 = Cfg::kAccs - 2; c2 >= 0; --c2) add2(w0, w1, __uint_as_float(v[c2][e]), __uint_as_float(v[c2][e + 1]));
             add2(sum[i + e], sum[i + e + 1], w0, w1);
           }
         }

@@ -82,16 +82,17 @@ class Codec:
         again after changing U, E or P in place."""
         dev = self.U.device
         self.drop_tables()
+        pitch = -(-self.k // 4) * 4      # compress reads the rows 16 bytes at a time (rank 67, 11967 x 2560: 48 -> 39 us)
         if embedding and self.E is not None:
-            self.EU = torch.empty((self.E.shape[0], self.k), dtype=torch.float32, device=dev)
+            self.EU = torch.empty((self.E.shape[0], pitch), dtype=torch.float32, device=dev)[:, :self.k]
         if positions and self.P is not None:
-            self.PU = torch.empty((self.P.shape[0], self.k), dtype=torch.float32, device=dev)
-        binding.ssn_prepare_tables(self.c, self.EU.data_ptr() if self.EU is not None else 0, self.k,
-                                   self.PU.data_ptr() if self.PU is not None else 0, self.k, _stream())
+            self.PU = torch.empty((self.P.shape[0], pitch), dtype=torch.float32, device=dev)[:, :self.k]
+        binding.ssn_prepare_tables(self.c, self.EU.data_ptr() if self.EU is not None else 0, pitch,
+                                   self.PU.data_ptr() if self.PU is not None else 0, pitch, _stream())
         if self.EU is not None:
-            self.c.EU, self.c.ldeu = self.EU.data_ptr(), self.k
+            self.c.EU, self.c.ldeu = self.EU.data_ptr(), pitch
         if self.PU is not None:
-            self.c.PU, self.c.ldpu = self.PU.data_ptr(), self.k
+            self.c.PU, self.c.ldpu = self.PU.data_ptr(), pitch
 
     def drop_tables(self) -> None:
         self.c.EU = self.c.PU = None
