@@ -149,12 +149,14 @@ bool codec_mma_supports(int d, int k) {
 
 cudaError_t launch_codec_mma(const MmaArgs &a, bool shift, int mode, int sm_count,
                              cudaStream_t stream) {
-  // Up to 16 tokens per SM the few-rows kernel has the shorter start: it wins until its own work (its warps
-  // read all of U) outgrows that, at about 65536 elements of U.  us, E and P rows, tcgen05 -> few rows: 2048
-  // tokens, rank 40: 512 columns 10.0 -> 6.8, 1536 columns 13.1 -> 10.5, 4096 columns 21.1 -> 21.1 (no tables: 15.9
-  // -> 18.9); rank 16, 4096 columns 20.2 -> 13.6.  Wire rows keep their kernel.
-  const bool few_rows = a.n <= 16 * (int64_t)sm_count && a.k <= 64 && (int64_t)a.d * a.k <= 65536 &&
-                        a.zout32 == nullptr && a.src2 == nullptr;
+  // Up to 16 tokens per SM the few-rows kernel has the shorter start, until its own work (its warps read all of U)
+  // outgrows that.  us, no tables, 2048 tokens, tcgen05 -> few rows: rank 8, 4096 columns 15.5 -> 7.8; rank 16, 512
+  // columns 6.4 -> 3.7, 4096 columns 15.1 -> 9.7; rank 40, 512 columns 7.1 -> 5.0, 1024 columns 8.3 -> 7.0; rank 64,
+  // 512 columns 7.6 -> 7.2, 1024 columns 8.9 -> 10.7.  Only without E and P: this kernel rounds the residual
+  // x - e - p to bf16, the tcgen05 one contracts X, E and P each as it is, or subtracts the rows of prepared tables.
+  // Wire rows keep their kernel.
+  const bool few_rows = !shift && a.n <= 16 * (int64_t)sm_count && a.k <= 64 &&
+                        (int64_t)a.d * a.k <= (a.k <= 32 ? 65536 : 45056) && a.zout32 == nullptr && a.src2 == nullptr;
   if (mode == kModeProject && !few_rows) {
     cudaError_t e = launch_codec_umma_project(a, shift, sm_count, stream);
     if (e != cudaErrorNotSupported) return e;
