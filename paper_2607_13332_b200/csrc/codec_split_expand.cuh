@@ -20,7 +20,8 @@
 //                the small ones (hm, mh, mm, hl, lh) into a second, two sets of both.  A warp of its own, since
 //                every MMA blocks its thread for about 80 clocks.
 //
-// Coordinates past k are zeroed once, rows past n or d repeat the last one and are never stored.
+// Coordinates past k are zeroed once (above rank 64, where a stage of U serves both groups of 64, with every tile
+// of U), rows past n or d repeat the last one and are never stored.
 #pragma once
 
 #include <type_traits>
@@ -165,6 +166,7 @@ __global__ void __launch_bounds__(kSplitExpandThreads, 1) codec_split_expand_ker
     const int row0 = ow * rpw + (lane >> lpr_log), pair = lane & ((1 << lpr_log) - 1);
     const int nit = kUmmaTile / (kSplitOperandWarps * rpw), row_step = kSplitOperandWarps * rpw;
     const uint32_t off0 = row0 * 128 + (((pair >> 2) ^ (row0 & 7)) << 4) + (pair & 3) * 4;
+    const int ksteps16 = (a.k + 15) & ~15;   // coordinates that the MMAs read
     // rows first .. first + 127 of a matrix (the last one repeated), coordinates 64 kg ..: parts into smem
     auto move_tile = [&](auto np, auto batch, const auto *M, int64_t ld, int64_t first, int64_t rows, int kg, bool vec_m,
                          uint32_t base, uint32_t part_bytes, int class_slot, auto wait_free) {
@@ -210,6 +212,14 @@ __global__ void __launch_bounds__(kSplitExpandThreads, 1) codec_split_expand_ker
 #pragma unroll
             for (int s = 0; s < NP; ++s) st_shared_b32(dst + (uint32_t)i * row_step * 128 + s * part_bytes, p[s]);
           }
+        } else if (KG == 2 && class_slot < 0 && j < ksteps16) {
+          // A stage of U that held the first 64 coordinates of another chunk now holds the second: what the last
+          // K step reads past k must be zero again, since 0 (of Z) times a stale infinity is no 0.
+          const uint32_t dst = base + off0 + (uint32_t)b * row_step * 128;
+#pragma unroll
+          for (int i = 0; i < B; ++i)
+#pragma unroll
+            for (int s = 0; s < NP; ++s) st_shared_b32(dst + (uint32_t)i * row_step * 128 + s * part_bytes, 0);
         }
       }
       return largest;

@@ -118,3 +118,26 @@ def test_rows_the_split_does_not_hold(n, d, k):
         _same_as_plain_sums(host64(codec.grad_project(to_device(finite["X"], dt)), dt), X @ U, "projection, U")
         _same_as_plain_sums(host64(codec.decompress(to_device(finite["Z0"], dt)), dt), Z @ U.T, "expansion, U")
     assert codec.take_status() == 0
+
+
+@pytest.mark.parametrize("k", [72, 100, 127])
+@pytest.mark.parametrize("bad", [np.inf, np.nan])
+def test_a_bad_basis_value_stays_in_its_column(k, bad):
+    """Above rank 64 a stage of U serves both groups of 64 coordinates, of one chunk of columns after the other:
+    an infinity or NaN in row r of U belongs to output column r and to no column of another chunk."""
+    n, d, dt = 4000, 1664, synth.BF16                   # 32 x 13 units, several per CTA
+    t = _inputs(n, d, k, dt, seed=k)
+    U = t["U"].copy()
+    U[[5, 700, 1663], [40, 15, 63]] = synth.to_storage(np.array([bad], np.float64), dt)[0]
+    codec = Codec(dt, _strided(U, dt, 3))
+    finite = np.setdiff1d(np.arange(d), [5, 700, 1663])
+    expect = f64(t["Z0"], dt) @ f64(t["U"], dt).T
+    out = host64(codec.decompress(_strided(t["Z0"], dt, 3)), dt)
+    assert B.ssn_last_kernel()[0] == B.SSN_KERNEL_SPLIT_EXPAND
+    assert_close(out[:, finite], expect[:, finite], dt, "decompress")
+    assert not np.isfinite(out[:, [5, 700, 1663]]).any()
+    wire = torch.from_numpy(f64(t["Z0"], dt).astype(np.float32)).cuda().view(torch.int32)
+    out = host64(codec.decompress_wire(wire, use_workspace=False), dt)
+    assert B.ssn_last_kernel()[0] == B.SSN_KERNEL_SPLIT_EXPAND
+    assert_close(out[:, finite], expect[:, finite], dt, "decompress_wire")
+    assert not np.isfinite(out[:, [5, 700, 1663]]).any()
