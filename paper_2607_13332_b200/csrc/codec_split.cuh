@@ -9,9 +9,11 @@
 // 1e-7).  Both kernels therefore keep the chains short: the small products have an accumulator of
 // their own, and the projection moves the leading one to registers (fp32 additions) every 64 columns.
 //
-// The split needs room below and above x: rows whose largest magnitude is under kSplitTiny (the low
-// terms would leave the range of bf16) or at or over kSplitHuge (h, or a partial sum of it, would
-// overflow; infinities too) are flagged and computed with plain fp32 FMAs instead.
+// The split needs room: the products of the low parts must not fall below the range of fp32 (2^-126), nor sums of the
+// leading ones rise above it.  A row whose largest magnitude is below kSplitTinyRow, or a row or column of an fp32
+// U below kSplitTinyU, is computed with plain sums instead, and so is what overflows: the expansion looks for magnitudes
+// from kSplitHugeRow and kSplitHugeU on (infinities too), the projection, whose sums are long, for
+// sums that are not finite.
 #pragma once
 
 #include "codec_umma.cuh"
@@ -19,13 +21,7 @@
 
 namespace ssn {
 
-constexpr float kSplitHuge = 0x1p120f, kSplitTiny = 0x1p-80f;
-
-// `largest`: by fmaxf over magnitudes, which skips NaN: a NaN stays one through its leading part, and makes
-// every sum it enters NaN, as it does in plain FMAs.
-__device__ __forceinline__ bool split_unsafe(float largest) {
-  return largest >= kSplitHuge || (largest != 0.f && largest < kSplitTiny);
-}
+constexpr float kSplitTinyRow = 0x1p-70f, kSplitTinyU = 0x1p-40f, kSplitHugeRow = 0x1p80f, kSplitHugeU = 0x1p40f;
 
 // Two fp32 operations in one instruction.
 __device__ __forceinline__ void sub2(float &a0, float &a1, float b0, float b1) {
@@ -162,6 +158,11 @@ template <typename T>
 __device__ __forceinline__ float pair_magnitude(const Pair<T> &v) {   // of the larger one
   if constexpr (sizeof(T) == 4) return fmaxf(fabsf(__uint_as_float(v.w[0])), fabsf(__uint_as_float(v.w[1])));
   else return fmaxf(fabsf(__uint_as_float(v.w[0] << 16)), fabsf(__uint_as_float(v.w[0] & 0xFFFF0000u)));
+}
+template <typename T>
+__device__ __forceinline__ void pair_maxima(const Pair<T> &v, float (&m)[2]) {   // of either one, into running maxima
+  m[0] = fmaxf(m[0], fabsf(__uint_as_float(sizeof(T) == 4 ? v.w[0] : v.w[0] << 16)));
+  m[1] = fmaxf(m[1], fabsf(__uint_as_float(sizeof(T) == 4 ? v.w[1] : v.w[0] & 0xFFFF0000u)));
 }
 // Its bf16 parts: three of an fp32 pair (or NP = 1), itself for a bf16 pair.
 template <typename T, int NP>

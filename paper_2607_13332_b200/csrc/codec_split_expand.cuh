@@ -76,10 +76,10 @@ struct SplitExpandConfig {
   static_assert(kSmemBytes <= 227 * 1024, "the operands do not fit in shared memory");
 };
 
-// What a row's largest magnitude says about its split, ordered so that the larger class of two halves is
-// that of the whole row.
+// What a row's largest magnitude (by fmaxf, which skips NaN: a NaN stays one through its leading part) says about its
+// split, ordered so that the larger class of two halves is that of the whole row.
 __device__ __forceinline__ unsigned char magnitude_class(float largest) {
-  return largest == 0.f ? 0 : (largest < kSplitTiny ? 1 : (largest < kSplitHuge ? 2 : 3));
+  return largest == 0.f ? 0 : (largest < kSplitTinyRow ? 1 : (largest < kSplitHugeRow ? 2 : 3));
 }
 
 template <typename T, typename TZ, int KG, int NSLOT>
@@ -174,6 +174,7 @@ __global__ void __launch_bounds__(kSplitExpandThreads, 1) codec_split_expand_ker
       using E = std::remove_const_t<std::remove_pointer_t<decltype(M)>>;
       const int j = kg * 64 + 2 * pair, valid = a.k - j;
       float largest = 0.f;
+      bool tiny = false;                                 // a row of U that its split does not hold
       const bool inside = first + kUmmaTile <= rows;
       const E *col = M + (first + row0) * ld + j;        // read only where `inside`
       const int64_t step = (int64_t)row_step * ld;
@@ -201,6 +202,24 @@ __global__ void __launch_bounds__(kSplitExpandThreads, 1) codec_split_expand_ker
             }
           }
         }
+        if (NP == 3 && class_slot < 0) {
+          float m[B];
+          bool some = false;
+#pragma unroll
+          for (int i = 0; i < B; ++i) {
+            m[i] = valid > 0 ? pair_magnitude<E>(joined<E>(v[i])) : 0.f;
+            some = some || (m[i] != 0.f && m[i] < kSplitTinyU);
+          }
+          if (__any_sync(0xffffffffu, some)) {           // hardly ever: look at whole rows
+#pragma unroll
+            for (int i = 0; i < B; ++i) {
+#pragma unroll
+              for (int off = 16; off > 0; off >>= 1)
+                if (off < (1 << lpr_log)) m[i] = fmaxf(m[i], __shfl_xor_sync(0xffffffffu, m[i], off));
+              tiny = tiny || (m[i] != 0.f && m[i] < kSplitTinyU);
+            }
+          }
+        }
         if (valid > 0) {
           const uint32_t dst = base + off0 + (uint32_t)b * row_step * 128;
 #pragma unroll
@@ -222,7 +241,7 @@ __global__ void __launch_bounds__(kSplitExpandThreads, 1) codec_split_expand_ker
             for (int s = 0; s < NP; ++s) st_shared_b32(dst + (uint32_t)i * row_step * 128 + s * part_bytes, 0);
         }
       }
-      return largest;
+      return tiny || largest >= kSplitHugeU;             // U only
     };
     using Eight = std::integral_constant<int, 8>;
     using Four = std::integral_constant<int, 4>;
@@ -249,7 +268,7 @@ __global__ void __launch_bounds__(kSplitExpandThreads, 1) codec_split_expand_ker
         if (lane == 0) mbar_arrive(z_full_bar(zb));
       }
       const int col0 = chunk * kChunkCols;
-      bool huge = false;
+      bool flagged = false;
       for (int kg = 0; kg < KG; ++kg) {
         auto u_tile = [&](auto batch) {
           return move_tile(std::integral_constant<int, NU>{}, batch, U, a.ldu, (int64_t)col0, (int64_t)a.d, kg, a.vec_u != 0,
@@ -257,10 +276,10 @@ __global__ void __launch_bounds__(kSplitExpandThreads, 1) codec_split_expand_ker
                              if (!dead && !mbar_wait(u_empty_bar(slot), parity)) timed_out();
                            });
         };
-        const float largest = nit >= 8 ? u_tile(Eight{}) : u_tile(Four{});
+        const bool bad = nit >= 8 ? u_tile(Eight{}) : u_tile(Four{});
         if (Cfg::kLow) {   // the slot's readers were eight units ago, and the ring holds fewer
-          huge = huge || __any_sync(0xffffffffu, largest >= kSplitHuge);
-          if (lane == 0) unit_flags[(unit % Cfg::kUnsafeSlots) * kSplitOperandWarps + ow] = huge ? 1 : 0;
+          flagged = flagged || __any_sync(0xffffffffu, bad);
+          if (lane == 0) unit_flags[(unit % Cfg::kUnsafeSlots) * kSplitOperandWarps + ow] = flagged ? 1 : 0;
         }
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
         __syncwarp();

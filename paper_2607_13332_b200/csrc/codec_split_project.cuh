@@ -69,7 +69,11 @@ struct SplitProjectConfig {
   static constexpr int kRawStepBytes = (1 + NSLOT) * kSplitRawBytes;
   static constexpr int kSumPitch = KN + 4;                  // floats per row of the exchanged sums
   static constexpr int kSumBytes = kUmmaTile * kSumPitch * 4;
-  static constexpr int kRoom = 227 * 1024 - 1024 - 256;
+  // barriers, TMEM address, largest magnitude per column of U, and of four tiles: rows the split does not hold
+  static constexpr int kBars = 8;
+  static constexpr int kTailBytes = kBars * 8 + 16 + 4 * KN + 4 * kUmmaTile;
+  static constexpr int kRoom = 227 * 1024 - 1024 - 1152;
+  static_assert(kTailBytes <= 1152, "the tail");
   // two operand stages unless that leaves no two steps of rows (bf16, three more operands)
   static constexpr int kStages = kRoom - 2 * kStageBytes >= 2 * kRawStepBytes ? 2 : 1;
   static constexpr int kFit = (kRoom - kStages * kStageBytes) / kRawStepBytes;
@@ -77,8 +81,7 @@ struct SplitProjectConfig {
   static_assert(kRaw >= 2, "no room for two steps of rows");
   static constexpr int kRingBytes = kStages * kStageBytes + kRaw * kRawStepBytes;
   static_assert(kRingBytes >= kSumBytes, "the exchanged sums take the place of the rings");
-  static constexpr int kBars = 8;
-  static constexpr int kSmemBytes = 1024 + kRingBytes + kBars * 8 + 16;   // barriers, TMEM address, unsafe-value flags
+  static constexpr int kSmemBytes = 1024 + kRingBytes + kTailBytes;
   static constexpr int kChain = 64 / kCols;                 // steps per accumulator
   static constexpr int kPairs = kCols * KN / 2 / kSplitRowThreads;   // pairs of U per thread and step
   static constexpr int kSums = KN / 4;                      // coordinates of one row per thread
@@ -109,42 +112,39 @@ __device__ __forceinline__ void store_coords4(const SplitProjectArgs &a, int64_t
   }
 }
 
-// Rows [row0, row0 + rows) of a tile again with plain FMAs, those whose residual the split does not hold
-// (all of them with `all`): one warp per row, lane = coordinate.
-template <typename T>
-__device__ __noinline__ void project_unsafe_rows(const SplitProjectArgs &a, int64_t tile, int row0, int rows, bool all) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (warp >= kSplitRowWarps) return;
-  const T *U = static_cast<const T *>(a.U);
-  for (int rr = row0 + warp; rr < row0 + rows; rr += kSplitRowWarps) {
-    const int64_t t = tile * kUmmaTile + rr;
-    if (t >= a.n) return;
-    const T *x = static_cast<const T *>(a.src) + t * a.lds;
-    const T *x2 = a.src2 != nullptr ? static_cast<const T *>(a.src2) + t * a.lds2 : nullptr;
-    const int64_t er = a.has_e ? embedding_row(a.shift, t) : -1, pr = a.has_p ? position_row(a.shift, t) : -1;
-    const T *e = er >= 0 ? static_cast<const T *>(a.shift.E) + er * a.shift.lde : nullptr;
-    const T *p = pr >= 0 ? static_cast<const T *>(a.shift.P) + pr * a.shift.ldp : nullptr;
-    auto residual = [&](int i) {
-      float r = to_f32(x[i]);
-      if (x2 != nullptr) r += to_f32(x2[i]);
-      if (e != nullptr) r -= to_f32(e[i]);
-      if (p != nullptr) r -= to_f32(p[i]);
-      return r;
-    };
-    float m = 0.f;
-    for (int i = lane; i < a.d; i += 32) m = fmaxf(m, fabsf(residual(i)));
+// Whether four finished sums stand: finite, and from columns of U that the split holds (largest magnitudes as bits;
+// zero columns are fine).
+__device__ __forceinline__ bool sums_stand(const float (&v)[4], const uint32_t *largest) {
+  bool ok = true;
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
-    if (!all && !split_unsafe(m)) continue;
-    for (int j = lane; j < a.k; j += 32) {
-      float acc = 0.f;
-      for (int i = 0; i < a.d; ++i) acc = fmaf(residual(i), to_f32(U[(int64_t)i * a.ldu + j]), acc);
-      if (a.wire || sizeof(T) == 4)
-        static_cast<float *>(a.zout)[t * a.ldzout + j] = acc;
-      else
-        static_cast<__nv_bfloat16 *>(a.zout)[t * a.ldzout + j] = __float2bfloat16_rn(acc);
-    }
+  for (int c = 0; c < 4; ++c) {
+    ok = ok && fabsf(v[c]) < __int_as_float(0x7f800000);
+    if (largest != nullptr) ok = ok && (largest[c] == 0 || largest[c] >= __float_as_uint(kSplitTinyU));
   }
+  return ok;
+}
+
+// Coordinates j .. j + 3 of token t again, as plain sums in 64 bits: for rows or columns of U that the split does not
+// hold, and for sums that left the range of fp32 on the way.
+template <typename T>
+__device__ __noinline__ void store_plain_coords4(const SplitProjectArgs &a, int64_t t, int j) {
+  const T *U = static_cast<const T *>(a.U), *x = static_cast<const T *>(a.src) + t * a.lds;
+  const T *x2 = a.src2 != nullptr ? static_cast<const T *>(a.src2) + t * a.lds2 : nullptr;
+  const int64_t er = a.has_e ? embedding_row(a.shift, t) : -1, pr = a.has_p ? position_row(a.shift, t) : -1;
+  const T *e = er >= 0 ? static_cast<const T *>(a.shift.E) + er * a.shift.lde : nullptr;
+  const T *p = pr >= 0 ? static_cast<const T *>(a.shift.P) + pr * a.shift.ldp : nullptr;
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 1
+  for (int i = 0; i < a.d; ++i) {
+    float r = to_f32(x[i]);
+    if (x2 != nullptr) r += to_f32(x2[i]);
+    if (e != nullptr) r -= to_f32(e[i]);
+    if (p != nullptr) r -= to_f32(p[i]);
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+      if (j + c < a.k) acc[c] = fma((double)r, (double)to_f32(U[(int64_t)i * a.ldu + j + c]), acc[c]);
+  }
+  store_coords4<T>(a, t, j, {(float)acc[0], (float)acc[1], (float)acc[2], (float)acc[3]});
 }
 
 template <typename T, int KN, int NSLOT>
@@ -174,8 +174,8 @@ __global__ void __launch_bounds__(kSplitProjectThreads, 1) codec_split_project_k
   auto acc_empty_bar = [&](int b) { return bars + (6 + b) * 8; };
   unsigned char *tail = smem_raw + (bars - smem_u) + Cfg::kBars * 8;
   volatile uint32_t *tmem_slot_ptr = reinterpret_cast<volatile uint32_t *>(tail);
-  // bit 0: some row may hold values its split does not; bit 1: U does
-  uint32_t *unsafe = reinterpret_cast<uint32_t *>(tail + 4);
+  uint32_t *u_largest = reinterpret_cast<uint32_t *>(tail + 16);       // [coordinate], as bits
+  volatile unsigned char *row_flags = tail + 16 + 4 * KN;              // [tile & 3][row]
 
   if (tid == 0) {
     for (int s = 0; s < 2; ++s) {
@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(kSplitProjectThreads, 1) codec_split_project_k
       mbar_init(acc_full_bar(s), 1);
       mbar_init(acc_empty_bar(s), kSplitRowWarps);
     }
-    *unsafe = 0;
+    for (int j = 0; j < KN; ++j) u_largest[j] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
   if (warp == kSplitRowWarps) {
@@ -376,17 +376,26 @@ __global__ void __launch_bounds__(kSplitProjectThreads, 1) codec_split_project_k
       if (lane == 0) mbar_arrive(acc_empty_bar(buf));
       if (last) {
         const int64_t t = (group + (int64_t)fin_tile * groups) * kUmmaTile + sum_row;
-        ++fin_tile;
         if (cluster_size == 1) {
           if (t < a.n) {
+            uint32_t bad = NX == 3 && row_flags[(fin_tile & 3) * kUmmaTile + sum_row] != 0 ? ~0u : 0u;
 #pragma unroll
-            for (int i = 0; i < Cfg::kSums; i += 4)
-              store_coords4<T>(a, t, sum_col + i, {sum[i], sum[i + 1], sum[i + 2], sum[i + 3]});
+            for (int i = 0; i < Cfg::kSums; i += 4) {
+              const float v[4] = {sum[i], sum[i + 1], sum[i + 2], sum[i + 3]};
+              store_coords4<T>(a, t, sum_col + i, v);
+              if (NX == 3 && !sums_stand(v, NU == 3 ? u_largest + sum_col + i : nullptr)) bad |= 1u << (i / 4);
+            }
+            if (bad != 0) {
+#pragma unroll 1
+              for (int i = 0; i < Cfg::kSums / 4 && sum_col + 4 * i < a.k; ++i)
+                if (bad >> i & 1) store_plain_coords4<T>(a, t, sum_col + 4 * i);
+            }
             if (a.wire_ids && part == 0) static_cast<int32_t *>(a.zout)[t * a.ldzout + a.k] = a.shift.ids[t];
           }
 #pragma unroll
           for (int i = 0; i < Cfg::kSums; ++i) sum[i] = 0.f;
         }
+        ++fin_tile;
       }
     };
 
@@ -410,8 +419,9 @@ __global__ void __launch_bounds__(kSplitProjectThreads, 1) codec_split_project_k
 
     int slot = 0, rslot = 0, st = 0, in_chain = 0;
     uint32_t parity = 1;
+    int tile = 0;                            // of this CTA, being filled
     bool prev_last = false;
-    float u_max = 0.f, row_max[2] = {0.f, 0.f};
+    float u_max[2] = {0.f, 0.f}, row_max[2] = {0.f, 0.f};
     const uint32_t a_off = Cfg::kF32 ? row * 64 + (((unit >> 1) ^ ((row >> 1) & 3)) << 4) + (unit & 1) * 8
                                      : row * 128 + ((unit ^ (row & 7)) << 4);   // + 64 rows: the second piece
     for (int step = 0; step < steps; ++step) {
@@ -462,7 +472,7 @@ __global__ void __launch_bounds__(kSplitProjectThreads, 1) codec_split_project_k
 #pragma unroll
       for (int i = 0; i < Cfg::kPairs; ++i) {
         const Pair<T> u = joined<T>(ureg[i]);
-        if (NX == 3) u_max = fmaxf(u_max, pair_magnitude<T>(u));
+        if (NU == 3) pair_maxima<T>(u, u_max);
         uint32_t up[NU];
         split_pair<T, NU>(u, up);
 #pragma unroll
@@ -470,6 +480,20 @@ __global__ void __launch_bounds__(kSplitProjectThreads, 1) codec_split_project_k
           const int n = s * KN + u_col;
           st_shared_b32(base + Cfg::kABytes + (n >> 6) * Cfg::kGroupBytes + (u_row + i * kURows) * 128 +
                             ((((n & 63) >> 3) ^ (u_row & 7)) << 4) + (n & 7) * 2, up[s]);
+        }
+      }
+      if (NX == 3 && next_st == 0) {
+        // the tile's rows, and U, are complete: the eight threads of a row agree on its largest magnitude
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+#pragma unroll
+          for (int off = 4; off > 0; off >>= 1) row_max[h] = fmaxf(row_max[h], __shfl_xor_sync(0xffffffffu, row_max[h], off));
+          if (unit == 0) row_flags[(tile & 3) * kUmmaTile + row + 64 * h] = row_max[h] != 0.f && row_max[h] < kSplitTinyRow ? 1 : 0;
+          row_max[h] = 0.f;
+        }
+        if (NU == 3 && tile == 0) {
+          atomicMax(u_largest + u_col, __float_as_uint(u_max[0]));
+          atomicMax(u_largest + u_col + 1, __float_as_uint(u_max[1]));
         }
       }
       asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
@@ -483,11 +507,7 @@ __global__ void __launch_bounds__(kSplitProjectThreads, 1) codec_split_project_k
       }
       if (++rslot == RD) rslot = 0;
       st = next_st;
-      if (st == 0 && NX == 3) {
-        // the tile's rows are complete: a row can be unsafe only if this thread's part of it is
-        if (split_unsafe(row_max[0]) || split_unsafe(row_max[1])) atomicOr(unsafe, 1u);
-        row_max[0] = row_max[1] = 0.f;
-      }
+      if (st == 0) ++tile;
       if (++in_chain == G || st == 0) {      // the accumulator before the one just filled
         if (chain > 0) take_chain(chain - 1, prev_last);
         prev_last = st == 0;
@@ -497,7 +517,6 @@ __global__ void __launch_bounds__(kSplitProjectThreads, 1) codec_split_project_k
     }
     take_chain(chain - 1, true);
     cp_async_wait<0>();
-    if (NX == 3 && u_max >= kSplitHuge) atomicOr(unsafe, 2u);
   }
 
   if (cluster_size > 1) {
@@ -517,32 +536,35 @@ __global__ void __launch_bounds__(kSplitProjectThreads, 1) codec_split_project_k
       asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(r) : "r"(addr), "r"(rank));
       return r;
     };
+    const uint32_t row_flags_addr = smem_u32(const_cast<unsigned char *>(row_flags));   // of tile 0, the only one
     for (int i = tid; i < rows * (KN / 4); i += kSplitProjectThreads) {
       const int rr = row0 + i / (KN / 4), j = 4 * (i % (KN / 4));
       const int64_t t = group * kUmmaTile + rr;
       if (t >= a.n || j >= a.k) continue;
       float v[4] = {0.f, 0.f, 0.f, 0.f};
+      uint32_t largest[4] = {0, 0, 0, 0}, bad_row = 0;
       for (uint32_t rk = 0; rk < cluster_size; ++rk) {
         float w0, w1, w2, w3;
         asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];\n"
                      : "=f"(w0), "=f"(w1), "=f"(w2), "=f"(w3)
                      : "r"(peer(smem0 + (uint32_t)(rr * Cfg::kSumPitch + j) * 4, rk)));
         v[0] += w0; v[1] += w1; v[2] += w2; v[3] += w3;
+        if (NX == 3) {
+          uint32_t m0, m1, m2, m3, f;
+          asm volatile("ld.shared::cluster.v4.u32 {%0,%1,%2,%3}, [%4];\n"
+                       : "=r"(m0), "=r"(m1), "=r"(m2), "=r"(m3) : "r"(peer(smem_u32(u_largest + j), rk)));
+          largest[0] = max(largest[0], m0); largest[1] = max(largest[1], m1);
+          largest[2] = max(largest[2], m2); largest[3] = max(largest[3], m3);
+          asm volatile("ld.shared::cluster.u8 %0, [%1];\n" : "=r"(f) : "r"(peer(row_flags_addr + rr, rk)));
+          bad_row |= f;
+        }
       }
       store_coords4<T>(a, t, j, v);
+      if (NX == 3 && (bad_row != 0 || !sums_stand(v, NU == 3 ? largest : nullptr))) store_plain_coords4<T>(a, t, j);
       if (a.wire_ids && j == 0) static_cast<int32_t *>(a.zout)[t * a.ldzout + a.k] = a.shift.ids[t];
     }
-    uint32_t bad = 0;
-    if (NX == 3) {
-      for (uint32_t rk = 0; rk < cluster_size; ++rk) {
-        uint32_t f;
-        asm volatile("ld.shared::cluster.u32 %0, [%1];\n" : "=r"(f) : "r"(peer(smem_u32(unsafe), rk)));
-        bad |= f;
-      }
-    }
-    // nobody leaves while its sums can still be read; and the rows above are stored
+    // nobody leaves while its sums can still be read
     asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
-    if (NX == 3 && bad != 0) project_unsafe_rows<T>(a, group, row0, rows, (bad & 2) != 0);
   }
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   __syncthreads();
@@ -550,11 +572,6 @@ __global__ void __launch_bounds__(kSplitProjectThreads, 1) codec_split_project_k
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem_base), "r"(Cfg::kTmemCols)
                  : "memory");
-  }
-  if (NX == 3 && cluster_size == 1) {      // the rows stored above are complete behind the barrier
-    const uint32_t bad = *unsafe;
-    if (bad != 0)
-      for (int i = 0; i < my_tiles; ++i) project_unsafe_rows<T>(a, group + i * groups, 0, kUmmaTile, (bad & 2) != 0);
   }
 }
 

@@ -141,3 +141,69 @@ def test_a_bad_basis_value_stays_in_its_column(k, bad):
     assert B.ssn_last_kernel()[0] == B.SSN_KERNEL_SPLIT_EXPAND
     assert_close(out[:, finite], expect[:, finite], dt, "decompress_wire")
     assert not np.isfinite(out[:, [5, 700, 1663]]).any()
+
+
+def _close_per_column(got, expect, what):
+    scale = np.abs(expect).max(axis=0)
+    assert (np.abs(got - expect).max(axis=0) <= 1e-5 * scale).all(), what
+
+
+@pytest.mark.parametrize("n,d,k", [(300, 256, 40), (19100, 130, 17), (700, 1100, 72)])
+@pytest.mark.parametrize("scale", [1e-33, 1e-37, 1e13])
+def test_columns_and_rows_of_a_basis_the_split_does_not_hold(n, d, k, scale):
+    """A column of U (projection) or a row of it (expansion) that is tiny or enormous as a whole keeps the precision of
+    fp32 against its own size; tiny values beside ordinary ones are no reason to compute anything again."""
+    dt = synth.F32
+    t = _inputs(n, d, k, dt, seed=5)
+    X, Z = f64(t["X"], dt), f64(t["Z0"], dt)
+    col, row = t["U"].copy(), t["U"].copy()
+    col[:, 3] *= np.float32(scale)
+    col[5, 2] = 1e-36
+    row[7] *= np.float32(scale)
+    row[9, 1] = 1e-36
+    dev = Codec(dt, to_device(col, dt))
+    _close_per_column(host64(dev.grad_project(to_device(t["X"], dt)), dt), X @ f64(col, dt), "projection")
+    dev = Codec(dt, to_device(row, dt))
+    _close_per_column(host64(dev.decompress(to_device(t["Z0"], dt)), dt), Z @ f64(row, dt).T, "expansion")
+
+
+@pytest.mark.parametrize("n,d", [(300, 256), (19100, 128)])     # one tile to a cluster of CTAs; a CTA with several tiles
+@pytest.mark.parametrize("dt", [synth.F32, synth.BF16])
+@pytest.mark.parametrize("addend", [False, True])
+def test_bad_rows_beside_tables_and_addends(n, d, dt, addend):
+    """Rows the split does not hold, beside E and P rows and a residual addend and as fp32 wire words; a row whose first
+    columns alone are tiny; every other row is what it is without them."""
+    k, ld = 40, 1
+    t = _inputs(n, d, k, dt, seed=11)
+    rng = np.random.default_rng(1)
+    pos = rng.integers(0, 50, n).astype(np.int32)
+    X, R = f64(t["X"], dt), f64(t["G"], dt)
+    X[0, 5], X[129, 9], X[130, 9] = np.inf, -np.inf, np.nan
+    X[20] *= 1e36
+    X[131, :32] = 1e-30
+    Xs, Rs = synth.to_storage(X, dt), synth.to_storage(R, dt)
+    X, R, E, P, U = f64(Xs, dt), f64(Rs, dt), f64(t["E"], dt), f64(t["P"][:50], dt), f64(t["U"], dt)
+    codec = Codec(dt, _strided(t["U"], dt, ld), _strided(t["E"], dt, ld), _strided(t["P"][:50], dt, ld))
+    ids, dpos = torch.from_numpy(t["ids"]).cuda(), torch.from_numpy(pos).cuda()
+    with np.errstate(invalid="ignore"):
+        if addend:
+            wire = codec.compress_sum(_strided(Xs, dt, ld), _strided(Rs, dt, ld), ids, pos=dpos, wire=True)
+            expect, _ = oracle.compress_sum(X, R, U, E, t["ids"], P, pos)
+        else:
+            wire = codec.compress_wire(_strided(Xs, dt, ld), ids, pos=dpos)
+            expect, _ = oracle.compress(X, U, E, t["ids"], P, pos)
+        assert B.ssn_last_kernel()[0] == B.SSN_KERNEL_SPLIT_PROJECT
+        got = wire.view(torch.float32).double().cpu().numpy()
+        _same_as_plain_sums(got, expect, "projection")
+        # fp32 coordinates into bf16 rows: tiny, enormous and infinite ones
+        Z = f64(t["Z0"], dt).astype(np.float32)
+        Z[3, 1], Z[4] = np.inf, Z[4] * np.float32(1e-30)
+        Z[5] *= np.float32(1e36)
+        out = host64(codec.decompress_wire(torch.from_numpy(Z).cuda().view(torch.int32), ids, pos=dpos, use_workspace=False), dt)
+        assert B.ssn_last_kernel()[0] == B.SSN_KERNEL_SPLIT_EXPAND
+        expect, _ = oracle.decompress(Z.astype(np.float64), U, E, t["ids"], P, pos)
+        rows = np.setdiff1d(np.arange(n), [3])
+        ok = np.abs(out[rows] - expect[rows]).max(axis=1) <= (1e-5 if dt == synth.F32 else 1e-2) * np.abs(expect[rows]).max(axis=1)
+        assert ok.all()
+        assert not np.isfinite(out[3]).any()
+    assert codec.take_status() == 0
