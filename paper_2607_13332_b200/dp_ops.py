@@ -60,6 +60,12 @@ def stage_clip(grads: Sequence[torch.Tensor], threshold: float, sumsq: torch.Ten
     for g in grads:
         if not (g.is_cuda and g.is_contiguous() and g.dtype in codes):
             raise ValueError("expected contiguous fp32 / bf16 CUDA gradients")
+    if len(grads) == 1:    # one tensor needs no list (100 elements: 27.4 -> 22.1 us, all of it host time)
+        g, stream = grads[0], _stream()
+        args = g.data_ptr(), g.numel(), codes[g.dtype], sumsq.data_ptr()
+        binding.stage_clip_sumsq(*args, stream)
+        binding.stage_clip_scale(*args, threshold, stream)
+        return sumsq
     spans = sorted((g.data_ptr(), g.data_ptr() + g.numel() * g.element_size()) for g in grads)
     if any(start < end for (_, end), (start, _) in zip(spans, spans[1:])):   # overlapping tensors: one after the other
         groups = [[g] for g in grads]

@@ -50,3 +50,16 @@ def test_overlapping_tensors_and_errors():
     binding.stage_clip_sumsq_list(binding.clip_list([], [], []), s.data_ptr())
     torch.cuda.synchronize()
     assert float(s.item()) == 0.0
+
+
+@pytest.mark.parametrize("dt", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("n", [0, 1, 4097])
+def test_one_tensor_alone(n, dt):
+    """A single tensor takes the launches without a list, to the same result."""
+    t = torch.randn(n, device="cuda", generator=torch.Generator(device="cuda").manual_seed(n)).to(dt)
+    before = t.double().cpu().numpy()
+    expect, norm, _ = dp.stage_clip([before], 0.01)
+    norm2 = float(dp_ops.stage_clip([t], 0.01).item())
+    assert abs(norm2 - norm * norm) <= 1e-6 * norm * norm
+    if n:
+        assert max_rel_err(t.double().cpu().numpy(), expect[0]) <= (2.0**-22 if dt == torch.float32 else 2.0**-8)
