@@ -6,8 +6,9 @@
 // 2^-16 (hh, hm, mh, mm, hl, lh) leave out less than the rounding of one fp32 operation.  bf16
 // products are exact in fp32, but the tensor cores TRUNCATE each addition to an accumulator (measured:
 // -6.6e-9 of the value per MMA, a bias of 8.5e-7 after 128 of them where a chain of FMAs errs by
-// 1e-7).  Both kernels therefore keep the chains short: the small products have an accumulator of
-// their own, and the projection moves the leading one to registers (fp32 additions) every 64 columns.
+// 1e-7).  Both kernels therefore keep the chains short: the small products have accumulators of
+// their own, and the projection moves the leading ones to registers every 64 or 128 columns and adds them up with
+// compensation, so that its results are no further from 64-bit sums than those of plain FMAs.
 //
 // The split needs room: the products of the low parts must not fall below the range of fp32 (2^-126), nor sums of the
 // leading ones rise above it.  A row whose largest magnitude is below kSplitTinyRow, or a row or column of an fp32
@@ -48,6 +49,10 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
                : "r"(taddr));
 }
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%8], {%0,%1,%2,%3,%4,%5,%6,%7};\n"
+               :: "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(taddr) : "memory");
+}
 __device__ __forceinline__ void st_shared_b32(uint32_t addr, uint32_t v) {
   asm volatile("st.shared.b32 [%0], %1;\n" ::"r"(addr), "r"(v) : "memory");
 }
@@ -64,22 +69,7 @@ __device__ __forceinline__ uint4 ld_shared_v4(uint32_t addr) {
   return v;
 }
 
-// Loads that are predicated where they have to be, never branched around, and not touched where they are
-// issued: the values are consumed a step later, and anything done to them here would wait for memory.
-__device__ __forceinline__ uint4 load_global_v4_if(const void *p, bool ok) {
-  uint4 v;
-  asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %5, 0;\n"
-               "mov.b32 %0, 0;\nmov.b32 %1, 0;\nmov.b32 %2, 0;\nmov.b32 %3, 0;\n"
-               "@p ld.global.nc.v4.b32 {%0,%1,%2,%3}, [%4];\n}\n"
-               : "=&r"(v.x), "=&r"(v.y), "=&r"(v.z), "=&r"(v.w) : "l"(p), "r"((int)ok));
-  return v;
-}
-__device__ __forceinline__ uint2 load_global_v2_if(const void *p, bool ok) {
-  uint2 v;
-  asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %3, 0;\nmov.b32 %0, 0;\nmov.b32 %1, 0;\n"
-               "@p ld.global.nc.v2.b32 {%0,%1}, [%2];\n}\n" : "=&r"(v.x), "=&r"(v.y) : "l"(p), "r"((int)ok));
-  return v;
-}
+// Loads that are predicated, not branched around.
 __device__ __forceinline__ uint32_t load_global_b32_if(const void *p, bool ok) {
   uint32_t v;
   asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %2, 0;\nmov.b32 %0, 0;\n@p ld.global.nc.b32 %0, [%1];\n}\n"

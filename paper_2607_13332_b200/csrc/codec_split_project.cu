@@ -29,39 +29,43 @@ int cluster_of(int64_t ntiles, int nst, int sms) {
   return best;
 }
 
-template <typename T, int KN, int NSLOT>
-cudaError_t launch_one(const SplitProjectArgs &a, int sms, cudaStream_t stream) {
-  auto kernel = codec_split_project_kernel<T, KN, NSLOT>;
-  constexpr int smem = SplitProjectConfig<T, KN, NSLOT>::kSmemBytes;
+int64_t units_of(const SplitProjectArgs &a) { return (a.n + kUmmaTile - 1) / kUmmaTile * a.halves; }   // tiles, or halves of them
+
+template <typename T, int KN, int NSLOT, bool CAREFUL>
+cudaError_t launch_one(const SplitProjectArgs &a, int c, int sms, cudaStream_t stream) {
+  using Cfg = SplitProjectConfig<T, KN, NSLOT, CAREFUL>;
+  auto kernel = codec_split_project_kernel<T, KN, NSLOT, CAREFUL>;
   static std::atomic<uint64_t> configured{0};
-  cudaError_t e = allow_dynamic_smem(kernel, smem, configured);
+  cudaError_t e = allow_dynamic_smem(kernel, Cfg::kSmemBytes, configured);
   if (e != cudaSuccess) return e;
-  const int64_t ntiles = (a.n + kUmmaTile - 1) / kUmmaTile;
-  const int c = cluster_of(ntiles, (a.d + 63) / 64, sms);
-  const int64_t single = ntiles < sms ? ntiles : sms, grid = c > 1 ? ntiles * c : single;
-  e = launch_dependent(kernel, (unsigned)grid, kSplitProjectThreads, smem, stream, c, a);
+  const int64_t units = units_of(a);
+  // whole tiles: as many CTAs for either half
+  const int64_t single = units < sms ? units : (sms > 1 ? sms - sms % a.halves : a.halves), grid = c > 1 ? units * c : single;
+  e = launch_dependent(kernel, (unsigned)grid, Cfg::kThreads, Cfg::kSmemBytes, stream, c, a);
   if (e != cudaSuccess && c > 1) {   // a device that cannot co-schedule the cluster
     cudaGetLastError();
-    e = launch_dependent(kernel, (unsigned)single, kSplitProjectThreads, smem, stream, 1, a);
+    e = launch_dependent(kernel, (unsigned)single, Cfg::kThreads, Cfg::kSmemBytes, stream, 1, a);
   }
-  note_kernel(SSN_KERNEL_SPLIT_PROJECT,
-              (a.has_e ? SSN_KVAR_E : 0) | (a.has_p ? SSN_KVAR_P : 0) | (KN > 64 ? SSN_KVAR_WIDE : 0) | (c > 1 ? SSN_KVAR_ALT : 0));
+  note_kernel(SSN_KERNEL_SPLIT_PROJECT, (a.has_e ? SSN_KVAR_E : 0) | (a.has_p ? SSN_KVAR_P : 0) |
+                                            (a.halves > 1 ? SSN_KVAR_WIDE : 0) | (c > 1 ? SSN_KVAR_ALT : 0));
   return e;
 }
 
-template <typename T, int KN>
-cudaError_t launch_slots(const SplitProjectArgs &a, int slots, int sms, cudaStream_t s) {
-  if (slots == 0) return launch_one<T, KN, 0>(a, sms, s);
-  if (slots == 1) return launch_one<T, KN, 1>(a, sms, s);
-  if (slots == 2) return launch_one<T, KN, 2>(a, sms, s);
-  return launch_one<T, KN, 3>(a, sms, s);
+template <typename T, int NSLOT>
+cudaError_t launch_rank(const SplitProjectArgs &a, int sms, cudaStream_t s) {
+  const int nst = (a.d + 63) / 64, c = cluster_of(units_of(a), nst, sms);
+  constexpr int careful = sizeof(T) == 2 && NSLOT == 0 ? kSplitCarefulColsPlain : kSplitCarefulCols;
+  if ((nst + c - 1) / c * 64 < careful) return launch_one<T, 64, NSLOT, true>(a, c, sms, s);
+  if (a.k <= 32) return launch_one<T, 32, NSLOT, false>(a, c, sms, s);
+  return launch_one<T, 64, NSLOT, false>(a, c, sms, s);
 }
 
 template <typename T>
-cudaError_t launch_rank(const SplitProjectArgs &a, int slots, int sms, cudaStream_t s) {
-  if (a.k <= 32) return launch_slots<T, 32>(a, slots, sms, s);
-  if (a.k <= 64) return launch_slots<T, 64>(a, slots, sms, s);
-  return launch_slots<T, 128>(a, slots, sms, s);
+cudaError_t launch_slots(const SplitProjectArgs &a, int slots, int sms, cudaStream_t s) {
+  if (slots == 0) return launch_rank<T, 0>(a, sms, s);
+  if (slots == 1) return launch_rank<T, 1>(a, sms, s);
+  if (slots == 2) return launch_rank<T, 2>(a, sms, s);
+  return launch_rank<T, 3>(a, sms, s);
 }
 
 bool rows16(const void *p, int64_t ld, int esz) {
@@ -87,6 +91,8 @@ cudaError_t launch_codec_split_project(const TokenArgs &a, int32_t dtype, int sm
   p.n = a.n;
   p.d = a.d;
   p.k = a.k;
+  p.halves = a.k > 64 ? 2 : 1;
+  p.k_half = a.k > 64 ? (a.k + 31) / 32 * 16 : a.k;
   p.wire = a.wire;
   p.wire_ids = a.wire_ids;
   p.shift = a.shift;
@@ -99,8 +105,8 @@ cudaError_t launch_codec_split_project(const TokenArgs &a, int32_t dtype, int sm
   // four coordinates are 16 bytes of words or 8 bytes of bf16
   p.vec_out = (a.ldzout & 3) == 0 && (reinterpret_cast<uintptr_t>(a.zout) & (a.wire || dtype == SSN_F32 ? 15 : 7)) == 0;
   const int slots = (a.src2 != nullptr) + p.has_e + p.has_p;
-  return dtype == SSN_F32 ? launch_rank<float>(p, slots, sm_count, stream)
-                          : launch_rank<__nv_bfloat16>(p, slots, sm_count, stream);
+  return dtype == SSN_F32 ? launch_slots<float>(p, slots, sm_count, stream)
+                          : launch_slots<__nv_bfloat16>(p, slots, sm_count, stream);
 }
 
 }  // namespace ssn

@@ -11,17 +11,18 @@
 //
 //   warps 0-15  every thread reads back the pieces it copied itself (no barrier), writes their parts and its
 //               share of U to the step's operand stage, and requests the rows of the step RD - 1 ahead.
-//               Every 64 columns a finished accumulator is added to fp32 sums in registers (see
-//               codec_split.cuh on why the chains are this short): warp w reads TMEM lanes 32 (w % 4) .. +31
-//               and a quarter of the columns.
-//   warp 16     one thread issues the MMAs: Ah x (Uh|Um|Ul), Am x (Uh|Um), Al x Uh, the parts of U side by
-//               side on N so that three instructions per K step cover the six products (rank above 64:
-//               five instructions, (Uh|Um) being 256 columns wide).  It is a warp of its own because each
-//               of these instructions blocks its thread for about 100 clocks.
+//               At the end of a chain of 64 or 128 columns its accumulators are added to compensated fp32 sums in
+//               registers (see SplitProjectConfig on the lengths): warp w reads TMEM lanes 32 (w % 4) .. +31 and a
+//               quarter of the columns.
+//   warp 16     one thread issues the MMAs: Ah x Uh into the leading accumulators; Ah x (Um|Ul), Am x (Uh|Um) and
+//               Al x Uh into the small ones, the parts of U side by side on N.  A warp of its own, because each of
+//               these instructions blocks its thread for about 100 clocks; above rank 32 warp 17 takes half of them.
 //
 // A CTA takes whole tiles of 128 tokens, or a cluster of 2 to 8 CTAs shares one tile where that fills the
 // SMs better: each contracts a slice of d, and the partial sums meet through distributed shared memory, every
-// CTA finishing its share of the rows.
+// CTA finishing its share of the rows.  Ranks above 64 are two halves on CTAs side by side: accumulators, sums and
+// their compensation for 128 coordinates do not fit a thread's registers (8192 x 2048 fp32, rank 100, E rows: one
+// CTA for all 136 us, halves 84).
 #pragma once
 
 #include "codec_split.cuh"
@@ -33,6 +34,7 @@ struct SplitProjectArgs {
   void *zout;
   int64_t lds, lds2, ldu, ldzout, n;
   int32_t d, k;
+  int32_t halves, k_half;      // ranks above 64: two halves, each CTA computes k_half coordinates or the rest; else one of k
   int32_t wire, wire_ids;      // fp32 words out, word k of a row = the token id
   int32_t has_e, has_p;
   int32_t vec_rows;            // every row operand may be read 16 bytes at a time and g_zero_row holds a row
@@ -41,24 +43,36 @@ struct SplitProjectArgs {
 };
 
 constexpr int kSplitRowWarps = 16, kSplitRowThreads = 32 * kSplitRowWarps;
-constexpr int kSplitProjectThreads = kSplitRowThreads + 32;
 constexpr int kSplitRawBytes = kUmmaTile * 128;       // one operand's rows of one step
 
-template <typename T, int KN, int NSLOT>
+// Slices of d of fewer columns take the CAREFUL kernel: over so few terms plain FMAs are at their best (products of
+// bf16 values add up exactly at first), and the additions among a chain's accumulators show.  Gradients of 128
+// columns in bf16, error against 64-bit sums: 5.1e-8, careful 4.7e-8, FMAs 4.8e-8.
+constexpr int kSplitCarefulCols = 256, kSplitCarefulColsPlain = 384;   // bf16 rows as they are
+
+template <typename T, int KN, int NSLOT, bool CAREFUL>
 struct SplitProjectConfig {
-  static_assert(KN == 32 || KN == 64 || KN == 128, "coordinates, rounded up");
+  static_assert(KN == 32 || KN == 64, "coordinates, rounded up");
   static constexpr bool kF32 = sizeof(T) == 4;
   static constexpr int kNX = kF32 || NSLOT > 0 ? 3 : 1;    // parts of the residual
   static constexpr int kNU = kF32 ? 3 : 1;                 // parts of U
-  static constexpr int kStack = kNU == 3 ? (KN <= 64 ? 3 : 2) : 1;   // parts of U under one Ah product
-  // KN-wide accumulators of a chain, all of them summed in fp32 where it ends.  fp32: hi and low products, side by
-  // side.  bf16 bases leave room to deal the K steps of the leading product to several: gradients
-  // of 4096 columns, rank 51, one accumulator 1.6e-7 from 64-bit sums, four 9.2e-8, plain FMAs 9.5e-8.
-  static constexpr int kHiAccs = kNU == 3 ? 1 : (kNX == 1 ? (KN <= 64 ? 4 : 2) : (KN <= 64 ? 2 : 1));
-  static constexpr int kAccs = kNU == 3 ? kStack : kHiAccs + (kNX == 3 ? 1 : 0);
-  static constexpr int kDCols = kAccs * KN;
-  static constexpr int kDStride = kDCols <= 32 ? 32 : (kDCols <= 64 ? 64 : (kDCols <= 128 ? 128 : 256));
-  static constexpr int kTmemCols = 2 * kDStride;
+  // Columns of d per chain and its accumulators, each KN columns of tensor memory, added up in fp32 where the chain
+  // ends: kHi for the leading products, which take turns with the K steps, and kLow for the small ones.  An
+  // accumulator is truncated with every MMA that is added to it.  Coordinates of 256 to 1024 columns, error against
+  // 64-bit sums, rank 8: four K steps in one accumulator 8.2e-8, in four 3.8e-8, plain FMAs 4.2e-8 (4.8e-8 at rank
+  // 33, 5.5e-8 at 100: there two K steps per accumulator are near enough, 4.5e-8 and 4.8e-8).  KN columns more hold
+  // the compensation of the sums over chains.  What is left decides whether there are two sets, so that a chain is
+  // summed while the next is written.
+  // CAREFUL (see kSplitCarefulCols) adds the accumulators one by one, with compensation.
+  static constexpr bool kOneStage = !kF32 && NSLOT == 3;   // see kStages: there a second set pays more than long chains
+  static constexpr int kChainCols = KN == 32 || kOneStage || kNX == 1 || CAREFUL ? 64 : 128;
+  static constexpr int kHi = KN == 32 || CAREFUL ? 4 : (kOneStage ? 2 : (kNX == 1 ? 3 : 4));
+  static constexpr int kLow = kNX == 1 ? 0 : (kF32 ? 2 : 1);
+  static constexpr int kDCols = (kHi + kLow) * KN;
+  static constexpr int kBufs = 2 * kDCols + KN <= 512 ? 2 : 1;
+  static constexpr int kCompCol = kBufs * kDCols;
+  static constexpr int kTmemCols = kCompCol + KN <= 256 ? 256 : 512;
+  static_assert(kCompCol + KN <= 512, "tensor memory");
   static constexpr int kCols = kF32 ? 32 : 64;              // columns of d per step
   static constexpr int kPartBytes = kUmmaTile * kCols * 2;  // one bf16 part of a [128 x kCols] operand
   static constexpr int kRowBytes = kCols * 2;               // its rows, swizzled within 64 or 128 bytes
@@ -72,42 +86,49 @@ struct SplitProjectConfig {
   // barriers, TMEM address, largest magnitude per column of U, and of four tiles: rows the split does not hold
   static constexpr int kBars = 8;
   static constexpr int kTailBytes = kBars * 8 + 16 + 4 * KN + 4 * kUmmaTile;
-  static constexpr int kRoom = 227 * 1024 - 1024 - 1152;
-  static_assert(kTailBytes <= 1152, "the tail");
+  // MMA-issuing warps.  Two where the instructions of one thread, about 100 clocks each, would take longer than the
+  // rows: one issues the leading products, the other the small ones (or they share the accumulators out).
+  static constexpr int kIssuers = KN == 64 ? 2 : 1;
+  static constexpr int kThreads = kSplitRowThreads + 32 * kIssuers;
+  static constexpr int kRoom = 227 * 1024 - 1024 - 896;
+  static_assert(kTailBytes <= 896, "the tail");
   // two operand stages unless that leaves no two steps of rows (bf16, three more operands)
   static constexpr int kStages = kRoom - 2 * kStageBytes >= 2 * kRawStepBytes ? 2 : 1;
+  static_assert(kStages == 2 || kOneStage, "chosen above without these sizes");
   static constexpr int kFit = (kRoom - kStages * kStageBytes) / kRawStepBytes;
   static constexpr int kRaw = kFit < 6 ? kFit : 6;          // steps of rows in flight or being read
   static_assert(kRaw >= 2, "no room for two steps of rows");
   static constexpr int kRingBytes = kStages * kStageBytes + kRaw * kRawStepBytes;
   static_assert(kRingBytes >= kSumBytes, "the exchanged sums take the place of the rings");
   static constexpr int kSmemBytes = 1024 + kRingBytes + kTailBytes;
-  static constexpr int kChain = 64 / kCols;                 // steps per accumulator
+  static constexpr int kChain = kChainCols / kCols;         // steps per chain
   static constexpr int kPairs = kCols * KN / 2 / kSplitRowThreads;   // pairs of U per thread and step
   static constexpr int kSums = KN / 4;                      // coordinates of one row per thread
+  // Place of part s of U on N.  Rank up to 32: m, l, h, so that the pair m | l and h alone both start a group.
+  __host__ __device__ static constexpr int b_part(int s) { return kF32 && KN == 32 ? (s + 2) % 3 : s; }
   static constexpr int kVecElems = kF32 ? 4 : 8;            // of a 16-byte piece; a thread has two per operand and step
 };
 
 template <typename T>
-__device__ __forceinline__ void store_coords4(const SplitProjectArgs &a, int64_t t, int j, const float (&v)[4]) {
-  if (j >= a.k) return;
+__device__ __forceinline__ void store_coords4(const SplitProjectArgs &a, int64_t t, int j, int j_end, const float (&v)[4]) {
+  if (j >= j_end) return;
   if (a.wire || sizeof(T) == 4) {
     float *z = static_cast<float *>(a.zout) + t * a.ldzout + j;
-    if (a.vec_out && j + 4 <= a.k) {
+    if (a.vec_out && j + 4 <= j_end) {
       *reinterpret_cast<float4 *>(z) = make_float4(v[0], v[1], v[2], v[3]);
     } else {
 #pragma unroll
       for (int e = 0; e < 4; ++e)
-        if (j + e < a.k) z[e] = v[e];
+        if (j + e < j_end) z[e] = v[e];
     }
   } else {
     __nv_bfloat16 *z = static_cast<__nv_bfloat16 *>(a.zout) + t * a.ldzout + j;
-    if (a.vec_out && j + 4 <= a.k) {
+    if (a.vec_out && j + 4 <= j_end) {
       *reinterpret_cast<uint2 *>(z) = make_uint2(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]));
     } else {
 #pragma unroll
       for (int e = 0; e < 4; ++e)
-        if (j + e < a.k) z[e] = __float2bfloat16_rn(v[e]);
+        if (j + e < j_end) z[e] = __float2bfloat16_rn(v[e]);
     }
   }
 }
@@ -124,10 +145,10 @@ __device__ __forceinline__ bool sums_stand(const float (&v)[4], const uint32_t *
   return ok;
 }
 
-// Coordinates j .. j + 3 of token t again, as plain sums in 64 bits: for rows or columns of U that the split does not
+// Coordinates j .. j + 3 (below j_end) of token t again, as plain sums in 64 bits: for rows or columns of U that the split does not
 // hold, and for sums that left the range of fp32 on the way.
 template <typename T>
-__device__ __noinline__ void store_plain_coords4(const SplitProjectArgs &a, int64_t t, int j) {
+__device__ __noinline__ void store_plain_coords4(const SplitProjectArgs &a, int64_t t, int j, int j_end) {
   const T *U = static_cast<const T *>(a.U), *x = static_cast<const T *>(a.src) + t * a.lds;
   const T *x2 = a.src2 != nullptr ? static_cast<const T *>(a.src2) + t * a.lds2 : nullptr;
   const int64_t er = a.has_e ? embedding_row(a.shift, t) : -1, pr = a.has_p ? position_row(a.shift, t) : -1;
@@ -142,15 +163,15 @@ __device__ __noinline__ void store_plain_coords4(const SplitProjectArgs &a, int6
     if (p != nullptr) r -= to_f32(p[i]);
 #pragma unroll
     for (int c = 0; c < 4; ++c)
-      if (j + c < a.k) acc[c] = fma((double)r, (double)to_f32(U[(int64_t)i * a.ldu + j + c]), acc[c]);
+      if (j + c < j_end) acc[c] = fma((double)r, (double)to_f32(U[(int64_t)i * a.ldu + j + c]), acc[c]);
   }
-  store_coords4<T>(a, t, j, {(float)acc[0], (float)acc[1], (float)acc[2], (float)acc[3]});
+  store_coords4<T>(a, t, j, j_end, {(float)acc[0], (float)acc[1], (float)acc[2], (float)acc[3]});
 }
 
-template <typename T, int KN, int NSLOT>
-__global__ void __launch_bounds__(kSplitProjectThreads, 1) codec_split_project_kernel(const SplitProjectArgs a) {
-  using Cfg = SplitProjectConfig<T, KN, NSLOT>;
-  constexpr int NX = Cfg::kNX, NU = Cfg::kNU, S = Cfg::kStages, RD = Cfg::kRaw, G = Cfg::kChain;
+template <typename T, int KN, int NSLOT, bool CAREFUL>
+__global__ void __launch_bounds__((SplitProjectConfig<T, KN, NSLOT, CAREFUL>::kThreads), 1) codec_split_project_kernel(const SplitProjectArgs a) {
+  using Cfg = SplitProjectConfig<T, KN, NSLOT, CAREFUL>;
+  constexpr int NX = Cfg::kNX, NU = Cfg::kNU, S = Cfg::kStages, RD = Cfg::kRaw, G = Cfg::kChain, NB = Cfg::kBufs;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -159,7 +180,13 @@ __global__ void __launch_bounds__(kSplitProjectThreads, 1) codec_split_project_k
   asm volatile("mov.u32 %0, %%cluster_nctaid.x;\n" : "=r"(cluster_size));
   asm volatile("mov.u32 %0, %%cluster_ctarank;\n" : "=r"(cta_rank));
   const int64_t ntiles = (a.n + kUmmaTile - 1) / kUmmaTile;
-  const int64_t groups = gridDim.x / cluster_size, group = blockIdx.x / cluster_size;
+  // the two halves of a tile's coordinates run side by side, so that its rows come from HBM once
+  const int64_t groups = gridDim.x / cluster_size / a.halves, group = blockIdx.x / cluster_size / a.halves;
+  const bool upper = a.halves > 1 && (blockIdx.x / cluster_size & 1) != 0;
+  auto lower = [&]() { return a.halves > 1 && !upper; };     // coordinates j_lo() to j_end()
+  auto j_lo = [&]() { return upper ? a.k_half : 0; };
+  auto j_end = [&]() { return lower() ? a.k_half : a.k; };
+  auto rank = [&]() { return j_end() - j_lo(); };
   const int nst = (a.d + Cfg::kCols - 1) / Cfg::kCols;
   const int st_lo = (int)((int64_t)nst * cta_rank / cluster_size);
   const int nloc = (int)((int64_t)nst * (cta_rank + 1) / cluster_size) - st_lo;   // >= 1: cluster_size <= nst
@@ -180,8 +207,8 @@ __global__ void __launch_bounds__(kSplitProjectThreads, 1) codec_split_project_k
   if (tid == 0) {
     for (int s = 0; s < 2; ++s) {
       mbar_init(full_bar(s), kSplitRowWarps);
-      mbar_init(empty_bar(s), 1);
-      mbar_init(acc_full_bar(s), 1);
+      mbar_init(empty_bar(s), Cfg::kIssuers);
+      mbar_init(acc_full_bar(s), Cfg::kIssuers);
       mbar_init(acc_empty_bar(s), kSplitRowWarps);
     }
     for (int j = 0; j < KN; ++j) u_largest[j] = 0;
@@ -210,47 +237,50 @@ __global__ void __launch_bounds__(kSplitProjectThreads, 1) codec_split_project_k
   const int quarter = warp & 3, part = warp >> 2;     // TMEM lanes and columns of this warp's sums
   const int sum_row = quarter * 32 + lane, sum_col = part * Cfg::kSums;
 
-  if (warp == kSplitRowWarps) {
-    // ------------------------------------------------------------------------- MMA issuer
+  if (warp >= kSplitRowWarps) {
+    // ------------------------------------------------------------------------- MMA issuers
     if (lane == 0) {
       // A: K-major rows of kRowBytes, 8-row groups 8 kRowBytes apart, one part after the other.  B: MN-major,
       // 64-coordinate groups kGroupBytes apart, 8-row groups 1024 bytes apart.
       constexpr uint32_t kLayoutA = Cfg::kF32 ? 4 : 2;       // 64- or 128-byte swizzle
-      constexpr uint32_t id1 = umma_idesc(KN, false), id2 = umma_idesc(Cfg::kStack >= 2 ? 2 * KN : KN, false),
-                         id3 = umma_idesc(Cfg::kStack == 3 ? 3 * KN : KN, false);
+      constexpr uint32_t id1 = umma_idesc(KN, false), id2 = umma_idesc(2 * KN, false);
       constexpr uint32_t kPart = Cfg::kPartBytes >> 4;                             // next part of A
-      constexpr uint32_t kBPart = (uint32_t)(KN / 64) * (Cfg::kGroupBytes >> 4);   // next part of B (KN = 128 only)
+      // where the parts of B start (see b_part)
+      constexpr uint32_t kGroup = Cfg::kGroupBytes >> 4;
+      constexpr uint32_t kBh = KN == 32 && NU == 3 ? kGroup : 0, kBm = KN == 32 ? 0 : kGroup;
+      const bool first = warp == kSplitRowWarps, lead = first || Cfg::kIssuers == 1, small = !first || Cfg::kIssuers == 1;
       int slot = 0, st = 0, in_chain = 0, chain = 0;
       uint32_t parity = 0;
       for (int step = 0; step < steps; ++step) {
-        const int buf = chain & 1;
-        if (in_chain == 0 && !dead && !mbar_wait(acc_empty_bar(buf), (uint32_t)(((chain >> 1) & 1) ^ 1))) timed_out();
+        const int buf = chain % NB;
+        if (in_chain == 0 && !dead && !mbar_wait(acc_empty_bar(buf), (uint32_t)(((chain / NB) & 1) ^ 1))) timed_out();
         if (!dead && !mbar_wait(full_bar(slot), parity)) timed_out();
         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
         const uint32_t base = smem0 + (uint32_t)slot * Cfg::kStageBytes;
-        const uint32_t D = tmem_base + (uint32_t)buf * Cfg::kDStride;
+        const uint32_t D = tmem_base + (uint32_t)buf * Cfg::kDCols, L0 = D + Cfg::kHi * KN, L1 = L0 + KN;
         const uint64_t ad = umma_desc(base, 16, 8 * Cfg::kRowBytes, kLayoutA);
         const uint64_t bd = umma_desc(base + Cfg::kABytes, Cfg::kGroupBytes, 1024, 2);
 #pragma unroll
         for (int j = 0; j < Cfg::kCols / 16; ++j) {
           const uint64_t A = ad + j * 2, B = bd + j * 128;   // 32 bytes of an A row; 16 rows of B
-          const uint32_t more = in_chain > 0 || j > 0 ? 1u : 0u;
-          if (NU == 1) {                       // a bf16 chain is one step
-            umma_bf16(D + (j % Cfg::kHiAccs) * KN, A, B, id1, j >= Cfg::kHiAccs ? 1u : 0u);
-            if (NX == 3) {
-              umma_bf16(D + Cfg::kHiAccs * KN, A + kPart, B, id1, more);
-              umma_bf16(D + Cfg::kHiAccs * KN, A + 2 * kPart, B, id1, 1u);
-            }
-          } else if (Cfg::kStack == 3) {
-            umma_bf16(D, A, B, id3, more);
-            umma_bf16(D + KN, A + kPart, B, id2, 1u);
-            umma_bf16(D + 2 * KN, A + 2 * kPart, B, id1, 1u);
+          const int ks = in_chain * (Cfg::kCols / 16) + j;   // K step of the chain
+          const uint32_t more = ks > 0 ? 1u : 0u;
+          // an accumulator belongs to one thread: its MMAs keep their order
+          if (NX == 1 && (Cfg::kHi % 2 != 0 ? ks % Cfg::kHi != 0 : j % 2 != 0) ? small : lead)
+            umma_bf16(D + (uint32_t)(ks % Cfg::kHi) * KN, A, B + kBh, id1, ks >= Cfg::kHi ? 1u : 0u);
+          if (NX == 1 || !small) continue;
+          if (NU == 1) {
+            umma_bf16(L0, A + kPart, B, id1, more);
+            umma_bf16(L0, A + 2 * kPart, B, id1, 1u);
           } else {
-            umma_bf16(D, A, B, id2, more);
-            umma_bf16(D + KN, A + kPart, B, id1, 1u);
-            umma_bf16(D + KN, A + kPart, B + kBPart, id1, 1u);
-            umma_bf16(D + KN, A + 2 * kPart, B, id1, 1u);
-            umma_bf16(D + KN, A, B + 2 * kBPart, id1, 1u);
+            umma_bf16(L0, A, B + kBm, id2, more);            // m and l side by side
+            if (KN == 64) {
+              umma_bf16(L0, A + kPart, B, id2, 1u);          // h and m
+            } else {
+              umma_bf16(L0, A + kPart, B + kBh, id1, 1u);
+              umma_bf16(L1, A + kPart, B + kBm, id1, 1u);
+            }
+            umma_bf16(L1, A + 2 * kPart, B + kBh, id1, 1u);
           }
         }
         umma_commit(empty_bar(slot));
@@ -274,10 +304,10 @@ __global__ void __launch_bounds__(kSplitProjectThreads, 1) codec_split_project_k
     const bool vec = a.vec_rows != 0;
     // the pairs of U this thread moves: rows u_row, u_row + kURows, ... of the step (8 divides kURows)
     constexpr int kURows = 2 * kSplitRowThreads / KN;
-    const int u_row = tid / (KN / 2), u_col = 2 * (tid % (KN / 2)), u_valid = max(a.k - u_col, 0);
+    const int u_row = tid / (KN / 2), u_col = 2 * (tid % (KN / 2)), u_valid = max(rank() - u_col, 0);
     const int64_t u_step = kURows * a.ldu;
     const bool vec_u = a.vec_u != 0;
-    const T *U = static_cast<const T *>(a.U);
+    const T *U = static_cast<const T *>(a.U) + j_lo();
     const T *ptr[1 + NSLOT][2];              // this thread's rows: X, then R, E, P as far as present
     Pair<T> ureg[Cfg::kPairs];
     const bool has_r = NSLOT > 0 && a.src2 != nullptr;
@@ -347,30 +377,96 @@ __global__ void __launch_bounds__(kSplitProjectThreads, 1) codec_split_project_k
         }
       }
     };
-    int chain = 0, fin_tile = 0;             // accumulators written so far, tiles finished
-    // adds accumulator c to the sums; `last`: it completes a tile
-    auto take_chain = [&](int c, bool last) {
-      const int buf = c & 1;
-      if (!dead && !mbar_wait(acc_full_bar(buf), (uint32_t)((c >> 1) & 1))) timed_out();
+    int chain = 0, fin_tile = 0;             // chains complete so far, tiles finished
+    bool fresh = true;                       // the next chain is a tile's first
+    // Adds chain c, of `chain_steps` steps, to the sums, with compensation: over 4096 columns of coherent rows 64 plain
+    // additions err by 1.2e-7, these by 3e-8.  `last`: it completes a tile.
+    auto take_chain = [&](int c, int chain_steps, bool last) {
+      const int buf = c % NB;
+      const int written = chain_steps * (Cfg::kCols / 16);   // leading accumulators that the chain has written
+      if (!dead && !mbar_wait(acc_full_bar(buf), (uint32_t)((c / NB) & 1))) timed_out();
       asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-      if (sum_col < a.k) {
-        const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)buf * Cfg::kDStride + sum_col;
+      if (sum_col < a.k_half) {
+        const uint32_t lane_addr = tmem_base + ((uint32_t)(quarter * 32) << 16) + sum_col;
+        const uint32_t taddr = lane_addr + (uint32_t)buf * Cfg::kDCols, caddr = lane_addr + Cfg::kCompCol;
+        asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");   // the compensation of the chain before
+        // s += x with compensation c
+        auto compensated = [](float &s0, float &s1, float &c0, float &c1, float x0, float x1) {
+          sub2(x0, x1, c0, c1);
+          float t0 = s0, t1 = s1;
+          add2(t0, t1, x0, x1);
+          c0 = t0, c1 = t1;
+          sub2(c0, c1, s0, s1);
+          sub2(c0, c1, x0, x1);
+          s0 = t0, s1 = t1;
+        };
+        constexpr int H0 = Cfg::kHi / 2, H1 = Cfg::kHi - H0;
 #pragma unroll
         for (int i = 0; i < Cfg::kSums; i += 8) {
-          uint32_t v[Cfg::kAccs][8];
+          if constexpr (CAREFUL) {
+            uint32_t comp[8], v[8];
+            tmem_ld8(caddr + i, comp);
 #pragma unroll
-          for (int c2 = 0; c2 < Cfg::kAccs; ++c2) tmem_ld8(taddr + c2 * KN + i, v[c2]);
-          asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+            for (int q = 0; q < Cfg::kHi + Cfg::kLow; ++q) {
+              if (q >= written && q < Cfg::kHi) continue;
+              tmem_ld8(taddr + q * KN + i, v);
+              asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
 #pragma unroll
-          for (int e = 0; e < 8; e += 2) {
-            // from the last on: the low products come last
-            float w0 = __uint_as_float(v[Cfg::kAccs - 1][e]), w1 = __uint_as_float(v[Cfg::kAccs - 1][e + 1]);
+              for (int e = 0; e < 8; e += 2) {
+                float c0 = q == 0 && fresh ? 0.f : __uint_as_float(comp[e]), c1 = q == 0 && fresh ? 0.f : __uint_as_float(comp[e + 1]);
+                compensated(sum[i + e], sum[i + e + 1], c0, c1, __uint_as_float(v[e]), __uint_as_float(v[e + 1]));
+                comp[e] = __float_as_uint(c0), comp[e + 1] = __float_as_uint(c1);
+              }
+            }
+            tmem_st8(caddr + i, comp);
+          } else {
+            // One half of the leading sums, then the other with the small ones: additions at half the sum's size.
+            float h[2][8];
+            uint32_t v[H1][8], w[Cfg::kLow + 1][8];
 #pragma unroll
-            for (int c2 = Cfg::kAccs - 2; c2 >= 0; --c2) add2(w0, w1, __uint_as_float(v[c2][e]), __uint_as_float(v[c2][e + 1]));
-            add2(sum[i + e], sum[i + e + 1], w0, w1);
+            for (int part2 = 0; part2 < 2; ++part2) {
+#pragma unroll
+              for (int q = 0; q < (part2 == 0 ? H0 : H1); ++q) {
+                if (part2 * H0 + q < Cfg::kCols / 16 || part2 * H0 + q < written) {
+                  tmem_ld8(taddr + (part2 * H0 + q) * KN + i, v[q]);
+                } else {
+#pragma unroll
+                  for (int e = 0; e < 8; ++e) v[q][e] = 0;
+                }
+              }
+              if (part2 == 1) {
+#pragma unroll
+                for (int q = 0; q < Cfg::kLow; ++q) tmem_ld8(taddr + (Cfg::kHi + q) * KN + i, w[q]);
+                tmem_ld8(caddr + i, w[Cfg::kLow]);
+              }
+              asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+#pragma unroll
+              for (int e = 0; e < 8; e += 2) {
+                float x0 = __uint_as_float(v[0][e]), x1 = __uint_as_float(v[0][e + 1]);
+#pragma unroll
+                for (int q = 1; q < (part2 == 0 ? H0 : H1); ++q) add2(x0, x1, __uint_as_float(v[q][e]), __uint_as_float(v[q][e + 1]));
+                h[part2][e] = x0, h[part2][e + 1] = x1;
+              }
+            }
+            uint32_t comp[8];
+#pragma unroll
+            for (int e = 0; e < 8; e += 2) {
+              float *const h0 = h[0], *const g = h[1];
+              if (Cfg::kLow > 0) {
+                float l0 = __uint_as_float(w[0][e]), l1 = __uint_as_float(w[0][e + 1]);
+                if (Cfg::kLow > 1) add2(l0, l1, __uint_as_float(w[Cfg::kLow - 1][e]), __uint_as_float(w[Cfg::kLow - 1][e + 1]));
+                add2(g[e], g[e + 1], l0, l1);
+              }
+              add2(h0[e], h0[e + 1], g[e], g[e + 1]);
+              float c0 = fresh ? 0.f : __uint_as_float(w[Cfg::kLow][e]), c1 = fresh ? 0.f : __uint_as_float(w[Cfg::kLow][e + 1]);
+              compensated(sum[i + e], sum[i + e + 1], c0, c1, h0[e], h0[e + 1]);
+              comp[e] = __float_as_uint(c0), comp[e + 1] = __float_as_uint(c1);
+            }
+            tmem_st8(caddr + i, comp);
           }
         }
       }
+      fresh = last;
       asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
       __syncwarp();
       if (lane == 0) mbar_arrive(acc_empty_bar(buf));
@@ -382,15 +478,15 @@ __global__ void __launch_bounds__(kSplitProjectThreads, 1) codec_split_project_k
 #pragma unroll
             for (int i = 0; i < Cfg::kSums; i += 4) {
               const float v[4] = {sum[i], sum[i + 1], sum[i + 2], sum[i + 3]};
-              store_coords4<T>(a, t, sum_col + i, v);
-              if (NX == 3 && !sums_stand(v, NU == 3 ? u_largest + sum_col + i : nullptr)) bad |= 1u << (i / 4);
+              store_coords4<T>(a, t, j_lo() + sum_col + i, j_end(), v);
+              if (!sums_stand(v, NU == 3 ? u_largest + sum_col + i : nullptr)) bad |= 1u << (i / 4);
             }
             if (bad != 0) {
 #pragma unroll 1
-              for (int i = 0; i < Cfg::kSums / 4 && sum_col + 4 * i < a.k; ++i)
-                if (bad >> i & 1) store_plain_coords4<T>(a, t, sum_col + 4 * i);
+              for (int i = 0; i < Cfg::kSums / 4 && sum_col + 4 * i < rank(); ++i)
+                if (bad >> i & 1) store_plain_coords4<T>(a, t, j_lo() + sum_col + 4 * i, j_end());
             }
-            if (a.wire_ids && part == 0) static_cast<int32_t *>(a.zout)[t * a.ldzout + a.k] = a.shift.ids[t];
+            if (a.wire_ids && part == 0 && !lower()) static_cast<int32_t *>(a.zout)[t * a.ldzout + a.k] = a.shift.ids[t];
           }
 #pragma unroll
           for (int i = 0; i < Cfg::kSums; ++i) sum[i] = 0.f;
@@ -421,6 +517,7 @@ __global__ void __launch_bounds__(kSplitProjectThreads, 1) codec_split_project_k
     uint32_t parity = 1;
     int tile = 0;                            // of this CTA, being filled
     bool prev_last = false;
+    int prev_steps = 0;
     float u_max[2] = {0.f, 0.f}, row_max[2] = {0.f, 0.f};
     const uint32_t a_off = Cfg::kF32 ? row * 64 + (((unit >> 1) ^ ((row >> 1) & 3)) << 4) + (unit & 1) * 8
                                      : row * 128 + ((unit ^ (row & 7)) << 4);   // + 64 rows: the second piece
@@ -477,7 +574,7 @@ __global__ void __launch_bounds__(kSplitProjectThreads, 1) codec_split_project_k
         split_pair<T, NU>(u, up);
 #pragma unroll
         for (int s = 0; s < NU; ++s) {
-          const int n = s * KN + u_col;
+          const int n = Cfg::b_part(s) * KN + u_col;
           st_shared_b32(base + Cfg::kABytes + (n >> 6) * Cfg::kGroupBytes + (u_row + i * kURows) * 128 +
                             ((((n & 63) >> 3) ^ (u_row & 7)) << 4) + (n & 7) * 2, up[s]);
         }
@@ -508,15 +605,20 @@ __global__ void __launch_bounds__(kSplitProjectThreads, 1) codec_split_project_k
       if (++rslot == RD) rslot = 0;
       st = next_st;
       if (st == 0) ++tile;
-      if (++in_chain == G || st == 0) {      // the accumulator before the one just filled
-        if (chain > 0) take_chain(chain - 1, prev_last);
+      // With two sets the chain before the one just filled; with one the chain before this one, as soon as this
+      // one's first step is filled, because its MMAs wait for it.
+      if (NB == 1 && in_chain == 0 && chain > 0) take_chain(chain - 1, prev_steps, prev_last);
+      if (++in_chain == G || st == 0) {
+        if (NB == 2 && chain > 0) take_chain(chain - 1, prev_steps, prev_last);
         prev_last = st == 0;
+        prev_steps = in_chain;
         in_chain = 0;
         ++chain;
       }
     }
-    take_chain(chain - 1, true);
+    take_chain(chain - 1, prev_steps, true);
     cp_async_wait<0>();
+    asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");   // before tensor memory is given back
   }
 
   if (cluster_size > 1) {
@@ -537,18 +639,19 @@ __global__ void __launch_bounds__(kSplitProjectThreads, 1) codec_split_project_k
       return r;
     };
     const uint32_t row_flags_addr = smem_u32(const_cast<unsigned char *>(row_flags));   // of tile 0, the only one
-    for (int i = tid; i < rows * (KN / 4); i += kSplitProjectThreads) {
+    for (int i = tid; i < rows * (KN / 4); i += Cfg::kThreads) {
       const int rr = row0 + i / (KN / 4), j = 4 * (i % (KN / 4));
       const int64_t t = group * kUmmaTile + rr;
-      if (t >= a.n || j >= a.k) continue;
-      float v[4] = {0.f, 0.f, 0.f, 0.f};
+      if (t >= a.n || j >= rank()) continue;
+      // up to eight slices of the sum in 64 bits: in fp32 their additions alone would err by 4e-8
+      double z[4] = {0.0, 0.0, 0.0, 0.0};
       uint32_t largest[4] = {0, 0, 0, 0}, bad_row = 0;
       for (uint32_t rk = 0; rk < cluster_size; ++rk) {
         float w0, w1, w2, w3;
         asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];\n"
                      : "=f"(w0), "=f"(w1), "=f"(w2), "=f"(w3)
                      : "r"(peer(smem0 + (uint32_t)(rr * Cfg::kSumPitch + j) * 4, rk)));
-        v[0] += w0; v[1] += w1; v[2] += w2; v[3] += w3;
+        z[0] += w0; z[1] += w1; z[2] += w2; z[3] += w3;
         if (NX == 3) {
           uint32_t m0, m1, m2, m3, f;
           asm volatile("ld.shared::cluster.v4.u32 {%0,%1,%2,%3}, [%4];\n"
@@ -559,9 +662,10 @@ __global__ void __launch_bounds__(kSplitProjectThreads, 1) codec_split_project_k
           bad_row |= f;
         }
       }
-      store_coords4<T>(a, t, j, v);
-      if (NX == 3 && (bad_row != 0 || !sums_stand(v, NU == 3 ? largest : nullptr))) store_plain_coords4<T>(a, t, j);
-      if (a.wire_ids && j == 0) static_cast<int32_t *>(a.zout)[t * a.ldzout + a.k] = a.shift.ids[t];
+      const float v[4] = {(float)z[0], (float)z[1], (float)z[2], (float)z[3]};
+      store_coords4<T>(a, t, j_lo() + j, j_end(), v);
+      if (bad_row != 0 || !sums_stand(v, NU == 3 ? largest : nullptr)) store_plain_coords4<T>(a, t, j_lo() + j, j_end());
+      if (a.wire_ids && j == 0 && !lower()) static_cast<int32_t *>(a.zout)[t * a.ldzout + a.k] = a.shift.ids[t];
     }
     // nobody leaves while its sums can still be read
     asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
