@@ -18,6 +18,22 @@ cudaError_t launch_tokens_ntp(const TokensArgs &t, const UmmaTokensMaps &maps, i
   note_kernel(SSN_KERNEL_UMMA_TOKENS, NTP > 8 ? SSN_KVAR_WIDE : 0);
   return e;
 }
+
+// CTAs for nblk blocks of nstage stages: one per SM, each with an equal range of all stages, or the same number for
+// every block, so that no range reaches into a second one and adds its sums twice.  Adding the sums of a block costs
+// a CTA about as much as k / kFlushRank stages, and more than kMostPerBlock CTAs get into one another's way there.
+constexpr int kFlushRank = 24, kMostPerBlock = 16;
+int grid_of(int64_t nblk, int64_t nstage, int k, int sms) {
+  int64_t all = nblk * nstage, per = nstage;
+  if (all > sms) all = sms;
+  if (all > kMostPerBlock * nblk) all = kMostPerBlock * nblk;
+  if (per > kMostPerBlock) per = kMostPerBlock;
+  if (per > sms / nblk) per = sms / nblk;
+  if (per < 1) return (int)all;
+  const double flush = (double)k / kFlushRank;
+  const double even = (double)((nstage + per - 1) / per) + flush, equal = (double)((nblk * nstage + all - 1) / all) + 2 * flush;
+  return (int)(even <= equal ? per * nblk : all);
+}
 }  // namespace
 
 cudaError_t launch_codec_umma_tokens(const __nv_bfloat16 *H, int64_t ldh, const __nv_bfloat16 *C, int64_t ldc,
@@ -31,17 +47,14 @@ cudaError_t launch_codec_umma_tokens(const __nv_bfloat16 *H, int64_t ldh, const 
   if (!make_sw128_map(&maps.c_wide, C, n, k <= 64 ? 64 : 128, ldc, kUmmaCols)) return cudaErrorNotSupported;
   const int nblk = (m + kUmmaTile - 1) / kUmmaTile;
   const int64_t nstage = (n + kUmmaCols - 1) / kUmmaCols;
-  // One CTA per SM, or the most of them that is a multiple of the blocks where that leaves few SMs out: no range
-  // then reaches into a second block (6443 tokens, 2048 columns, rank 64: forward, backward and this 66.3 -> 64.5 us).
-  const int64_t units = nblk * nstage, aligned = nblk <= sm_count ? nblk * (sm_count / nblk) : 0;
-  const int most = 20 * aligned >= 19 * (int64_t)sm_count ? (int)aligned : sm_count;
-  const int grid = (int)(units < most ? units : most);
+  const int grid = grid_of(nblk, nstage, k, sm_count);
   TokensArgs t{};
   t.out = out;
   t.ldout = ldout;
   t.n = n;
   t.m = m;
   t.k = k;
+  t.vec = k % 4 == 0 && ldout % 4 == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0;
   t.dev_status = dev_status;
   if (nblk % grid != 0 || nstage > kTokensChain) {   // some block is summed in parts
     cudaError_t e = cudaMemset2DAsync(out, (size_t)ldout * sizeof(float), 0, (size_t)k * sizeof(float), (size_t)m, stream);

@@ -34,6 +34,7 @@ struct TokensArgs {
   int64_t ldout;
   int64_t n;         // tokens
   int32_t m, k;
+  int32_t vec;       // rows of out take 16 bytes at a time
   int32_t *dev_status;
 };
 
@@ -41,6 +42,16 @@ struct UmmaTokensMaps {
   CUtensorMap h;             // H: boxes of 64 token rows x 64 columns
   CUtensorMap c, c_wide;     // C: boxes of 64 token rows x 64 coordinates (c_wide: see UmmaMaps)
 };
+
+// Four neighbouring sums.  The lanes of a warp hold rows, so that every access is a sector per lane: one for four
+// sums instead of one each.
+__device__ __forceinline__ void store_or_add4(float *p, uint32_t a, uint32_t b, uint32_t c, uint32_t d, bool store) {
+  if (store)
+    asm volatile("st.global.v4.b32 [%0], {%1,%2,%3,%4};\n" ::"l"(p), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+  else
+    asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1,%2,%3,%4};\n"
+                 ::"l"(p), "f"(__uint_as_float(a)), "f"(__uint_as_float(b)), "f"(__uint_as_float(c)), "f"(__uint_as_float(d)) : "memory");
+}
 
 template <int NTP>
 struct UmmaTokensConfig {
@@ -197,13 +208,18 @@ codec_umma_tokens_kernel(const TokensArgs a, const __grid_constant__ UmmaTokensM
         if (row < a.m) {
           float *orow = a.out + (int64_t)row * a.ldout;
 #pragma unroll
-          for (int i = 0; i < 16; ++i) {
+          for (int i = 0; i < 16; i += 4) {
             const int col = q * 16 + i;
-            if (col < a.k) {
-              if (whole)
-                orow[col] = __uint_as_float(v[i]);
-              else
-                atomicAdd(orow + col, __uint_as_float(v[i]));
+            if (a.vec) {
+              if (col < a.k) store_or_add4(orow + col, v[i], v[i + 1], v[i + 2], v[i + 3], whole);
+            } else {
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                if (col + e < a.k) {
+                  if (whole) orow[col + e] = __uint_as_float(v[i + e]);
+                  else atomicAdd(orow + col + e, __uint_as_float(v[i + e]));
+                }
+              }
             }
           }
         }
