@@ -9,9 +9,12 @@ namespace {
 // Whether the P rows may be gathered: us against the mma.sync kernels, E and P rows (theirs -> this one),
 // 10007 tokens: 512 columns 28 -> 16, 2048 columns 56 -> 25; 40000 x 512: 32 -> 28.  Narrower rows gain nothing
 // (10007 x 256, rank 72: 12 -> 15), nor do E and P rows of up to 16 tokens per SM (2155 x 2048: 13.6 -> 13.8,
-// rank 24 11.0 -> 13.6) unless the rank or a second run of coordinates needs their wide tiles (45 -> 14).
+// rank 24 11.0 -> 13.6) unless the rank or a second run of coordinates needs their wide tiles (45 -> 14), nor small
+// ranks up to 32 tokens per SM (4096 tokens, rank 16: 1024 columns 9.4 -> 13.7, 2048 columns 12.9 -> 16.4, 4096 columns
+// 20.3 -> 20.5).
 bool gathers_positions(const MmaArgs &a, bool has_e, int sm_count) {
   if (a.d < 512 || a.rowsumsq != nullptr) return false;
+  if (a.k <= 16 && a.d <= 2048 && a.zin2 == nullptr && a.n <= 32 * (int64_t)sm_count) return false;
   return !has_e || a.k > 64 || a.zin2 != nullptr || a.n > 16 * (int64_t)sm_count;
 }
 

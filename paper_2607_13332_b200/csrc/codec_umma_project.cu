@@ -54,7 +54,10 @@ cudaError_t launch_codec_umma_project(const MmaArgs &a, bool shift, int sm_count
     // win at every width (rank 40: 2155 x 512 6.9 -> 11.3, 2155 x 2048 13.0 -> 16.7), above it this one does
     // (10007 x 256 22 -> 11, 10007 x 2048 51 -> 23) except on narrow rows in large batches (40000 x 256
     // 17.5 -> 22); ranks above 64 from 512 columns on (2155 x 512 13.8 -> 13.3, 2155 x 2048 45 -> 18.5).
+    // Up to 32 tokens per SM small ranks keep theirs too (4096 tokens: rank 8, 512 columns 6.8 -> 11.0, 4096 columns
+    // 20.6 -> 24.3; rank 16 7.7 -> 10.3, 19.6 -> 21.6; rank 40, 256 columns 8.4 -> 10.3, 2048 columns 17.1 -> 16.5).
     const bool narrow = a.d < 512;
+    if (a.n <= 32 * (int64_t)sm_count && a.k <= 64 && (a.k <= 16 || narrow || (a.k <= 32 && a.d <= 1024))) return cudaErrorNotSupported;
     if (a.k > 64 ? narrow : a.n <= 16 * (int64_t)sm_count || (narrow && a.n > 128 * (int64_t)sm_count))
       return cudaErrorNotSupported;
   }

@@ -65,3 +65,23 @@ def test_few_rows_and_wire_rows_keep_their_kernels():
     wire = codec.compress_wire(X, ids, pos=dpos)
     assert B.ssn_last_kernel()[0] == B.SSN_KERNEL_SPLIT_PROJECT
     assert_close(wire.view(torch.float32).double().cpu().numpy(), expect, DT, "wire", tol=1e-6)
+
+
+@pytest.mark.parametrize("n,d,k,project,expand", [
+    (3000, 1024, 16, B.SSN_KERNEL_MMA_SYNC_DSPLIT, B.SSN_KERNEL_MMA_SYNC_DSPLIT),
+    (3000, 4096, 8, B.SSN_KERNEL_MMA_SYNC_DSPLIT, B.SSN_KERNEL_UMMA_EXPAND),
+    (4736, 256, 64, B.SSN_KERNEL_MMA_SYNC_DSPLIT, None), (4736, 1024, 40, B.SSN_KERNEL_UMMA_PROJECT, B.SSN_KERNEL_UMMA_EXPAND),
+    (4737, 512, 16, B.SSN_KERNEL_UMMA_PROJECT, None)])
+def test_small_ranks_of_mid_sized_calls_keep_the_mma_sync_kernels(n, d, k, project, expand):
+    wl = synth.Workload("mid", d, k, 100, 1, n, DT)
+    t = synth.codec_inputs(wl, seed=n + k, noise_std=0.05)
+    pos = np.random.default_rng(0).integers(0, 200, n).astype(np.int32)
+    codec = Codec(DT, to_device(t["U"], DT), to_device(t["E"], DT), to_device(t["P"][:200], DT))
+    ids, dpos = torch.from_numpy(t["ids"]).cuda(), torch.from_numpy(pos).cuda()
+    U, E, P = f64(t["U"], DT), f64(t["E"], DT), f64(t["P"][:200], DT)
+    Z = codec.compress(to_device(t["X"], DT), ids, pos=dpos)
+    assert B.ssn_last_kernel()[0] == project
+    assert_close(host64(Z, DT), oracle.compress(f64(t["X"], DT), U, E, t["ids"], P, pos)[0], DT, "compress")
+    X = codec.decompress(to_device(t["Z0"], DT), ids, pos=dpos)
+    assert expand is None or B.ssn_last_kernel()[0] == expand
+    assert_close(host64(X, DT), oracle.decompress(f64(t["Z0"], DT), U, E, t["ids"], P, pos)[0], DT, "decompress")
