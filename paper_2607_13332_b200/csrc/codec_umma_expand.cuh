@@ -95,16 +95,19 @@ struct UmmaExpandConfig {
       kZBufs * kZBytes + kSelBytes + kUStages * kUStageBytes + kStagingBytes;
   static constexpr int kMaxSmem = 227 * 1024;
   static constexpr int kEFit = (kMaxSmem - 1024 - 1024 - kFixedBytes) / kEStageBytes;
-  // A chunk takes 2 kGathered stages and the two epilogue groups take alternate chunks, so with E and P pieces a
-  // ring of 8 brings every group back to stages it consumed itself.  (A wait on a phase is only sound when the
-  // phase before it is known to be over; with 10 stages that would be the other group's, two chunks back.)
+  // A chunk takes 2 kGathered stages and the two epilogue groups take alternate chunks.  A wait on a phase is only
+  // sound when the phase before it is known to be over, so a group must see every phase of a barrier it waits on: with
+  // a ring of whole pairs of chunks every stage always serves the same group; with one of an odd number of chunks
+  // the groups take turns on every stage, and each has full barriers of its own (kTurns).
   static constexpr int kEMost = kGathered == 2 ? 8 : 12;
   static constexpr int kEStages = kGathered > 0 ? (kEFit < kEMost ? kEFit : kEMost) : 0;
   static_assert(kGathered == 0 || kEStages >= 4, "no room for the E ring");
+  static_assert(kGathered == 0 || kEStages % (2 * kGathered) == 0, "the ring holds whole chunks");
+  static constexpr bool kTurns = kGathered > 0 && kEStages % (4 * kGathered) != 0;
   static constexpr int kDBufs = 2;                 // accumulators of 128 columns: one per epilogue group
   static constexpr int kTmemCols = 256;
   static constexpr int SE = kGathered > 0 ? kEStages : 1;
-  static constexpr int kBars = 4 + 2 * kUStages + 8 * SE + 2 * kDBufs;   // the E ring has a full and an empty barrier per stage and QUARTER
+  static constexpr int kBars = 4 + 2 * kUStages + (kTurns ? 12 : 8) * SE + 2 * kDBufs;   // the E ring has a full and an empty barrier per stage and QUARTER
   static constexpr int kSmemBytes = 1024 + kFixedBytes + kEStages * kEStageBytes + kBars * 8 + 16;
   static_assert(kSmemBytes <= kMaxSmem, "the rings do not fit in shared memory");
 };
@@ -158,7 +161,10 @@ codec_umma_expand_kernel(const MmaArgs a, const ExpandGeometry geo, const __grid
   auto u_empty_bar = [&](int s) { return bars + (4 + SU + s) * 8; };
   // The E ring is handed over per QUARTER of a stage (32 rows: one gather warp fills them, one
   // epilogue warp of either group consumes them), so that a late row holds up only its own quarter.
-  auto e_full_bar = [&](int s, int q) { return bars + (4 + 2 * SU + 4 * s + q) * 8; };
+  auto e_full_bar = [&](int s, int q, int group) {   // of either epilogue group, if they take turns
+    return bars + (4 + 2 * SU + 4 * s + q + (Cfg::kTurns && group != 0 ? 8 * SE + 2 * Cfg::kDBufs : 0)) * 8;
+  };
+  auto e_full_parity = [&](int64_t count) { return (uint32_t)((Cfg::kTurns ? count / SE / 2 : count / SE) & 1); };
   auto e_empty_bar = [&](int s, int q) { return bars + (4 + 2 * SU + 4 * SE + 4 * s + q) * 8; };
   auto d_full_bar = [&](int b) { return bars + (4 + 2 * SU + 8 * SE + b) * 8; };
   auto d_empty_bar = [&](int b) { return bars + (4 + 2 * SU + 8 * SE + Cfg::kDBufs + b) * 8; };
@@ -201,7 +207,8 @@ codec_umma_expand_kernel(const MmaArgs a, const ExpandGeometry geo, const __grid
     }
     for (int s = 0; s < SE; ++s) {
       for (int q = 0; q < 4; ++q) {
-        mbar_init(e_full_bar(s, q), 32);             // one arrival per thread of the quarter's gather warp
+        mbar_init(e_full_bar(s, q, 0), 32);          // one arrival per thread of the quarter's gather warp
+        if (Cfg::kTurns) mbar_init(e_full_bar(s, q, 1), 32);
         mbar_init(e_empty_bar(s, q), 1);             // the epilogue warp that consumed the quarter
       }
     }
@@ -350,7 +357,7 @@ codec_umma_expand_kernel(const MmaArgs a, const ExpandGeometry geo, const __grid
       const int gw = warp - 10;                // rows 32*gw .. 32*gw+31 of the tile
       const int piece = lane & 7, sub = lane >> 3;
       int slot = 0;
-      uint32_t parity = 1;
+      uint32_t parity = 1, turn = 0;           // turn: 64-column groups so far
       for (int64_t tile = tile_lo; tile <= tile_hi; ++tile) {
         int c1, c2;
         tile_coords(tile, c1, c2);
@@ -377,14 +384,15 @@ codec_umma_expand_kernel(const MmaArgs a, const ExpandGeometry geo, const __grid
         }
         int q0, q1;
         chunk_range(tile, q0, q1);
-        for (int qg = 2 * q0; qg < 2 * q1; ++qg) {     // 64-column groups of the row
+        for (int qg = 2 * q0; qg < 2 * q1; ++qg, ++turn) {     // 64-column groups of the row
 #pragma unroll
           for (int o = 0; o < NG; ++o) {
             if (!dead && !mbar_wait(e_empty_bar(slot, gw), parity)) timed_out();
             const uint32_t base = e_ring + (uint32_t)slot * Cfg::kEStageBytes;
 #pragma unroll
             for (int i = 0; i < 8; ++i) cp_async16_cg(base + dst[i], src[o][i] + qg * 128);
-            asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];\n" ::"r"(e_full_bar(slot, gw)) : "memory");
+            asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];\n" ::"r"(e_full_bar(slot, gw, (int)(turn >> 1 & 1)))
+                         : "memory");
             if (++slot == SE) {
               slot = 0;
               parity ^= 1u;
@@ -439,7 +447,7 @@ codec_umma_expand_kernel(const MmaArgs a, const ExpandGeometry geo, const __grid
           }
           uint32_t slab;   // 32 rows x 128 B handed to the TMA store
           if (NG > 0) {
-            if (!dead && !mbar_wait(e_full_bar(eslot, quarter), (uint32_t)((ecount / SE) & 1))) timed_out();
+            if (!dead && !mbar_wait(e_full_bar(eslot, quarter, group), e_full_parity(ecount))) timed_out();
             slab = e_ring + (uint32_t)eslot * Cfg::kEStageBytes + (uint32_t)quarter * 4096;
           } else {
             // the store that last read this slab (two stores ago) must be done reading it
@@ -451,7 +459,7 @@ codec_umma_expand_kernel(const MmaArgs a, const ExpandGeometry geo, const __grid
           if (NG == 2) {   // the P pieces from the next stage, which goes back at once
             const int64_t pcount = ecount + 1;
             const int pslot = (int)(pcount % SE);
-            if (!dead && !mbar_wait(e_full_bar(pslot, quarter), (uint32_t)((pcount / SE) & 1))) timed_out();
+            if (!dead && !mbar_wait(e_full_bar(pslot, quarter, group), e_full_parity(pcount))) timed_out();
             const uint32_t prow = e_ring + (uint32_t)pslot * Cfg::kEStageBytes + (uint32_t)quarter * 4096 + lane * 128;
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
