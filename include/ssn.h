@@ -128,7 +128,8 @@ typedef struct ssn_codec {
  * fixed and known to both ends, and U_k is fixed, so by linearity Eq. (ssn_compress) is
  *     Z[t,:] = X[t,:] U - EU[ids[t],:] - PU[pos(t),:]
  * and a codec whose EU / PU fields point at these tables lets ssn_compress read only X, ids
- * and 2k floats per token instead of the E and P rows.  Either output may be NULL (then that
+ * and 2k floats per token instead of the E and P rows (the TMA kernels, from 512 tokens on; the
+ * other kernels, fp32 storage among them, give the same result from the rows).  Either output may be NULL (then that
  * table is not made; it must be NULL when the codec has no such term).  The tables must be
  * made again whenever U, E or P change.  The codec passed in is read for U, E, P only.
  */

@@ -271,7 +271,7 @@ struct UmmaProjectConfig {
   // Warps: 0 producer; 1-3 the first three issuers; 4-7 epilogue; with E rows 8-11 gather them and
   // warp 12 is the fourth issuer (E only, k <= 64).  A launch has only the warps its roles need, so
   // that the register budget of the epilogue (a whole accumulator row per thread) is not cut by
-  // warps that would idle: 256 threads without E rows, 384 or 416 with them.
+  // warps that would idle: 256 threads where nothing is gathered, 384 or 416 where E or P rows are.
   static constexpr int kWarps = !kGathers ? 8 : (kIssuers == 4 ? 13 : 12);
   static constexpr int kThreads = 32 * kWarps;
   static constexpr int kBufs = 2 * kIssuers * kAccCols <= 512 ? 2 : 1;   // accumulator sets (tiles in flight)

@@ -1,6 +1,6 @@
 """GPU parity on batches of whole sequences at 512 to 8192 tokens, against the CPU oracle element
-by element.  At these sizes the projections (compress, grad-project) and the fused
-project-then-expand run on the tcgen05 kernels, while decompress takes the few-rows-per-SM
+by element.  At these sizes compress with E or P and the fused project-then-expand run on the tcgen05
+kernels (compress without either takes the few-rows kernel up to 2368 tokens), while decompress takes the few-rows-per-SM
 mma.sync kernel; the tcgen05 expansion and the large-batch mma.sync kernels are covered, with an
 assertion of which kernel ran, in test_gpu_dispatch_coverage.py.  Also here: the prepared tables
 EU = E U, PU = P U, the re-projection lists, guard bands and odd leading dimensions."""
