@@ -203,7 +203,7 @@ class Codec:
         Xh = out if out is not None else self._empty(n, self.d)
         if workspace is None:
             nbytes = binding.ssn_decompress_wire_workspace_bytes(self.c, n, with_ids)
-            if not use_workspace:   # only what the ids need: the general kernel runs
+            if not use_workspace:   # only what the ids need: the fp32 words are split in the expansion
                 nbytes = (n * 4 + 255) // 256 * 256 if with_ids else 0
             workspace = torch.empty(nbytes, dtype=torch.uint8, device=self.U.device) if nbytes else None
         binding.ssn_decompress_wire(self.c, wire.data_ptr(), _ld(wire), with_ids,
