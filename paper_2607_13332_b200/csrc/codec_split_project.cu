@@ -1,8 +1,13 @@
-// Launcher of the split-operand projection kernel (see codec_split_project.cuh).
+// Launchers of the split-operand projection kernel (codec_split_project.cuh) and of its form for bf16 rows as they are
+// (codec_plain_project.cuh).
 #include "codec_split_project.cuh"
 
+#include <algorithm>
+
 #include "codec_mma_launch.h"
+#include "codec_plain_project.cuh"
 #include "codec_split.h"
+#include "codec_tensor_maps.h"
 
 namespace ssn {
 namespace {
@@ -31,24 +36,62 @@ int cluster_of(int64_t ntiles, int nst, int sms) {
 
 int64_t units_of(const SplitProjectArgs &a) { return (a.n + kUmmaTile - 1) / kUmmaTile * a.halves; }   // tiles, or halves of them
 
+// Launches either kernel with clusters of c, or with single CTAs on a device that cannot co-schedule them.
+template <typename Kernel, typename... Args>
+cudaError_t launch_slices(Kernel kernel, int threads, int smem, const SplitProjectArgs &a, int c, int sms, cudaStream_t stream,
+                          Args... args) {
+  const int64_t units = units_of(a);
+  // whole tiles: as many CTAs for either half
+  const int64_t single = units < sms ? units : (sms > 1 ? sms - sms % a.halves : a.halves), grid = c > 1 ? units * c : single;
+  cudaError_t e = launch_dependent(kernel, (unsigned)grid, threads, smem, stream, c, a, args...);
+  if (e != cudaSuccess && c > 1) {
+    cudaGetLastError();
+    e = launch_dependent(kernel, (unsigned)single, threads, smem, stream, 1, a, args...);
+  }
+  note_kernel(SSN_KERNEL_SPLIT_PROJECT, (a.has_e ? SSN_KVAR_E : 0) | (a.has_p ? SSN_KVAR_P : 0) |
+                                            (a.halves > 1 ? SSN_KVAR_WIDE : 0) | (c > 1 ? SSN_KVAR_ALT : 0));
+  return e;
+}
+
 template <typename T, int KN, int NSLOT, bool CAREFUL>
 cudaError_t launch_one(const SplitProjectArgs &a, int c, int sms, cudaStream_t stream) {
   using Cfg = SplitProjectConfig<T, KN, NSLOT, CAREFUL>;
   auto kernel = codec_split_project_kernel<T, KN, NSLOT, CAREFUL>;
   static std::atomic<uint64_t> configured{0};
-  cudaError_t e = allow_dynamic_smem(kernel, Cfg::kSmemBytes, configured);
+  const cudaError_t e = allow_dynamic_smem(kernel, Cfg::kSmemBytes, configured);
   if (e != cudaSuccess) return e;
+  return launch_slices(kernel, Cfg::kThreads, Cfg::kSmemBytes, a, c, sms, stream);
+}
+
+// The plain kernel's CTAs per tile.  A stage takes a CTA kPlainStageNs, or the time of the 16 KB that every CTA at work
+// takes from HBM, whichever is longer; a wave of clusters kPlainWaveNs besides.  Single CTAs are persistent.
+constexpr double kPlainStageNs = 260, kPlainHbmNs = 2.65, kPlainWaveNs = 4000;
+int plain_cluster_of(const SplitProjectArgs &a, int nst, int sms) {
   const int64_t units = units_of(a);
-  // whole tiles: as many CTAs for either half
-  const int64_t single = units < sms ? units : (sms > 1 ? sms - sms % a.halves : a.halves), grid = c > 1 ? units * c : single;
-  e = launch_dependent(kernel, (unsigned)grid, Cfg::kThreads, Cfg::kSmemBytes, stream, c, a);
-  if (e != cudaSuccess && c > 1) {   // a device that cannot co-schedule the cluster
-    cudaGetLastError();
-    e = launch_dependent(kernel, (unsigned)single, Cfg::kThreads, Cfg::kSmemBytes, stream, 1, a);
+  auto stage_ns = [&](int64_t ctas) { return std::max(kPlainStageNs, kPlainHbmNs * (double)ctas / a.halves); };
+  int best = 1;
+  double best_ns = kPlainWaveNs + (double)((units + sms - 1) / sms) * nst * stage_ns(units < sms ? units : sms);
+  for (int c = 2; c <= 8 && c <= nst; ++c) {
+    const int64_t at_once = kClustersAtOnce[c - 1] * sms / 148;
+    if (at_once < 1) break;
+    const double ns = (double)((units + at_once - 1) / at_once) *
+                      (kPlainWaveNs + (double)((nst + c - 1) / c) * stage_ns((units < at_once ? units : at_once) * c));
+    if (ns < 0.97 * best_ns) {
+      best = c;
+      best_ns = ns;
+    }
   }
-  note_kernel(SSN_KERNEL_SPLIT_PROJECT, (a.has_e ? SSN_KVAR_E : 0) | (a.has_p ? SSN_KVAR_P : 0) |
-                                            (a.halves > 1 ? SSN_KVAR_WIDE : 0) | (c > 1 ? SSN_KVAR_ALT : 0));
-  return e;
+  return best;
+}
+
+template <int KN>
+cudaError_t launch_plain(const SplitProjectArgs &a, const CUtensorMap &x, int sms, cudaStream_t stream) {
+  auto kernel = codec_plain_project_kernel<KN>;
+  constexpr int smem = PlainProjectConfig<KN>::kSmemBytes;
+  static std::atomic<uint64_t> configured{0};
+  const cudaError_t e = allow_dynamic_smem(kernel, smem, configured);
+  if (e != cudaSuccess) return e;
+  return launch_slices(kernel, kPlainThreads, smem, a, plain_cluster_of(a, (a.d + kUmmaCols - 1) / kUmmaCols, sms), sms, stream, x);
 }
 
 template <typename T, int NSLOT>
@@ -105,6 +148,11 @@ cudaError_t launch_codec_split_project(const TokenArgs &a, int32_t dtype, int sm
   // four coordinates are 16 bytes of words or 8 bytes of bf16
   p.vec_out = (a.ldzout & 3) == 0 && (reinterpret_cast<uintptr_t>(a.zout) & (a.wire || dtype == SSN_F32 ? 15 : 7)) == 0;
   const int slots = (a.src2 != nullptr) + p.has_e + p.has_p;
+  if (dtype == SSN_BF16 && slots == 0 && rows16(a.src, a.lds, esz)) {   // rows that TMA can fetch, and nothing to add to them
+    CUtensorMap x;
+    if (make_sw128_map(&x, a.src, a.n, a.d, a.lds, kUmmaTile))
+      return a.k <= 32 ? launch_plain<32>(p, x, sm_count, stream) : launch_plain<64>(p, x, sm_count, stream);
+  }
   return dtype == SSN_F32 ? launch_slots<float>(p, slots, sm_count, stream)
                           : launch_slots<__nv_bfloat16>(p, slots, sm_count, stream);
 }

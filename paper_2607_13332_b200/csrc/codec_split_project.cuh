@@ -168,6 +168,88 @@ __device__ __noinline__ void store_plain_coords4(const SplitProjectArgs &a, int6
   store_coords4<T>(a, t, j, j_end, {(float)acc[0], (float)acc[1], (float)acc[2], (float)acc[3]});
 }
 
+// What a CTA of a launch with a.halves halves computes: its tiles, columns of d and coordinates.
+struct SplitSchedule {
+  uint32_t cluster_size, cta_rank;
+  int64_t groups, group;       // CTAs (clusters) side by side, and this one
+  bool upper;
+  int st_lo, nloc, my_tiles;   // steps of d; one tile with clusters
+  const SplitProjectArgs &a;
+  __device__ __forceinline__ SplitSchedule(const SplitProjectArgs &args, int cols) : a(args) {
+    asm volatile("mov.u32 %0, %%cluster_nctaid.x;\n" : "=r"(cluster_size));
+    asm volatile("mov.u32 %0, %%cluster_ctarank;\n" : "=r"(cta_rank));
+    const int64_t ntiles = (a.n + kUmmaTile - 1) / kUmmaTile;
+    // the two halves of a tile's coordinates run side by side, so that its rows come from HBM once
+    groups = gridDim.x / cluster_size / a.halves;
+    group = blockIdx.x / cluster_size / a.halves;
+    upper = a.halves > 1 && (blockIdx.x / cluster_size & 1) != 0;
+    const int nst = (a.d + cols - 1) / cols;
+    st_lo = (int)((int64_t)nst * cta_rank / cluster_size);
+    nloc = (int)((int64_t)nst * (cta_rank + 1) / cluster_size) - st_lo;   // >= 1: cluster_size <= nst
+    my_tiles = (int)((ntiles - group + groups - 1) / groups);
+  }
+  __device__ __forceinline__ int64_t tile(int i) const { return group + (int64_t)i * groups; }
+  __device__ __forceinline__ bool lower() const { return a.halves > 1 && !upper; }   // coordinates j_lo() to j_end()
+  __device__ __forceinline__ int j_lo() const { return upper ? a.k_half : 0; }
+  __device__ __forceinline__ int j_end() const { return lower() ? a.k_half : a.k; }
+  __device__ __forceinline__ int rank() const { return j_end() - j_lo(); }
+};
+
+// s += x with compensation c, two sums at a time.
+__device__ __forceinline__ void add_compensated2(float &s0, float &s1, float &c0, float &c1, float x0, float x1) {
+  sub2(x0, x1, c0, c1);
+  float t0 = s0, t1 = s1;
+  add2(t0, t1, x0, x1);
+  c0 = t0, c1 = t1;
+  sub2(c0, c1, s0, s1);
+  sub2(c0, c1, x0, x1);
+  s0 = t0, s1 = t1;
+}
+
+// The CTAs of a cluster have left their sums [128][KN + 4] at smem0; each adds up, and stores, its share of the rows.
+// FLAGS: beside them lie the largest magnitudes per column of U and, per row, whether the split does not hold it.
+template <typename T, int KN, int THREADS, bool FLAGS>
+__device__ __forceinline__ void finish_slices(const SplitProjectArgs &a, const SplitSchedule &s, uint32_t smem0, uint32_t u_largest_addr,
+                                              uint32_t row_flags_addr) {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+  const int row0 = (int)(kUmmaTile * s.cta_rank / s.cluster_size), rows = (int)(kUmmaTile * (s.cta_rank + 1) / s.cluster_size) - row0;
+  auto peer = [](uint32_t addr, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+  };
+  for (int i = threadIdx.x; i < rows * (KN / 4); i += THREADS) {
+    const int rr = row0 + i / (KN / 4), j = 4 * (i % (KN / 4));
+    const int64_t t = s.group * kUmmaTile + rr;
+    if (t >= a.n || j >= s.rank()) continue;
+    // up to eight slices of the sum in 64 bits: in fp32 their additions alone would err by 4e-8
+    double z[4] = {0.0, 0.0, 0.0, 0.0};
+    uint32_t largest[4] = {0, 0, 0, 0}, bad_row = 0;
+    for (uint32_t rk = 0; rk < s.cluster_size; ++rk) {
+      float w0, w1, w2, w3;
+      asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];\n"
+                   : "=f"(w0), "=f"(w1), "=f"(w2), "=f"(w3)
+                   : "r"(peer(smem0 + (uint32_t)(rr * (KN + 4) + j) * 4, rk)));
+      z[0] += w0; z[1] += w1; z[2] += w2; z[3] += w3;
+      if (FLAGS) {
+        uint32_t m0, m1, m2, m3, f;
+        asm volatile("ld.shared::cluster.v4.u32 {%0,%1,%2,%3}, [%4];\n"
+                     : "=r"(m0), "=r"(m1), "=r"(m2), "=r"(m3) : "r"(peer(u_largest_addr + j * 4, rk)));
+        largest[0] = max(largest[0], m0); largest[1] = max(largest[1], m1);
+        largest[2] = max(largest[2], m2); largest[3] = max(largest[3], m3);
+        asm volatile("ld.shared::cluster.u8 %0, [%1];\n" : "=r"(f) : "r"(peer(row_flags_addr + rr, rk)));
+        bad_row |= f;
+      }
+    }
+    const float v[4] = {(float)z[0], (float)z[1], (float)z[2], (float)z[3]};
+    store_coords4<T>(a, t, s.j_lo() + j, s.j_end(), v);
+    if (bad_row != 0 || !sums_stand(v, FLAGS && sizeof(T) == 4 ? largest : nullptr)) store_plain_coords4<T>(a, t, s.j_lo() + j, s.j_end());
+    if (a.wire_ids && j == 0 && !s.lower()) static_cast<int32_t *>(a.zout)[t * a.ldzout + a.k] = a.shift.ids[t];
+  }
+  // nobody leaves while its sums can still be read
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+}
+
 template <typename T, int KN, int NSLOT, bool CAREFUL>
 __global__ void __launch_bounds__((SplitProjectConfig<T, KN, NSLOT, CAREFUL>::kThreads), 1) codec_split_project_kernel(const SplitProjectArgs a) {
   using Cfg = SplitProjectConfig<T, KN, NSLOT, CAREFUL>;
@@ -176,22 +258,9 @@ __global__ void __launch_bounds__((SplitProjectConfig<T, KN, NSLOT, CAREFUL>::kT
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
-  uint32_t cluster_size, cta_rank;
-  asm volatile("mov.u32 %0, %%cluster_nctaid.x;\n" : "=r"(cluster_size));
-  asm volatile("mov.u32 %0, %%cluster_ctarank;\n" : "=r"(cta_rank));
-  const int64_t ntiles = (a.n + kUmmaTile - 1) / kUmmaTile;
-  // the two halves of a tile's coordinates run side by side, so that its rows come from HBM once
-  const int64_t groups = gridDim.x / cluster_size / a.halves, group = blockIdx.x / cluster_size / a.halves;
-  const bool upper = a.halves > 1 && (blockIdx.x / cluster_size & 1) != 0;
-  auto lower = [&]() { return a.halves > 1 && !upper; };     // coordinates j_lo() to j_end()
-  auto j_lo = [&]() { return upper ? a.k_half : 0; };
-  auto j_end = [&]() { return lower() ? a.k_half : a.k; };
-  auto rank = [&]() { return j_end() - j_lo(); };
-  const int nst = (a.d + Cfg::kCols - 1) / Cfg::kCols;
-  const int st_lo = (int)((int64_t)nst * cta_rank / cluster_size);
-  const int nloc = (int)((int64_t)nst * (cta_rank + 1) / cluster_size) - st_lo;   // >= 1: cluster_size <= nst
-  const int my_tiles = (int)((ntiles - group + groups - 1) / groups);             // 1 with clusters
-  const int steps = my_tiles * nloc;
+  const SplitSchedule sched(a, Cfg::kCols);
+  const int st_lo = sched.st_lo, nloc = sched.nloc;
+  const int steps = sched.my_tiles * nloc;
 
   const uint32_t smem_u = smem_u32(smem_raw), smem0 = (smem_u + 1023u) & ~1023u;
   const uint32_t raw0 = smem0 + S * Cfg::kStageBytes, bars = smem0 + Cfg::kRingBytes;
@@ -304,10 +373,10 @@ __global__ void __launch_bounds__((SplitProjectConfig<T, KN, NSLOT, CAREFUL>::kT
     const bool vec = a.vec_rows != 0;
     // the pairs of U this thread moves: rows u_row, u_row + kURows, ... of the step (8 divides kURows)
     constexpr int kURows = 2 * kSplitRowThreads / KN;
-    const int u_row = tid / (KN / 2), u_col = 2 * (tid % (KN / 2)), u_valid = max(rank() - u_col, 0);
+    const int u_row = tid / (KN / 2), u_col = 2 * (tid % (KN / 2)), u_valid = max(sched.rank() - u_col, 0);
     const int64_t u_step = kURows * a.ldu;
     const bool vec_u = a.vec_u != 0;
-    const T *U = static_cast<const T *>(a.U) + j_lo();
+    const T *U = static_cast<const T *>(a.U) + sched.j_lo();
     const T *ptr[1 + NSLOT][2];              // this thread's rows: X, then R, E, P as far as present
     Pair<T> ureg[Cfg::kPairs];
     const bool has_r = NSLOT > 0 && a.src2 != nullptr;
@@ -390,16 +459,6 @@ __global__ void __launch_bounds__((SplitProjectConfig<T, KN, NSLOT, CAREFUL>::kT
         const uint32_t lane_addr = tmem_base + ((uint32_t)(quarter * 32) << 16) + sum_col;
         const uint32_t taddr = lane_addr + (uint32_t)buf * Cfg::kDCols, caddr = lane_addr + Cfg::kCompCol;
         asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");   // the compensation of the chain before
-        // s += x with compensation c
-        auto compensated = [](float &s0, float &s1, float &c0, float &c1, float x0, float x1) {
-          sub2(x0, x1, c0, c1);
-          float t0 = s0, t1 = s1;
-          add2(t0, t1, x0, x1);
-          c0 = t0, c1 = t1;
-          sub2(c0, c1, s0, s1);
-          sub2(c0, c1, x0, x1);
-          s0 = t0, s1 = t1;
-        };
         constexpr int H0 = Cfg::kHi / 2, H1 = Cfg::kHi - H0;
 #pragma unroll
         for (int i = 0; i < Cfg::kSums; i += 8) {
@@ -414,7 +473,7 @@ __global__ void __launch_bounds__((SplitProjectConfig<T, KN, NSLOT, CAREFUL>::kT
 #pragma unroll
               for (int e = 0; e < 8; e += 2) {
                 float c0 = q == 0 && fresh ? 0.f : __uint_as_float(comp[e]), c1 = q == 0 && fresh ? 0.f : __uint_as_float(comp[e + 1]);
-                compensated(sum[i + e], sum[i + e + 1], c0, c1, __uint_as_float(v[e]), __uint_as_float(v[e + 1]));
+                add_compensated2(sum[i + e], sum[i + e + 1], c0, c1, __uint_as_float(v[e]), __uint_as_float(v[e + 1]));
                 comp[e] = __float_as_uint(c0), comp[e + 1] = __float_as_uint(c1);
               }
             }
@@ -459,7 +518,7 @@ __global__ void __launch_bounds__((SplitProjectConfig<T, KN, NSLOT, CAREFUL>::kT
               }
               add2(h0[e], h0[e + 1], g[e], g[e + 1]);
               float c0 = fresh ? 0.f : __uint_as_float(w[Cfg::kLow][e]), c1 = fresh ? 0.f : __uint_as_float(w[Cfg::kLow][e + 1]);
-              compensated(sum[i + e], sum[i + e + 1], c0, c1, h0[e], h0[e + 1]);
+              add_compensated2(sum[i + e], sum[i + e + 1], c0, c1, h0[e], h0[e + 1]);
               comp[e] = __float_as_uint(c0), comp[e + 1] = __float_as_uint(c1);
             }
             tmem_st8(caddr + i, comp);
@@ -471,22 +530,22 @@ __global__ void __launch_bounds__((SplitProjectConfig<T, KN, NSLOT, CAREFUL>::kT
       __syncwarp();
       if (lane == 0) mbar_arrive(acc_empty_bar(buf));
       if (last) {
-        const int64_t t = (group + (int64_t)fin_tile * groups) * kUmmaTile + sum_row;
-        if (cluster_size == 1) {
+        const int64_t t = sched.tile(fin_tile) * kUmmaTile + sum_row;
+        if (sched.cluster_size == 1) {
           if (t < a.n) {
             uint32_t bad = NX == 3 && row_flags[(fin_tile & 3) * kUmmaTile + sum_row] != 0 ? ~0u : 0u;
 #pragma unroll
             for (int i = 0; i < Cfg::kSums; i += 4) {
               const float v[4] = {sum[i], sum[i + 1], sum[i + 2], sum[i + 3]};
-              store_coords4<T>(a, t, j_lo() + sum_col + i, j_end(), v);
+              store_coords4<T>(a, t, sched.j_lo() + sum_col + i, sched.j_end(), v);
               if (!sums_stand(v, NU == 3 ? u_largest + sum_col + i : nullptr)) bad |= 1u << (i / 4);
             }
             if (bad != 0) {
 #pragma unroll 1
-              for (int i = 0; i < Cfg::kSums / 4 && sum_col + 4 * i < rank(); ++i)
-                if (bad >> i & 1) store_plain_coords4<T>(a, t, j_lo() + sum_col + 4 * i, j_end());
+              for (int i = 0; i < Cfg::kSums / 4 && sum_col + 4 * i < sched.rank(); ++i)
+                if (bad >> i & 1) store_plain_coords4<T>(a, t, sched.j_lo() + sum_col + 4 * i, sched.j_end());
             }
-            if (a.wire_ids && part == 0 && !lower()) static_cast<int32_t *>(a.zout)[t * a.ldzout + a.k] = a.shift.ids[t];
+            if (a.wire_ids && part == 0 && !sched.lower()) static_cast<int32_t *>(a.zout)[t * a.ldzout + a.k] = a.shift.ids[t];
           }
 #pragma unroll
           for (int i = 0; i < Cfg::kSums; ++i) sum[i] = 0.f;
@@ -498,7 +557,7 @@ __global__ void __launch_bounds__((SplitProjectConfig<T, KN, NSLOT, CAREFUL>::kT
     int ld_tile = 0, ld_st = 0, ld_slot = 0;
     auto advance_rows = [&](bool more) {     // requests one more step (or commits an empty group)
       if (more) {
-        if (ld_st == 0) row_pointers(group + (int64_t)ld_tile * groups);
+        if (ld_st == 0) row_pointers(sched.tile(ld_tile));
         issue_rows(ld_st, ld_slot);
         if (++ld_st == nloc) {
           ld_st = 0;
@@ -621,7 +680,7 @@ __global__ void __launch_bounds__((SplitProjectConfig<T, KN, NSLOT, CAREFUL>::kT
     asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");   // before tensor memory is given back
   }
 
-  if (cluster_size > 1) {
+  if (sched.cluster_size > 1) {
     // Every accumulator has been read, so every stage is consumed and the rings can carry the sums.
     __syncthreads();
     if (warp < kSplitRowWarps) {
@@ -631,44 +690,7 @@ __global__ void __launch_bounds__((SplitProjectConfig<T, KN, NSLOT, CAREFUL>::kT
         st_shared_v4(dst + c * 4, __float_as_uint(sum[c]), __float_as_uint(sum[c + 1]), __float_as_uint(sum[c + 2]),
                      __float_as_uint(sum[c + 3]));
     }
-    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
-    const int row0 = (int)(kUmmaTile * cta_rank / cluster_size), rows = (int)(kUmmaTile * (cta_rank + 1) / cluster_size) - row0;
-    auto peer = [](uint32_t addr, uint32_t rank) {
-      uint32_t r;
-      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(r) : "r"(addr), "r"(rank));
-      return r;
-    };
-    const uint32_t row_flags_addr = smem_u32(const_cast<unsigned char *>(row_flags));   // of tile 0, the only one
-    for (int i = tid; i < rows * (KN / 4); i += Cfg::kThreads) {
-      const int rr = row0 + i / (KN / 4), j = 4 * (i % (KN / 4));
-      const int64_t t = group * kUmmaTile + rr;
-      if (t >= a.n || j >= rank()) continue;
-      // up to eight slices of the sum in 64 bits: in fp32 their additions alone would err by 4e-8
-      double z[4] = {0.0, 0.0, 0.0, 0.0};
-      uint32_t largest[4] = {0, 0, 0, 0}, bad_row = 0;
-      for (uint32_t rk = 0; rk < cluster_size; ++rk) {
-        float w0, w1, w2, w3;
-        asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];\n"
-                     : "=f"(w0), "=f"(w1), "=f"(w2), "=f"(w3)
-                     : "r"(peer(smem0 + (uint32_t)(rr * Cfg::kSumPitch + j) * 4, rk)));
-        z[0] += w0; z[1] += w1; z[2] += w2; z[3] += w3;
-        if (NX == 3) {
-          uint32_t m0, m1, m2, m3, f;
-          asm volatile("ld.shared::cluster.v4.u32 {%0,%1,%2,%3}, [%4];\n"
-                       : "=r"(m0), "=r"(m1), "=r"(m2), "=r"(m3) : "r"(peer(smem_u32(u_largest + j), rk)));
-          largest[0] = max(largest[0], m0); largest[1] = max(largest[1], m1);
-          largest[2] = max(largest[2], m2); largest[3] = max(largest[3], m3);
-          asm volatile("ld.shared::cluster.u8 %0, [%1];\n" : "=r"(f) : "r"(peer(row_flags_addr + rr, rk)));
-          bad_row |= f;
-        }
-      }
-      const float v[4] = {(float)z[0], (float)z[1], (float)z[2], (float)z[3]};
-      store_coords4<T>(a, t, j_lo() + j, j_end(), v);
-      if (bad_row != 0 || !sums_stand(v, NU == 3 ? largest : nullptr)) store_plain_coords4<T>(a, t, j_lo() + j, j_end());
-      if (a.wire_ids && j == 0 && !lower()) static_cast<int32_t *>(a.zout)[t * a.ldzout + a.k] = a.shift.ids[t];
-    }
-    // nobody leaves while its sums can still be read
-    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+    finish_slices<T, KN, Cfg::kThreads, NX == 3>(a, sched, smem0, smem_u32(u_largest), smem_u32(const_cast<unsigned char *>(row_flags)));
   }
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   __syncthreads();

@@ -1,0 +1,74 @@
+"""Projection of bf16 rows as they are, with a basis at any address and pitch: rows of U that start on and between 4-byte
+words, ranks on both sides of a lane's pair and of the 32- and 64-coordinate kernels, widths that end inside a stage, one
+tile to several CTAs and several tiles to one; NaN around every operand, and infinite and NaN rows."""
+
+import numpy as np
+import pytest
+import torch
+
+from paper_2607_13332_b200 import binding as B
+from paper_2607_13332_b200 import synth
+from tests.harness import Codec, assert_close
+
+pytestmark = pytest.mark.gpu
+
+# fp32 words of exact products, up to 4096 of them added with compensation: the rounding of the result, 6e-8, and a few 2^-24
+# of the partial sums, which are no larger than the rms at these inputs
+WORD_TOL = 1e-6
+
+
+def _rand(shape, seed, std=1.0):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    return (torch.randn(shape, device="cuda", generator=g) * std).bfloat16()
+
+
+def _inside_nan(t, pitch, offset):
+    """t at `offset` elements into a buffer of NaN, rows `pitch` apart."""
+    rows, cols = t.shape
+    buf = torch.full((offset + rows * pitch + 8,), float("nan"), dtype=t.dtype, device="cuda")
+    view = torch.as_strided(buf, (rows, cols), (pitch, 1), offset)
+    view.copy_(t)
+    return view
+
+
+@pytest.mark.parametrize("n,d", [(1, 64), (127, 72), (128, 128), (129, 200), (700, 1000), (3000, 4096), (19100, 136)])
+@pytest.mark.parametrize("k", [1, 2, 31, 32, 33, 51, 63, 64, 65, 99, 127, 128])
+@pytest.mark.parametrize("excess,offset", [(0, 0), (1, 1), (2, 3), (3, 8)])
+def test_any_basis(n, d, k, excess, offset):
+    if k > d or (k + excess) % 8 == 0 and offset % 8 == 0:
+        pytest.skip("an aligned basis belongs to the TMA kernels")
+    X = _inside_nan(_rand((n, d), n), (d + 15) // 8 * 8, 64)
+    U = _inside_nan(_rand((d, k), k, d ** -0.5), k + excess, offset)
+    codec = Codec(synth.BF16, U)
+    expect = (X.double() @ U.double()).cpu().numpy()
+    words = torch.full((n, k + 2), -1, dtype=torch.int32, device="cuda")
+    codec.grad_project_wire(X, out=words.view(torch.float32)[:, :k])
+    assert B.ssn_last_kernel()[0] == B.SSN_KERNEL_SPLIT_PROJECT
+    assert_close(words.view(torch.float32)[:, :k].double().cpu().numpy(), expect, synth.F32, "words", tol=WORD_TOL)
+    assert (words[:, k:] == -1).all()
+    Z = codec.grad_project(X)
+    assert_close(Z.double().cpu().numpy(), expect, synth.BF16, "rows")
+    ids = torch.arange(n, dtype=torch.int32, device="cuda")
+    wire = codec.compress_wire(X, ids, with_ids=True)
+    assert torch.equal(wire[:, k], ids) and torch.equal(wire[:, :k], words[:, :k])
+    assert codec.take_status() == 0
+
+
+@pytest.mark.parametrize("n", [300, 20000])
+def test_bad_rows(n):
+    d, k = 256, 51
+    X, U = _rand((n, d), 1), _rand((d, k), 2, d ** -0.5)
+    X[0, 5], X[129, 9], X[130, 9] = float("inf"), -float("inf"), float("nan")
+    X[20] *= 1e36
+    codec = Codec(synth.BF16, U)
+    got = codec.grad_project_wire(X).double().cpu().numpy()
+    expect = (X.double() @ U.double()).cpu().numpy()
+    assert np.array_equal(np.isnan(got), np.isnan(expect))
+    assert np.array_equal(np.isinf(got), np.isinf(expect))
+    rows = np.isfinite(expect).all(axis=1)
+    scale = np.abs(expect[rows]).max(axis=1, keepdims=True)
+    assert (np.abs(got[rows] - expect[rows]) <= 1e-5 * scale).all()
+    # a bad value of the basis stays in its column
+    U[7, 3] = float("nan")
+    got = Codec(synth.BF16, U).grad_project_wire(X[200:]).cpu().numpy()
+    assert np.isnan(got[:, 3]).all() and np.isfinite(np.delete(got, 3, axis=1)).all()
