@@ -226,11 +226,14 @@ ssn_status_t ssn_weight_reproject(const ssn_codec_t *codec, void *const *W_ptrs,
  *   SSN_SIDE_LEFT : W_i is [d x extent[i]],  W_i <- U (U^T W_i)
  *   W_ptrs, extent, ldw   HOST arrays of `count` device pointers, extents (>= 1) and leading
  *                         dimensions (>= d for RIGHT, >= extent[i] for LEFT); distinct buffers.
- *   workspace   only read for SSN_SIDE_LEFT weights that the fused tensor-core kernel does not
+ *   workspace   needed for SSN_SIDE_LEFT weights that the fused tensor-core kernel does not
  *               take (fp32, k > 128, d not a multiple of 128, leading dimension not a multiple of
  *               8 elements, unaligned base): k * max(extent) * 4 bytes, 16-byte aligned; such a
  *               weight without enough workspace gives SSN_ERR_WORKSPACE (weights before it in the
- *               list have been re-projected then).  May be NULL otherwise.
+ *               list have been re-projected then).  For SSN_SIDE_RIGHT it is optional: weights that
+ *               the fused kernel does not take run on the tensor cores when it has
+ *               ssn_coords_workspace_bytes(codec, max(extent)) bytes, on the general kernel else.
+ *               Garbage afterwards.
  * Same arithmetic as ssn_weight_reproject.
  */
 ssn_status_t ssn_weight_reproject_list(const ssn_codec_t *codec, void *const *W_ptrs,
@@ -254,6 +257,18 @@ ssn_status_t ssn_weight_reproject_list(const ssn_codec_t *codec, void *const *W_
 ssn_status_t ssn_reparam_project(const ssn_codec_t *codec, const void *H, int64_t ldh, int64_t m,
                                  const void *Zw, int64_t ldzw, int64_t n_tokens, void *Y,
                                  int64_t ldy, void *coords, int64_t ldc, void *stream);
+
+/*
+ * The same with device scratch for the fp32 coordinates, 16-byte aligned, of
+ * ssn_coords_workspace_bytes(codec, n_tokens) bytes (0 for ranks that have no use for it).  It
+ * is used where the fused kernel does not take the call (fp32, leading dimension not a multiple of 8
+ * elements, unaligned base, ...), which then runs on the tensor cores; NULL or too small: the general kernel.
+ */
+size_t ssn_coords_workspace_bytes(const ssn_codec_t *codec, int64_t rows);
+ssn_status_t ssn_reparam_project_ws(const ssn_codec_t *codec, const void *H, int64_t ldh, int64_t m,
+                                    const void *Zw, int64_t ldzw, int64_t n_tokens, void *Y,
+                                    int64_t ldy, void *coords, int64_t ldc, void *workspace,
+                                    size_t workspace_bytes, void *stream);
 
 /*
  * Gradient of a reparameterized projection's factor (the chain rule stated with Eq. reparam:

@@ -75,6 +75,8 @@ _SIGNATURES = {
     "ssn_weight_reproject_left_static": (_i32, [_codec_p, _vp, _i64, _i64, _vp]),
     "ssn_prepare_tables": (_i32, [_codec_p, _vp, _i64, _vp, _i64, _vp]),
     "ssn_reparam_project": (_i32, [_codec_p, _vp, _i64, _i64, _vp, _i64, _i64, _vp, _i64, _vp, _i64, _vp]),
+    "ssn_coords_workspace_bytes": (_sz, [_codec_p, _i64]),
+    "ssn_reparam_project_ws": (_i32, [_codec_p, _vp, _i64, _i64, _vp, _i64, _i64, _vp, _i64, _vp, _i64, _vp, _sz, _vp]),
     "ssn_reparam_grad_factor": (_i32, [_codec_p, _vp, _i64, _i64, _vp, _i64, _i64, _vp, _i64, _vp, _sz, _vp]),
     "ssn_head_embed": (_i32, [_codec_p, _vp, _i64, _i64, _vp, _vp, _i64, _i32, _vp, _i64, _vp, _sz, _vp, _vp]),
     "ssn_compress_wire": (_i32, [_codec_p, _vp, _i64, _vp, _vp, _i64, _i32, _vp, _i64, _i32, _vp, _vp]),
@@ -231,6 +233,19 @@ def ssn_reparam_project(codec: ssn_codec_t, H: int, ldh: int, m: int, Zw: int, l
     _check(_lib.ssn_reparam_project(ctypes.byref(codec), H or None, ldh, m, Zw or None, ldzw, n_tokens,
                                     Y or None, ldy, coords or None, ldc, stream or None),
            "ssn_reparam_project")
+
+
+def ssn_coords_workspace_bytes(codec: ssn_codec_t, rows: int) -> int:
+    return int(_lib.ssn_coords_workspace_bytes(ctypes.byref(codec), rows))
+
+
+def ssn_reparam_project_ws(codec: ssn_codec_t, H: int, ldh: int, m: int, Zw: int, ldzw: int, n_tokens: int,
+                           Y: int, ldy: int, coords: int, ldc: int, workspace: int, workspace_bytes: int,
+                           stream: int = 0) -> None:
+    """ssn_reparam_project with scratch for the fp32 coordinates of calls that the fused kernel does not take."""
+    _check(_lib.ssn_reparam_project_ws(ctypes.byref(codec), H or None, ldh, m, Zw or None, ldzw, n_tokens, Y or None,
+                                       ldy, coords or None, ldc, workspace or None, workspace_bytes, stream or None),
+           "ssn_reparam_project_ws")
 
 
 def ssn_reparam_grad_factor(codec: ssn_codec_t, H: int, ldh: int, m: int, dY: int, lddy: int, n_tokens: int,

@@ -172,6 +172,46 @@ ssn_status_t launch_token_kernel(const TokenArgs &a, int32_t dtype, cudaStream_t
   return launch_generic_token_kernel(a, dtype, stream);
 }
 
+// Scratch for the fp32 coordinates of project_then_expand: rows on a 16-byte pitch.
+inline int64_t coords_pitch(int32_t k) { return ((int64_t)k + 3) & ~3LL; }
+inline size_t coords_bytes(int64_t rows, int32_t k) { return (size_t)rows * (size_t)coords_pitch(k) * sizeof(float); }
+
+// D = (S U) U2^T of rows the fused kernels do not take (a.src and a.dst; fp32 storage, operands off the 16-byte grid).
+// With scratch for the fp32 coordinates and a rank that the split-operand kernels take it is a projection and an expansion on
+// these, on the tensor cores; without it the general kernel.  us, general -> split: fp32 weights [2048 + 7168] x 2048 twice,
+// rank 40 1389 -> 239; bf16 ones, rank 51 packed 1482 -> 176; H [8192 x 7168] to 2048 columns, fp32 1633 -> 166.  fp32 results
+// are closer to 64-bit sums too (1.9e-7 -> 1.0e-7).
+ssn_status_t project_then_expand(const TokenArgs &a, int32_t dtype, void *scratch, size_t scratch_bytes, cudaStream_t stream) {
+  // The general kernel's time grows with the columns per pass of 32 coordinates, the two launches' hardly does: 512 rows x 64
+  // columns, rank 51 10 us against 25 (fp32), 512 columns, rank 8 22 against 19, rank 51 43 against 26, 2048 columns 184
+  // against 32; the same for 1 to 2000 rows.  Above that it grows with the rows, too.
+  const int64_t columns = a.U2 != nullptr ? ((int64_t)a.d + a.d2) / 2 : a.d;
+  const bool wide = columns * ((a.k + 31) / 32) >= 512 || a.n > 4096;
+  const bool split = wide && (a.U2 != nullptr || !mma_eligible(a, dtype)) && a.k <= kSplitMaxRank && scratch != nullptr &&
+                     aligned16(scratch) && scratch_bytes >= coords_bytes(a.n, a.k) && (a.zout == nullptr || dtype == SSN_F32);
+  if (!split) return a.U2 != nullptr ? launch_generic_token_kernel(a, dtype, stream) : launch_token_kernel(a, dtype, stream);
+  TokenArgs p = a, e = a;
+  p.dst = nullptr;
+  p.U2 = nullptr;
+  p.zout = a.zout != nullptr ? a.zout : scratch;   // fp32 coordinates that the caller asked for serve as they are
+  p.ldzout = a.zout != nullptr ? a.ldzout : coords_pitch(a.k);
+  p.wire = 1;
+  ssn_status_t st = launch_token_kernel(p, dtype, stream);
+  if (st != SSN_OK) return st;
+  e.src = nullptr;
+  e.zin = p.zout;
+  e.ldzin = p.ldzout;
+  e.zout = nullptr;
+  e.wire = 1;
+  if (a.U2 != nullptr) {
+    e.U = a.U2;
+    e.ldu = a.ldu2;
+    e.d = a.d2;
+    e.U2 = nullptr;
+  }
+  return launch_token_kernel(e, dtype, stream);
+}
+
 }  // namespace
 
 void note_kernel(int family, int variant) { g_last_kernel = family | (variant << 8); }
@@ -184,7 +224,8 @@ namespace {
 // RIGHT re-projection of `count` matrices [rows[i] x d]: groups of up to kMaxFusedMatrices go to the fused
 // tcgen05 kernel in one launch each; what that kernel does not take goes matrix by matrix.
 ssn_status_t reproject_right_list(const ssn_codec_t *codec, void *const *W_ptrs, const int64_t *rows,
-                                  const int64_t *ldw, int32_t count, cudaStream_t s) {
+                                  const int64_t *ldw, int32_t count, void *workspace, size_t workspace_bytes,
+                                  cudaStream_t s) {
   const int sms = sm_count_of_current_device();
   int32_t done = 0;
   while (done < count) {
@@ -223,7 +264,7 @@ ssn_status_t reproject_right_list(const ssn_codec_t *codec, void *const *W_ptrs,
         a.d = codec->d;
         a.k = codec->k;
         a.shift.dev_status = codec->dev_status;
-        ssn_status_t st = launch_token_kernel(a, codec->dtype, s);
+        ssn_status_t st = project_then_expand(a, codec->dtype, workspace, workspace_bytes, s);
         if (st != SSN_OK) return st;
       }
     }
@@ -698,6 +739,17 @@ ssn_status_t ssn_decompress_wire(const ssn_codec_t *codec, const void *wire, int
 ssn_status_t ssn_reparam_project(const ssn_codec_t *codec, const void *H, int64_t ldh, int64_t m,
                                  const void *Zw, int64_t ldzw, int64_t n_tokens, void *Y,
                                  int64_t ldy, void *coords, int64_t ldc, void *stream) {
+  return ssn_reparam_project_ws(codec, H, ldh, m, Zw, ldzw, n_tokens, Y, ldy, coords, ldc, nullptr, 0, stream);
+}
+
+size_t ssn_coords_workspace_bytes(const ssn_codec_t *codec, int64_t rows) {
+  return check_codec(codec) != SSN_OK || rows < 1 || codec->k > kSplitMaxRank ? 0 : coords_bytes(rows, codec->k);
+}
+
+ssn_status_t ssn_reparam_project_ws(const ssn_codec_t *codec, const void *H, int64_t ldh, int64_t m,
+                                    const void *Zw, int64_t ldzw, int64_t n_tokens, void *Y,
+                                    int64_t ldy, void *coords, int64_t ldc, void *workspace,
+                                    size_t workspace_bytes, void *stream) {
   ssn_status_t st = check_codec(codec);
   if (st != SSN_OK) return st;
   if (n_tokens < 0 || m < 1 || m > 0x7fffffffLL || ldh < m || ldzw < codec->k || ldy < codec->d) return SSN_ERR_SHAPE;
@@ -728,8 +780,7 @@ ssn_status_t ssn_reparam_project(const ssn_codec_t *codec, const void *H, int64_
     }
     if (e != cudaErrorNotSupported) return SSN_ERR_CUDA;
   }
-  // general path: one launch of the general kernel, the coordinates stay in fp32 in shared memory
-  TokenArgs p{};
+  TokenArgs p{};      // the coordinates stay in fp32, in the workspace or in shared memory
   p.src = H;
   p.lds = ldh;
   p.zout = coords;
@@ -744,7 +795,8 @@ ssn_status_t ssn_reparam_project(const ssn_codec_t *codec, const void *H, int64_
   p.d2 = codec->d;
   p.n = n_tokens;
   p.k = codec->k;
-  return launch_generic_token_kernel(p, codec->dtype, s);
+  p.shift.dev_status = codec->dev_status;
+  return project_then_expand(p, codec->dtype, workspace, workspace_bytes, s);
 }
 
 ssn_status_t ssn_reparam_grad_factor(const ssn_codec_t *codec, const void *H, int64_t ldh, int64_t m,
@@ -876,7 +928,7 @@ ssn_status_t ssn_weight_reproject_list(const ssn_codec_t *codec, void *const *W_
     if (extent[b] < 1 || ldw[b] < (side == SSN_SIDE_RIGHT ? (int64_t)codec->d : extent[b])) return SSN_ERR_SHAPE;
   }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (side == SSN_SIDE_RIGHT) return reproject_right_list(codec, W_ptrs, extent, ldw, count, s);
+  if (side == SSN_SIDE_RIGHT) return reproject_right_list(codec, W_ptrs, extent, ldw, count, workspace, workspace_bytes, s);
   return reproject_left_list(codec, W_ptrs, extent, ldw, count, workspace, workspace_bytes, s);
 }
 
@@ -898,7 +950,7 @@ ssn_status_t ssn_weight_reproject(const ssn_codec_t *codec, void *const *W_ptrs,
 
   if (side == SSN_SIDE_RIGHT) {
     std::vector<int64_t> nrows((size_t)batch, rows), lds((size_t)batch, ldw);
-    return reproject_right_list(codec, W_ptrs, nrows.data(), lds.data(), batch, s);
+    return reproject_right_list(codec, W_ptrs, nrows.data(), lds.data(), batch, workspace, workspace_bytes, s);
   }
 
   std::vector<int64_t> ncols((size_t)batch, cols), lds((size_t)batch, ldw);

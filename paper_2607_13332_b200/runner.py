@@ -214,6 +214,15 @@ class Codec:
                                     self.dev_status.data_ptr(), _stream())
         return Xh
 
+    def _fetchable(self, *matrices: torch.Tensor) -> bool:
+        """Whether TMA can fetch the basis and these matrices: what the fused kernels take needs no scratch."""
+        return self.dtype == synth.BF16 and all(t.data_ptr() % 16 == 0 and _ld(t) % 8 == 0 for t in (self.U, *matrices))
+
+    def _coords_workspace(self, rows: int) -> Optional[torch.Tensor]:
+        """Scratch for the fp32 coordinates of `rows` rows."""
+        nbytes = binding.ssn_coords_workspace_bytes(self.c, rows)
+        return torch.empty(nbytes, dtype=torch.uint8, device=self.U.device) if nbytes else None
+
     def reproject_workspace(self, rows: int, cols: int, side: str, batch: int) -> Optional[torch.Tensor]:
         nbytes = binding.ssn_weight_reproject_workspace_bytes(self.c, rows, cols, binding.SIDES[side], batch)
         if nbytes == 0:
@@ -225,9 +234,11 @@ class Codec:
         """Y = (H Zw) U^T for a projection stored as its factor Zw [m, k] (Eq. reparam)."""
         n, m = H.shape
         Y = out if out is not None else self._empty(n, self.d)
-        binding.ssn_reparam_project(self.c, H.data_ptr(), _ld(H), m, Zw.data_ptr(), _ld(Zw), n, Y.data_ptr(),
-                                    _ld(Y), coords.data_ptr() if coords is not None else 0,
-                                    _ld(coords) if coords is not None else 0, _stream())
+        ws = None if self._fetchable(H, Zw, Y) else self._coords_workspace(n)
+        binding.ssn_reparam_project_ws(self.c, H.data_ptr(), _ld(H), m, Zw.data_ptr(), _ld(Zw), n, Y.data_ptr(),
+                                       _ld(Y), coords.data_ptr() if coords is not None else 0,
+                                       _ld(coords) if coords is not None else 0,
+                                       ws.data_ptr() if ws is not None else 0, ws.numel() if ws is not None else 0, _stream())
         return Y
 
     def reparam_grad_factor(self, H: torch.Tensor, dY: torch.Tensor) -> torch.Tensor:
@@ -263,6 +274,8 @@ class Codec:
         if side == "left" and workspace is None:
             workspace = torch.empty(self.k * max(w.shape[1] for w in weights) * 4, dtype=torch.uint8,
                                     device=self.U.device)
+        if side == "right" and workspace is None and not self._fetchable(*weights):
+            workspace = self._coords_workspace(max(w.shape[0] for w in weights))
         binding.ssn_weight_reproject_list(self.c, [w.data_ptr() for w in weights],
                                           [w.shape[axis] for w in weights], [_ld(w) for w in weights],
                                           binding.SIDES[side],
@@ -284,6 +297,8 @@ class Codec:
                 raise ValueError("weights of one call must share shape and leading dimension")
         if workspace is None:
             workspace = self.reproject_workspace(rows, cols, side, len(weights))
+        if side == "right" and workspace is None and not self._fetchable(*weights):
+            workspace = self._coords_workspace(rows)
         binding.ssn_weight_reproject(self.c, [w.data_ptr() for w in weights], rows, cols, ldw,
                                      binding.SIDES[side],
                                      workspace.data_ptr() if workspace is not None else 0,

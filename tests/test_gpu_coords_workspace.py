@@ -1,0 +1,63 @@
+"""Project-then-expand of rows the fused kernel does not take (fp32 storage, operands off the 16-byte grid), through
+fp32 coordinates in scratch: edges of the 128-row tiles and 128-column chunks, both rank groups, with and without the
+coordinates as an output, and the general kernel where there is no scratch."""
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import ssn_oracle as oracle
+from paper_2607_13332_b200 import binding as B
+from paper_2607_13332_b200 import synth
+from tests.harness import Codec, assert_close, f64, guards_intact, host64, padded, to_device
+
+pytestmark = pytest.mark.gpu
+
+SPLIT = (B.SSN_KERNEL_SPLIT_PROJECT, B.SSN_KERNEL_SPLIT_EXPAND)
+
+
+def _rand(rng, shape, dt, std=1.0):
+    return synth.to_storage(rng.standard_normal(shape) * std, dt)
+
+
+@pytest.mark.parametrize("dt", [synth.F32, synth.BF16])
+@pytest.mark.parametrize("d,k,rows", [(130, 7, (300,)), (130, 7, (5000,)), (520, 7, (1, 127, 300)), (256, 51, (128, 129)), (384, 99, (700,)), (2048, 128, (513, 64))])
+@pytest.mark.parametrize("scratch", [True, False])
+def test_reprojection_of_rows(d, k, rows, dt, scratch):
+    rng = np.random.default_rng(d + k)
+    U0 = synth.to_storage(np.linalg.qr(rng.standard_normal((d, k)))[0], dt)
+    W0 = [_rand(rng, (r, d), dt, 0.02) for r in rows]
+    U, _ = padded(d, k, k + 1, dt, fill=to_device(U0, dt))       # off the 16-byte grid
+    pairs = [padded(r, d, d + 3, dt, fill=to_device(w, dt)) for r, w in zip(rows, W0)]
+    codec = Codec(dt, U)
+    short = torch.empty(16, dtype=torch.uint8, device="cuda")    # too small to be of use
+    codec.weight_reproject_list([w for w, _ in pairs], "right", workspace=None if scratch else short)
+    # narrow rows, and calls without scratch, are the general kernel's
+    assert (B.ssn_last_kernel()[0] in SPLIT) == (scratch and (d, rows) != (130, (300,)))
+    for (w, buf), w0 in zip(pairs, W0):
+        assert_close(host64(w, dt), oracle.weight_reproject(f64(w0, dt), f64(U0, dt), "right"), dt, "reproject")
+        assert guards_intact(w, buf, dt)
+    assert codec.take_status() == 0
+
+
+@pytest.mark.parametrize("dt", [synth.F32, synth.BF16])
+@pytest.mark.parametrize("n,m,d,k", [(1, 1000, 130, 5), (129, 320, 256, 51), (700, 130, 1100, 100), (3000, 512, 640, 17)])
+@pytest.mark.parametrize("coords", [False, True])
+def test_reparameterised_projection(n, m, d, k, dt, coords):
+    rng = np.random.default_rng(n + m)
+    H0, Zw0 = _rand(rng, (n, m), dt), _rand(rng, (m, k), dt, 0.02)
+    U0 = synth.to_storage(np.linalg.qr(rng.standard_normal((d, k)))[0], dt)
+    Zw, _ = padded(m, k, k + 1, dt, fill=to_device(Zw0, dt))
+    out, buf = padded(n, d, d + 1, dt)
+    C, cbuf = padded(n, k, k + 1, dt) if coords else (None, None)
+    codec = Codec(dt, to_device(U0, dt))
+    codec.reparam_project(to_device(H0, dt), Zw, out=out, coords=C)
+    # bf16 coordinates as an output are the general kernel's
+    assert (B.ssn_last_kernel()[0] in SPLIT) == (dt == synth.F32 or not coords)
+    H, Z, U = f64(H0, dt), f64(Zw0, dt), f64(U0, dt)
+    assert_close(host64(out, dt), oracle.reparam_project(H, Z, U), dt, "Y")
+    assert guards_intact(out, buf, dt)
+    if coords:
+        assert_close(host64(C, dt), H @ Z, dt, "coordinates")
+        assert guards_intact(C, cbuf, dt)
+    assert codec.take_status() == 0
