@@ -582,6 +582,9 @@ __global__ void __launch_bounds__((SplitProjectConfig<T, KN, NSLOT, CAREFUL>::kT
                                      : row * 128 + ((unit ^ (row & 7)) << 4);   // + 64 rows: the second piece
     for (int step = 0; step < steps; ++step) {
       cp_async_wait<RD - 2>();
+      // Into the slot read in the step before: at once where the next step is the only one ahead (bf16, three operands or
+      // more: 152 -> 141 us for X, R and E rows of 12288 x 5120), else after this step's work (fp32 E and P: 53 against 55).
+      if (RD == 2) advance_rows(step + RD - 1 < steps);
       const int next_st = st + 1 == nloc ? 0 : st + 1;
       uint4 x[2], w[NSLOT > 0 ? NSLOT : 1][2];
       const uint32_t src = raw0 + (uint32_t)rslot * Cfg::kRawStepBytes + raw_off;
@@ -656,7 +659,7 @@ __global__ void __launch_bounds__((SplitProjectConfig<T, KN, NSLOT, CAREFUL>::kT
       __syncwarp();
       if (lane == 0) mbar_arrive(full_bar(slot));
       if (step + 1 < steps) issue_u(next_st);
-      advance_rows(step + RD - 1 < steps);   // into the slot read in the step before
+      if (RD > 2) advance_rows(step + RD - 1 < steps);
       if (++slot == S) {
         slot = 0;
         parity ^= 1u;
