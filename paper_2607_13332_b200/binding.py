@@ -312,6 +312,16 @@ def ssn_prepare_tables(codec: ssn_codec_t, EU: int, ldeu: int, PU: int, ldpu: in
                                    stream or None), "ssn_prepare_tables")
 
 
+def library() -> ctypes.CDLL:
+    """The loaded library: its functions return the status instead of raising; 0 is NULL."""
+    return _lib
+
+
+def reference(codec: ssn_codec_t):
+    """A prepared reference to the codec; what is changed in the codec later is seen through it."""
+    return ctypes.byref(codec)
+
+
 def raw(name: str):
     """The raw ctypes function (returns the status instead of raising); used by error tests."""
     return getattr(_lib, name)
