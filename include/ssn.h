@@ -208,7 +208,8 @@ ssn_status_t ssn_grad_project(const ssn_codec_t *codec, const void *G, int64_t l
  *            dimension ldw >= cols; the weights must be distinct buffers.
  *   workspace  device scratch of at least ssn_weight_reproject_workspace_bytes(...) bytes,
  *              16-byte aligned; may be NULL only when that size is 0.  Its contents are
- *              garbage afterwards; calls that share it must be ordered on one stream.
+ *              garbage afterwards; calls that share it must be ordered on one stream.  For
+ *              SSN_SIDE_RIGHT it is optional, as in ssn_weight_reproject_list.
  * The k coordinates are kept in fp32 between the two products.
  */
 size_t ssn_weight_reproject_workspace_bytes(const ssn_codec_t *codec, int64_t rows,
@@ -421,7 +422,7 @@ enum {
   SSN_KERNEL_UMMA_EXPAND = 6,      /* tcgen05 + TMA expansion                                  */
   SSN_KERNEL_UMMA_ROUNDTRIP = 7,   /* tcgen05 + TMA project-then-expand                        */
   SSN_KERNEL_UMMA_TOKENS = 8,      /* tcgen05 + TMA contraction over tokens                    */
-  SSN_KERNEL_SPLIT_PROJECT = 9,    /* tcgen05 projection, operands split into bf16 parts: fp32 and
+  SSN_KERNEL_SPLIT_PROJECT = 9,    /* tcgen05 projection, operands split into bf16 parts where they need it: fp32 and
                                       the bf16 calls TMA cannot fetch                          */
   SSN_KERNEL_SPLIT_EXPAND = 10     /* the same for the expansion                               */
 };
