@@ -111,6 +111,16 @@ cudaError_t launch_slots(const SplitProjectArgs &a, int slots, int sms, cudaStre
   return launch_rank<T, 3>(a, sms, s);
 }
 
+// Above rank 32 the first and last rows of the basis, fetched half a word at a time, cost the plain kernel 3 us that wide rows
+// or many of them have to earn.  us, split -> plain: rank 51 1500 x 512 10.7 -> 13.8, x 1024 12.5 -> 14.4, x 2048
+// 15.8 -> 15.7, x 4096 20.0 -> 18.4; 9000 x 1024 20.9 -> 21.6, 16000 x 1024 34.9 -> 30.7, x 512 24.2 -> 25.3; rank 99 1500 x 2048
+// 18.5 -> 19.3, 3000 x 2048 30.5 -> 26.7.  Rank 27: 600 x 512 9.7 -> 9.8, 1500 x 1024 11.5 -> 10.3, 9000 x 4096 41 -> 27.
+bool plain_pays(const SplitProjectArgs &a) {
+  if (a.k <= 32) return true;
+  if (a.d >= 2048 && (a.k <= 64 || a.n >= 2048)) return true;
+  return a.d >= 1024 && a.n * a.d >= 16000LL * 1024;
+}
+
 bool rows16(const void *p, int64_t ld, int esz) {
   return (reinterpret_cast<uintptr_t>(p) & 15) == 0 && (ld * esz) % 16 == 0;
 }
@@ -148,7 +158,7 @@ cudaError_t launch_codec_split_project(const TokenArgs &a, int32_t dtype, int sm
   // four coordinates are 16 bytes of words or 8 bytes of bf16
   p.vec_out = (a.ldzout & 3) == 0 && (reinterpret_cast<uintptr_t>(a.zout) & (a.wire || dtype == SSN_F32 ? 15 : 7)) == 0;
   const int slots = (a.src2 != nullptr) + p.has_e + p.has_p;
-  if (dtype == SSN_BF16 && slots == 0 && rows16(a.src, a.lds, esz)) {   // rows that TMA can fetch, and nothing to add to them
+  if (dtype == SSN_BF16 && slots == 0 && rows16(a.src, a.lds, esz) && plain_pays(p)) {   // rows that TMA can fetch, and nothing to add
     CUtensorMap x;
     if (make_sw128_map(&x, a.src, a.n, a.d, a.lds, kUmmaTile))
       return a.k <= 32 ? launch_plain<32>(p, x, sm_count, stream) : launch_plain<64>(p, x, sm_count, stream);

@@ -31,7 +31,7 @@ def _inside_nan(t, pitch, offset):
     return view
 
 
-@pytest.mark.parametrize("n,d", [(1, 64), (127, 72), (128, 128), (129, 200), (700, 1000), (3000, 4096), (19100, 136)])
+@pytest.mark.parametrize("n,d", [(1, 64), (127, 72), (128, 128), (129, 200), (700, 1000), (3000, 4096), (1, 2056), (2100, 2056), (19100, 136)])
 @pytest.mark.parametrize("k", [1, 2, 31, 32, 33, 51, 63, 64, 65, 99, 127, 128])
 @pytest.mark.parametrize("excess,offset", [(0, 0), (1, 1), (2, 3), (3, 8)])
 def test_any_basis(n, d, k, excess, offset):
