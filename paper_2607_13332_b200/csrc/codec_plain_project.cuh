@@ -17,6 +17,9 @@
 // Before -> now, us: 12288 x 5120, rank 51, fp32 words 104 -> 67; 40000 x 1536, rank 27, bf16 rows 87 -> 50; 700 x 1024,
 // rank 19 11.3 -> 10.2.
 //
+// CAREFUL (see kSplitCarefulCols) adds the four accumulators one by one, with compensation: the same sums as the split kernel's.
+// 20000 x 320, rank 32: 4.1e-8 from 64-bit sums instead of 5.3e-8, 13.0 us instead of 12.0 (the split kernel 21).
+//
 // Clusters and halves as in the split kernel.  Every wait is bounded; one that runs out sets SSN_DEV_TIMEOUT and the
 // kernel still runs to its end.
 #pragma once
@@ -39,7 +42,7 @@ struct PlainProjectConfig {
   static_assert(kAccs == 4 && kBufs % 2 == 0, "two issuers take turns with the sets of accumulators");
   static constexpr int kSums = KN / 2;                        // coordinates of one row per thread
   static constexpr int kRingBytes = kStagesN * kStageBytes;
-  static_assert(kRingBytes >= kUmmaTile * (KN + 4) * 4, "the exchanged sums take the place of the ring");
+  static_assert(kRingBytes >= 2 * kUmmaTile * (KN + 4) * 4, "the exchanged sums take the place of the ring");
   static constexpr int kBars = 2 * kStagesN + 2 * kBufs;
   static constexpr int kSmemBytes = 1024 + kRingBytes + kBars * 8 + 16;
   static_assert(kSmemBytes <= 227 * 1024, "the ring does not fit in shared memory");
@@ -121,7 +124,7 @@ struct BasisPairs {
   }
 };
 
-template <int KN>
+template <int KN, bool CAREFUL>
 __global__ void __launch_bounds__(kPlainThreads, 1)
 codec_plain_project_kernel(const SplitProjectArgs a, const __grid_constant__ CUtensorMap x_map) {
   using Cfg = PlainProjectConfig<KN>;
@@ -282,6 +285,13 @@ codec_plain_project_kernel(const SplitProjectArgs a, const __grid_constant__ CUt
           const int i = h / 2 * 8;
 #pragma unroll
           for (int e = 0; e < 8; e += 2) {
+            if constexpr (CAREFUL) {
+#pragma unroll
+              for (int q = 0; q < 2; ++q)
+                add_compensated2(sum[i + e], sum[i + e + 1], comp[i + e], comp[i + e + 1], __uint_as_float(v[h & 1][q][e]),
+                                 __uint_as_float(v[h & 1][q][e + 1]));
+              continue;
+            }
             float y0 = __uint_as_float(v[h & 1][0][e]), y1 = __uint_as_float(v[h & 1][0][e + 1]);
             add2(y0, y1, __uint_as_float(v[h & 1][1][e]), __uint_as_float(v[h & 1][1][e + 1]));
             if ((h & 1) == 0) {
@@ -322,13 +332,17 @@ codec_plain_project_kernel(const SplitProjectArgs a, const __grid_constant__ CUt
     if (s.cluster_size > 1) {   // the last accumulators are complete, so every stage is consumed: the ring carries the sums
       const uint32_t dst = smem0 + (uint32_t)(row * (KN + 4) + col0) * 4;
 #pragma unroll
-      for (int c = 0; c < Cfg::kSums; c += 4)
+      for (int c = 0; c < Cfg::kSums; c += 4) {
         st_shared_v4(dst + c * 4, __float_as_uint(sum[c]), __float_as_uint(sum[c + 1]), __float_as_uint(sum[c + 2]),
                      __float_as_uint(sum[c + 3]));
+        if (!CAREFUL && s.cluster_size <= kFewSlices)
+          st_shared_v4(dst + kUmmaTile * (KN + 4) * 4 + c * 4, __float_as_uint(comp[c]), __float_as_uint(comp[c + 1]),
+                       __float_as_uint(comp[c + 2]), __float_as_uint(comp[c + 3]));
+      }
     }
   }
 
-  if (s.cluster_size > 1) finish_slices<T, KN, kPlainThreads, false>(a, s, smem0, 0, 0);
+  if (s.cluster_size > 1) finish_slices<T, KN, kPlainThreads, false, !CAREFUL>(a, s, smem0, 0, 0);
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   __syncthreads();
   if (warp == 1) {

@@ -84,14 +84,21 @@ int plain_cluster_of(const SplitProjectArgs &a, int nst, int sms) {
   return best;
 }
 
-template <int KN>
-cudaError_t launch_plain(const SplitProjectArgs &a, const CUtensorMap &x, int sms, cudaStream_t stream) {
-  auto kernel = codec_plain_project_kernel<KN>;
+template <int KN, bool CAREFUL>
+cudaError_t launch_plain(const SplitProjectArgs &a, const CUtensorMap &x, int c, int sms, cudaStream_t stream) {
+  auto kernel = codec_plain_project_kernel<KN, CAREFUL>;
   constexpr int smem = PlainProjectConfig<KN>::kSmemBytes;
   static std::atomic<uint64_t> configured{0};
   const cudaError_t e = allow_dynamic_smem(kernel, smem, configured);
   if (e != cudaSuccess) return e;
-  return launch_slices(kernel, kPlainThreads, smem, a, plain_cluster_of(a, (a.d + kUmmaCols - 1) / kUmmaCols, sms), sms, stream, x);
+  return launch_slices(kernel, kPlainThreads, smem, a, c, sms, stream, x);
+}
+
+cudaError_t launch_plain_rank(const SplitProjectArgs &a, const CUtensorMap &x, int sms, cudaStream_t s) {
+  const int nst = (a.d + kUmmaCols - 1) / kUmmaCols, c = plain_cluster_of(a, nst, sms);
+  const bool careful = (nst + c - 1) / c * kUmmaCols < kSplitCarefulColsPlain;
+  if (a.k <= 32) return careful ? launch_plain<32, true>(a, x, c, sms, s) : launch_plain<32, false>(a, x, c, sms, s);
+  return careful ? launch_plain<64, true>(a, x, c, sms, s) : launch_plain<64, false>(a, x, c, sms, s);
 }
 
 template <typename T, int NSLOT>
@@ -161,7 +168,7 @@ cudaError_t launch_codec_split_project(const TokenArgs &a, int32_t dtype, int sm
   if (dtype == SSN_BF16 && slots == 0 && rows16(a.src, a.lds, esz) && plain_pays(p)) {   // rows that TMA can fetch, and nothing to add
     CUtensorMap x;
     if (make_sw128_map(&x, a.src, a.n, a.d, a.lds, kUmmaTile))
-      return a.k <= 32 ? launch_plain<32>(p, x, sm_count, stream) : launch_plain<64>(p, x, sm_count, stream);
+      return launch_plain_rank(p, x, sm_count, stream);
   }
   return dtype == SSN_F32 ? launch_slots<float>(p, slots, sm_count, stream)
                           : launch_slots<__nv_bfloat16>(p, slots, sm_count, stream);

@@ -168,6 +168,11 @@ __device__ __noinline__ void store_plain_coords4(const SplitProjectArgs &a, int6
   store_coords4<T>(a, t, j, j_end, {(float)acc[0], (float)acc[1], (float)acc[2], (float)acc[3]});
 }
 
+// Clusters of few CTAs pass on the compensations as well: the rounding of a slice's sum shows where the slices are few.  Rows
+// of the subspace, error against 64-bit sums without and with: 20000 x 4096 in three slices 3.4e-8, 3.2e-8; 3000 x 5120,
+// rank 99 in two 3.8e-8, 3.0e-8.  Eight slices err by 3.1e-8 without.  It takes 1 us (3000 x 2048, rank 51 in four 17.2 -> 18.2).
+constexpr uint32_t kFewSlices = 4;
+
 // What a CTA of a launch with a.halves halves computes: its tiles, columns of d and coordinates.
 struct SplitSchedule {
   uint32_t cluster_size, cta_rank;
@@ -208,7 +213,8 @@ __device__ __forceinline__ void add_compensated2(float &s0, float &s1, float &c0
 
 // The CTAs of a cluster have left their sums [128][KN + 4] at smem0; each adds up, and stores, its share of the rows.
 // FLAGS: beside them lie the largest magnitudes per column of U and, per row, whether the split does not hold it.
-template <typename T, int KN, int THREADS, bool FLAGS>
+// COMP: in clusters of up to kFewSlices, behind them lie the compensations of the sums, [128][KN + 4] too.
+template <typename T, int KN, int THREADS, bool FLAGS, bool COMP>
 __device__ __forceinline__ void finish_slices(const SplitProjectArgs &a, const SplitSchedule &s, uint32_t smem0, uint32_t u_largest_addr,
                                               uint32_t row_flags_addr) {
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
@@ -222,26 +228,53 @@ __device__ __forceinline__ void finish_slices(const SplitProjectArgs &a, const S
     const int rr = row0 + i / (KN / 4), j = 4 * (i % (KN / 4));
     const int64_t t = s.group * kUmmaTile + rr;
     if (t >= a.n || j >= s.rank()) continue;
-    // up to eight slices of the sum in 64 bits: in fp32 their additions alone would err by 4e-8
-    double z[4] = {0.0, 0.0, 0.0, 0.0};
+    float v[4] = {0.f, 0.f, 0.f, 0.f};
     uint32_t largest[4] = {0, 0, 0, 0}, bad_row = 0;
-    for (uint32_t rk = 0; rk < s.cluster_size; ++rk) {
-      float w0, w1, w2, w3;
+    auto slice = [&](int row, uint32_t rk, float (&w)[4]) {
       asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];\n"
-                   : "=f"(w0), "=f"(w1), "=f"(w2), "=f"(w3)
-                   : "r"(peer(smem0 + (uint32_t)(rr * (KN + 4) + j) * 4, rk)));
-      z[0] += w0; z[1] += w1; z[2] += w2; z[3] += w3;
-      if (FLAGS) {
-        uint32_t m0, m1, m2, m3, f;
-        asm volatile("ld.shared::cluster.v4.u32 {%0,%1,%2,%3}, [%4];\n"
-                     : "=r"(m0), "=r"(m1), "=r"(m2), "=r"(m3) : "r"(peer(u_largest_addr + j * 4, rk)));
-        largest[0] = max(largest[0], m0); largest[1] = max(largest[1], m1);
-        largest[2] = max(largest[2], m2); largest[3] = max(largest[3], m3);
-        asm volatile("ld.shared::cluster.u8 %0, [%1];\n" : "=r"(f) : "r"(peer(row_flags_addr + rr, rk)));
-        bad_row |= f;
+                   : "=f"(w[0]), "=f"(w[1]), "=f"(w[2]), "=f"(w[3])
+                   : "r"(peer(smem0 + (uint32_t)(row * (KN + 4) + j) * 4, rk)));
+    };
+    if (COMP && s.cluster_size <= kFewSlices) {
+      // sums and compensations, all on their way at a time, the rounding of each addition kept with the latter
+      float w[kFewSlices][4], c[kFewSlices][4], rest[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (uint32_t rk = 0; rk < kFewSlices; ++rk)
+        if (rk < s.cluster_size) {
+          slice(rr, rk, w[rk]);
+          slice(kUmmaTile + rr, rk, c[rk]);
+        }
+#pragma unroll
+      for (uint32_t rk = 0; rk < kFewSlices; ++rk)
+        if (rk < s.cluster_size) {
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const float t = v[e] + w[rk][e], b = t - v[e];
+            rest[e] += ((v[e] - (t - b)) + (w[rk][e] - b)) - c[rk][e];
+            v[e] = t;
+          }
+        }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) v[e] += rest[e];
+    } else {
+      // up to eight slices of the sum in 64 bits: in fp32 their additions alone would err by 4e-8
+      double z[4] = {0.0, 0.0, 0.0, 0.0};
+      for (uint32_t rk = 0; rk < s.cluster_size; ++rk) {
+        float w[4];
+        slice(rr, rk, w);
+        z[0] += w[0]; z[1] += w[1]; z[2] += w[2]; z[3] += w[3];
+        if (FLAGS) {
+          uint32_t m0, m1, m2, m3, f;
+          asm volatile("ld.shared::cluster.v4.u32 {%0,%1,%2,%3}, [%4];\n"
+                       : "=r"(m0), "=r"(m1), "=r"(m2), "=r"(m3) : "r"(peer(u_largest_addr + j * 4, rk)));
+          largest[0] = max(largest[0], m0); largest[1] = max(largest[1], m1);
+          largest[2] = max(largest[2], m2); largest[3] = max(largest[3], m3);
+          asm volatile("ld.shared::cluster.u8 %0, [%1];\n" : "=r"(f) : "r"(peer(row_flags_addr + rr, rk)));
+          bad_row |= f;
+        }
       }
+      v[0] = (float)z[0]; v[1] = (float)z[1]; v[2] = (float)z[2]; v[3] = (float)z[3];
     }
-    const float v[4] = {(float)z[0], (float)z[1], (float)z[2], (float)z[3]};
     store_coords4<T>(a, t, s.j_lo() + j, s.j_end(), v);
     if (bad_row != 0 || !sums_stand(v, FLAGS && sizeof(T) == 4 ? largest : nullptr)) store_plain_coords4<T>(a, t, s.j_lo() + j, s.j_end());
     if (a.wire_ids && j == 0 && !s.lower()) static_cast<int32_t *>(a.zout)[t * a.ldzout + a.k] = a.shift.ids[t];
@@ -693,7 +726,7 @@ __global__ void __launch_bounds__((SplitProjectConfig<T, KN, NSLOT, CAREFUL>::kT
         st_shared_v4(dst + c * 4, __float_as_uint(sum[c]), __float_as_uint(sum[c + 1]), __float_as_uint(sum[c + 2]),
                      __float_as_uint(sum[c + 3]));
     }
-    finish_slices<T, KN, Cfg::kThreads, NX == 3>(a, sched, smem0, smem_u32(u_largest), smem_u32(const_cast<unsigned char *>(row_flags)));
+    finish_slices<T, KN, Cfg::kThreads, NX == 3, false>(a, sched, smem0, smem_u32(u_largest), smem_u32(const_cast<unsigned char *>(row_flags)));
   }
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   __syncthreads();
