@@ -36,19 +36,20 @@ template <int KN>
 struct PlainProjectConfig {
   static_assert(KN == 32 || KN == 64, "coordinates, rounded up");
   static constexpr int kXBytes = kUmmaTile * 128, kUBytes = kUmmaCols * 128, kStageBytes = kXBytes + kUBytes;
-  static constexpr int kStagesN = 9;
+  static constexpr int kStagesN = 8;
   static constexpr int kAccs = kUmmaCols / 16;                // one accumulator per K step of a stage
   static constexpr int kAccCols = kAccs * KN, kBufs = 512 / kAccCols, kTmemCols = 512;
-  static_assert(kAccs == 4 && kBufs % 2 == 0, "two issuers take turns with the sets of accumulators");
+  static_assert(kAccs == 4, "the sums add up four accumulators per stage");
   static constexpr int kSums = KN / 2;                        // coordinates of one row per thread
   static constexpr int kRingBytes = kStagesN * kStageBytes;
   static_assert(kRingBytes >= 2 * kUmmaTile * (KN + 4) * 4, "the exchanged sums take the place of the ring");
   static constexpr int kBars = 2 * kStagesN + 2 * kBufs;
   static constexpr int kSmemBytes = 1024 + kRingBytes + kBars * 8 + 16;
   static_assert(kSmemBytes <= 227 * 1024, "the ring does not fit in shared memory");
-  // A basis warp waits for the release of stage i - S having seen that of stage i - S - kPlainBasisWarps, which must
-  // come after that of stage i - 2 S: a parity tells only the current phase from the one before it.
-  static_assert(kStagesN > kPlainBasisWarps, "a wait of the basis warps would span two phases");
+  // A parity tells only the current phase of a barrier from the one before it, so whoever waits has to see every phase.  Stage i
+  // belongs to issuer i % 2 and basis warp i % 4; with these numbers a slot, or a set of accumulators, keeps its owners, and
+  // an owner waits for each of its phases in turn.
+  static_assert(kStagesN % kPlainBasisWarps == 0 && kStagesN % 2 == 0 && kBufs % 2 == 0, "a wait would span two phases");
 };
 
 // 64 rows of a bf16 U, at any address and pitch, as a swizzled MN-major operand: one warp, a 4-byte word per lane and row,
@@ -199,28 +200,27 @@ codec_plain_project_kernel(const SplitProjectArgs a, const __grid_constant__ CUt
     if (lane == 0) {
       constexpr uint32_t idesc = umma_idesc(KN, false);
       const uint64_t adesc0 = umma_desc(0, 16, 1024, 2), bdesc0 = umma_desc(0, Cfg::kUBytes, 1024, 2);
-      int slot = 0, buf = 0;
+      int slot = warp - 1, buf = warp - 1;
       uint32_t parity = 0, acc_parity = 1;
-      for (int step = 0; step < steps; ++step) {
-        // every stage's barrier, the partner's too: a parity tells only the current phase from the one before it
+      for (int step = warp - 1; step < steps; step += 2) {
         if (!dead && !mbar_wait(full_bar(slot), parity)) timed_out();
-        if ((step & 1) == warp - 1) {                 // this thread's stage, and accumulators
-          if (!dead && !mbar_wait(acc_empty_bar(buf), acc_parity)) timed_out();
-          const uint32_t acc = tmem_base + (uint32_t)buf * Cfg::kAccCols;
-          asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-          const uint32_t base = smem0 + (uint32_t)slot * Cfg::kStageBytes;
-          const uint64_t ad = adesc0 + umma_desc_addr(base), bd = bdesc0 + umma_desc_addr(base + Cfg::kXBytes);
+        if (!dead && !mbar_wait(acc_empty_bar(buf), acc_parity)) timed_out();
+        const uint32_t acc = tmem_base + (uint32_t)buf * Cfg::kAccCols;
+        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+        const uint32_t base = smem0 + (uint32_t)slot * Cfg::kStageBytes;
+        const uint64_t ad = adesc0 + umma_desc_addr(base), bd = bdesc0 + umma_desc_addr(base + Cfg::kXBytes);
 #pragma unroll
-          for (int j = 0; j < Cfg::kAccs; ++j) umma_bf16(acc + (uint32_t)j * KN, ad + j * 2, bd + j * 128, idesc, 0u);
-          umma_commit(empty_bar(slot));
-          umma_commit(acc_full_bar(buf));
-        }
-        if (++slot == S) {
-          slot = 0;
+        for (int j = 0; j < Cfg::kAccs; ++j) umma_bf16(acc + (uint32_t)j * KN, ad + j * 2, bd + j * 128, idesc, 0u);
+        umma_commit(empty_bar(slot));
+        umma_commit(acc_full_bar(buf));
+        slot += 2;
+        if (slot >= S) {
+          slot -= S;
           parity ^= 1u;
         }
-        if (++buf == Cfg::kBufs) {
-          buf = 0;
+        buf += 2;
+        if (buf >= Cfg::kBufs) {
+          buf -= Cfg::kBufs;
           acc_parity ^= 1u;
         }
       }
