@@ -268,6 +268,8 @@ struct UmmaProjectConfig {
   static constexpr int kXIssuers = (!HAS_E || (kN <= 64 && !HAS_P)) ? 2 : 1;
   static constexpr int kEIssuers = HAS_E ? kXIssuers : 0;
   static constexpr int kIssuers = kXIssuers + kEIssuers + (HAS_P ? 1 : 0);
+  // What frees a stage: a commit per operand, and an arrival of the thread whose turn it is not where two take turns.
+  static constexpr int kFrees = kATiles + (kXIssuers == 2 ? 1 : 0) + (kEIssuers == 2 ? 1 : 0);
   // Warps: 0 producer; 1-3 the first three issuers; 4-7 epilogue; with E rows 8-11 gather them and
   // warp 12 is the fourth issuer (E only, k <= 64).  A launch has only the warps its roles need, so
   // that the register budget of the epilogue (a whole accumulator row per thread) is not cut by
@@ -405,7 +407,7 @@ codec_umma_project_kernel(const MmaArgs a, const __grid_constant__ UmmaMaps maps
     mbar_init(ring_free_bar, 2);        // the peer's two receiving warps
     for (int s = 0; s < S; ++s) {
       mbar_init(full_bar(s), Cfg::kGathers ? 5 : 1);
-      mbar_init(empty_bar(s), Cfg::kATiles);   // one commit per operand (the X threads take turns)
+      mbar_init(empty_bar(s), Cfg::kFrees);
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(acc_full_bar(b), Cfg::kIssuers);
@@ -515,7 +517,9 @@ codec_umma_project_kernel(const MmaArgs a, const __grid_constant__ UmmaMaps maps
           // the current phase of a barrier and the one before it: a thread that skipped its
           // partner's stages could reach a slot while the load of the slot's previous use (a
           // partner's stage, loads complete out of order) was still in flight, take that earlier
-          // phase for its own, consume a half-written stage and arrive on "empty" once too often.
+          // phase for its own, consume a half-written stage and arrive on "empty" once too often.  And it frees them
+          // too: its partner's commit alone would let the slot be filled again before this thread has looked, whose
+          // wait would then be for a phase that has gone by.
           if (!dead && !mbar_wait(full_bar(slot), parity)) timed_out();
           if (mine) {
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
@@ -531,6 +535,8 @@ codec_umma_project_kernel(const MmaArgs a, const __grid_constant__ UmmaMaps maps
                 umma_bf16(d_tmem, adesc + j * 2, bdesc + j * 128, idesc, (st > first_st || j > 0) ? 1u : 0u);
             }
             umma_commit(empty_bar(slot));
+          } else {
+            mbar_arrive(empty_bar(slot));
           }
           if (++slot == S) {
             slot = 0;

@@ -144,7 +144,7 @@ codec_umma_roundtrip_kernel(const MmaArgs a, const __grid_constant__ UmmaRoundTr
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
       mbar_init(full_bar(s), 1);
-      mbar_init(empty_bar(s), 1);
+      mbar_init(empty_bar(s), 2);   // both pass-1 issuers: one commits, the other has looked
     }
     mbar_init(acc1_full_bar, 2);   // both pass-1 issuers
     mbar_init(c_ready_bar, 4);
@@ -247,7 +247,8 @@ codec_umma_roundtrip_kernel(const MmaArgs a, const __grid_constant__ UmmaRoundTr
         const uint32_t acc1 = tmem_base + Cfg::kAcc1Col;
         for (int st = 0; st < nstage; ++st) {
           // both pass-1 issuers wait on every stage (a thread that skipped a barrier's phase could
-          // take the phase before it for the one it wants); the odd stages are warp 7's
+          // take the phase before it for the one it wants), and free it, so that no phase goes by before both have
+          // looked; the odd stages are warp 7's
           if (!dead && !mbar_wait(full_bar(slot), parity)) timed_out();
           if ((st & 1) == 0) {
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
@@ -257,6 +258,8 @@ codec_umma_roundtrip_kernel(const MmaArgs a, const __grid_constant__ UmmaRoundTr
             for (int j = 0; j < kUmmaCols / 16; ++j)   // a K step: 32 bytes of a K-major row, 16 rows of an MN-major tile
               umma_bf16(acc1, ad + j * (LEFT ? 128 : 2), bd + j * 128, idesc1, (st > 0 || j > 0) ? 1u : 0u);
             umma_commit(empty_bar(slot));
+          } else {
+            mbar_arrive(empty_bar(slot));
           }
           if (++slot == S) {
             slot = 0;
@@ -317,6 +320,8 @@ codec_umma_roundtrip_kernel(const MmaArgs a, const __grid_constant__ UmmaRoundTr
             for (int j = 0; j < kUmmaCols / 16; ++j)
               umma_bf16(acc1b, ad + j * (LEFT ? 128 : 2), bd + j * 128, idesc1, (st > 1 || j > 0) ? 1u : 0u);
             umma_commit(empty_bar(slot));
+          } else {
+            mbar_arrive(empty_bar(slot));
           }
           if (++slot == S) {
             slot = 0;

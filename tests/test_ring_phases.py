@@ -133,3 +133,56 @@ def test_an_issuer_that_looks_at_its_partners_stages_can_miss_one():
     with pytest.raises(AssertionError):
         for seed in range(150):
             plain_ring(41, 9, 4, 2, wait_all=True).run(random.Random(seed))
+
+
+def tma_ring(steps_of_tiles, slots, pairs, singles, bufs, partner_frees):
+    """codec_umma.cuh, and pass 1 of codec_umma_roundtrip.cuh: one load per stage, `pairs` operands whose two issuers take
+    alternate stages of a tile and `singles` with one, an accumulator per issuer; partner_frees: the issuer whose turn it is
+    not frees the stage as well."""
+    ops = pairs + singles
+    r = Ring(slots, 1, ops + (pairs if partner_frees else 0), bufs, 2 * pairs + singles, 1)
+
+    def issuer(op, half, halves):
+        step = 0
+        for tile, nst in enumerate(steps_of_tiles):
+            yield r.acc_empty[tile % bufs], 1 - tile // bufs % 2
+            for st in range(nst):
+                slot = step % slots
+                yield r.full[slot], step // slots % 2
+                if halves == 1 or st % 2 == half:
+                    r.consume("rows", slot, step)
+                    r.later(("mma", op, half), lambda slot=slot, step=step: free(slot, step))
+                elif partner_frees:
+                    free(slot, step)
+                step += 1
+                yield None
+            r.later(("mma", op, half), lambda buf=tile % bufs: r.acc_full[buf].arrive())
+
+    def free(slot, step):
+        r.consume("rows", slot, step)
+        if r.empty[slot].pending == 1:
+            r.release(slot, ("rows",))
+        r.empty[slot].arrive()
+
+    def epilogue():
+        for tile in range(len(steps_of_tiles)):
+            yield r.acc_full[tile % bufs], tile // bufs % 2
+            r.acc_empty[tile % bufs].arrive()
+
+    r.roles = [_producer(r, "rows", sum(steps_of_tiles), True), epilogue()]
+    r.roles += [issuer(op, half, 2) for op in range(pairs) for half in (0, 1)] + [issuer(pairs + op, 0, 1) for op in range(singles)]
+    return r
+
+
+@pytest.mark.parametrize("pairs,singles,bufs", [(1, 0, 2), (1, 1, 2), (2, 0, 2), (2, 0, 1), (0, 3, 1)])
+@pytest.mark.parametrize("slots", [2, 4, 5, 10])
+@pytest.mark.parametrize("tiles", [(1,), (1, 1, 1), (8, 4), (7, 7, 7, 3), (16, 16, 8)])
+def test_tma_projection(tiles, slots, pairs, singles, bufs):
+    for seed in range(60):
+        tma_ring(tiles, slots, pairs, singles, bufs, partner_frees=True).run(random.Random(seed))
+
+
+def test_a_stage_its_reader_alone_frees_can_pass_by_the_partner():
+    with pytest.raises(AssertionError):
+        for seed in range(300):
+            tma_ring((16, 16, 8), 5, 1, 0, 2, partner_frees=False).run(random.Random(seed))
