@@ -317,9 +317,7 @@ def library() -> ctypes.CDLL:
     return _lib
 
 
-def reference(codec: ssn_codec_t):
-    """A prepared reference to the codec; what is changed in the codec later is seen through it."""
-    return ctypes.byref(codec)
+check = _check   # raises SsnError for a status other than SSN_OK
 
 
 def raw(name: str):

@@ -7,6 +7,7 @@ Python and nothing here works without the CUDA library.
 
 from __future__ import annotations
 
+from ctypes import byref
 from typing import List, Optional, Sequence
 
 import numpy as np
@@ -46,8 +47,8 @@ def padded_columns(t: torch.Tensor, multiple: int = 8) -> torch.Tensor:
 
 
 # The calls below are often shorter on the GPU than on the host, so what every one of them does is kept short: the raw
-# handle of the current stream, one look at shape and strides, the C function itself with a prepared reference to the codec.
-# Four calls of a step: 57 -> 35 us of host time.
+# handle of the current stream, one look at shape and strides, the C function itself.  Four calls of a step: 57 -> 35 us of
+# host time.
 _lib = binding.library()
 
 
@@ -88,7 +89,6 @@ class Codec:
             E.shape[0] if E is not None else 0,
             P.data_ptr() if P is not None else 0, _ld(P) if P is not None else None,
             P.shape[0] if P is not None else 0, dev_status=self.dev_status.data_ptr())
-        self._c = binding.reference(self.c)
 
     def prepare_tables(self, embedding: bool = True, positions: bool = True) -> None:
         """Project the codec's constant tables once (EU = E U, PU = P U, fp32) and attach them,
@@ -135,20 +135,18 @@ class Codec:
                  pos: Optional[torch.Tensor] = None, out: Optional[torch.Tensor] = None) -> torch.Tensor:
         n = X.shape[0]
         Z = out if out is not None else self._empty(n, self.k)
-        st = _lib.ssn_compress(self._c, X.data_ptr(), _ld(X), _ptr(ids), _ptr(pos), n, seq_len, Z.data_ptr(), _ld(Z),
+        st = _lib.ssn_compress(byref(self.c), X.data_ptr(), _ld(X), _ptr(ids), _ptr(pos), n, seq_len, Z.data_ptr(), _ld(Z),
                                self.dev_status.data_ptr(), _stream())
-        if st:
-            raise binding.SsnError(st, "ssn_compress")
+        binding.check(st, "ssn_compress")
         return Z
 
     def decompress(self, Z: torch.Tensor, ids: Optional[torch.Tensor] = None, seq_len: int = 1,
                    pos: Optional[torch.Tensor] = None, out: Optional[torch.Tensor] = None) -> torch.Tensor:
         n = Z.shape[0]
         Xh = out if out is not None else self._empty(n, self.d)
-        st = _lib.ssn_decompress(self._c, Z.data_ptr(), _ld(Z), _ptr(ids), _ptr(pos), n, seq_len, Xh.data_ptr(), _ld(Xh),
+        st = _lib.ssn_decompress(byref(self.c), Z.data_ptr(), _ld(Z), _ptr(ids), _ptr(pos), n, seq_len, Xh.data_ptr(), _ld(Xh),
                                  self.dev_status.data_ptr(), _stream())
-        if st:
-            raise binding.SsnError(st, "ssn_decompress")
+        binding.check(st, "ssn_decompress")
         return Xh
 
     def decompress_rowsumsq(self, Z: torch.Tensor, ids: Optional[torch.Tensor] = None, seq_len: int = 1,
@@ -169,10 +167,9 @@ class Codec:
         mode = (binding.SSN_GRAD_COEFF if coeff else 0) | (binding.SSN_GRAD_FULL if full else 0)
         dZ = (out if out is not None else self._empty(n, self.k)) if coeff else None
         Gp = (out_full if out_full is not None else self._empty(n, self.d)) if full else None
-        st = _lib.ssn_grad_project(self._c, G.data_ptr(), _ld(G), n, mode, dZ.data_ptr() if coeff else 0,
+        st = _lib.ssn_grad_project(byref(self.c), G.data_ptr(), _ld(G), n, mode, dZ.data_ptr() if coeff else 0,
                                    _ld(dZ) if coeff else 0, Gp.data_ptr() if full else 0, _ld(Gp) if full else 0, _stream())
-        if st:
-            raise binding.SsnError(st, "ssn_grad_project")
+        binding.check(st, "ssn_grad_project")
         if coeff and full:
             return dZ, Gp
         return dZ if coeff else Gp
