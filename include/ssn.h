@@ -209,7 +209,7 @@ ssn_status_t ssn_grad_project(const ssn_codec_t *codec, const void *G, int64_t l
  *   workspace  device scratch of at least ssn_weight_reproject_workspace_bytes(...) bytes,
  *              16-byte aligned; may be NULL only when that size is 0.  Its contents are
  *              garbage afterwards; calls that share it must be ordered on one stream.  For
- *              SSN_SIDE_RIGHT it is optional, as in ssn_weight_reproject_list.
+ *              SSN_SIDE_RIGHT it is optional, as in ssn_weight_reproject_list_ws.
  * The k coordinates are kept in fp32 between the two products.
  */
 size_t ssn_weight_reproject_workspace_bytes(const ssn_codec_t *codec, int64_t rows,
@@ -227,20 +227,30 @@ ssn_status_t ssn_weight_reproject(const ssn_codec_t *codec, void *const *W_ptrs,
  *   SSN_SIDE_LEFT : W_i is [d x extent[i]],  W_i <- U (U^T W_i)
  *   W_ptrs, extent, ldw   HOST arrays of `count` device pointers, extents (>= 1) and leading
  *                         dimensions (>= d for RIGHT, >= extent[i] for LEFT); distinct buffers.
- *   workspace   needed for SSN_SIDE_LEFT weights that the fused tensor-core kernel does not
+ *   workspace   only read for SSN_SIDE_LEFT weights that the fused tensor-core kernel does not
  *               take (fp32, k > 128, d not a multiple of 128, leading dimension not a multiple of
  *               8 elements, unaligned base): k * max(extent) * 4 bytes, 16-byte aligned; such a
  *               weight without enough workspace gives SSN_ERR_WORKSPACE (weights before it in the
- *               list have been re-projected then).  For SSN_SIDE_RIGHT it is optional: weights that
- *               the fused kernel does not take run on the tensor cores when it has
- *               ssn_coords_workspace_bytes(codec, max(extent)) bytes, on the general kernel else.
- *               Garbage afterwards.
+ *               list have been re-projected then).  May be NULL otherwise.  Its contents are garbage
+ *               after a LEFT call, and LEFT calls that share it must be ordered on one stream; a
+ *               RIGHT call leaves it alone.
  * Same arithmetic as ssn_weight_reproject.
  */
 ssn_status_t ssn_weight_reproject_list(const ssn_codec_t *codec, void *const *W_ptrs,
                                        const int64_t *extent, const int64_t *ldw, int32_t count,
                                        int32_t side, void *workspace, size_t workspace_bytes,
                                        void *stream);
+
+/*
+ * The same with a workspace that RIGHT calls use as well: for SSN_SIDE_RIGHT weights that the fused kernel
+ * does not take, ssn_coords_workspace_bytes(codec, max(extent)) bytes, 16-byte aligned, put them on the
+ * tensor cores (see ssn_reparam_project_ws on the exceptions); NULL or too small: the general kernel.
+ * Garbage afterwards; calls that share it must be ordered on one stream, whichever side they are.
+ */
+ssn_status_t ssn_weight_reproject_list_ws(const ssn_codec_t *codec, void *const *W_ptrs,
+                                          const int64_t *extent, const int64_t *ldw, int32_t count,
+                                          int32_t side, void *workspace, size_t workspace_bytes,
+                                          void *stream);
 
 /*
  * Reparameterized SSN (Eq. reparam): an output projection is stored as its low-dimensional

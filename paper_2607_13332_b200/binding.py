@@ -87,6 +87,8 @@ _SIGNATURES = {
                                    _vp, _vp]),
     "ssn_weight_reproject_list": (_i32, [_codec_p, ctypes.POINTER(_vp), ctypes.POINTER(_i64),
                                          ctypes.POINTER(_i64), _i32, _i32, _vp, _sz, _vp]),
+    "ssn_weight_reproject_list_ws": (_i32, [_codec_p, ctypes.POINTER(_vp), ctypes.POINTER(_i64),
+                                            ctypes.POINTER(_i64), _i32, _i32, _vp, _sz, _vp]),
     "ssn_static_scratch_bytes": (_sz, []),
     "sparta_segment": (_i32, [_i64, _i32, _i64, ctypes.POINTER(_i64), ctypes.POINTER(_i64)]),
     "sparta_snapshot": (_i32, [_vp, _i64, _i64, _vp, _vp]),
@@ -219,12 +221,13 @@ def ssn_weight_reproject_left_static(codec: ssn_codec_t, W: int, cols: int, ldw:
 
 
 def ssn_weight_reproject_list(codec: ssn_codec_t, W_ptrs, extent, ldw, side: int, workspace: int = 0,
-                              workspace_bytes: int = 0, stream: int = 0) -> None:
-    """Re-projection of weights [extent[i] x d] (RIGHT) or [d x extent[i]] (LEFT), in place."""
+                              workspace_bytes: int = 0, stream: int = 0, right_workspace: bool = False) -> None:
+    """Re-projection of weights [extent[i] x d] (RIGHT) or [d x extent[i]] (LEFT), in place.  A RIGHT call leaves the
+    workspace alone unless right_workspace is set (ssn_weight_reproject_list_ws)."""
     n = len(W_ptrs)
-    _check(_lib.ssn_weight_reproject_list(ctypes.byref(codec), (_vp * n)(*W_ptrs), (_i64 * n)(*extent),
-                                          (_i64 * n)(*ldw), n, side, workspace or None, workspace_bytes,
-                                          stream or None), "ssn_weight_reproject_list")
+    fn = _lib.ssn_weight_reproject_list_ws if right_workspace else _lib.ssn_weight_reproject_list
+    _check(fn(ctypes.byref(codec), (_vp * n)(*W_ptrs), (_i64 * n)(*extent), (_i64 * n)(*ldw), n, side, workspace or None,
+              workspace_bytes, stream or None), fn.__name__)
 
 
 def ssn_reparam_project(codec: ssn_codec_t, H: int, ldh: int, m: int, Zw: int, ldzw: int, n_tokens: int,

@@ -917,6 +917,14 @@ ssn_status_t ssn_weight_reproject_list(const ssn_codec_t *codec, void *const *W_
                                        const int64_t *extent, const int64_t *ldw, int32_t count,
                                        int32_t side, void *workspace, size_t workspace_bytes,
                                        void *stream) {
+  if (side == SSN_SIDE_RIGHT) workspace = nullptr, workspace_bytes = 0;   // left alone
+  return ssn_weight_reproject_list_ws(codec, W_ptrs, extent, ldw, count, side, workspace, workspace_bytes, stream);
+}
+
+ssn_status_t ssn_weight_reproject_list_ws(const ssn_codec_t *codec, void *const *W_ptrs,
+                                          const int64_t *extent, const int64_t *ldw, int32_t count,
+                                          int32_t side, void *workspace, size_t workspace_bytes,
+                                          void *stream) {
   ssn_status_t st = check_codec(codec);
   if (st != SSN_OK) return st;
   if (side != SSN_SIDE_LEFT && side != SSN_SIDE_RIGHT) return SSN_ERR_DTYPE;

@@ -282,27 +282,30 @@ class Codec:
                               workspace: Optional[torch.Tensor] = None) -> None:
         """In place, for weights [rows_i x d] ("right") or [d x cols_i] ("left") of any free
         extents.  A LEFT weight the fused kernel does not take needs k * cols * 4 bytes of workspace;
-        one is allocated here when none is given."""
+        one is allocated here when none is given.  LEFT calls that share a given one must be ordered on one
+        stream; RIGHT calls leave it alone, and have scratch of their own only when none is given."""
         if not weights:
             return
         axis = 0 if side == "right" else 1
+        lend = side == "right" and workspace is None and not self._fetchable(*weights)
         if side == "left" and workspace is None:
             workspace = torch.empty(self.k * max(w.shape[1] for w in weights) * 4, dtype=torch.uint8,
                                     device=self.U.device)
-        if side == "right" and workspace is None and not self._fetchable(*weights):
+        if lend:
             workspace = self._coords_workspace(max(w.shape[0] for w in weights))
         binding.ssn_weight_reproject_list(self.c, [w.data_ptr() for w in weights],
                                           [w.shape[axis] for w in weights], [_ld(w) for w in weights],
                                           binding.SIDES[side],
                                           workspace.data_ptr() if workspace is not None else 0,
-                                          workspace.numel() if workspace is not None else 0, _stream())
+                                          workspace.numel() if workspace is not None else 0, _stream(), right_workspace=lend)
 
     def weight_reproject_rows(self, weights: Sequence[torch.Tensor]) -> None:
         self.weight_reproject_list(weights, "right")
 
     def weight_reproject(self, weights: Sequence[torch.Tensor], side: str,
                          workspace: Optional[torch.Tensor] = None) -> None:
-        """In place, for a list of equally shaped weights."""
+        """In place, for a list of equally shaped weights.  A given workspace is garbage afterwards, and calls that share it
+        must be ordered on one stream."""
         if not weights:
             return
         rows, cols = weights[0].shape

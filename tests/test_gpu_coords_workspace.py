@@ -61,3 +61,20 @@ def test_reparameterised_projection(n, m, d, k, dt, coords):
         assert_close(host64(C, dt), H @ Z, dt, "coordinates")
         assert guards_intact(C, cbuf, dt)
     assert codec.take_status() == 0
+
+
+def test_a_workspace_given_to_a_right_list_is_left_alone():
+    """Two such calls on two streams may be handed the same one; their weights would come out wrong if either wrote it."""
+    d, k = 512, 40
+    rng = np.random.default_rng(3)
+    U0 = np.linalg.qr(rng.standard_normal((d, k)))[0].astype(np.float32)
+    codec = Codec(synth.F32, to_device(U0, synth.F32))
+    W0 = _rand(rng, (300, d), synth.F32, 0.02)
+    given = torch.full((B.ssn_coords_workspace_bytes(codec.c, 300),), 0xA5, dtype=torch.uint8, device="cuda")
+    weights = [to_device(W0, synth.F32) for _ in range(2)]
+    codec.weight_reproject_list(weights[:1], "right", workspace=given)
+    B.ssn_weight_reproject_list(codec.c, [weights[1].data_ptr()], [300], [d], B.SSN_SIDE_RIGHT, given.data_ptr(), given.numel(),
+                                torch.cuda.current_stream().cuda_stream)
+    assert bool((given == 0xA5).all())
+    for w in weights:
+        assert_close(host64(w, synth.F32), oracle.weight_reproject(f64(W0, synth.F32), f64(U0, synth.F32), "right"), synth.F32, "reproject")
