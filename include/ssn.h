@@ -271,9 +271,13 @@ ssn_status_t ssn_reparam_project(const ssn_codec_t *codec, const void *H, int64_
 
 /*
  * The same with device scratch for the fp32 coordinates, 16-byte aligned, of
- * ssn_coords_workspace_bytes(codec, n_tokens) bytes (0 for ranks that have no use for it).  It
- * is used where the fused kernel does not take the call (fp32, leading dimension not a multiple of 8
- * elements, unaligned base, ...), which then runs on the tensor cores; NULL or too small: the general kernel.
+ * ssn_coords_workspace_bytes(codec, n_tokens) bytes (0 for ranks that have no use for it).  With it a
+ * call that the fused kernel does not take (fp32, fewer than 512 tokens, d not a multiple of 128 or m of 64,
+ * leading dimension not a multiple of 8 elements, unaligned base) runs on the tensor cores; with NULL or
+ * too little on the general kernel.  Exceptions, scratch or not: fp32 `coords` take the place of the scratch,
+ * which is not touched then; bf16 `coords`, and narrow calls ((m + d) / 2 columns times k / 32, rounded up,
+ * below 512, and at most 4096 tokens), run on the general kernel.
+ * The scratch is garbage afterwards; calls that share it must be ordered on one stream.
  */
 size_t ssn_coords_workspace_bytes(const ssn_codec_t *codec, int64_t rows);
 ssn_status_t ssn_reparam_project_ws(const ssn_codec_t *codec, const void *H, int64_t ldh, int64_t m,

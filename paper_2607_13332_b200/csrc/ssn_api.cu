@@ -177,8 +177,8 @@ inline int64_t coords_pitch(int32_t k) { return ((int64_t)k + 3) & ~3LL; }
 inline size_t coords_bytes(int64_t rows, int32_t k) { return (size_t)rows * (size_t)coords_pitch(k) * sizeof(float); }
 
 // D = (S U) U2^T of rows the fused kernels do not take (a.src and a.dst; fp32 storage, operands off the 16-byte grid).
-// With scratch for the fp32 coordinates and a rank that the split-operand kernels take it is a projection and an expansion on
-// these, on the tensor cores; without it the general kernel.  us, general -> split: fp32 weights [2048 + 7168] x 2048 twice,
+// With room for the fp32 coordinates and a rank that the split-operand kernels take it is a projection and an expansion on
+// the tensor cores; without it the general kernel.  us, general -> split: fp32 weights [2048 + 7168] x 2048 twice,
 // rank 40 1389 -> 239; bf16 ones, rank 51 packed 1482 -> 176; H [8192 x 7168] to 2048 columns, fp32 1633 -> 166.  fp32 results
 // are closer to 64-bit sums too (1.9e-7 -> 1.0e-7).
 ssn_status_t project_then_expand(const TokenArgs &a, int32_t dtype, void *scratch, size_t scratch_bytes, cudaStream_t stream) {
@@ -187,13 +187,15 @@ ssn_status_t project_then_expand(const TokenArgs &a, int32_t dtype, void *scratc
   // against 32; the same for 1 to 2000 rows.  Above that it grows with the rows, too.
   const int64_t columns = a.U2 != nullptr ? ((int64_t)a.d + a.d2) / 2 : a.d;
   const bool wide = columns * ((a.k + 31) / 32) >= 512 || a.n > 4096;
-  const bool split = wide && (a.U2 != nullptr || !mma_eligible(a, dtype)) && a.k <= kSplitMaxRank && scratch != nullptr &&
-                     aligned16(scratch) && scratch_bytes >= coords_bytes(a.n, a.k) && (a.zout == nullptr || dtype == SSN_F32);
+  // fp32 coordinates that the caller asked for serve as they are; bf16 ones are rounded by the general kernel
+  const bool held = a.zout != nullptr ? dtype == SSN_F32
+                                      : scratch != nullptr && aligned16(scratch) && scratch_bytes >= coords_bytes(a.n, a.k);
+  const bool split = wide && held && (a.U2 != nullptr || !mma_eligible(a, dtype)) && a.k <= kSplitMaxRank;
   if (!split) return a.U2 != nullptr ? launch_generic_token_kernel(a, dtype, stream) : launch_token_kernel(a, dtype, stream);
   TokenArgs p = a, e = a;
   p.dst = nullptr;
   p.U2 = nullptr;
-  p.zout = a.zout != nullptr ? a.zout : scratch;   // fp32 coordinates that the caller asked for serve as they are
+  p.zout = a.zout != nullptr ? a.zout : scratch;
   p.ldzout = a.zout != nullptr ? a.ldzout : coords_pitch(a.k);
   p.wire = 1;
   ssn_status_t st = launch_token_kernel(p, dtype, stream);

@@ -249,7 +249,8 @@ class Codec:
         """Y = (H Zw) U^T for a projection stored as its factor Zw [m, k] (Eq. reparam)."""
         n, m = H.shape
         Y = out if out is not None else self._empty(n, self.d)
-        ws = None if self._fetchable(H, Zw, Y) else self._coords_workspace(n)
+        # coordinates that the caller asked for are kept there
+        ws = None if coords is not None or self._fetchable(H, Zw, Y) else self._coords_workspace(n)
         binding.ssn_reparam_project_ws(self.c, H.data_ptr(), _ld(H), m, Zw.data_ptr(), _ld(Zw), n, Y.data_ptr(),
                                        _ld(Y), coords.data_ptr() if coords is not None else 0,
                                        _ld(coords) if coords is not None else 0,

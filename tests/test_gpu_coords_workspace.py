@@ -78,3 +78,22 @@ def test_a_workspace_given_to_a_right_list_is_left_alone():
     assert bool((given == 0xA5).all())
     for w in weights:
         assert_close(host64(w, synth.F32), oracle.weight_reproject(f64(W0, synth.F32), f64(U0, synth.F32), "right"), synth.F32, "reproject")
+
+
+def _reparam(seed, n=200, m=640, d=512, k=24):
+    rng = np.random.default_rng(seed)
+    H0, Zw0 = _rand(rng, (n, m), synth.F32), _rand(rng, (m, k), synth.F32, 0.02)
+    U0 = np.linalg.qr(rng.standard_normal((d, k)))[0].astype(np.float32)
+    expect = oracle.reparam_project(f64(H0, synth.F32), f64(Zw0, synth.F32), f64(U0, synth.F32))
+    return Codec(synth.F32, to_device(U0, synth.F32)), to_device(H0, synth.F32), to_device(Zw0, synth.F32), expect
+
+
+def test_requested_coordinates_need_no_scratch():
+    codec, H, Zw, expect = _reparam(7)
+    (n, m), k, d = H.shape, codec.k, codec.d
+    Y, C = torch.empty((n, d), device="cuda"), torch.empty((n, k), device="cuda")
+    B.ssn_reparam_project(codec.c, H.data_ptr(), m, m, Zw.data_ptr(), k, n, Y.data_ptr(), d, C.data_ptr(), k,
+                          torch.cuda.current_stream().cuda_stream)
+    assert B.ssn_last_kernel()[0] == B.SSN_KERNEL_SPLIT_EXPAND
+    assert_close(Y.double().cpu().numpy(), expect, synth.F32, "Y")
+    assert_close(C.double().cpu().numpy(), (H.double() @ Zw.double()).cpu().numpy(), synth.F32, "coordinates")
