@@ -229,9 +229,11 @@ class Codec:
                                     self.dev_status.data_ptr(), _stream())
         return Xh
 
-    def _fetchable(self, *matrices: torch.Tensor) -> bool:
-        """Whether TMA can fetch the basis and these matrices: what the fused kernels take needs no scratch."""
-        return self.dtype == synth.BF16 and all(t.data_ptr() % 16 == 0 and _ld(t) % 8 == 0 for t in (self.U, *matrices))
+    def _fused(self, rows: int, inner: int, *matrices: torch.Tensor) -> bool:
+        """Whether the fused project-then-expand kernel takes a call over this many rows, the contraction `inner` wide: bf16
+        that TMA can fetch, four row tiles or more, whole stages and chunks of columns.  Such a call has no use for scratch."""
+        return (self.dtype == synth.BF16 and rows >= 512 and inner % 64 == 0 and self.d % 128 == 0
+                and all(t.data_ptr() % 16 == 0 and _ld(t) % 8 == 0 for t in (self.U, *matrices)))
 
     def _coords_workspace(self, rows: int) -> Optional[torch.Tensor]:
         """Scratch for the fp32 coordinates of `rows` rows."""
@@ -250,7 +252,7 @@ class Codec:
         n, m = H.shape
         Y = out if out is not None else self._empty(n, self.d)
         # coordinates that the caller asked for are kept there
-        ws = None if coords is not None or self._fetchable(H, Zw, Y) else self._coords_workspace(n)
+        ws = None if coords is not None or self._fused(n, m, H, Zw, Y) else self._coords_workspace(n)
         binding.ssn_reparam_project_ws(self.c, H.data_ptr(), _ld(H), m, Zw.data_ptr(), _ld(Zw), n, Y.data_ptr(),
                                        _ld(Y), coords.data_ptr() if coords is not None else 0,
                                        _ld(coords) if coords is not None else 0,
@@ -288,7 +290,7 @@ class Codec:
         if not weights:
             return
         axis = 0 if side == "right" else 1
-        lend = side == "right" and workspace is None and not self._fetchable(*weights)
+        lend = side == "right" and workspace is None and not self._fused(min(w.shape[0] for w in weights), self.d, *weights)
         if side == "left" and workspace is None:
             workspace = torch.empty(self.k * max(w.shape[1] for w in weights) * 4, dtype=torch.uint8,
                                     device=self.U.device)
@@ -316,7 +318,7 @@ class Codec:
                 raise ValueError("weights of one call must share shape and leading dimension")
         if workspace is None:
             workspace = self.reproject_workspace(rows, cols, side, len(weights))
-        if side == "right" and workspace is None and not self._fetchable(*weights):
+        if side == "right" and workspace is None and not self._fused(rows * len(weights), self.d, *weights):
             workspace = self._coords_workspace(rows)
         binding.ssn_weight_reproject(self.c, [w.data_ptr() for w in weights], rows, cols, ldw,
                                      binding.SIDES[side],

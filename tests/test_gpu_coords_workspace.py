@@ -97,3 +97,30 @@ def test_requested_coordinates_need_no_scratch():
     assert B.ssn_last_kernel()[0] == B.SSN_KERNEL_SPLIT_EXPAND
     assert_close(Y.double().cpu().numpy(), expect, synth.F32, "Y")
     assert_close(C.double().cpu().numpy(), (H.double() @ Zw.double()).cpu().numpy(), synth.F32, "coordinates")
+
+
+# calls on the 16-byte grid, but with fewer rows or other widths than the fused kernel takes
+@pytest.mark.parametrize("n,m,d", [(300, 1024, 512), (700, 1024, 520), (700, 1000, 512), (511, 2048, 1024)])
+@pytest.mark.parametrize("k", [8, 56])
+def test_aligned_calls_the_fused_kernel_refuses(n, m, d, k):
+    dt = synth.BF16
+    rng = np.random.default_rng(n + m)
+    H0, Zw0 = _rand(rng, (n, m), dt), _rand(rng, (m, k), dt, 0.02)
+    U0 = synth.to_storage(np.linalg.qr(rng.standard_normal((d, k)))[0], dt)
+    codec = Codec(dt, to_device(U0, dt))
+    out = codec.reparam_project(to_device(H0, dt), to_device(Zw0, dt))
+    assert B.ssn_last_kernel()[0] == B.SSN_KERNEL_SPLIT_EXPAND
+    assert_close(host64(out, dt), oracle.reparam_project(f64(H0, dt), f64(Zw0, dt), f64(U0, dt)), dt, "Y")
+
+
+def test_aligned_weights_the_fused_kernel_refuses():
+    d, k, dt = 1000, 40, synth.BF16
+    rng = np.random.default_rng(5)
+    U0 = synth.to_storage(np.linalg.qr(rng.standard_normal((d, k)))[0], dt)
+    W0 = _rand(rng, (600, d), dt, 0.02)
+    codec = Codec(dt, to_device(U0, dt))
+    for call in (codec.weight_reproject, codec.weight_reproject_list):
+        W = to_device(W0, dt)
+        call([W], "right")
+        assert B.ssn_last_kernel()[0] == B.SSN_KERNEL_SPLIT_EXPAND
+        assert_close(host64(W, dt), oracle.weight_reproject(f64(W0, dt), f64(U0, dt), "right"), dt, "reproject")
