@@ -236,9 +236,13 @@ class Codec:
                 and all(t.data_ptr() % 16 == 0 and _ld(t) % 8 == 0 for t in (self.U, *matrices)))
 
     def _coords_workspace(self, rows: int) -> Optional[torch.Tensor]:
-        """Scratch for the fp32 coordinates of `rows` rows."""
+        """Scratch for the fp32 coordinates of `rows` rows; None, and the general kernel takes the call, where there is no
+        use for it or no memory left."""
         nbytes = binding.ssn_coords_workspace_bytes(self.c, rows)
-        return torch.empty(nbytes, dtype=torch.uint8, device=self.U.device) if nbytes else None
+        try:
+            return torch.empty(nbytes, dtype=torch.uint8, device=self.U.device) if nbytes else None
+        except torch.OutOfMemoryError:
+            return None
 
     def reproject_workspace(self, rows: int, cols: int, side: str, batch: int) -> Optional[torch.Tensor]:
         nbytes = binding.ssn_weight_reproject_workspace_bytes(self.c, rows, cols, binding.SIDES[side], batch)

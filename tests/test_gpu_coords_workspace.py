@@ -124,3 +124,16 @@ def test_aligned_weights_the_fused_kernel_refuses():
         call([W], "right")
         assert B.ssn_last_kernel()[0] == B.SSN_KERNEL_SPLIT_EXPAND
         assert_close(host64(W, dt), oracle.weight_reproject(f64(W0, dt), f64(U0, dt), "right"), dt, "reproject")
+
+
+def test_no_memory_for_scratch(monkeypatch):
+    codec, H, Zw, expect = _reparam(8)
+    out = torch.empty((H.shape[0], codec.d), device="cuda")
+
+    def full(*args, **kwargs):
+        raise torch.OutOfMemoryError("no memory left")
+    with monkeypatch.context() as m:
+        m.setattr(torch, "empty", full)
+        codec.reparam_project(H, Zw, out=out)
+    assert B.ssn_last_kernel()[0] == B.SSN_KERNEL_GENERIC
+    assert_close(out.double().cpu().numpy(), expect, synth.F32, "Y")
