@@ -449,6 +449,7 @@ enum {
                              SPLIT_PROJECT: several CTAs per tile; SPLIT_EXPAND: fp32 wire rows */
 #define SSN_KVAR_ROWSUMSQ 16 /* UMMA_EXPAND / GENERIC: the row statistic is produced              */
 #define SSN_KVAR_TWO_RUNS 64  /* UMMA_EXPAND: head and remainder of fp32 wire rows as two runs against one chunk of U */
+#define SSN_KVAR_PLAIN 128    /* SPLIT_PROJECT: the kernel for bf16 rows as they are, fetched by TMA      */
 #define SSN_KVAR_FEWSEQ 32   /* UMMA_EXPAND: tiles of 4, 2 or 1 sequences (a batch that is not groups of 8) */
 int32_t ssn_last_kernel(void);
 

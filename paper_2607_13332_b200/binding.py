@@ -26,6 +26,7 @@ SSN_DEV_BAD_ID, SSN_DEV_BAD_POS, SSN_DEV_TIMEOUT = 1, 2, 4
  SSN_KERNEL_UMMA_PROJECT, SSN_KERNEL_UMMA_EXPAND, SSN_KERNEL_UMMA_ROUNDTRIP, SSN_KERNEL_UMMA_TOKENS,
  SSN_KERNEL_SPLIT_PROJECT, SSN_KERNEL_SPLIT_EXPAND) = range(11)
 SSN_KVAR_E, SSN_KVAR_P, SSN_KVAR_WIDE, SSN_KVAR_ALT, SSN_KVAR_ROWSUMSQ, SSN_KVAR_FEWSEQ, SSN_KVAR_TWO_RUNS = 1, 2, 4, 8, 16, 32, 64
+SSN_KVAR_PLAIN = 128
 
 DTYPES = {"f32": SSN_F32, "bf16": SSN_BF16}
 SIDES = {"left": SSN_SIDE_LEFT, "right": SSN_SIDE_RIGHT}

@@ -38,8 +38,8 @@ int64_t units_of(const SplitProjectArgs &a) { return (a.n + kUmmaTile - 1) / kUm
 
 // Launches either kernel with clusters of c, or with single CTAs on a device that cannot co-schedule them.
 template <typename Kernel, typename... Args>
-cudaError_t launch_slices(Kernel kernel, int threads, int smem, const SplitProjectArgs &a, int c, int sms, cudaStream_t stream,
-                          Args... args) {
+cudaError_t launch_slices(Kernel kernel, int threads, int smem, int variant, const SplitProjectArgs &a, int c, int sms,
+                          cudaStream_t stream, Args... args) {
   const int64_t units = units_of(a);
   // whole tiles: as many CTAs for either half
   const int64_t single = units < sms ? units : (sms > 1 ? sms - sms % a.halves : a.halves), grid = c > 1 ? units * c : single;
@@ -48,7 +48,7 @@ cudaError_t launch_slices(Kernel kernel, int threads, int smem, const SplitProje
     cudaGetLastError();
     e = launch_dependent(kernel, (unsigned)single, threads, smem, stream, 1, a, args...);
   }
-  note_kernel(SSN_KERNEL_SPLIT_PROJECT, (a.has_e ? SSN_KVAR_E : 0) | (a.has_p ? SSN_KVAR_P : 0) |
+  note_kernel(SSN_KERNEL_SPLIT_PROJECT, variant | (a.has_e ? SSN_KVAR_E : 0) | (a.has_p ? SSN_KVAR_P : 0) |
                                             (a.halves > 1 ? SSN_KVAR_WIDE : 0) | (c > 1 ? SSN_KVAR_ALT : 0));
   return e;
 }
@@ -60,7 +60,7 @@ cudaError_t launch_one(const SplitProjectArgs &a, int c, int sms, cudaStream_t s
   static std::atomic<uint64_t> configured{0};
   const cudaError_t e = allow_dynamic_smem(kernel, Cfg::kSmemBytes, configured);
   if (e != cudaSuccess) return e;
-  return launch_slices(kernel, Cfg::kThreads, Cfg::kSmemBytes, a, c, sms, stream);
+  return launch_slices(kernel, Cfg::kThreads, Cfg::kSmemBytes, 0, a, c, sms, stream);
 }
 
 // The plain kernel's CTAs per tile.  A stage takes a CTA kPlainStageNs, or the time of the 16 KB that every CTA at work
@@ -91,7 +91,7 @@ cudaError_t launch_plain(const SplitProjectArgs &a, const CUtensorMap &x, int c,
   static std::atomic<uint64_t> configured{0};
   const cudaError_t e = allow_dynamic_smem(kernel, smem, configured);
   if (e != cudaSuccess) return e;
-  return launch_slices(kernel, kPlainThreads, smem, a, c, sms, stream, x);
+  return launch_slices(kernel, kPlainThreads, smem, SSN_KVAR_PLAIN, a, c, sms, stream, x);
 }
 
 cudaError_t launch_plain_rank(const SplitProjectArgs &a, const CUtensorMap &x, int sms, cudaStream_t s) {

@@ -31,43 +31,66 @@ def _inside_nan(t, pitch, offset):
     return view
 
 
-@pytest.mark.parametrize("n,d", [(1, 64), (127, 72), (128, 128), (129, 200), (700, 1000), (3000, 4096), (1, 2056), (2100, 2056), (19100, 136)])
-@pytest.mark.parametrize("k", [1, 2, 31, 32, 33, 51, 63, 64, 65, 99, 127, 128])
+def _variant():
+    family, variant = B.ssn_last_kernel()
+    assert family == B.SSN_KERNEL_SPLIT_PROJECT
+    return variant
+
+
+# up to 32 coordinates any size; more of them only wide rows, or many
+NARROW = [(n, d, k) for n, d in [(1, 24), (1, 64), (127, 72), (129, 200), (700, 1000), (3000, 4096), (19100, 136)] for k in (1, 2, 31, 32)]
+WIDE = ([(n, d, k) for n, d in [(2100, 2056), (19100, 1032)] for k in (33, 51, 63, 64, 65, 99, 127, 128)]
+        + [(3000, 4096, k) for k in (51, 64, 127)] + [(1, 2056, k) for k in (33, 64)])
+
+
+@pytest.mark.parametrize("n,d,k", [c for c in NARROW if c[2] <= c[1]] + WIDE)
 @pytest.mark.parametrize("excess,offset", [(0, 0), (1, 1), (2, 3), (3, 8)])
 def test_any_basis(n, d, k, excess, offset):
-    if k > d or (k + excess) % 8 == 0 and offset % 8 == 0:
-        pytest.skip("an aligned basis belongs to the TMA kernels")
+    if (k + excess) % 8 == 0 and offset % 8 == 0:
+        excess += 2   # an aligned basis belongs to the TMA kernels
     X = _inside_nan(_rand((n, d), n), (d + 15) // 8 * 8, 64)
     U = _inside_nan(_rand((d, k), k, d ** -0.5), k + excess, offset)
     codec = Codec(synth.BF16, U)
     expect = (X.double() @ U.double()).cpu().numpy()
     words = torch.full((n, k + 2), -1, dtype=torch.int32, device="cuda")
     codec.grad_project_wire(X, out=words.view(torch.float32)[:, :k])
-    assert B.ssn_last_kernel()[0] == B.SSN_KERNEL_SPLIT_PROJECT
+    variant = _variant()
+    assert variant & B.SSN_KVAR_PLAIN and bool(variant & B.SSN_KVAR_WIDE) == (k > 64)
+    # 150 tiles: several to a CTA; few tiles of wide rows: several CTAs to a tile
+    if n == 19100 or d >= 2056:
+        assert bool(variant & B.SSN_KVAR_ALT) == (n < 19100)
     assert_close(words.view(torch.float32)[:, :k].double().cpu().numpy(), expect, synth.F32, "words", tol=WORD_TOL)
     assert (words[:, k:] == -1).all()
     Z = codec.grad_project(X)
+    assert _variant() & B.SSN_KVAR_PLAIN
     assert_close(Z.double().cpu().numpy(), expect, synth.BF16, "rows")
     ids = torch.arange(n, dtype=torch.int32, device="cuda")
     wire = codec.compress_wire(X, ids, with_ids=True)
+    assert _variant() & B.SSN_KVAR_PLAIN
     assert torch.equal(wire[:, k], ids) and torch.equal(wire[:, :k], words[:, :k])
     assert codec.take_status() == 0
 
 
-@pytest.mark.parametrize("n", [300, 20000])
-def test_bad_rows(n):
-    d, k = 256, 51
-    X, U = _rand((n, d), 1), _rand((d, k), 2, d ** -0.5)
+# clusters and single CTAs of both kernels for few and for many coordinates; the last two are the split kernel's
+@pytest.mark.parametrize("n,d,k,plain,cluster", [(300, 256, 27, True, True), (20000, 256, 27, True, False), (300, 2048, 51, True, True),
+                                                 (20000, 1032, 64, True, False), (300, 256, 51, False, True), (20000, 256, 51, False, False)])
+def test_bad_rows(n, d, k, plain, cluster):
+    X, U = _rand((n, d), 1), _inside_nan(_rand((d, k), 2, d ** -0.5), k + 1 + k % 2, 0)
     X[0, 5], X[129, 9], X[130, 9] = float("inf"), -float("inf"), float("nan")
     X[20] *= 1e36
+    X[21] = 3e38                                  # sums out of the range of fp32, at the end or on the way
     codec = Codec(synth.BF16, U)
     got = codec.grad_project_wire(X).double().cpu().numpy()
-    expect = (X.double() @ U.double()).cpu().numpy()
+    variant = _variant()
+    assert bool(variant & B.SSN_KVAR_PLAIN) == plain and bool(variant & B.SSN_KVAR_ALT) == cluster
+    expect = (X.double() @ U.double()).float().double().cpu().numpy()
     assert np.array_equal(np.isnan(got), np.isnan(expect))
     assert np.array_equal(np.isinf(got), np.isinf(expect))
     rows = np.isfinite(expect).all(axis=1)
     scale = np.abs(expect[rows]).max(axis=1, keepdims=True)
     assert (np.abs(got[rows] - expect[rows]) <= 1e-5 * scale).all()
+    finite = np.isfinite(expect[21])
+    assert np.allclose(got[21, finite], expect[21, finite], rtol=1e-5)
     # a bad value of the basis stays in its column
     U[7, 3] = float("nan")
     got = Codec(synth.BF16, U).grad_project_wire(X[200:]).cpu().numpy()
@@ -85,6 +108,6 @@ def test_words_of_few_terms(n, d, k, coherent, bound):
     if coherent:
         X = (_rand((n, k), 3, 3.0).float() @ U.float().T + 0.3 * X.float()).bfloat16()
     got = Codec(synth.BF16, _inside_nan(U, k + 1 + k % 2, 0)).grad_project_wire(X).double()
-    assert B.ssn_last_kernel()[0] == B.SSN_KERNEL_SPLIT_PROJECT
+    assert _variant() & B.SSN_KVAR_PLAIN
     expect = X.double() @ U.double()
     assert (got - expect).norm() <= bound * expect.norm()
