@@ -11,11 +11,13 @@
 //   warps 4-11       sums: of every stage, the four accumulators and the compensated running sum of 32 (or 16)
 //                    coordinates of a row per thread, all in registers.  The issuers take turns with two or four sets of accumulators.
 //
-// What bounds a stage: the stream alone takes 35 us at the size below (96 CTAs, one tile each), the hand-over of the
-// accumulators another 7; the additions of eight warps (~480 clocks a stage) and the basis take the rest.  In the split
-// kernel the warps that add also copied rows and basis through registers, and a tile was spread over four CTAs in three waves.
-// Before -> now, us: 12288 x 5120, rank 51, fp32 words 104 -> 67; 40000 x 1536, rank 27, bf16 rows 87 -> 50; 700 x 1024,
-// rank 19 11.3 -> 10.2.
+// What bounds it: no unit by itself.  A stage of 12288 x 5120, rank 51 takes a CTA 0.76 us; the stream alone would take 35 us in all
+// (96 CTAs, one tile each), its four MMAs take about 0.2 us, and without the additions, or without the loads of the basis,
+// the call takes 59.8 us instead of 63.6.  What is left is the hand-over: from the commit of a stage to the release of its
+// accumulators a sum warp reads them in eight rounds of two loads, and two sets of accumulators are in turn.
+// In the split kernel the warps that add also copied rows and basis through registers, and a tile was spread over four CTAs
+// in three waves.  us, split -> this kernel: 12288 x 5120, rank 51 103 -> 63.6; 40000 x 1536, rank 27 85 -> 41.5; 700 x 1024, rank 19
+// 10.7 -> 9.1 (fp32 words out).  Issuers that wait for their own stages only: 12288 x 5120, rank 32 45.9 -> 36.2.
 //
 // CAREFUL (see kSplitCarefulCols) adds the four accumulators one by one, with compensation: the same sums as the split kernel's.
 // 20000 x 320, rank 32: 4.1e-8 from 64-bit sums instead of 5.3e-8, 13.0 us instead of 12.0 (the split kernel 21).

@@ -63,8 +63,11 @@ cudaError_t launch_one(const SplitProjectArgs &a, int c, int sms, cudaStream_t s
   return launch_slices(kernel, Cfg::kThreads, Cfg::kSmemBytes, 0, a, c, sms, stream);
 }
 
-// The plain kernel's CTAs per tile.  A stage takes a CTA kPlainStageNs, or the time of the 16 KB that every CTA at work
-// takes from HBM, whichever is longer; a wave of clusters kPlainWaveNs besides.  Single CTAs are persistent.
+// The plain kernel's CTAs per tile, by a rough cost that orders the choices: a stage takes a CTA kPlainStageNs, or the time of
+// the 16 KB that every CTA at work takes from HBM, whichever is longer; a wave of clusters kPlainWaveNs besides.  Single CTAs are
+// persistent.  us with 1, 2, 3, ... CTAs, the chosen number in brackets: 100 x 2048, rank 27 19.1 14.2 12.2 11.6 10.7 [10.7] 10.6 10.5;
+// 3000 x 4096, rank 27 31.7 20.9 16.7 [15.4] 14.3 24.3; 9000 x 4096, rank 51 53.7 [36.1] 52.1 66.9; 5000 x 4096, rank 51 53.0 33.1 [27.3]
+// 45.3; 12288 x 5120, rank 51 [63.5] 76.2 84.2; 20000 x 2048, rank 51 [59.8] 68.4 75.0; it errs at 20000 x 4096, rank 27 58.7 62.1 [66.4].
 constexpr double kPlainStageNs = 260, kPlainHbmNs = 2.65, kPlainWaveNs = 4000;
 int plain_cluster_of(const SplitProjectArgs &a, int nst, int sms) {
   const int64_t units = units_of(a);
@@ -118,14 +121,19 @@ cudaError_t launch_slots(const SplitProjectArgs &a, int slots, int sms, cudaStre
   return launch_rank<T, 3>(a, sms, s);
 }
 
-// Above rank 32 the first and last rows of the basis, fetched half a word at a time, cost the plain kernel 3 us that wide rows
-// or many of them have to earn.  us, split -> plain: rank 51 1500 x 512 10.7 -> 13.8, x 1024 12.5 -> 14.4, x 2048
-// 15.8 -> 15.7, x 4096 20.0 -> 18.4; 9000 x 1024 20.9 -> 21.6, 16000 x 1024 34.9 -> 30.7, x 512 24.2 -> 25.3; rank 99 1500 x 2048
-// 18.5 -> 19.3, 3000 x 2048 30.5 -> 26.7.  Rank 27: 600 x 512 9.7 -> 9.8, 1500 x 1024 11.5 -> 10.3, 9000 x 4096 41 -> 27.
+// Where the plain kernel is the faster one, us, split -> plain.  One stage is too little for its set-up, and above rank 32 the
+// first and last rows of the basis, fetched half a word at a time, cost it 3 us that wide rows, or many, have to earn.
+//   rank 27: 16000 x 64 9.5 -> 10.2 (rank 8 7.5 -> 8.3, 20000 rows 9.1 -> 8.8), 40000 x 64 15.4 -> 14.8, 100 x 72 9.1 -> 8.9, 9000 x 128 9.8 -> 10.1, 20000 x 128 15.2 -> 12.2,
+//            3000 x 256 9.1 -> 9.4, 6000 x 256 11.3 -> 10.1, 100 x 640 10.5 -> 9.5, 9000 x 4096 41 -> 23; rank 32, the most of one
+//            group, 1500 x 256 9.0 -> 9.6
+//   rank 51: 9000 x 1024 20.4 -> 21.5, 16000 x 1024 31.9 -> 27.3, 100 x 2048 14.7 -> 14.9, 3000 x 2048 18.7 -> 18.9, 5000 x 2048
+//            23.9 -> 20.8, 1500 x 2304 16.9 -> 15.2, 100 x 4096 18.4 -> 17.0; rank 64 loses up to 2 us more
+//   rank 99: 2048 x 2048 19.2 -> 22.2, 3000 x 2048 29.9 -> 26.5, 2048 x 3072 24.6 -> 24.6, 1500 x 4096 26.2 -> 23.8
 bool plain_pays(const SplitProjectArgs &a) {
-  if (a.k <= 32) return true;
-  if (a.d >= 2048 && (a.k <= 64 || a.n >= 2048)) return true;
-  return a.d >= 1024 && a.n * a.d >= 16000LL * 1024;
+  const double size = (double)a.n * a.d;
+  if (a.k <= 32) return a.d > kUmmaCols || a.n >= 20000;
+  if (a.d >= 2048 && (a.k <= 64 || size >= 6e6)) return true;
+  return a.d >= 1024 && size >= 16000. * 1024;
 }
 
 bool rows16(const void *p, int64_t ld, int esz) {

@@ -37,9 +37,9 @@ def _variant():
     return variant
 
 
-# up to 32 coordinates any size; more of them only wide rows, or many
-NARROW = [(n, d, k) for n, d in [(1, 24), (1, 64), (127, 72), (129, 200), (700, 1000), (3000, 4096), (19100, 136)] for k in (1, 2, 31, 32)]
-WIDE = ([(n, d, k) for n, d in [(2100, 2056), (19100, 1032)] for k in (33, 51, 63, 64, 65, 99, 127, 128)]
+# up to 32 coordinates rows of more than one stage, or many; above that only wide rows, or many
+NARROW = [(n, d, k) for n, d in [(1, 72), (127, 72), (129, 200), (700, 1000), (3000, 4096), (19100, 136), (30001, 24)] for k in (1, 2, 31, 32)]
+WIDE = ([(n, d, k) for n, d in [(5000, 2056), (19100, 1032)] for k in (33, 51, 63, 64, 65, 99, 127, 128)]
         + [(3000, 4096, k) for k in (51, 64, 127)] + [(1, 2056, k) for k in (33, 64)])
 
 
@@ -56,9 +56,8 @@ def test_any_basis(n, d, k, excess, offset):
     codec.grad_project_wire(X, out=words.view(torch.float32)[:, :k])
     variant = _variant()
     assert variant & B.SSN_KVAR_PLAIN and bool(variant & B.SSN_KVAR_WIDE) == (k > 64)
-    # 150 tiles: several to a CTA; few tiles of wide rows: several CTAs to a tile
-    if n == 19100 or d >= 2056:
-        assert bool(variant & B.SSN_KVAR_ALT) == (n < 19100)
+    # 150 tiles and more, or 80 halves of tiles: single CTAs; fewer, of two stages or more: several CTAs to a tile
+    assert bool(variant & B.SSN_KVAR_ALT) == (n < 5000 or n == 5000 and k <= 64)
     assert_close(words.view(torch.float32)[:, :k].double().cpu().numpy(), expect, synth.F32, "words", tol=WORD_TOL)
     assert (words[:, k:] == -1).all()
     Z = codec.grad_project(X)
@@ -71,9 +70,10 @@ def test_any_basis(n, d, k, excess, offset):
     assert codec.take_status() == 0
 
 
-# clusters and single CTAs of both kernels for few and for many coordinates; the last two are the split kernel's
+# clusters and single CTAs of both kernels, for few and for many coordinates
 @pytest.mark.parametrize("n,d,k,plain,cluster", [(300, 256, 27, True, True), (20000, 256, 27, True, False), (300, 2048, 51, True, True),
-                                                 (20000, 1032, 64, True, False), (300, 256, 51, False, True), (20000, 256, 51, False, False)])
+                                                 (20000, 1032, 64, True, False), (300, 256, 51, False, True), (20000, 256, 51, False, False),
+                                                 (300, 64, 27, False, False)])
 def test_bad_rows(n, d, k, plain, cluster):
     X, U = _rand((n, d), 1), _inside_nan(_rand((d, k), 2, d ** -0.5), k + 1 + k % 2, 0)
     X[0, 5], X[129, 9], X[130, 9] = float("inf"), -float("inf"), float("nan")
