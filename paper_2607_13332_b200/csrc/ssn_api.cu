@@ -176,10 +176,12 @@ ssn_status_t launch_token_kernel(const TokenArgs &a, int32_t dtype, cudaStream_t
 inline int64_t coords_pitch(int32_t k) { return ((int64_t)k + 3) & ~3LL; }
 inline size_t coords_bytes(int64_t rows, int32_t k) { return (size_t)rows * (size_t)coords_pitch(k) * sizeof(float); }
 
-// D = (S U) U2^T of rows the fused kernels do not take (a.src and a.dst; fp32 storage, operands off the 16-byte grid).
+// D = (S U) U2^T of rows the fused kernels do not take (a.src and a.dst; fp32 storage, operands off the 16-byte grid, few rows,
+// odd widths).
 // With room for the fp32 coordinates and a rank that the split-operand kernels take it is a projection and an expansion on
 // the tensor cores; without it the general kernel.  us, general -> split: fp32 weights [2048 + 7168] x 2048 twice,
-// rank 40 1389 -> 239; bf16 ones, rank 51 packed 1482 -> 176; H [8192 x 7168] to 2048 columns, fp32 1633 -> 166.  fp32 results
+// rank 40 1389 -> 239; bf16 ones, rank 51 packed 1482 -> 176; H [8192 x 7168] to 2048 columns, fp32 1633 -> 166; bf16 on
+// the grid, H [400 x 14336] to 4096 columns, rank 40 922 -> 41, [256 x 512] to 512, rank 8 27 -> 17.  fp32 results
 // are closer to 64-bit sums too (1.9e-7 -> 1.0e-7).
 ssn_status_t project_then_expand(const TokenArgs &a, int32_t dtype, void *scratch, size_t scratch_bytes, cudaStream_t stream) {
   // The general kernel's time grows with the columns per pass of 32 coordinates, the two launches' hardly does: 512 rows x 64
